@@ -579,7 +579,6 @@ bool use_tc(const hopf_ctx* ctx, int m, int p) {
 hopf_status tc_reserve_bytes(hopf_ctx* ctx, size_t need) {
   if (need <= ctx->tcbytes) return HOPF_OK;
   dfree(ctx->tcbuf);
-  dfree(ctx->ev_idx); dfree(ctx->ev_vals); dfree(ctx->ev_out);
   ctx->tcbuf = nullptr;
   ctx->tcbytes = 0;
   CK(hk::dev_alloc(&ctx->tcbuf, need));
