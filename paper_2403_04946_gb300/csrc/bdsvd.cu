@@ -9,24 +9,35 @@
 //     upper bidiagonal, with the reflector conventions of LAPACK's zgebrd.
 //     One cooperative launch; CTA g keeps the rows r = g (mod G) of R in
 //     shared memory and the CTAs meet once per column (see gebrd_kernel).
-//  2. Singular values of B: eigenvalues of the Golub-Kahan tridiagonal T_GK
-//     (order 2n, zero diagonal, off-diagonals d_1, e_1, d_2, ..., d_n, whose
-//     eigenvalues are +-sigma) by Sturm-count multisection, one warp per
-//     value.  Counts are taken in double-float arithmetic (hi + lo FP32
-//     pair, ~2^-47 relative): a Sturm count is exact for a matrix whose
-//     entries are perturbed by a few units of the working precision, and
-//     the singular values of a bidiagonal move by a relative amount of the
-//     same order under such perturbations (Demmel & Kahan 1990), so every
-//     value, large or small, is found to a relative accuracy of ~1e-13.
-//  3. Left singular vectors of B for the kept values: inverse iteration on
-//     T_GK - sigma I (the eigenvector for +sigma is (v_1, u_1, ..., v_n,
-//     u_n)/sqrt 2), FP64, tridiagonal LU with partial pivoting, modified
-//     Gram-Schmidt inside clusters of close values (as in LAPACK's dstein).
-//     Kept values at the rounding-noise level of R get an orthonormal
-//     completion instead (their vectors are not determined by R).
+//  2. Singular values of B: eigenvalues sigma^2 of B B^T by counting with the
+//     differential qd transform of B B^T - x^2 I (Fernando & Parlett 1994),
+//     one CTA of 32 W threads per value and 32 W points per round of
+//     multisection.  Counts are taken in double-float arithmetic (hi + lo FP32
+//     pair, ~2^-45 relative): a count is exact for a bidiagonal whose entries
+//     are perturbed by a few units of the working precision, and the singular
+//     values of a bidiagonal move by a relative amount of the same order under
+//     such perturbations (Demmel & Kahan 1990), so every value above 2^-50 of
+//     the largest entry is found to a relative accuracy of ~1e-13; the ones
+//     below (FP64 rounding of the bidiagonalisation) to 2^-8 by Sturm counts
+//     of the Golub-Kahan tridiagonal T_GK (order 2n, zero diagonal,
+//     off-diagonals d_1, e_1, d_2, ..., d_n), whose pivots stay in FP32 range.
+//  3. Left singular vectors of B for the kept values: eigenvectors of B B^T
+//     by twisted factorisation (Dhillon & Parlett 2004): the stationary and
+//     the progressive differential qd transforms of B B^T - lambda I meet at
+//     the index where the residual is smallest, one Rayleigh-quotient
+//     correction of lambda, then again, FP64.  Every vector is computed by
+//     itself, all of them at once; their orthogonality error is the rounding
+//     over the relative gap of the values and is removed by two Newton-Schulz
+//     steps of the polar factor.  Only if values agree to ~1e-11 (repeated
+//     singular values) are all vectors computed again one cluster after
+//     another, by inverse iteration on T_GK with modified Gram-Schmidt inside
+//     clusters (as in LAPACK's dstein).  Kept values at the rounding-noise
+//     level of R get an orthonormal completion (their vectors are not
+//     determined by R).
 //  4. U = Q [u_1 .. u_rho] by applying the left reflectors.
 #include <algorithm>
 #include <cfloat>
+#include <utility>
 
 #include "kernels.h"
 
@@ -367,9 +378,9 @@ DV dfr df_of(double x) {
   return dfr{h, (float)(x - (double)h)};
 }
 
-// Prepare the scaled squared off-diagonals of T_GK: a_k = d[k/2] (k even),
-// e[k/2] (k odd), k < 2n-1; a2[k] = (a_k / amax)^2 as double-float;
-// info[0] = amax, info[1] = Gershgorin bound of T_GK / amax.
+// Prepare the scaled squares a2[2i] = (d_i / amax)^2, a2[2i+1] = (e_i / amax)^2
+// (the squared off-diagonals of T_GK in order) as double-float; info[0] = amax,
+// info[1] = Gershgorin bound of T_GK / amax (2n entries, the last one zero).
 __global__ void bd_prep_kernel(const double* __restrict__ d, const double* __restrict__ e, int n,
                                float2* __restrict__ a2, double* __restrict__ info) {
   __shared__ double red[32];
@@ -407,6 +418,8 @@ __global__ void bd_prep_kernel(const double* __restrict__ d, const double* __res
     for (int w = 0; w < nw; ++w) b = fmax(b, red[w]);
     info[0] = amax;
     info[1] = b * (1.0 + 1e-6) + 1e-30;
+    info[2] = 0.0;  // set when the vectors of nearly equal values need the clustered path
+    a2[N - 1] = make_float2(0.f, 0.f);
   }
 }
 
@@ -429,10 +442,118 @@ __device__ __forceinline__ int sturm_count_df(const float2* __restrict__ a2, int
   return cnt;
 }
 
-// One warp per value: sig[k] = k-th largest singular value of B.  The
+// a + b with an error of a few 2^-48 of the *result* (both parts summed
+// without error first), so that it also holds when the operands cancel: the
+// relative accuracy of the qd recurrence rests on it.
+DV dfr df_add_rel(dfr a, dfr b) {
+  const float s = a.h + b.h, sb = s - a.h;
+  const float se = (a.h - (s - sb)) + (b.h - sb);
+  const float t = a.l + b.l, tb = t - a.l;
+  const float te = (a.l - (t - tb)) + (b.l - tb);
+  const dfr v = df_quick(s, se + t);
+  return df_quick(v.h, te + v.l);
+}
+DV dfr df_mul(dfr a, dfr b) {
+  const float p = a.h * b.h;
+  return df_quick(p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h));
+}
+
+// Number of singular values below x (x >= 2^-50: x^2 and the pivots stay far
+// inside the FP32 range): negative pivots p_i of B B^T - x^2 I = L D L^T from
+// the top, in differential form: with q_i = d_i^2 and eps_i = e_i^2,
+//   s_1 = q_1 - x^2,  p_i = s_i + eps_i,  s_{i+1} = q_{i+1} (s_i / p_i) - x^2
+// (the quotient first: s_i q_{i+1} would leave the FP32 range).  Per row one
+// division, one product and two additions, against two divisions and two
+// additions in the two T_GK rows it replaces.
+__device__ __forceinline__ int qd_count_df(const float4* __restrict__ qe, int n, double x) {
+  const float pivmin = 1e-36f;
+  const dfr lam = df_of(x * x);
+  const dfr ml{-lam.h, -lam.l};
+  float4 cur = __ldg(qe);
+  dfr s = df_add_rel(dfr{cur.x, cur.y}, ml);
+  int cnt = 0;
+  for (int i = 0; i < n; ++i) {
+    const float4 nxt = __ldg(qe + (i + 1 < n ? i + 1 : i));
+    const dfr ep{cur.z, cur.w};
+    dfr p = df_add_rel(s, ep);
+    if (fabsf(p.h) < pivmin) {
+      p = dfr{p.h < 0.f ? -pivmin : pivmin, 0.f};
+      s = df_add_rel(p, dfr{-ep.h, -ep.l});
+    }
+    cnt += (p.h < 0.f);
+    s = df_add_rel(df_mul(df_div(s, p), dfr{nxt.x, nxt.y}), ml);
+    cur = nxt;
+  }
+  return cnt;
+}
+
+// One CTA of 32 W threads per value: sig[k] = k-th largest singular value of
+// B.  The bracket [lo, hi) keeps #{sigma < lo} < target <= #{sigma < hi} with
+// target = n - k; each round the threads count at 32 W interior points, the
+// first round's spaced geometrically from 2^-50, so that small values cost no
+// more rounds than large ones.  Bound: the latency of the count's dependent
+// chain (n rows of ~50 FP32 operations), times the rounds.  32 W points per
+// round cut the rounds to 7 (W = 4); W = 1 once n values of 4 warps would
+// queue for the issue slots instead of waiting for latency.  A value below
+// 2^-50 amax is rounding noise of the FP64 bidiagonalisation and is found to
+// 2^-8 relative by two rounds of T_GK counts.
+template <int W>
+__global__ void __launch_bounds__(32 * W)
+bd_sigma_kernel(const float2* __restrict__ a2, const double* __restrict__ info, int n, double* __restrict__ sig) {
+  const int P = 32 * W, t = threadIdx.x, k = blockIdx.x;
+  const double amax = info[0];
+  if (amax == 0.0) {
+    if (t == 0) sig[k] = 0.0;
+    return;
+  }
+  const int target = n - k;
+  const float4* qe = reinterpret_cast<const float4*>(a2);
+  const double bound = info[1], floor_hi = 0x1p-50;
+  double lo = floor_hi, hi = bound;
+  bool tiny = false;
+  {
+    // point 0 is the floor itself
+    const double step = log2(bound / floor_hi) / P;
+    auto at = [&](int j) { return floor_hi * exp2(step * j); };
+    const int first = __syncthreads_count(qd_count_df(qe, n, at(t)) < target);
+    if (first == 0) tiny = true;
+    else {
+      lo = at(first - 1);
+      if (first < P) hi = at(first);
+    }
+  }
+  if (tiny) {
+    const double base = 0x1p-106;
+    lo = 0.0;
+    hi = floor_hi;
+    for (int it = 0; it < 2; ++it) {
+      const double l0 = lo, h0 = hi;
+      auto at = [&](int j) {
+        return it == 0 ? base * exp2(56.0 / P * j) : l0 + (h0 - l0) * (double)(j + 1) * (1.0 / (P + 1));
+      };
+      const int first = __syncthreads_count(sturm_count_df(a2, 2 * n, at(t)) - n < target);
+      if (first > 0) lo = at(first - 1);
+      if (first < P) hi = at(first);
+      if (lo == 0.0) break;  // below 2^-106
+    }
+  } else {
+    for (int it = 0; it < 24; ++it) {
+      if (hi - lo <= 0x1p-42 * hi) break;
+      const double l0 = lo, h0 = hi;
+      auto at = [&](int j) { return l0 + (h0 - l0) * (double)(j + 1) * (1.0 / (P + 1)); };
+      const int first = __syncthreads_count(qd_count_df(qe, n, at(t)) < target);
+      if (first > 0) lo = at(first - 1);
+      if (first < P) hi = at(first);
+    }
+  }
+  if (t == 0) sig[k] = 0.5 * (lo + hi) * amax;
+}
+
+// The mixed path's values (see bd_invit_kernel): one warp per value on T_GK,
+// sig[k] = k-th largest singular value of B.  The
 // bracket [lo, hi) keeps #{sigma < lo} < target <= #{sigma < hi} with
 // target = n - k; each round the lanes count at 32 interior points.
-__global__ void bd_sigma_kernel(const float2* __restrict__ a2, const double* __restrict__ info, int n,
+__global__ void bd_sigma_gk_kernel(const float2* __restrict__ a2, const double* __restrict__ info, int n,
                                 double* __restrict__ sig) {
   const int lane = threadIdx.x & 31;
   const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -459,13 +580,14 @@ __global__ void bd_sigma_kernel(const float2* __restrict__ a2, const double* __r
 }
 
 cudaError_t bd_sigma(const double* d, const double* e, int n, float2* a2, double* info, double* sig,
-                     cudaStream_t s) {
+                     int mixed, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   bd_prep_kernel<<<1, 256, 0, s>>>(d, e, n, a2, info);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  const int warps = 4;
-  bd_sigma_kernel<<<(n + warps - 1) / warps, 32 * warps, 0, s>>>(a2, info, n, sig);
+  if (mixed) bd_sigma_gk_kernel<<<(n + 3) / 4, 128, 0, s>>>(a2, info, n, sig);
+  else if (n <= 512) bd_sigma_kernel<4><<<n, 128, 0, s>>>(a2, info, n, sig);
+  else bd_sigma_kernel<1><<<n, 32, 0, s>>>(a2, info, n, sig);
   return cudaGetLastError();
 }
 // Rank rule on the sorted values (the same rule as rank_select), one CTA:
@@ -545,6 +667,9 @@ DV double hash_unit(unsigned a, unsigned b) {
   h ^= h >> 15;
   return (double)(h & 0xFFFFFFu) * (1.0 / 16777216.0) - 0.5;
 }
+
+// Entry i of the start vector of inverse iteration for value k.
+DV double start_value(int i, int k) { return 1.0 + 0.25 * hash_unit((unsigned)i, (unsigned)k); }
 
 // Solver arrays of T_GK - lam I (length N each) in shared memory, and the
 // scaled off-diagonals (staged once per launch).
@@ -628,19 +753,203 @@ DV void gk_solve(int N, double* w) {
   }
 }
 
-// One warp per cluster of kept values (consecutive values closer than
-// 1e-3 sigma_max): inverse iteration for each member, re-orthogonalised
+// Reciprocal to FP64 rounding level: the hardware's 20-bit seed and one
+// third-order step of Householder's iteration, y (1 + e + e^2) with
+// e = 1 - x y (error e^3).  The serial chains below wait on one of these per
+// row: about 230 cycles of dependent operations against 640 measured for the
+// IEEE division.  |x| in [1e-150, 1e150] here (pivots are clamped).
+DV double rcp_fast(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// One warp per kept value: left vector u_k of B as the eigenvector of B B^T
+// by twisted factorisation.  With q_i = d_i^2, eps_i = e_i^2 (scaled by
+// 1 / amax^2) and lambda = (sig_k / amax)^2, lane 0 runs
+//   s_1 = q_1 - lambda, p_i = s_i + eps_i, s_{i+1} = q_{i+1} s_i / p_i - lambda
+// from the top while lane 1 runs
+//   t_n = -lambda, r_i = q_i + t_i, t_{i-1} = eps_{i-1} t_i / r_i - lambda
+// from the bottom; gamma_i = s_i + t_i + lambda is the residual of the vector
+// that solves every equation but row i, and the row where it is smallest
+// starts the two products z_{i} = -(d_{i+1} e_i / p_i) z_{i+1} upwards and
+// z_{i+1} = -(d_{i+1} e_i / r_{i+1}) z_i downwards.  lambda + gamma / |z|^2 is
+// the Rayleigh quotient: one correction brings the multisection's 2^-42 to
+// rounding level.  Bound by the latency of the FP64 chain, two sweeps of n
+// rows of one reciprocal and three dependent operations.  The serial form it
+// replaces (one warp per cluster, LU with pivoting and three solves of 2n
+// rows per vector, one vector after another in a cluster) needed 14.3 ms per
+// factor at n = 384 and 64 kept values when the values decay.
+enum { V_Q = 0, V_EP = 1, V_OFF = 2, V_S = 3, V_T = 4, V_P = 5, V_R = 6, V_Z = 7 };
+constexpr int kVecArrays = 8;
+
+__global__ void __launch_bounds__(32)
+bd_vectors_kernel(const double* __restrict__ d, const double* __restrict__ e, int n,
+                  const double* __restrict__ info, const double* __restrict__ sig, double* __restrict__ X,
+                  int ldx) {
+  extern __shared__ __align__(16) double vsm[];
+  const int k = blockIdx.x, lane = threadIdx.x;
+  const double amax = info[0];
+  if (amax == 0.0) return;
+  const double inv = 1.0 / amax;
+  double *Q = vsm + V_Q * n, *EP = vsm + V_EP * n, *OFF = vsm + V_OFF * n, *Sv = vsm + V_S * n, *Tv = vsm + V_T * n,
+         *Pi = vsm + V_P * n, *Ri = vsm + V_R * n, *Z = vsm + V_Z * n;
+  for (int i = lane; i < n; i += 32) {
+    const double di = d[i] * inv, ei = (i + 1 < n) ? e[i] * inv : 0.0;
+    Q[i] = di * di;
+    EP[i] = ei * ei;
+    OFF[i] = (i + 1 < n) ? d[i + 1] * inv * ei : 0.0;
+  }
+  __syncwarp();
+  double lam = sig[k] * inv;
+  lam *= lam;
+  const double tiny = 1e-150;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (lane < 2) {
+      const bool up = lane == 1;  // lane 1 walks from the bottom
+      double v = up ? -lam : Q[0] - lam;
+      double* V = up ? Tv : Sv;
+      double* C = up ? Ri : Pi;
+      int i = up ? n - 1 : 0;
+      const int di = up ? -1 : 1;
+      double add = up ? Q[i] : EP[i];
+      for (int step = 0; step < n; ++step) {
+        // the next row's inputs are loaded ahead of the chain
+        const int in = (step + 1 < n) ? i + di : i;
+        const double mul = up ? EP[in] : Q[in];
+        const double addn = up ? Q[in] : EP[in];
+        double piv = v + add;
+        if (fabs(piv) < tiny) {
+          piv = piv < 0.0 ? -tiny : tiny;
+          v = piv - add;
+        }
+        V[i] = v;
+        const double vm = v * mul;
+        const double rc = rcp_fast(piv);
+        C[i] = rc;
+        v = fma(vm, rc, -lam);
+        add = addn;
+        i = in;
+      }
+    }
+    __syncwarp();
+    // twist row: smallest |gamma|
+    double best = 1e300;
+    int tw = 0;
+    for (int i = lane; i < n; i += 32) {
+      const double g = fabs(Sv[i] + Tv[i] + lam);
+      if (g < best) {
+        best = g;
+        tw = i;
+      }
+    }
+    for (int o = 16; o >= 1; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int ot = __shfl_xor_sync(0xffffffffu, tw, o);
+      if (ob < best || (ob == best && ot < tw)) {
+        best = ob;
+        tw = ot;
+      }
+    }
+    const double gam = Sv[tw] + Tv[tw] + lam;
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+      Pi[i] *= -OFF[i];
+      if (i > 0) Ri[i] *= -OFF[i - 1];
+    }
+    __syncwarp();
+    if (lane < 2) {
+      double v = 1.0;
+      if (lane == 0) {
+        Z[tw] = 1.0;
+        for (int i = tw - 1; i >= 0; --i) {
+          v *= Pi[i];
+          Z[i] = v;
+        }
+      } else {
+        for (int i = tw + 1; i < n; ++i) {
+          v *= Ri[i];
+          Z[i] = v;
+        }
+      }
+    }
+    __syncwarp();
+    double nrm = 0.0;
+    for (int i = lane; i < n; i += 32) nrm = fma(Z[i], Z[i], nrm);
+    nrm = warp_sum(nrm);
+    if (pass == 0) {
+      const double corr = gam / nrm;
+      if (fabs(corr) <= 1e-9 * lam) lam += corr;
+    } else {
+      const double s = 1.0 / sqrt(nrm);
+      for (int i = lane; i < n; i += 32) X[i + (size_t)ldx * k] = Z[i] * s;
+    }
+  }
+}
+
+// One Newton-Schulz step towards the polar factor of X (n x k, columns of
+// norm one and nearly orthogonal): X_out = X + X (I - X^T X) / 2, whose
+// orthogonality error is 3/4 of the square of X's; the columns' span is
+// unchanged.  One CTA per column: its k dot products, then its row of the
+// update.  The first step sets info[2] when a pair of columns is not even
+// orthogonal to 1e-4 (values equal to ~1e-11): the clustered path then
+// computes all vectors again.
+constexpr int kOrthThreads = 256;
+__global__ void __launch_bounds__(kOrthThreads)
+bd_orth_kernel(int n, int k, const double* __restrict__ X, int ldx, double* __restrict__ Xo, int ldo,
+               double* __restrict__ info, int check) {
+  extern __shared__ __align__(16) double osm[];  // column j [n], e_j [k]
+  double* xj = osm;
+  double* ej = osm + n;
+  const int j = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kOrthThreads >> 5;
+  for (int i = threadIdx.x; i < n; i += kOrthThreads) xj[i] = X[i + (size_t)ldx * j];
+  __syncthreads();
+  // two columns at a time per warp: independent chains
+  for (int c = 2 * wid; c < k; c += 2 * nw) {
+    const bool two = c + 1 < k;
+    const double *a = X + (size_t)ldx * c, *b = X + (size_t)ldx * (two ? c + 1 : c);
+    double s0 = 0.0, s1 = 0.0;
+    for (int i = lane; i < n; i += 32) {
+      s0 = fma(a[i], xj[i], s0);
+      s1 = fma(b[i], xj[i], s1);
+    }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    if (lane < 2 && c + lane < k) {
+      const double g = lane ? s1 : s0;
+      const double ee = (c + lane == j) ? 1.0 - g : -g;
+      ej[c + lane] = 0.5 * ee;
+      if (check && !(fabs(ee) <= 1e-4)) info[2] = 1.0;  // also for NaN
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += kOrthThreads) {
+    double v0 = 0.0, v1 = 0.0;
+    int c = 0;
+    for (; c + 1 < k; c += 2) {
+      v0 = fma(X[i + (size_t)ldx * c], ej[c], v0);
+      v1 = fma(X[i + (size_t)ldx * (c + 1)], ej[c + 1], v1);
+    }
+    if (c < k) v0 = fma(X[i + (size_t)ldx * c], ej[c], v0);
+    Xo[i + (size_t)ldo * j] = xj[i] + (v0 + v1);
+  }
+}
+
+// The path for repeated values (runs when bd_orth_kernel has set info[2]): one
+// warp per cluster of kept values (consecutive values closer than 1e-3
+// sigma_max): inverse iteration for each member, re-orthogonalised
 // against the members before it.  Lane 0 runs the tridiagonal recurrences
 // out of shared memory; the warp does the products and norms.  X (n x
 // nvec, ldx) receives the normalised left vectors u_k.  Every k < nvec is
 // above the noise level (the caller passes the count of such values).
-__global__ void bd_vectors_kernel(const double* __restrict__ d, const double* __restrict__ e, int n,
+__global__ void bd_cluster_kernel(const double* __restrict__ d, const double* __restrict__ e, int n,
                                   const double* __restrict__ info, const double* __restrict__ sig,
                                   int nvec, double* __restrict__ X, int ldx, double* __restrict__ Zs) {
   extern __shared__ __align__(16) double vsm[];  // kSolveArrays * N
   const int k0 = blockIdx.x, lane = threadIdx.x;
   const int N = 2 * n;
-  if (k0 >= nvec) return;
+  if (k0 >= nvec || info[2] == 0.0) return;
   const double amax = info[0];
   if (amax == 0.0) return;
   const double gap_tol = 1e-3 * sig[0];
@@ -654,7 +963,7 @@ __global__ void bd_vectors_kernel(const double* __restrict__ d, const double* __
   __syncwarp();
   for (int k = k0; k < k1; ++k) {
     if (lane == 0) gk_factor(N, sig[k] * inv, vsm);
-    for (int i = lane; i < N; i += 32) B[i] = 1.0 + 0.25 * hash_unit((unsigned)i, (unsigned)k);
+    for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
     __syncwarp();
     for (int it = 0; it < 3; ++it) {
       if (lane == 0) gk_solve(N, vsm);
@@ -686,6 +995,97 @@ __global__ void bd_vectors_kernel(const double* __restrict__ d, const double* __
     for (int i = lane; i < n; i += 32) X[i + (size_t)ldx * k] = B[2 * i + 1] * s;
     __syncwarp();
   }
+}
+
+// ---- vectors of the mixed path ------------------------------------------------
+// The digit products cut U at 2^-40 of its largest entry, about the 1e-12 by
+// which a vector in a cluster of values (gaps below 1e-3 sigma_max) moves with
+// the rounding of its computation, so another method shows in the mixed
+// path's results at 1e-2 of their error (1e-9 of a covariance).  Here the
+// vectors stay those of three steps of inverse iteration on T_GK - lambda I
+// with Gram-Schmidt inside clusters, at the T_GK values, but all of them at
+// once: the LU factors and the solves of every value are independent, and
+// since each step leaves the vectors orthogonal to about 1e-9 already,
+// Gram-Schmidt in order is its first-order form
+//   z_k <- z_k (1 - (g_kk - 1) / 2) - sum_{j < k, same cluster} g_jk z_j
+// with g the Gram before the step.  One serial warp per cluster took 14.3 ms
+// per factor on average at n = 384 (up to 43 ms).  Values so close that a
+// step leaves 1e-4 or more set info[2]: the serial kernel then runs.
+// lu: per value the five factor arrays (5 N); Z: N per value.
+__global__ void __launch_bounds__(32)
+bd_invit_kernel(const double* __restrict__ d, const double* __restrict__ e, int n, const double* __restrict__ info,
+                const double* __restrict__ sig, int first, double* __restrict__ lu, double* __restrict__ Z) {
+  extern __shared__ __align__(16) double vsm[];  // kSolveArrays * N
+  const int k = blockIdx.x, lane = threadIdx.x, N = 2 * n;
+  const double amax = info[0];
+  if (amax == 0.0) return;
+  double* B = vsm + L_B * N;
+  double* f = lu + (size_t)k * 5 * N;
+  double* z = Z + (size_t)k * N;
+  if (first) {
+    const double inv = 1.0 / amax;
+    double* off = vsm + L_OFF * N;
+    for (int i = lane; i < N - 1; i += 32) off[i] = ((i & 1) ? e[i >> 1] : d[i >> 1]) * inv;
+    __syncwarp();
+    if (lane == 0) gk_factor(N, sig[k] * inv, vsm);
+    for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
+    __syncwarp();
+    // (the last rows of C1, C2, DL, PV are never written or read)
+    for (int i = lane; i < 5 * N; i += 32)
+      if (i < N || i % N < N - 1) f[i] = vsm[i];
+  } else {
+    for (int i = lane; i < 5 * N; i += 32)
+      if (i < N || i % N < N - 1) vsm[i] = f[i];
+    for (int i = lane; i < N; i += 32) B[i] = z[i];
+    __syncwarp();
+  }
+  if (lane == 0) gk_solve(N, vsm);
+  __syncwarp();
+  double nrm = 0.0;
+  for (int i = lane; i < N; i += 32) nrm += B[i] * B[i];
+  nrm = warp_sum(nrm);
+  const double s = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
+  for (int i = lane; i < N; i += 32) z[i] = B[i] * s;
+}
+
+// The ordered Gram-Schmidt step, one CTA per vector; with X, the result is
+// the normalised left part (entries 1, 3, ..) instead.
+__global__ void __launch_bounds__(kOrthThreads)
+bd_gs_kernel(int n, const double* __restrict__ sig, const double* __restrict__ Z, double* __restrict__ Zo,
+             double* __restrict__ X, int ldx, double* __restrict__ info) {
+  extern __shared__ __align__(16) double osm[];  // z_k [N], g [k + 1]
+  __shared__ double red[32];
+  const int N = 2 * n, k = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kOrthThreads >> 5;
+  double *zk = osm, *g = osm + N;
+  for (int i = threadIdx.x; i < N; i += kOrthThreads) zk[i] = Z[(size_t)k * N + i];
+  const double gap_tol = 1e-3 * sig[0];
+  int k0 = k;  // first member of the cluster
+  while (k0 > 0 && sig[k0 - 1] - sig[k0] < gap_tol) --k0;
+  __syncthreads();
+  for (int j = k0 + wid; j <= k; j += nw) {
+    const double* zj = Z + (size_t)j * N;
+    double s = 0.0;
+    for (int i = lane; i < N; i += 32) s = fma(zj[i], zk[i], s);
+    s = warp_sum(s);
+    if (lane == 0) {
+      g[j - k0] = (j == k) ? 0.5 * (s - 1.0) : s;
+      if (!(fabs(j == k ? s - 1.0 : s) <= 1e-4)) info[2] = 1.0;
+    }
+  }
+  __syncthreads();
+  double un = 0.0;
+  for (int i = threadIdx.x; i < N; i += kOrthThreads) {
+    double v = 0.0;
+    for (int j = k0; j <= k; ++j) v = fma(Z[(size_t)j * N + i], g[j - k0], v);
+    v = zk[i] - v;
+    if (!X) Zo[(size_t)k * N + i] = v;
+    else if (i & 1) un = fma(v, v, un);
+    if (X) zk[i] = v;
+  }
+  if (!X) return;
+  un = block_sum(un, red);
+  const double s = un > 0.0 ? 1.0 / sqrt(un) : 0.0;
+  for (int i = threadIdx.x; i < n; i += kOrthThreads) X[i + (size_t)ldx * k] = zk[2 * i + 1] * s;
 }
 
 // Orthonormal completion for kept values at the noise level (indices
@@ -725,14 +1125,34 @@ __global__ void bd_complete_kernel(int n, int kt, int nvec, double* __restrict__
 }
 
 
-cudaError_t bd_vectors(const double* d, const double* e, int n, const double* info, const double* sig,
-                       int kt, int nvec, double* X, int ldx, double* Zs, cudaStream_t s) {
+size_t bd_lu_elems(int n, int kt) { return (size_t)14 * n * kt; }
+
+cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, const double* sig,
+                       int kt, int nvec, double* X, int ldx, double* Zs, double* lu, cudaStream_t s) {
+  const bool mixed = lu != nullptr;
   if (nvec <= 0) return cudaSuccess;
   if (kt > 0) {
-    const size_t smem = bd_vectors_smem(n);
-    cudaError_t err = allow_smem((const void*)bd_vectors_kernel, smem);
+    const size_t vsmem = sizeof(double) * kVecArrays * (size_t)n, csmem = bd_vectors_smem(n);
+    const size_t osmem = sizeof(double) * ((mixed ? 2 : 1) * (size_t)n + kt);
+    cudaError_t err = allow_smem(mixed ? (const void*)bd_gs_kernel : (const void*)bd_orth_kernel, osmem);
+    if (err == cudaSuccess) err = allow_smem((const void*)bd_cluster_kernel, csmem);
+    if (err == cudaSuccess)
+      err = mixed ? allow_smem((const void*)bd_invit_kernel, csmem) : allow_smem((const void*)bd_vectors_kernel, vsmem);
     if (err != cudaSuccess) return err;
-    bd_vectors_kernel<<<kt, 32, smem, s>>>(d, e, n, info, sig, kt, X, ldx, Zs);
+    if (mixed) {
+      const size_t nz = (size_t)2 * n * kt;
+      double *Z = lu + 5 * nz, *Zo = Z + nz;
+      for (int it = 0; it < 3; ++it) {
+        bd_invit_kernel<<<kt, 32, csmem, s>>>(d, e, n, info, sig, it == 0, lu, Z);
+        bd_gs_kernel<<<kt, kOrthThreads, osmem, s>>>(n, sig, Z, Zo, it == 2 ? X : nullptr, ldx, info);
+        std::swap(Z, Zo);
+      }
+    } else {
+      bd_vectors_kernel<<<kt, 32, vsmem, s>>>(d, e, n, info, sig, X, ldx);
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, 1);
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, 0);
+    }
+    bd_cluster_kernel<<<kt, 32, csmem, s>>>(d, e, n, info, sig, kt, X, ldx, Zs);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }

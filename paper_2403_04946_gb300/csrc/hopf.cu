@@ -57,6 +57,8 @@ struct RoundWs {
   double* bd_info = nullptr;  // 4
   double* bd_X = nullptr;     // kcap * kcap
   double* bd_Zs = nullptr;    // kcap * 2 kcap
+  double* bd_lu = nullptr;    // mixed: factors of the inverse iteration, grown on demand
+  size_t bd_lu_elems = 0;
   // mixed precision, tensor-core QR: per core the Gram blocks of the
   // phase-1 reflectors (gstride elements each), and those of phase 2's QR
   cplx* G = nullptr;
@@ -431,7 +433,7 @@ hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
   dfree(w.Rb); dfree(w.Mb); dfree(w.Jb); dfree(w.Ub); dfree(w.Sb);
   dfree(w.sig); dfree(w.perm);
   dfree(w.bd_d); dfree(w.bd_e); dfree(w.bd_tauq); dfree(w.bd_taup); dfree(w.bd_a2);
-  dfree(w.bd_info); dfree(w.bd_X); dfree(w.bd_Zs);
+  dfree(w.bd_info); dfree(w.bd_X); dfree(w.bd_Zs); dfree(w.bd_lu);
   dfree(w.G); dfree(w.G2); dfree(w.bd_rows);
   w = RoundWs{};
   const size_t elems = std::max(need, w.elems);
@@ -468,6 +470,17 @@ hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
   w.d = d;
   w.kcap = K;
   return coop_reserve(ctx, K);
+}
+
+hopf_status bd_lu_reserve(hopf_ctx* ctx, size_t elems) {
+  RoundWs& w = ctx->rw;
+  if (elems <= w.bd_lu_elems) return HOPF_OK;
+  dfree(w.bd_lu);
+  w.bd_lu = nullptr;
+  w.bd_lu_elems = 0;
+  CK(dalloc(&w.bd_lu, elems));
+  w.bd_lu_elems = elems;
+  return HOPF_OK;
 }
 
 hopf_status tt_alloc(hopf_ctx* ctx, int cap_rank, hopf_tt** out) {
@@ -893,7 +906,7 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Jb, pp, pp, pp, w.Mb, pp, ctx->stream));
       }
       LAUNCH(HOPF_K_SVD, gebrd_flops(pp), 0, 1, hk::gebrd(w.Mb, pp, pp, w.bd_d, w.bd_e, w.bd_tauq, w.bd_taup, ctx->coop, ctx->stream, w.bd_rows));
-      LAUNCH(HOPF_K_SVD, 0, 0, 2, hk::bd_sigma(w.bd_d, w.bd_e, pp, w.bd_a2, w.bd_info, w.sig, ctx->stream));
+      LAUNCH(HOPF_K_SVD, 0, 0, 2, hk::bd_sigma(w.bd_d, w.bd_e, pp, w.bd_a2, w.bd_info, w.sig, MIXED_FLAG, ctx->stream));
       LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::bd_rank(w.sig, pp, ctx->d_dbl + 1, cap, forced_c, ctx->d_int, ctx->d_dbl + 2, w.sig + pp, ctx->stream));
       TRY(read_small_checked(ctx, 3, 5));
       ctx->prof.svd_count += 1;
@@ -936,7 +949,8 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
     // new core c = Q [U_rho; 0]
     if (use_bd) {
       const int kt = std::min(ctx->h_int[2], rnew);
-      LAUNCH(HOPF_K_SVD, 0, 0, (kt > 0) + (kt < rnew), hk::bd_vectors(w.bd_d, w.bd_e, pp, w.bd_info, w.sig, kt, rnew, w.bd_X, pp, w.bd_Zs, ctx->stream));
+      if (MIXED_FLAG) TRY(bd_lu_reserve(ctx, hk::bd_lu_elems(pp, kt)));
+      LAUNCH(HOPF_K_SVD, 0, 0, (kt > 0 ? 4 + 3 * MIXED_FLAG : 0) + (kt < rnew), hk::bd_vectors(w.bd_d, w.bd_e, pp, w.bd_info, w.sig, kt, rnew, w.bd_X, pp, w.bd_Zs, MIXED_FLAG ? w.bd_lu : nullptr, ctx->stream));
       LAUNCH(HOPF_K_SVD, 0, 0, 1, hk::bd_back(w.Mb, pp, w.bd_tauq, pp, w.bd_X, pp, rnew, w.Ub, pp, t->cores[c], Mrows, Mrows, ctx->stream));
     } else if (case1) {
       LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::gather_u(w.Mb, pp, pp, w.perm, w.sig, 1, rnew, t->cores[c], Mrows, Mrows, w.Ub, pp, ctx->stream));
@@ -1472,7 +1486,7 @@ void hopf_destroy(hopf_ctx* ctx) {
   dfree(w.Rb); dfree(w.Mb); dfree(w.Jb); dfree(w.Ub); dfree(w.Sb);
   dfree(w.sig); dfree(w.perm);
   dfree(w.bd_d); dfree(w.bd_e); dfree(w.bd_tauq); dfree(w.bd_taup); dfree(w.bd_a2);
-  dfree(w.bd_info); dfree(w.bd_X); dfree(w.bd_Zs);
+  dfree(w.bd_info); dfree(w.bd_X); dfree(w.bd_Zs); dfree(w.bd_lu);
   dfree(w.G); dfree(w.G2); dfree(w.bd_rows);
   dfree(ctx->tcbuf);
   dfree(ctx->ev_idx); dfree(ctx->ev_vals); dfree(ctx->ev_out);

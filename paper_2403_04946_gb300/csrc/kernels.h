@@ -91,19 +91,22 @@ cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cpl
 bool gebrd_fits(int n, const CoopWs& ws, bool have_rows_ws = false);
 size_t gebrd_rows_elems(int n, int sms);
 // All singular values of B, sorted descending, into sig[n]; a2 (float2
-// [2n]) and info (double [4]) are scratch kept for bd_vectors.
+// [2n]) and info (double [4]) are scratch kept for bd_vectors.  mixed: the
+// values of the mixed path, see bd_invit_kernel.
 cudaError_t bd_sigma(const double* d, const double* e, int n, float2* a2, double* info, double* sig,
-                     cudaStream_t s);
+                     int mixed, cudaStream_t s);
 // Rank rule on sorted values: out_int[0] = rho, [1] = rho by tolerance,
 // [2] = number of kept values above the noise level 2 n eps ||B||_F;
 // out_dbl as rank_select; tail2[n+1] scratch.
 cudaError_t bd_rank(const double* sig, int n, const double* eps_hat, int cap, int forced, int* out_int,
                     double* out_dbl, double* tail2, cudaStream_t s);
-// Left singular vectors of B: columns k < kt by inverse iteration, columns
+// Left singular vectors of B: columns k < kt by twisted factorisation, columns
 // kt..nvec-1 by orthonormal completion; X (n x nvec, ldx), real.
-// Zs: nvec x 2n doubles of scratch (the T_GK eigenvectors).
-cudaError_t bd_vectors(const double* d, const double* e, int n, const double* info, const double* sig,
-                       int kt, int nvec, double* X, int ldx, double* Zs, cudaStream_t s);
+// Zs: nvec x 2n doubles of scratch; lu (NULL in FP64): bd_lu_elems(n, kt)
+// doubles for the mixed path's inverse iteration.
+size_t bd_lu_elems(int n, int kt);
+cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, const double* sig,
+                       int kt, int nvec, double* X, int ldx, double* Zs, double* lu, cudaStream_t s);
 // U = Q X -> U (n x nvec, ldu) and Xp (mrows x nvec, ldp, zero below row n).
 cudaError_t bd_back(const cplx* A, int lda, const cplx* tauq, int n, const double* X, int ldx, int nvec,
                     cplx* U, int ldu, cplx* Xp, int ldp, int mrows, cudaStream_t s);
