@@ -180,8 +180,7 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     if (tid == 0) pr[g] = sq;
     if (owner)
       for (int c = i + tid; c < n; c += blockDim.x) rowb[c] = R(i / G, c);
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // (b1) left reflector of column i (every CTA), reduction of its columns
     if (wid == 0) {
       const double s2 = warp_sum(sum_published(pr, G));
@@ -207,8 +206,7 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
         nrg[c] = csub(a_ic, f);
       }
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // (b2) left update of own rows r > i: A[r,c] -= v_r conj(tau) w_c;
     // column i keeps v_r
     for (int lr = lr0 + tid; lr < nact; lr += blockDim.x) vloc[lr] = cmul(R(lr, i), scq);

@@ -232,8 +232,8 @@ struct GridBar {
 // k * gridDim, so no CTA has to reset anything between barriers (one atomic
 // and one polled load per CTA per barrier).  Every wait is bounded: after
 // kBarrierTimeoutNs of wall time (or the context's limit_us) the CTA records
-// the expiry in err and leaves; callers check grid_failed() and return
-// early.
+// the expiry in err, and every CTA of the launch leaves (grid_sync returns
+// true).
 constexpr uint64_t kBarrierTimeoutNs = 4000000000ull;  // 4 s
 
 struct GridSync {
@@ -255,35 +255,44 @@ DV unsigned int ld_acquire_gpu(const unsigned int* p) {
   return v;
 }
 
-DV void grid_sync(GridSync& gs) {
+// Set in the arrival counter by an expired wait (a launch counts far below).
+constexpr unsigned int kBarFail = 0x80000000u;
+
+// Returns true if a wait expired (to every thread of the CTA: all leave).
+// The expiry travels in the arrival counter itself, so that a column of a
+// factorisation waits for one L2 round trip after the last arrival and no
+// more: reading the err record before arriving and after leaving cost two
+// further round trips per barrier.  err is read once per launch (an expiry of
+// an earlier one still ends the later ones at once).
+DV bool grid_sync(GridSync& gs) {
   __syncthreads();
+  int failed = 0;
   if (threadIdx.x == 0) {
-    volatile int* verr = &gs.bar->err;
+    unsigned int* cnt = &gs.bar->count;
+    const bool first = gs.target == 0u;
     gs.target += gridDim.x * gridDim.y * gridDim.z;
-    if (*verr == 0) {
-      bar_arrive_release(&gs.bar->count);
-      const unsigned int lim = *((volatile unsigned int*)&gs.bar->limit_us);
-      const uint64_t limit_ns = lim ? (uint64_t)lim * 1000ull : kBarrierTimeoutNs;
-      uint64_t t0 = 0;
-      unsigned int spins = 0;
-      while ((int)(ld_acquire_gpu(&gs.bar->count) - gs.target) < 0) {
-        if (((++spins) & 31u) == 0u) {
-          if (*verr != 0) break;
-          const uint64_t now = global_ns();
-          if (t0 == 0) {
-            t0 = now;
-          } else if (now - t0 > limit_ns) {
-            atomicExch(&gs.bar->err, 1);
-            break;
-          }
+    bar_arrive_release(cnt);
+    if (first && *((volatile int*)&gs.bar->err) != 0) failed = 1;
+    uint64_t t0 = 0, limit_ns = 0;
+    for (unsigned int spins = 1; !failed; ++spins) {
+      const unsigned int v = ld_acquire_gpu(cnt);
+      if (v & kBarFail) failed = 1;
+      else if (v >= gs.target) break;
+      else if ((spins & 31u) == 0u) {
+        const uint64_t now = global_ns();
+        if (t0 == 0) {
+          const unsigned int lim = *((volatile unsigned int*)&gs.bar->limit_us);
+          limit_ns = lim ? (uint64_t)lim * 1000ull : kBarrierTimeoutNs;
+          t0 = now;
+        } else if (now - t0 > limit_ns) {
+          atomicExch(&gs.bar->err, 1);
+          atomicOr(cnt, kBarFail);
+          failed = 1;
+        } else {
+          __nanosleep(32);
         }
-        __nanosleep(32);
       }
     }
   }
-  __syncthreads();
-}
-
-DV bool grid_failed(const GridBar* bar) {
-  return *((volatile const int*)&bar->err) != 0;
+  return __syncthreads_or(failed) != 0;
 }

@@ -148,8 +148,7 @@ cross_pivots_kernel(const cplx* __restrict__ A, int M, int c, int R, double rel_
         }
       cand[g] = mk(b, (double)ee);  // flat index < 2^53: exact in a double
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     if (tid == 0) {
       double b = -1.0;
       long long ee = 0;

@@ -10,6 +10,7 @@
 // trailing update (three per panel of width nb).  Reductions over CTAs are
 // done in a fixed order, so results are bitwise reproducible.
 #include <algorithm>
+#include <climits>
 
 #include "kernels.h"
 
@@ -264,9 +265,11 @@ __device__ void rows_to_fp64(cplx* A, int lda, int r0, int r1, int c0, int c1, i
 
 // Power-of-two exponent E with max |entry| * 2^-E < 1 over rows [r0, r1) of
 // columns [0, k) of every CTA: one grid barrier; the per-CTA maxima go to
-// slot[0..G).  Returns E (0 for an all-zero matrix).
+// slot[0..G).  Returns E (0 for an all-zero matrix), kScaleFailed if the
+// barrier's wait expired.
+constexpr int kScaleFailed = INT_MIN;
 __device__ int grid_scale_exponent(const cplx* A, int lda, int r0, int r1, int k, double* slot,
-                                   double* red, GridSync& gs, const GridBar* bar) {
+                                   double* red, GridSync& gs) {
   const int nr = r1 - r0;
   double mx = 0.0;
   if (nr > 0)
@@ -283,8 +286,7 @@ __device__ int grid_scale_exponent(const cplx* A, int lda, int r0, int r1, int k
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b = fmax(b, red[w]);
     slot[blockIdx.x] = b;
   }
-  grid_sync(gs);
-  if (grid_failed(bar)) return 0;
+  if (grid_sync(gs)) return kScaleFailed;
   // every warp takes the maximum over the CTAs' values, lanes in parallel
   double g = 0.0;
   for (int c = threadIdx.x & 31; c < (int)gridDim.x; c += 32) g = fmax(g, __ldcg(slot + c));
@@ -348,8 +350,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
   int E = 0;
   __shared__ int esc_sh;
   if (MIXED) {
-    E = grid_scale_exponent(A, lda, r0, r1, k, ws.pr + 2 * G, dred, gs, ws.bar);
-    if (grid_failed(ws.bar)) return;
+    E = grid_scale_exponent(A, lda, r0, r1, k, ws.pr + 2 * G, dred, gs);
+    if (E == kScaleFailed) return;
     rows_to_df(A, lda, r0, r1, 0, k, E);
     __syncthreads();
   }
@@ -475,8 +477,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (g == gown)
           for (int c = tid; c < nbk - t; c += blockDim.x) rowp[c] = P[(size_t)(t + c) * R + (jj - r0)];
       }
-      grid_sync(gs);
-      if (grid_failed(ws.bar)) return;
+      if (grid_sync(gs)) return;
       // (b) the reflector (zlarfg conventions: beta real, v_jj = 1), in FP64
       if (wid == 0) {
         // the pivot row's entry alpha is loaded with the first batch of
@@ -700,8 +701,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       __syncthreads();
       if (nt > 0) partial_vhx<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, out + (size_t)nbk * nbk);
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // S2: reduce columns l % G == g into wfin
     for (int l = g; l < ncol; l += G) {
       for (int s = wid; s < nbk; s += nw) {
@@ -709,8 +709,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (lane == 0) ws.wfin[s + (size_t)nbk * l] = v;
       }
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // S3: W2 = T^H W for the trailing columns this CTA reduced, without
     // forming T: applying H_0^H, H_1^H, ... in turn gives, with
     // Gram[s,u] = v_s^H v_u,
@@ -740,8 +739,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (lane < nbk) ws.wfin[lane + (size_t)nbk * l] = mine;
       }
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // S4: trailing update over this CTA's rows
     if (nt > 0) {
       if (MIXED)
@@ -774,8 +772,8 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
   __shared__ double dred[32];
   int E = 0;
   if (MIXED) {
-    E = grid_scale_exponent(C, ldc, r0, r1, q, ws.pr, dred, gs, ws.bar);
-    if (grid_failed(ws.bar)) return;
+    E = grid_scale_exponent(C, ldc, r0, r1, q, ws.pr, dred, gs);
+    if (E == kScaleFailed) return;
     rows_to_df(C, ldc, r0, r1, 0, q, E);
     __syncthreads();
   }
@@ -801,8 +799,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
                         ws.pc + (size_t)g * pstride);
     else
       partial_vhx<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride);
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     // reduce, then W2 = T W (apply Q, not Q^H) from the stored Gram and tau:
     // applying H_{nbk-1}, ..., H_0 in turn gives
     //   w2_s = tau_s (W[s] - sum_{u>s} Gram[s,u] w2_u),  Gram[s,u] = v_s^H v_u
@@ -828,8 +825,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
         if (lane < nbk) ws.wfin[lane + (size_t)nbk * l] = mine;
       }
     }
-    grid_sync(gs);
-    if (grid_failed(ws.bar)) return;
+    if (grid_sync(gs)) return;
     if (MIXED)
       update_x_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<df2*>(C), ldc, q, ws.wfin);
     else

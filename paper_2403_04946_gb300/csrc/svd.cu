@@ -68,8 +68,7 @@ jacobi_kernel(cplx* M, int ldm, int nr, int nc, cplx* J, int ldj, int accumJ, do
   for (int c = g * blockDim.x + threadIdx.x; c < nc; c += G * blockDim.x) colver[c] = 0u;
   for (size_t e = (size_t)g * blockDim.x + threadIdx.x; e < (size_t)nc * nc; e += (size_t)G * blockDim.x)
     pairchk[e] = ~0ull;
-  grid_sync(gs);
-  if (grid_failed(ws.bar)) return;
+  if (grid_sync(gs)) return;
   double fro2 = 0.0;
   for (int c = 0; c < nc; ++c) fro2 += __ldcg(colnorm + c);
   // A pair is left alone once its smaller column is below theta: a column of
@@ -91,8 +90,7 @@ jacobi_kernel(cplx* M, int ldm, int nr, int nc, cplx* J, int ldj, int accumJ, do
       // the rotations below update the norms incrementally; start each sweep
       // from exact ones, so the final (rotation-free) sweep tests exactly
       column_norms();
-      grid_sync(gs);
-      if (grid_failed(ws.bar)) return;
+      if (grid_sync(gs)) return;
     }
     for (int r = 0; r < N - 1; ++r) {
       for (int base = 2 * g; base < npairs; base += 2 * G) {
@@ -189,8 +187,7 @@ jacobi_kernel(cplx* M, int ldm, int nr, int nc, cplx* J, int ldj, int accumJ, do
           pairchk[(size_t)i * nc + j] = key;
         }
       }
-      grid_sync(gs);
-      if (grid_failed(ws.bar)) return;
+      if (grid_sync(gs)) return;
     }
     // every CTA sees the same count after the last round's barrier
     const int rotations = __ldcg(ws.counters + (sweep & 31));
