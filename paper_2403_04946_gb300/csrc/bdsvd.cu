@@ -894,9 +894,14 @@ bd_vectors_kernel(const double* __restrict__ d, const double* __restrict__ e, in
 // orthogonal to 1e-4 (values equal to ~1e-11): the clustered path then
 // computes all vectors again.
 constexpr int kOrthThreads = 256;
+// The clustered path's vectors take two steps of their own (only where it
+// ran): orthogonal vectors of T_GK leave their left parts orthogonal to
+// rounding times sigma_max / sigma only.
+enum { kOrthFirst = 1, kOrthNext = 0, kOrthClustered = 2 };
 __global__ void __launch_bounds__(kOrthThreads)
 bd_orth_kernel(int n, int k, const double* __restrict__ X, int ldx, double* __restrict__ Xo, int ldo,
-               double* __restrict__ info, int check) {
+               double* __restrict__ info, int mode) {
+  if (mode == kOrthClustered && info[2] == 0.0) return;
   extern __shared__ __align__(16) double osm[];  // column j [n], e_j [k]
   double* xj = osm;
   double* ej = osm + n;
@@ -918,7 +923,7 @@ bd_orth_kernel(int n, int k, const double* __restrict__ X, int ldx, double* __re
       const double g = lane ? s1 : s0;
       const double ee = (c + lane == j) ? 1.0 - g : -g;
       ej[c + lane] = 0.5 * ee;
-      if (check && !(fabs(ee) <= 1e-4)) info[2] = 1.0;  // also for NaN
+      if (mode == kOrthFirst && !(fabs(ee) <= 1e-4)) info[2] = 1.0;  // also for NaN
     }
   }
   __syncthreads();
@@ -1147,10 +1152,14 @@ cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, co
       }
     } else {
       bd_vectors_kernel<<<kt, 32, vsmem, s>>>(d, e, n, info, sig, X, ldx);
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, 1);
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, 0);
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthFirst);
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthNext);
     }
     bd_cluster_kernel<<<kt, 32, csmem, s>>>(d, e, n, info, sig, kt, X, ldx, Zs);
+    if (!mixed) {
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthClustered);
+      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthClustered);
+    }
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
