@@ -498,8 +498,14 @@ cudaError_t check_finite(const cplx* x, size_t count, int* flag, cudaStream_t s)
   return cudaGetLastError();
 }
 
-// ---- FP64 complex GEMM (64 x 64 tiles, 4 x 4 outputs per thread) -------------------------
-constexpr int GT = 64, GK = 16;
+// ---- FP64 complex GEMM ----------------------------------------------------------------------
+// GT x GT tiles, (GT / GS)^2 outputs for each of GS^2 threads.  The FP64 unit
+// retires two multiply-adds per clock and SM, so a tile of any size is bound
+// by it alone, and what counts is that all SMs have tiles: 64 x 64 for large
+// products, down to 8 x 8 for the projections and merges of small bonds
+// (gemm_tile; 16 x 96 x 96 took 186 us on two 64 x 64 tiles).
+constexpr int GK = 16;
+constexpr int gemm_side(int GT) { return GT < 16 ? GT : 16; }
 
 struct LoadA_N {  // A(i, t) = A[i + lda t]
   const cplx* A;
@@ -543,19 +549,20 @@ struct StoreC {  // mode 0: C[i + ldc j]; mode 1: conj into the H^H layout
   }
 };
 
-template <class LA, class LB, class ST>
-__global__ void __launch_bounds__(256) gemm_kernel(LA la, LB lb, ST st, int M, int N, int K) {
+template <int GT, class LA, class LB, class ST>
+__global__ void __launch_bounds__(gemm_side(GT) * gemm_side(GT)) gemm_kernel(LA la, LB lb, ST st, int M, int N, int K) {
+  constexpr int GS = gemm_side(GT), Q = GT / GS;
   __shared__ cplx As[GK][GT + 1];
   __shared__ cplx Bs[GK][GT + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int tx = threadIdx.x % GS, ty = threadIdx.x / GS;
   const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
-  cplx acc[4][4];
+  cplx acc[Q][Q];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < Q; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = mk(0, 0);
+    for (int b = 0; b < Q; ++b) acc[a][b] = mk(0, 0);
   for (int t0 = 0; t0 < K; t0 += GK) {
-    for (int e = threadIdx.x; e < GT * GK; e += 256) {
+    for (int e = threadIdx.x; e < GT * GK; e += GS * GS) {
       const int r = e % GT, kk = e / GT;
       As[kk][r] = la(i0 + r, t0 + kk);
       const int kk2 = e % GK, cc = e / GK;
@@ -564,40 +571,41 @@ __global__ void __launch_bounds__(256) gemm_kernel(LA la, LB lb, ST st, int M, i
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      cplx av[4], bv[4];
+      cplx av[Q], bv[Q];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + 16 * a];
+      for (int a = 0; a < Q; ++a) av[a] = As[kk][tx + GS * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][ty + 16 * b];
+      for (int b = 0; b < Q; ++b) bv[b] = Bs[kk][ty + GS * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < Q; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = cfma(av[a], bv[b], acc[a][b]);
+        for (int b = 0; b < Q; ++b) acc[a][b] = cfma(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < Q; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) st(i0 + tx + 16 * a, j0 + ty + 16 * b, acc[a][b]);
+    for (int b = 0; b < Q; ++b) st(i0 + tx + GS * a, j0 + ty + GS * b, acc[a][b]);
 }
 
 // Mixed-precision variant: operands split into double-float (hi, lo) when
 // staged, products and sums in double-float arithmetic on the FP32 pipe,
 // result stored in FP64.
-template <class LA, class LB, class ST>
-__global__ void __launch_bounds__(256) gemm_kernel_f(LA la, LB lb, ST st, int M, int N, int K) {
+template <int GT, class LA, class LB, class ST>
+__global__ void __launch_bounds__(gemm_side(GT) * gemm_side(GT)) gemm_kernel_f(LA la, LB lb, ST st, int M, int N, int K) {
+  constexpr int GS = gemm_side(GT), Q = GT / GS;
   __shared__ df2 As[GK][GT + 1];
   __shared__ df2 Bs[GK][GT + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int tx = threadIdx.x % GS, ty = threadIdx.x / GS;
   const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
-  df2 acc[4][4];
+  df2 acc[Q][Q];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < Q; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = df_zero();
+    for (int b = 0; b < Q; ++b) acc[a][b] = df_zero();
   for (int t0 = 0; t0 < K; t0 += GK) {
-    for (int e = threadIdx.x; e < GT * GK; e += 256) {
+    for (int e = threadIdx.x; e < GT * GK; e += GS * GS) {
       const int r = e % GT, kk = e / GT;
       As[kk][r] = df_from(la(i0 + r, t0 + kk));
       const int kk2 = e % GK, cc = e / GK;
@@ -606,48 +614,61 @@ __global__ void __launch_bounds__(256) gemm_kernel_f(LA la, LB lb, ST st, int M,
     __syncthreads();
 #pragma unroll 4
     for (int kk = 0; kk < GK; ++kk) {
-      df2 av[4], bv[4];
+      df2 av[Q], bv[Q];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + 16 * a];
+      for (int a = 0; a < Q; ++a) av[a] = As[kk][tx + GS * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][ty + 16 * b];
+      for (int b = 0; b < Q; ++b) bv[b] = Bs[kk][ty + GS * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < Q; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) df_cmac(acc[a][b], av[a], bv[b]);
+        for (int b = 0; b < Q; ++b) df_cmac(acc[a][b], av[a], bv[b]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < Q; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) st(i0 + tx + 16 * a, j0 + ty + 16 * b, df_to(acc[a][b]));
+    for (int b = 0; b < Q; ++b) st(i0 + tx + GS * a, j0 + ty + GS * b, df_to(acc[a][b]));
+}
+
+// Largest tile that still gives every SM one (8 x 8 if none does).
+static int gemm_tile(int M, int N) {
+  for (int T = 64; T > 8; T >>= 1)
+    if ((size_t)((M + T - 1) / T) * ((N + T - 1) / T) >= (size_t)dev_info().sm_count) return T;
+  return 8;
+}
+
+template <int GT, class LA, class LB, class ST>
+static cudaError_t gemm_launch_t(LA la, LB lb, ST st, int M, int N, int K, cudaStream_t s, int mixed) {
+  const dim3 grid((M + GT - 1) / GT, (N + GT - 1) / GT);
+  constexpr int threads = gemm_side(GT) * gemm_side(GT);
+  if (mixed) gemm_kernel_f<GT><<<grid, threads, 0, s>>>(la, lb, st, M, N, K);
+  else gemm_kernel<GT><<<grid, threads, 0, s>>>(la, lb, st, M, N, K);
+  return cudaGetLastError();
+}
+
+template <class LA, class LB, class ST>
+static cudaError_t gemm_launch(LA la, LB lb, ST st, int M, int N, int K, cudaStream_t s, int mixed) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  switch (gemm_tile(M, N)) {
+    case 64: return gemm_launch_t<64>(la, lb, st, M, N, K, s, mixed);
+    case 32: return gemm_launch_t<32>(la, lb, st, M, N, K, s, mixed);
+    case 16: return gemm_launch_t<16>(la, lb, st, M, N, K, s, mixed);
+    default: return gemm_launch_t<8>(la, lb, st, M, N, K, s, mixed);
+  }
 }
 
 cudaError_t gemm_a_rh(const cplx* A, int lda, int M, int K, const cplx* R, int ldr, int N,
                       cplx* C, int ldc, int mode, int rl, int n, cudaStream_t s, int mixed) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((M + GT - 1) / GT, (N + GT - 1) / GT);
-  if (mixed)
-    gemm_kernel_f<<<grid, 256, 0, s>>>(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, 0},
-                                       StoreC{C, ldc, M, N, mode, rl, n}, M, N, K);
-  else
-    gemm_kernel<<<grid, 256, 0, s>>>(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, 0},
-                                     StoreC{C, ldc, M, N, mode, rl, n}, M, N, K);
-  return cudaGetLastError();
+  return gemm_launch(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, 0}, StoreC{C, ldc, M, N, mode, rl, n}, M, N, K, s,
+                     mixed);
 }
 
 cudaError_t gemm_a_rblk_h(const cplx* A, int lda, int M, int K, const cplx* R, int ldr, int coff,
                           int N, cplx* C, int ldc, cudaStream_t s, int mixed) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((M + GT - 1) / GT, (N + GT - 1) / GT);
-  if (mixed)
-    gemm_kernel_f<<<grid, 256, 0, s>>>(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, coff},
-                                       StoreC{C, ldc, M, N, 0, 1, 1}, M, N, K);
-  else
-    gemm_kernel<<<grid, 256, 0, s>>>(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, coff},
-                                     StoreC{C, ldc, M, N, 0, 1, 1}, M, N, K);
-  return cudaGetLastError();
+  return gemm_launch(LoadA_N{A, lda, M, K}, LoadB_RH{R, ldr, K, N, coff}, StoreC{C, ldc, M, N, 0, 1, 1}, M, N, K, s,
+                     mixed);
 }
 
 // out(alpha, i, m, q) = sum_beta W[alpha, beta] applied along m to
@@ -803,11 +824,7 @@ cudaError_t stencil_combine(const cplx* T, int r, int n, int p, int Bn, int Al, 
 
 cudaError_t gemm_uh_r(const cplx* U, int ldu, int M, int K, const cplx* R, int ldr, int N,
                       cplx* C, int ldc, cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((M + GT - 1) / GT, (N + GT - 1) / GT);
-  gemm_kernel<<<grid, 256, 0, s>>>(LoadA_UH{U, ldu, M, K}, LoadB_N{R, ldr, K, N},
-                                   StoreC{C, ldc, M, N, 0, 1, 1}, M, N, K);
-  return cudaGetLastError();
+  return gemm_launch(LoadA_UH{U, ldu, M, K}, LoadB_N{R, ldr, K, N}, StoreC{C, ldc, M, N, 0, 1, 1}, M, N, K, s, 0);
 }
 
 // ---- watchdog check -----------------------------------------------------------
