@@ -1987,30 +1987,14 @@ hopf_status hopf_eval_moments(hopf_ctx* ctx, const hopf_tt* t, double* mean, dou
   if (!ctx || !t || !mean || !cov) return ctx ? fail(ctx, HOPF_EINVAL, "hopf_eval_moments: null argument") : HOPF_EINVAL;
   if (!(ctx->L > 0.0)) return fail(ctx, HOPF_EINVAL, "L is not set");
   if (ctx->equation != HOPF_EQ_PHI) return fail(ctx, HOPF_EINVAL, "hopf_eval_moments: moments come from Phi, not a CDF");
-  const int d = t->d, n = t->n, c = n / 2;
+  const int d = t->d, n = t->n;
   const int npts = 1 + 2 * d + 2 * d * (d - 1);
-  std::vector<int> idx((size_t)npts * d, c);
-  auto at = [&](int pt, int ax, int off) { idx[(size_t)pt * d + ax] = c + off; };
-  int pt = 1;
-  for (int k = 0; k < d; ++k) {
-    at(pt, k, 1); ++pt;
-    at(pt, k, -1); ++pt;
-  }
-  for (int j = 0; j < d; ++j)
-    for (int k = j + 1; k < d; ++k) {
-      at(pt, j, 1); at(pt, k, 1); ++pt;
-      at(pt, j, 1); at(pt, k, -1); ++pt;
-      at(pt, j, -1); at(pt, k, 1); ++pt;
-      at(pt, j, -1); at(pt, k, -1); ++pt;
-    }
   int maxr = 1;
   for (int r : t->ranks) maxr = std::max(maxr, r);
-  TRY(ev_reserve(ctx, idx.size(), (size_t)npts, (size_t)d + (size_t)d * d + 1));
-  int* didx = ctx->ev_idx;
+  TRY(ev_reserve(ctx, 0, (size_t)npts + hk::moment_env_elems(d, maxr), (size_t)d + (size_t)d * d + 1));
   cplx* dv = ctx->ev_vals;
   double* dout = ctx->ev_out;
-  cudaError_t e = cudaMemcpyAsync(didx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-  if (e == cudaSuccess) e = hk::eval_points(t->d_ptrs, t->d_ranks, d, n, maxr, npts, didx, dv, ctx->stream);
+  cudaError_t e = hk::moment_values(t->d_ptrs, t->d_ranks, d, n, maxr, dv + npts, dv, ctx->stream);
   const double da = 2.0 * ctx->L / n;
   if (e == cudaSuccess) e = hk::moments_combine(dv, d, da, dout, dout + d, dout + d + (size_t)d * d, ctx->stream);
   double ir = 0.0;

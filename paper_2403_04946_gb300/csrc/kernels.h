@@ -227,6 +227,11 @@ cudaError_t init_sh_pad(const cplx* S, int lds, int q, int p, cplx* X, int ldx, 
 cudaError_t gather_u(const cplx* src, int lds, int pp, const int* perm, const double* sigma,
                      int use_sigma, int rho, cplx* X, int ldx, int mrows, cplx* Ub, int ldub,
                      cudaStream_t s);
+// The point values of the moment stencil, in the order moments_combine reads
+// them (1 + 2 d + 2 d (d - 1) of them); env: moment_env_elems of scratch.
+size_t moment_env_elems(int d, int rmax);
+cudaError_t moment_values(const cplx* const* cores_dev, const int* ranks_dev, int d, int n, int rmax, cplx* env,
+                          cplx* vals, cudaStream_t s);
 // Combine the point values of the moment stencil into mean/cov.
 cudaError_t moments_combine(const cplx* vals, int d, double da, double* mean, double* cov,
                             double* imag_resid, cudaStream_t s);
