@@ -137,42 +137,90 @@ cudaError_t sum_core(const SumTerm* terms_dev, int nterms, int kind, int n, cplx
 }
 
 // ---- point evaluation --------------------------------------------------------------
-// Phi[i_1..i_d] = C_1[0,i_1,:] C_2[:,i_2,:] ... C_d[:,i_d,0]; one CTA per point.
-__global__ void eval_points_kernel(const cplx* const* __restrict__ cores,
-                                   const int* __restrict__ ranks, int d, int n,
-                                   const int* __restrict__ idx, cplx* __restrict__ vals) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  const int maxr = blockDim.y;  // unused, kept for clarity
-  (void)maxr;
-  cplx* v = reinterpret_cast<cplx*>(sm);
-  const int pt = blockIdx.x;
-  int rmax = 1;
-  for (int k = 0; k <= d; ++k) rmax = max(rmax, ranks[k]);
-  cplx* w = v + rmax;
-  if (threadIdx.x == 0) v[0] = mk(1, 0);
-  __syncthreads();
-  for (int k = 0; k < d; ++k) {
-    const int a = ranks[k], c = ranks[k + 1];
-    const int ik = idx[(size_t)pt * d + k];
-    const cplx* C = cores[k] + (size_t)a * ik;  // C[:, ik, :] with column stride a*n
-    for (int j = threadIdx.x; j < c; j += blockDim.x) {
-      const cplx* col = C + (size_t)a * n * j;
-      cplx acc = mk(0, 0);
-      for (int i = 0; i < a; ++i) acc = cfma(v[i], col[i], acc);
-      w[j] = acc;
+// Phi[i_1..i_d] = C_1[0,i_1,:] C_2[:,i_2,:] ... C_d[:,i_d,0]; one CTA per
+// point, the running row vector in shared memory.  S adjacent lanes share a
+// column of the slice (interleaved rows: contiguous in memory) and add their
+// parts by shuffles; S = 4 for many columns (the additions across lanes cost
+// FP64 time), more when the columns do not fill the CTA.  Many points are
+// bound by the FP64 units (r^2 complex multiply-adds per mode, 2 per clock
+// and SM).  Few points are bound by latency, d dependent products: the
+// indices are known ahead, so every slice is prefetched into L2 first, and
+// each thread keeps four loads and two sums in flight (one thread per column
+// walking all rows took 6.7 us per mode at r = 32).
+constexpr int kEvThreads = 256;
+template <int S>
+DV void eval_mode(const cplx* __restrict__ C, size_t cs, int a, int c, const cplx* v, cplx* w) {
+  const int seg = threadIdx.x % S;
+  constexpr int per = kEvThreads / S;
+  for (int jb = 0; jb < c; jb += per) {
+    const int j = jb + threadIdx.x / S;
+    cplx s0 = mk(0, 0), s1 = mk(0, 0);
+    if (j < c) {
+      const cplx* col = C + cs * j;
+      int i = seg;
+      for (; i + 3 * S < a; i += 4 * S) {
+        const cplx e0 = __ldg(col + i), e1 = __ldg(col + i + S), e2 = __ldg(col + i + 2 * S), e3 = __ldg(col + i + 3 * S);
+        s0 = cfma(v[i], e0, s0);
+        s1 = cfma(v[i + S], e1, s1);
+        s0 = cfma(v[i + 2 * S], e2, s0);
+        s1 = cfma(v[i + 3 * S], e3, s1);
+      }
+      for (; i < a; i += S) s0 = cfma(v[i], __ldg(col + i), s0);
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < c; j += blockDim.x) v[j] = w[j];
+    s0 = cadd(s0, s1);
+#pragma unroll
+    for (int o = 1; o < S; o <<= 1) {
+      s0.x += __shfl_xor_sync(0xffffffffu, s0.x, o);
+      s0.y += __shfl_xor_sync(0xffffffffu, s0.y, o);
+    }
+    if (seg == 0 && j < c) w[j] = s0;
+  }
+}
+
+__global__ void __launch_bounds__(kEvThreads)
+eval_points_kernel(const cplx* const* __restrict__ cores, const int* __restrict__ ranks, int d, int n, int rmax,
+                   int prefetch, const int* __restrict__ idx, cplx* __restrict__ vals) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  cplx* vb = reinterpret_cast<cplx*>(sm);  // [2][rmax]
+  const int pt = blockIdx.x;
+  const int* ip = idx + (size_t)pt * d;
+  if (prefetch) {
+    // one 128-byte line (8 values of a column) per thread and step
+    for (int k = 0; k < d; ++k) {
+      const int a = ranks[k], c = ranks[k + 1], lines = (a + 7) / 8;
+      const cplx* C = cores[k] + (size_t)a * ip[k];
+      for (int t = threadIdx.x; t < lines * c; t += kEvThreads)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(C + (size_t)a * n * (t / lines) + 8 * (t % lines)));
+    }
+  }
+  if (threadIdx.x == 0) vb[0] = mk(1, 0);
+  __syncthreads();
+  int cur = 0;
+  for (int k = 0; k < d; ++k, cur ^= 1) {
+    const int a = ranks[k], c = ranks[k + 1];
+    const cplx* C = cores[k] + (size_t)a * ip[k];  // C[:, i_k, :], column stride a n
+    const cplx* v = vb + (size_t)cur * rmax;
+    cplx* w = vb + (size_t)(cur ^ 1) * rmax;
+    const size_t cs = (size_t)a * n;
+    if (c > 32) eval_mode<4>(C, cs, a, c, v, w);
+    else if (c > 16) eval_mode<8>(C, cs, a, c, v, w);
+    else if (c > 8) eval_mode<16>(C, cs, a, c, v, w);
+    else eval_mode<32>(C, cs, a, c, v, w);
     __syncthreads();
   }
-  if (threadIdx.x == 0) vals[pt] = v[0];
+  if (threadIdx.x == 0) vals[pt] = vb[(size_t)cur * rmax];
 }
 
 cudaError_t eval_points(const cplx* const* cores_dev, const int* ranks_dev, int d, int n, int maxr,
                         int npts, const int* idx_dev, cplx* vals, cudaStream_t s) {
   if (npts <= 0) return cudaSuccess;
-  const size_t smem = sizeof(cplx) * 2 * (size_t)std::max(maxr, 1);
-  eval_points_kernel<<<npts, 128, smem, s>>>(cores_dev, ranks_dev, d, n, idx_dev, vals);
+  const int rmax = std::max(maxr, 1);
+  const size_t smem = sizeof(cplx) * 2 * (size_t)rmax;
+  cudaError_t e = allow_smem((const void*)eval_points_kernel, smem);
+  if (e != cudaSuccess) return e;
+  // with several points per SM the next point's loads hide the latency
+  const int prefetch = npts <= 2 * dev_info().sm_count;
+  eval_points_kernel<<<npts, kEvThreads, smem, s>>>(cores_dev, ranks_dev, d, n, rmax, prefetch, idx_dev, vals);
   return cudaGetLastError();
 }
 
