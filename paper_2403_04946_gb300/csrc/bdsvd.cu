@@ -751,18 +751,6 @@ DV void gk_solve(int N, double* w) {
   }
 }
 
-// Reciprocal to FP64 rounding level: the hardware's 20-bit seed and one
-// third-order step of Householder's iteration, y (1 + e + e^2) with
-// e = 1 - x y (error e^3).  The serial chains below wait on one of these per
-// row: about 230 cycles of dependent operations against 640 measured for the
-// IEEE division.  |x| in [1e-150, 1e150] here (pivots are clamped).
-DV double rcp_fast(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
 // One warp per kept value: left vector u_k of B as the eigenvector of B B^T
 // by twisted factorisation.  With q_i = d_i^2, eps_i = e_i^2 (scaled by
 // 1 / amax^2) and lambda = (sig_k / amax)^2, lane 0 runs

@@ -453,49 +453,73 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           for (int c = tid; c < nbk - t; c += blockDim.x)
             reinterpret_cast<df2*>(rowp)[c] = Pd[(size_t)(t + c) * R + (jj - r0)];
       } else {
-        const cplx* xt = P + (size_t)t * R;
-        double sq = 0.0;
-        for (int i = ilo + tid; i < r1; i += blockDim.x) sq += cabs2(xt[i - r0]);
-        sq = block_sum(sq, dred);
-        if (tid == 0) prp[g] = sq;
-        for (int cb = wid; cb < nrem; cb += 4 * nw) {
-          cplx acc[4] = {mk(0, 0), mk(0, 0), mk(0, 0), mk(0, 0)};
-          for (int i = ilo + lane; i < r1; i += 32) {
-            const cplx x = xt[i - r0];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (cb + q * nw < nrem) acc[q] = cfmac(x, P[(size_t)(t + 1 + cb + q * nw) * R + (i - r0)], acc[q]);
+        // columns t (its norm) .. nbk-1 at once: S lanes per column, so that
+        // 32, 16 or 8 columns fill the CTA (a warp per column would spend
+        // more FP64 time on the additions across 32 lanes than on the sums)
+        const int S = nrem + 1 > 16 ? 8 : (nrem + 1 > 8 ? 16 : 32);
+        const int c = tid / S, seg = tid % S;
+        cplx a0 = mk(0, 0), a1 = mk(0, 0);
+        if (c <= nrem) {
+          const cplx* xt = P + (size_t)t * R;
+          const cplx* ac = xt + (size_t)c * R;
+          int i = ilo - r0 + seg;
+          for (; i + S < r1 - r0; i += 2 * S) {
+            a0 = cfmac(xt[i], ac[i], a0);
+            a1 = cfmac(xt[i + S], ac[i + S], a1);
           }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (cb + q * nw < nrem) {
-              acc[q] = warp_sum(acc[q]);
-              if (lane == 0) myp[cb + q * nw] = acc[q];
-            }
-          }
+          if (i < r1 - r0) a0 = cfmac(xt[i], ac[i], a0);
         }
+        a0 = cadd(a0, a1);
+        for (int o = 1; o < S; o <<= 1) {
+          a0.x += __shfl_xor_sync(0xffffffffu, a0.x, o);
+          a0.y += __shfl_xor_sync(0xffffffffu, a0.y, o);
+        }
+        if (seg == 0 && c <= nrem) myp[c] = a0;
         if (g == gown)
-          for (int c = tid; c < nbk - t; c += blockDim.x) rowp[c] = P[(size_t)(t + c) * R + (jj - r0)];
+          for (int q = tid; q < nbk - t; q += blockDim.x) rowp[q] = P[(size_t)(t + q) * R + (jj - r0)];
       }
-      if (grid_sync(gs)) return;
+      if constexpr (MIXED) {
+        if (grid_sync(gs)) return;
+      } else {
+        // while the other CTAs arrive: column t-1 becomes its reflector
+        grid_arrive(gs);
+        if (t > 0) {
+          const cplx psc = bc[1];
+          cplx* xp = P + (size_t)(t - 1) * R;
+          for (int i = max(lo, jj) + tid; i < r1; i += blockDim.x) xp[i - r0] = cmul(xp[i - r0], psc);
+        }
+        if (grid_wait(gs)) return;
+      }
       // (b) the reflector (zlarfg conventions: beta real, v_jj = 1), in FP64
+      cplx rv = mk(0, 0);  // entry t + 1 + tid of the pivot row (warp 0)
       if (wid == 0) {
-        // the pivot row's entry alpha is loaded with the first batch of
-        // partial norms (both are one L2 round trip away)
+        // the pivot row is loaded with the first batch of partial norms (all
+        // one L2 round trip away)
+        if (lane < nrem) rv = ld_cg(rowp + 1 + lane);
         cplx al;
         if constexpr (MIXED) al = df_to_scaled(ld_cg_df(rowp), 0);
         else al = ld_cg(rowp);
         double s2 = 0.0;
+        const double* nsrc = MIXED ? prp : reinterpret_cast<const double*>(ws.pc + tail0 + (size_t)par * nb);
+        const size_t nstride = MIXED ? 1 : 2 * pstride;
         for (int g0 = lane; g0 < G; g0 += 32 * kLoadBatch) {
           double v[kLoadBatch];
 #pragma unroll
-          for (int u = 0; u < kLoadBatch; ++u) v[u] = (g0 + 32 * u < G) ? ld_cg(prp + g0 + 32 * u) : 0.0;
+          for (int u = 0; u < kLoadBatch; ++u) v[u] = (g0 + 32 * u < G) ? ld_cg(nsrc + nstride * (g0 + 32 * u)) : 0.0;
 #pragma unroll
           for (int u = 0; u < kLoadBatch; ++u)
             if (g0 + 32 * u < G) s2 += v[u];
         }
         s2 = warp_sum(s2);
-        if (lane == 0) {
+        if (!MIXED && lane == 0) {
+          cplx tu, sc;
+          double beta;
+          house_fast(al, s2, &tu, &sc, &beta);
+          bc[0] = tu;
+          bc[1] = sc;
+          bc[2] = mk(beta, 0.0);
+        }
+        if (MIXED && lane == 0) {
           cplx tu, sc;
           double beta;
           if (s2 == 0.0 && al.y == 0.0) {
@@ -510,7 +534,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
             tu = mk((beta - al.x) * ib, -al.y * ib);
             sc = cinv(mk(al.x - beta, al.y));
           }
-          if (MIXED) {
+          {
             // the scale can leave the FP32 range (tiny columns): keep it as
             // mantissa x 2^esc
             const double smax = fmax(fabs(sc.x), fabs(sc.y));
@@ -528,9 +552,9 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         }
       }
       // raw sums over the CTAs of the dot products (tpc threads per
-      // column); in mixed precision warp 0 is left out, so that these sums
-      // run while it forms the reflector
-      const int skip = MIXED ? 32 : 0;
+      // column); warp 0 is left out, so that these sums run while it forms
+      // the reflector
+      constexpr int skip = 32;
       if (nrem > 0 && tid >= skip) {
         const int nthr = blockDim.x - skip, t2 = tid - skip;
         int tpc = 32;
@@ -539,7 +563,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         for (int base = 0; base < nrem; base += per) {
           const int c = base + t2 / tpc;
           const bool valid = c < nrem && t2 / tpc < per;
-          const cplx* src = ws.pc + tail0 + (size_t)par * nb + c;
+          const cplx* src = ws.pc + tail0 + (size_t)par * nb + c + (MIXED ? 0 : 1);
           if constexpr (MIXED) {
             df2 acc = df_zero();
             if (valid)
@@ -566,8 +590,11 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
                   const int gg = g0 + tpc * u;
                   v[u] = (gg < G) ? ld_cg(src + (size_t)gg * pstride) : mk(0, 0);
                 }
+                // pairs first: half the dependent FP64 additions
 #pragma unroll
-                for (int u = 0; u < kLoadBatch; ++u)
+                for (int u = 0; u < kLoadBatch; u += 2) v[u] = cadd(v[u], v[u + 1]);
+#pragma unroll
+                for (int u = 0; u < kLoadBatch; u += 2)
                   if (g0 + tpc * u < G) acc = cadd(acc, v[u]);
               }
             for (int o = 1; o < tpc; o <<= 1) {
@@ -585,10 +612,11 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         df2* Pd = reinterpret_cast<df2*>(P);
         const df2 ctu = bcd[0], csc = bcd[1], scd = bcd[2];
         const int es = esc_sh;
-        for (int c = tid; c < nrem; c += blockDim.x) {
+        if (tid < nrem) {
+          const int c = tid;
           df2 cr = df_zero();
           df_cmac(cr, csc, reinterpret_cast<const df2*>(praw)[c]);
-          const df2 w = df_cadd(ld_cg_df(rowp + 1 + c), df_scalb(cr, es));
+          const df2 w = df_cadd(*reinterpret_cast<const df2*>(&rv), df_scalb(cr, es));
           df2 f = df_zero();
           df_cmac(f, ctu, w);
           f = df_cadd(f, df_zero());
@@ -602,14 +630,16 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         }
         if (tid == 0 && jj >= r0 && jj < r1) xt[jj - r0] = bcd[3];
       } else {
-        for (int c = tid; c < nrem; c += blockDim.x) {
-          const cplx w = cadd(ld_cg(rowp + 1 + c), cmul(cconj(sc), praw[c]));
-          const cplx f = cmul(cconj(tu), w);
-          wl[c] = mk(-f.x, -f.y);  // -f
+        // -f for the pivot row (v = 1), -scale f for the rows below, which
+        // hold x until the next column's barrier
+        if (tid < nrem) {
+          const int c = tid;
+          const cplx w = cadd(rv, cmul(cconj(sc), praw[c]));
+          const cplx f = cmul(cconj(tu), w), sf = cmul(sc, f);
+          wl[c] = mk(-f.x, -f.y);
+          wl[kNbMax + c] = mk(-sf.x, -sf.y);
         }
-        cplx* xt = P + (size_t)t * R;
-        for (int i = ilo + tid; i < r1; i += blockDim.x) xt[i - r0] = cmul(xt[i - r0], sc);
-        if (tid == 0 && jj >= r0 && jj < r1) xt[jj - r0] = bc[2];
+        if (tid == 0 && jj >= r0 && jj < r1) P[(size_t)t * R + (jj - r0)] = bc[2];
       }
       if (tid == 0 && g == 0) tau[jj] = tu;
       __syncthreads();
@@ -631,15 +661,30 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
             a = df_cadd(a, dlt);
           }
         } else {
+          // L lanes along the rows (few rows: several columns per warp)
           const cplx* xt = P + (size_t)t * R;
-          for (int e = tid; e < nrow * nrem; e += blockDim.x) {
-            const int c = e / nrow, i = ifrom + e % nrow;
-            const cplx v = (i == jj) ? mk(1, 0) : xt[i - r0];
-            cplx& a = P[(size_t)(t + 1 + c) * R + (i - r0)];
-            a = cfma(v, wl[c], a);
+          const int nx = r1 - ilo;
+          int L = 32;
+          while (L > 4 && L / 2 >= nx) L >>= 1;
+          const int cw = 32 / L;
+          for (int c = wid * cw + lane / L; c < nrem; c += nw * cw) {
+            cplx* ac = P + (size_t)(t + 1 + c) * R;
+            const cplx sf = wl[kNbMax + c];
+            for (int i = ilo - r0 + lane % L; i < r1 - r0; i += L) ac[i] = cfma(xt[i], sf, ac[i]);
           }
+          if (g == gown)
+            for (int c = tid; c < nrem; c += blockDim.x) {
+              cplx& ap = P[(size_t)(t + 1 + c) * R + (jj - r0)];
+              ap = cadd(ap, wl[c]);
+            }
         }
       }
+      __syncthreads();
+    }
+    if constexpr (!MIXED) {
+      const cplx psc = bc[1];
+      cplx* xp = P + (size_t)(nbk - 1) * R;
+      for (int i = max(lo, j0 + nbk) + tid; i < r1; i += blockDim.x) xp[i - r0] = cmul(xp[i - r0], psc);
       __syncthreads();
     }
     // write the factored panel back in FP64 (R on/above the diagonal, V below)
