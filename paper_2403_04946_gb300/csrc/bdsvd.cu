@@ -129,6 +129,11 @@ DV void house_scalars(cplx alpha, double xnorm2, cplx* tau, cplx* scale, double*
 // alternate between two halves by column parity: a CTA writing column
 // i+2's data has passed both barriers of column i+1, so every reader of
 // column i's half is done.
+// FAST (FP64 contexts): reflector scalars from the reciprocal root and
+// reciprocal of common.cuh, about 800 cycles less on each of a column's two
+// scalar chains.  The mixed path keeps the IEEE forms (bd_invit_kernel says
+// why its factors are kept to the last bit).
+template <bool FAST>
 __global__ void __launch_bounds__(kBdThreads, 1)
 gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* tauq, cplx* taup,
              CoopWs ws, cplx* rows_global) {
@@ -181,31 +186,44 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     if (owner)
       for (int c = i + tid; c < n; c += blockDim.x) rowb[c] = R(i / G, c);
     if (grid_sync(gs)) return;
-    // (b1) left reflector of column i (every CTA), reduction of its columns
+    // (b1) left reflector of column i (every CTA, warp 0) while the other
+    // warps sum this CTA's columns; a second round only where a CTA has more
+    // columns than warps
+    cplx acc = mk(0, 0), a_ic = mk(0, 0);
+    int cc = g + (wid - 1) * G;
     if (wid == 0) {
+      const cplx al = __ldcg(rowb + i);
       const double s2 = warp_sum(sum_published(pr, G));
       if (lane == 0) {
         cplx tq, sc;
         double beta;
-        house_scalars(__ldcg(rowb + i), s2, &tq, &sc, &beta);
+        if (FAST) house_fast(al, s2, &tq, &sc, &beta);
+        else house_scalars(al, s2, &tq, &sc, &beta);
         bc[0] = tq;
         bc[1] = sc;
         bc[2] = mk(beta, 0.0);
       }
+    } else if (cc < C) {
+      a_ic = __ldcg(rowb + i + 1 + cc);
+      acc = warp_sum(sum_published(pc + i + 1 + cc, pstride, G));
     }
     __syncthreads();
     const cplx tq = bc[0], scq = bc[1];
     const cplx ctq = cconj(tq), cscq = cconj(scq);
-    for (int cc = g + wid * G; cc < C; cc += nw * G) {
-      const int c = i + 1 + cc;
-      const cplx acc = warp_sum(sum_published(pc + c, pstride, G));
-      if (lane == 0) {
-        const cplx a_ic = __ldcg(rowb + c);
-        const cplx f = cmul(ctq, cadd(a_ic, cmul(cscq, acc)));
-        fvg[c] = f;
-        nrg[c] = csub(a_ic, f);
+    if (wid > 0)
+      while (cc < C) {
+        const int c = i + 1 + cc;
+        if (lane == 0) {
+          const cplx f = cmul(ctq, cadd(a_ic, cmul(cscq, acc)));
+          fvg[c] = f;
+          nrg[c] = csub(a_ic, f);
+        }
+        cc += (nw - 1) * G;
+        if (cc < C) {
+          a_ic = __ldcg(rowb + i + 1 + cc);
+          acc = warp_sum(sum_published(pc + i + 1 + cc, pstride, G));
+        }
       }
-    }
     if (grid_sync(gs)) return;
     // (b2) left update of own rows r > i: A[r,c] -= v_r conj(tau) w_c;
     // column i keeps v_r
@@ -231,7 +249,8 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
       if (lane == 0 && i + 1 < n) {
         cplx tp, sp;
         double beta;
-        house_scalars(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
+        if (FAST) house_fast(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
+        else house_scalars(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
         bcr[0] = tp;
         bcr[1] = sp;
         bcr[2] = mk(beta, 0.0);
@@ -328,7 +347,7 @@ bool gebrd_fits(int n, const CoopWs& ws, bool have_rows_ws) {
 }
 
 cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cplx* taup,
-                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws) {
+                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int mixed) {
   if (n <= 0) return cudaSuccess;
   int nloc;
   size_t smem;
@@ -338,13 +357,14 @@ cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cpl
   cplx* rows_global = glob ? rows_ws : nullptr;
   if ((size_t)2 * G * (n + 1) > ws.pc_elems || (size_t)6 * n > ws.wfin_elems || 2 * G > 1024)
     return cudaErrorInvalidValue;
-  cudaError_t err = allow_smem((const void*)gebrd_kernel, smem);
+  void* fn = mixed ? (void*)gebrd_kernel<false> : (void*)gebrd_kernel<true>;
+  cudaError_t err = allow_smem(fn, smem);
   if (err != cudaSuccess) return err;
   err = cudaMemsetAsync(&ws.bar->count, 0, sizeof(unsigned int), s);
   if (err != cudaSuccess) return err;
   CoopWs w = ws;
   void* args[] = {&A, &lda, &n, &nloc, &d, &e, &tauq, &taup, &w, &rows_global};
-  return cudaLaunchCooperativeKernel((void*)gebrd_kernel, dim3(G), dim3(kBdThreads), args, smem, s);
+  return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBdThreads), args, smem, s);
 }
 
 // ---- 2. singular values ------------------------------------------------------------

@@ -87,7 +87,7 @@ cudaError_t rank_select(const cplx* M, int ldm, int nr, int nc, const double* ep
 // rows_ws (may be NULL): gebrd_rows_elems(n) elements where the rows go when
 // they do not fit in shared memory (L2-resident for the sizes met here).
 cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cplx* taup,
-                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws = nullptr);
+                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int mixed);
 bool gebrd_fits(int n, const CoopWs& ws, bool have_rows_ws = false);
 size_t gebrd_rows_elems(int n, int sms);
 // All singular values of B, sorted descending, into sig[n]; a2 (float2
