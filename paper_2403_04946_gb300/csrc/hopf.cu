@@ -1080,15 +1080,16 @@ hopf_status apply_impl(hopf_ctx* ctx, const hopf_tt* in, hopf_tt* out) {
   std::vector<int> r(d + 1, 1);
   for (int k = 1; k < d; ++k) r[k] = 6 * in->ranks[k];
   TRY(check_fit(ctx, out, r));
-  hk::OpTable ops{ctx->d_coef, n};
+  const hk::OpTable ops{ctx->d_coef, n, ctx->op_forms};
+  double bytes = 0.0;
+  int maxr = 1;
   for (int k = 0; k < d; ++k) {
-    const int kind = (k == 0) ? 0 : (k == d - 1 ? 2 : 1);
     const int Al = (k == 0) ? 1 : 6, Ar = (k == d - 1) ? 1 : 6;
-    const double rd = (double)in->ranks[k] * n * in->ranks[k + 1];
-    LAUNCH(HOPF_K_APPLY, 0, 16.0 * rd * (1.0 + (double)Al * Ar), 1,
-           hk::apply_core(in->cores[k], in->ranks[k], n, in->ranks[k + 1], out->cores[k], Al, Ar,
-                          ctx->d_blocks + 36 * kind, ops, ctx->stream));
+    bytes += 16.0 * in->ranks[k] * n * in->ranks[k + 1] * (1.0 + (double)Al * Ar);
+    maxr = std::max(maxr, in->ranks[k]);
   }
+  LAUNCH(HOPF_K_APPLY, 0, bytes, 1,
+         hk::apply_cores(in->d_ptrs, in->d_ranks, d, n, maxr, out->d_ptrs, ctx->d_blocks, ops, ctx->stream));
   out->ranks = r;
   return sync_meta(ctx, out);
 }

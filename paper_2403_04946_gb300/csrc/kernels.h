@@ -189,10 +189,12 @@ DV cplx op_apply(const cplx* coef, int op, int n, const cplx* x, size_t s, int m
 cudaError_t stencil_combine(const cplx* T, int r, int n, int p, int Bn, int Al, int Ar,
                             const unsigned char* blocks_dev, const OpTable& ops, cplx* out,
                             int mode, int ldo, cudaStream_t s);
-// out core (Al*a) x n x (Ar*c) from in core a x n x c; blocks[alpha*Ar+beta]
-// holds the op index (OP_NONE = zero block).
-cudaError_t apply_core(const cplx* in, int a, int n, int c, cplx* out, int Al, int Ar,
-                       const unsigned char* blocks_dev, const OpTable& ops, cudaStream_t s);
+// All cores of Y = G X: out core k is (Al a) x n x (Ar c) from in core a x n x c
+// (Al = 1 for the first core, Ar = 1 for the last, else 6); blocks: 3 site
+// kinds x 36 op indices (alpha * Ar + beta, OP_NONE = zero block); maxr >= every
+// rank of X.
+cudaError_t apply_cores(const cplx* const* in_dev, const int* ranks_dev, int d, int n, int maxr, cplx* const* out_dev,
+                        const unsigned char* blocks_dev, const OpTable& ops, cudaStream_t s);
 // Block concatenation of one core of a TT sum.  kind: 0 first, 1 interior,
 // 2 last.  Term t has core pointer ptrs[t], dims (ra[t], n, rc[t]) and
 // coefficient coef[t] (applied on the first core only).

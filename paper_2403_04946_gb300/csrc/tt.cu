@@ -46,44 +46,91 @@ const DevInfo& dev_info() {
 
 static inline int nblk(size_t n, int t) { return (int)((n + t - 1) / t); }
 
+// acc += (op x)[m] from the taps xl = x[m-1], x0 = x[m], xu = x[m+1]
+// (zero beyond the edges), using the parts of the coefficients that f marks.
+DV void op_acc(const cplx* __restrict__ cf, int n, int m, unsigned f, const cplx& xl, const cplx& x0,
+               const cplx& xu, cplx& acc) {
+  if (f & 0x40) {
+    acc.x += x0.x;
+    acc.y += x0.y;
+    return;
+  }
+  if (f & 0x03) {
+    const cplx c = cf[m];
+    if (f & 0x01) { acc.x = fma(c.x, xl.x, acc.x); acc.y = fma(c.x, xl.y, acc.y); }
+    if (f & 0x02) { acc.x = fma(-c.y, xl.y, acc.x); acc.y = fma(c.y, xl.x, acc.y); }
+  }
+  if (f & 0x0C) {
+    const cplx c = cf[n + m];
+    if (f & 0x04) { acc.x = fma(c.x, x0.x, acc.x); acc.y = fma(c.x, x0.y, acc.y); }
+    if (f & 0x08) { acc.x = fma(-c.y, x0.y, acc.x); acc.y = fma(c.y, x0.x, acc.y); }
+  }
+  if (f & 0x30) {
+    const cplx c = cf[2 * n + m];
+    if (f & 0x10) { acc.x = fma(c.x, xu.x, acc.x); acc.y = fma(c.x, xu.y, acc.y); }
+    if (f & 0x20) { acc.x = fma(-c.y, xu.y, acc.x); acc.y = fma(c.y, xu.x, acc.y); }
+  }
+}
+
 // ---- operator apply ------------------------------------------------------------
 // Y[(alpha, i), m, (beta, j)] = sum_m' W[alpha, beta][m, m'] X[i, m', j] with
-// every W block one of the per-mode operators (op_apply): tridiagonal in
-// (m, m'), or the CDF equation's cumulative K.  One thread per
-// output element, consecutive threads along the fastest (left-rank) index, so
-// loads of X and stores of Y are both coalesced 16-byte accesses.  The grid's
-// y index walks the right-rank index q = (beta, j) and x the (alpha, i, m)
-// plane, so that every index comes from 32-bit arithmetic (the plane is
-// below 2^31 elements, checked by the launcher).
-__global__ void apply_core_kernel(const cplx* __restrict__ X, int a, int n, int c,
-                                  cplx* __restrict__ Y, int Al, int Ar,
-                                  const unsigned char* __restrict__ blocks,
-                                  const cplx* __restrict__ coef) {
-  const int rows = Al * a;
-  const int plane = rows * n;
+// every W block one of the per-mode operators: tridiagonal in (m, m'), or the
+// CDF equation's cumulative K.  Bound by the stores (36 values out per value
+// in, 27 of them zero in an interior core), so that what matters is to issue
+// little else: all cores in one launch (grid z), a thread keeps its row
+// (alpha, i) and column (beta, j) and walks kApM grid points with the three
+// taps in registers (no index division, one load per value), and of an
+// operator only the coefficient parts that are nonzero are applied (12 FP64
+// multiply-adds per value for all of them would alone take 1.5 times the
+// stores' time).
+constexpr int kApRow = 64;  // consecutive rows per CTA: 1 KB store segments
+constexpr int kApSub = 4;   // groups of grid points per CTA
+constexpr int kApM = 8;     // grid points per thread
+__global__ void __launch_bounds__(kApRow* kApSub)
+apply_cores_kernel(const cplx* const* __restrict__ in, const int* __restrict__ ranks, int d, int n,
+                   cplx* const* __restrict__ out, const unsigned char* __restrict__ blocks,
+                   const cplx* __restrict__ coef, unsigned long long forms, int mtiles) {
+  const int k = blockIdx.z, a = ranks[k], c = ranks[k + 1];
+  const int Al = k == 0 ? 1 : 6, Ar = k == d - 1 ? 1 : 6, kind = k == 0 ? 0 : (k == d - 1 ? 2 : 1);
+  const int rows = Al * a, p = (blockIdx.x / mtiles) * kApRow + threadIdx.x;
+  if (p >= rows) return;
+  const int al = p / a, i = p - al * a;
+  const int m0 = ((blockIdx.x % mtiles) * kApSub + threadIdx.y) * kApM, m1 = min(n, m0 + kApM);
   for (int q = blockIdx.y; q < Ar * c; q += gridDim.y) {
     const int be = q / c, j = q - be * c;
-    const cplx* Xj = X + (size_t)a * n * j;
-    cplx* Yq = Y + (size_t)plane * q;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < plane; idx += gridDim.x * blockDim.x) {
-      const int m = idx / rows, p = idx - m * rows;
-      const int al = p / a, i = p - al * a;
-      const int op = blocks[al * Ar + be];
+    const int op = blocks[36 * kind + al * Ar + be];
+    cplx* y = out[k] + p + (size_t)rows * ((size_t)n * q);
+    if (op == OP_NONE) {
+      for (int m = m0; m < m1; ++m) y[(size_t)rows * m] = mk(0, 0);
+      continue;
+    }
+    const cplx* x = in[k] + i + (size_t)a * n * j;  // X[i, :, j], stride a
+    if (!(forms >> 63)) {
+      for (int m = m0; m < m1; ++m) y[(size_t)rows * m] = op_apply(coef, op, n, x, (size_t)a, m);
+      continue;
+    }
+    const unsigned f = (unsigned)(forms >> (8 * op)) & 0xFFu;
+    const cplx* cf = coef + (size_t)op * 3 * n;
+    cplx xl = m0 > 0 && m0 < n ? __ldg(x + (size_t)a * (m0 - 1)) : mk(0, 0);
+    cplx x0 = m0 < n ? __ldg(x + (size_t)a * m0) : mk(0, 0);
+#pragma unroll 4
+    for (int m = m0; m < m1; ++m) {
+      const cplx xu = m + 1 < n ? __ldg(x + (size_t)a * (m + 1)) : mk(0, 0);
       cplx v = mk(0, 0);
-      if (op != OP_NONE) v = op_apply(coef, op, n, Xj + i, (size_t)a, m);  // X[i, :, j], stride a
-      Yq[idx] = v;
+      op_acc(cf, n, m, f, xl, x0, xu, v);
+      y[(size_t)rows * m] = v;
+      xl = x0;
+      x0 = xu;
     }
   }
 }
 
-cudaError_t apply_core(const cplx* in, int a, int n, int c, cplx* out, int Al, int Ar,
-                       const unsigned char* blocks_dev, const OpTable& ops, cudaStream_t s) {
-  const size_t plane = (size_t)Al * a * n;
-  const size_t nq = (size_t)Ar * c;
-  if (plane == 0 || nq == 0) return cudaSuccess;
-  if (plane >= (1u << 31) || nq >= (1u << 31)) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)std::min<size_t>(nblk(plane, 256), 1024), (unsigned)std::min<size_t>(nq, 65535));
-  apply_core_kernel<<<grid, 256, 0, s>>>(in, a, n, c, out, Al, Ar, blocks_dev, ops.coef);
+cudaError_t apply_cores(const cplx* const* in_dev, const int* ranks_dev, int d, int n, int maxr, cplx* const* out_dev,
+                        const unsigned char* blocks_dev, const OpTable& ops, cudaStream_t s) {
+  const int mtiles = (n + kApSub * kApM - 1) / (kApSub * kApM);
+  const dim3 grid((6 * maxr + kApRow - 1) / kApRow * mtiles, std::min(6 * maxr, 65535), d);
+  apply_cores_kernel<<<grid, dim3(kApRow, kApSub), 0, s>>>(in_dev, ranks_dev, d, n, out_dev, blocks_dev, ops.coef,
+                                                           ops.forms, mtiles);
   return cudaGetLastError();
 }
 
@@ -767,32 +814,6 @@ size_t stencil_tile_smem(int Bn) { return (size_t)Bn * (kStTM + 2) * kStLd * siz
 DV void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-}
-
-// acc += (op x)[m] from the taps xl = x[m-1], x0 = x[m], xu = x[m+1]
-// (zero beyond the edges), using the parts of the coefficients that f marks.
-DV void op_acc(const cplx* __restrict__ cf, int n, int m, unsigned f, const cplx& xl, const cplx& x0,
-               const cplx& xu, cplx& acc) {
-  if (f & 0x40) {
-    acc.x += x0.x;
-    acc.y += x0.y;
-    return;
-  }
-  if (f & 0x03) {
-    const cplx c = cf[m];
-    if (f & 0x01) { acc.x = fma(c.x, xl.x, acc.x); acc.y = fma(c.x, xl.y, acc.y); }
-    if (f & 0x02) { acc.x = fma(-c.y, xl.y, acc.x); acc.y = fma(c.y, xl.x, acc.y); }
-  }
-  if (f & 0x0C) {
-    const cplx c = cf[n + m];
-    if (f & 0x04) { acc.x = fma(c.x, x0.x, acc.x); acc.y = fma(c.x, x0.y, acc.y); }
-    if (f & 0x08) { acc.x = fma(-c.y, x0.y, acc.x); acc.y = fma(c.y, x0.x, acc.y); }
-  }
-  if (f & 0x30) {
-    const cplx c = cf[2 * n + m];
-    if (f & 0x10) { acc.x = fma(c.x, xu.x, acc.x); acc.y = fma(c.x, xu.y, acc.y); }
-    if (f & 0x20) { acc.x = fma(-c.y, xu.y, acc.x); acc.y = fma(c.y, xu.x, acc.y); }
-  }
 }
 
 __global__ void __launch_bounds__(kStThreads, 3)
