@@ -69,7 +69,9 @@ typedef struct {
                   /* hopf_init_gaussian to sqrt(36.8 / min_k C0_kk)       */
   double tol;     /* relative rounding tolerance used by hopf_step        */
   int rank_cap;   /* rank cap used by hopf_step                           */
-  int precision;  /* HOPF_FP64: every step in FP64.  HOPF_MIXED: the    */
+  int precision;  /* HOPF_FP64: every step at FP64 accuracy (products of   */
+                  /* tall factors as eight-digit BF16 splits on the tensor */
+                  /* cores, exact to 2^-60).  HOPF_MIXED: the              */
                   /* dense products of the rounding (QR trailing updates,  */
                   /* Q applications, merges, U^H R) run on the tensor     */
                   /* cores as digit-split BF16 products with exact FP32   */
@@ -139,7 +141,8 @@ hopf_status hopf_set_wait_limit(hopf_ctx* ctx, double seconds);
  * CUDA error.  Nothing faults; the call blocks for the wait limit. */
 hopf_status hopf_check_watchdog(hopf_ctx* ctx);
 /* How the mixed-precision rounding factors its tall flattenings (QR of
- * n p x K matrices, App. A Alg. 1/2; in HOPF_FP64 every QR is FP64).
+ * n p x K matrices, App. A Alg. 1/2; in HOPF_FP64 every QR is accurate to
+ * FP64 rounding and this choice has no effect).
  * HOPF_QR_TENSOR (the default): for factors of at least 4096 rows,
  * blocked Householder in outer panels of 128 columns whose Gram, trailing
  * products and Q applications run on the tensor cores (digit-split BF16

@@ -585,9 +585,13 @@ hopf_status check_barrier(hopf_ctx* ctx) {
 // |A||B| per product).
 constexpr int kTcDigits = 5;
 
+// Products of an m-row factor on the tensor cores: in mixed precision with
+// the tensor-core QR, in FP64 with the wide digits (FP64 accuracy).
 bool use_tc(const hopf_ctx* ctx, int m, int p) {
-  return ctx->p.precision == HOPF_MIXED && ctx->qr_method == HOPF_QR_TENSOR && hk::qr_tc_applies(m, p);
+  if (ctx->p.precision == HOPF_FP64) return hk::qr_wide_applies(m, p);
+  return ctx->qr_method == HOPF_QR_TENSOR && hk::qr_tc_applies(m, p);
 }
+int product_digits(const hopf_ctx* ctx) { return ctx->p.precision == HOPF_FP64 ? hk::tc_wide_digits() : kTcDigits; }
 
 hopf_status tc_reserve_bytes(hopf_ctx* ctx, size_t need) {
   if (need <= ctx->tcbytes) return HOPF_OK;
@@ -599,24 +603,27 @@ hopf_status tc_reserve_bytes(hopf_ctx* ctx, size_t need) {
   return HOPF_OK;
 }
 
-hopf_status tc_reserve(hopf_ctx* ctx, int m, int k) { return tc_reserve_bytes(ctx, hk::qr_tc_scratch_bytes(m, k, kTcDigits)); }
+hopf_status tc_reserve(hopf_ctx* ctx, int m, int k) {
+  return tc_reserve_bytes(ctx, ctx->p.precision == HOPF_FP64 ? hk::qr_wide_scratch_bytes(m, k)
+                                                             : hk::qr_tc_scratch_bytes(m, k, kTcDigits));
+}
 
 // out (a.R x b.R, column-major, ldo) = A B^T of two operand views on the
 // tensor cores (digit splits in the context's scratch), profiled as one
 // HOPF_K_TC phase with the given FLOP count.
 hopf_status tc_product(hopf_ctx* ctx, const hk::TcOperandView& a, const hk::TcOperandView& b, cplx* out, long long ldo,
                        double flops) {
-  const int Kc = hk::tc_chunk();
-  const size_t ba = (hk::tc_operand_bytes(a.R, a.K, kTcDigits, Kc) + 255) & ~(size_t)255;
-  const size_t bb = (hk::tc_operand_bytes(b.R, b.K, kTcDigits, Kc) + 255) & ~(size_t)255;
-  const size_t np = hk::tc_part_elems(a.R, b.R, a.K);
+  const int S = product_digits(ctx), Kc = hk::tc_chunk(S);
+  const size_t ba = (hk::tc_operand_bytes(a.R, a.K, S, Kc) + 255) & ~(size_t)255;
+  const size_t bb = (hk::tc_operand_bytes(b.R, b.K, S, Kc) + 255) & ~(size_t)255;
+  const size_t np = hk::tc_part_elems(a.R, b.R, a.K, S);
   TRY(tc_reserve_bytes(ctx, ba + bb + np * sizeof(cplx) + 256));
   unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
   hk::TcOperand oa, ob;
   const int slot = prof_begin(ctx);
-  CK(hk::tc_split(a, kTcDigits, &oa, buf, ctx->stream));
-  CK(hk::tc_split(b, kTcDigits, &ob, buf + ba, ctx->stream));
-  CK(hk::tc_zgemm(oa, ob, out, ldo, 1.0, 0, np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr, np,
+  CK(hk::tc_split(a, S, &oa, buf, ctx->stream));
+  CK(hk::tc_split(b, S, &ob, buf + ba, ctx->stream));
+  CK(hk::tc_zgemm(oa, ob, out, 1, ldo, 1.0, 0, np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr, np,
                   &ctx->coop.bar->err, ctx->stream));
   prof_end(ctx, slot, HOPF_K_TC, flops, 0.0, np ? 4 : 3);
   return HOPF_OK;
@@ -676,6 +683,13 @@ bool conf_tc(const hopf_ctx* ctx, const QrConf& c, int m, int p) {
 hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int m, int k, cplx* tau, cplx* T,
                            int* nb, cplx* G) {
   CtaCap cap(ctx, c.ctas);
+  if (ctx->p.precision == HOPF_FP64 && hk::qr_wide_applies(m, std::min(m, k))) {
+    TRY(tc_reserve(ctx, m, k));
+    *nb = 32;
+    CK(hk::geqrf_wide(A, lda, m, k, tau, T, ctx->tcbuf, ctx->tcbytes, ctx->coop, 0, ctx->stream,
+                      phase_timer(ctx, HOPF_K_QR)));
+    return HOPF_OK;
+  }
   if (conf_tc(ctx, c, m, std::min(m, k))) {
     TRY(tc_reserve(ctx, m, k));
     *nb = 32;
@@ -773,6 +787,12 @@ hopf_status qr_apply(hopf_ctx* ctx, const cplx* A, int lda, int m, int p, const 
                      const cplx* G, cplx* C, int ldc, int q) {
   const QrConf c = qr_conf(ctx, m, p);
   CtaCap cap(ctx, c.ctas);
+  if (ctx->p.precision == HOPF_FP64 && hk::qr_wide_applies(m, p)) {
+    TRY(tc_reserve(ctx, m, q));
+    CK(hk::ormqr_wide(A, lda, m, p, T, C, ldc, q, ctx->tcbuf, ctx->tcbytes, &ctx->coop.bar->err, ctx->stream,
+                      phase_timer(ctx, HOPF_K_APPLYQ)));
+    return HOPF_OK;
+  }
   if (conf_tc(ctx, c, m, p)) {
     TRY(tc_reserve(ctx, m, q));
     CK(hk::ormqr_tc(A, lda, m, p, tau, G, C, ldc, q, ctx->tcbuf, ctx->tcbytes, &ctx->coop.bar->err, kTcDigits,
@@ -959,7 +979,9 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
     }
     TRY(qr_apply(ctx, Z, Mrows, Mrows, pp, w.tau2, w.T2, nb2, w.G2, t->cores[c], Mrows, rnew));
     // S = U_rho^H R (rho x cols)
-    if (use_tc(ctx, 4096, pp)) {
+    // (FP64: below about 4e6 multiply-adds the product's and the splits'
+    // launches cost more than the FP64 units' time on all SMs, 14 us)
+    if (use_tc(ctx, 4096, pp) && (MIXED_FLAG || (double)rnew * pp * cols > 4e6)) {
       TRY(tc_product(ctx, hk::TcOperandView{w.Ub, pp, 1, rnew, pp, 1, 0, 0}, hk::TcOperandView{w.Rb, pp, 1, cols, pp, 0, 0, 0},
                      w.Sb, rnew, 8.0 * rnew * pp * cols));
     } else {
@@ -1027,23 +1049,23 @@ hopf_status orth_sweep_apply(hopf_ctx* ctx, const hopf_tt* X, std::vector<int>& 
     if (use_tc(ctx, rl * n, 64)) {
       // the six products on the tensor cores: X_{c-1} (rl n x r) split once,
       // each block of R^H (conjugated, upper trapezoid) split in turn
-      const int Kc = hk::tc_chunk();
-      const size_t ba = (hk::tc_operand_bytes(rl * n, r[c], kTcDigits, Kc) + 255) & ~(size_t)255;
-      const size_t bb = (hk::tc_operand_bytes(p[c], r[c], kTcDigits, Kc) + 255) & ~(size_t)255;
-      const size_t np = hk::tc_part_elems(rl * n, p[c], r[c]);
+      const int S = product_digits(ctx), Kc = hk::tc_chunk(S);
+      const size_t ba = (hk::tc_operand_bytes(rl * n, r[c], S, Kc) + 255) & ~(size_t)255;
+      const size_t bb = (hk::tc_operand_bytes(p[c], r[c], S, Kc) + 255) & ~(size_t)255;
+      const size_t np = hk::tc_part_elems(rl * n, p[c], r[c], S);
       TRY(tc_reserve_bytes(ctx, ba + bb + np * sizeof(cplx) + 256));
       unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
       cplx* part = np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr;
       hk::TcOperand oX, oR;
       int slot = prof_begin(ctx);
-      CK(hk::tc_split(hk::TcOperandView{X->cores[c - 1], 1, (long long)rl * n, rl * n, r[c], 0, 0, 0}, kTcDigits, &oX, buf,
+      CK(hk::tc_split(hk::TcOperandView{X->cores[c - 1], 1, (long long)rl * n, rl * n, r[c], 0, 0, 0}, S, &oX, buf,
                       ctx->stream));
       prof_end(ctx, slot, HOPF_K_TC, 0.0, 0.0, 1);
       for (int be = 0; be < 6; ++be) {
         slot = prof_begin(ctx);
-        CK(hk::tc_split(hk::TcOperandView{w.B[c] + (size_t)m * be * r[c], 1, m, p[c], r[c], 1, 1, be * r[c]}, kTcDigits,
+        CK(hk::tc_split(hk::TcOperandView{w.B[c] + (size_t)m * be * r[c], 1, m, p[c], r[c], 1, 1, be * r[c]}, S,
                         &oR, buf + ba, ctx->stream));
-        CK(hk::tc_zgemm(oX, oR, w.W1 + be * blk, rl * n, 1.0, 0, part, np, &ctx->coop.bar->err, ctx->stream));
+        CK(hk::tc_zgemm(oX, oR, w.W1 + be * blk, 1, rl * n, 1.0, 0, part, np, &ctx->coop.bar->err, ctx->stream));
         prof_end(ctx, slot, HOPF_K_TC, rblk_flops((double)rl * n, r[c], p[c], be * r[c]), 0.0, np ? 3 : 2);
       }
     } else {
@@ -2113,9 +2135,9 @@ hopf_status hopf_tc_zgemm(hopf_ctx* ctx, int M, int N, int K, const double* A, i
       digits < 1 || digits > hk::tc_max_digits() || ldc < M || lda < (opA ? K : M) || ldb < (opB ? N : K))
     return fail(ctx, HOPF_EINVAL, "hopf_tc_zgemm: bad arguments");
   const size_t na = (size_t)lda * (opA ? M : K), nb = (size_t)ldb * (opB ? K : N), nc = (size_t)ldc * N;
-  const int Kc = hk::tc_chunk();
+  const int Kc = hk::tc_chunk(digits);
   const size_t oa = hk::tc_operand_bytes(M, K, digits, Kc), ob = hk::tc_operand_bytes(N, K, digits, Kc);
-  const size_t np = hk::tc_part_elems(M, N, K);
+  const size_t np = hk::tc_part_elems(M, N, K, digits);
   cplx *dA = nullptr, *dB = nullptr, *dC = nullptr, *dP = nullptr;
   unsigned char *bufA = nullptr, *bufB = nullptr;
   auto release = [&]() {
@@ -2137,7 +2159,7 @@ hopf_status hopf_tc_zgemm(hopf_ctx* ctx, int M, int N, int K, const double* A, i
   if (e == cudaSuccess) e = hk::tc_split(va, digits, &oA, bufA, ctx->stream);
   if (e == cudaSuccess) e = hk::tc_split(vb, digits, &oB, bufB, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(dC, 0, nc * sizeof(cplx), ctx->stream);
-  if (e == cudaSuccess) e = hk::tc_zgemm(oA, oB, dC, ldc, 1.0, 0, dP, np, &ctx->coop.bar->err, ctx->stream);
+  if (e == cudaSuccess) e = hk::tc_zgemm(oA, oB, dC, 1, ldc, 1.0, 0, dP, np, &ctx->coop.bar->err, ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(C, dC, nc * sizeof(cplx), cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   release();

@@ -246,7 +246,8 @@ cudaError_t check_finite(const cplx* x, size_t count, int* flag, cudaStream_t s)
 // conj).  tri_mode 1: zero where r > k + tri (upper trapezoid); 2: rows are
 // Householder reflectors s and columns their entries i, zero where
 // k < r + tri, one where k == r + tri; 3: the same reflectors with rows i and
-// columns s (zero where r < k + tri, one where r == k + tri).
+// columns s (zero where r < k + tri, one where r == k + tri); 4: the first
+// tri rows are reflectors as in mode 2 (with tri = 0), the others stored.
 struct TcOperandView {
   const cplx* X;
   long long rs, ks;
@@ -265,17 +266,19 @@ struct TcOperand {
 };
 // Bytes of device memory an operand's digits take (planes + exponents).
 size_t tc_operand_bytes(int R, int K, int S, int Kc);
-int tc_chunk();       // K-chunk with exact FP32 accumulation (192)
-int tc_max_digits();  // 5
+int tc_chunk(int S);   // K-chunk with exact FP32 accumulation (192; 128 for the wide digits)
+int tc_max_digits();   // 5
+int tc_wide_digits();  // 8: products at FP64 accuracy
 // Splits the operand into S digit planes in `buf` (tc_operand_bytes).
 cudaError_t tc_split(const TcOperandView& v, int S, TcOperand* out, void* buf, cudaStream_t s);
-// out (M x N, column-major, ldo) = alpha * A B^T (+ out if accumulate), with
-// alpha a signed power of two, A (M x K) and B (N x K) split operands, i.e. out[m, n] =
+// out[rso m + ldo n] = alpha * A B^T (+ out if accumulate), with alpha a
+// signed power of two, A (M x K) and B (N x K) split operands (5 digits at
+// most, or the wide digits; rso != 1 only for those or beyond one chunk), i.e.
 // alpha sum_k A(m, k) B(n, k).  K beyond one chunk: per-chunk partials in
 // part (tc_part_elems), summed in a fixed order.  err: expiry record.
-cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long ldo, double alpha, int accumulate,
-                     cplx* part, size_t part_elems, int* err, cudaStream_t s);
-size_t tc_part_elems(int M, int N, int K);
+cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long rso, long long ldo, double alpha,
+                     int accumulate, cplx* part, size_t part_elems, int* err, cudaStream_t s);
+size_t tc_part_elems(int M, int N, int K, int S);
 
 // ---- blocked QR / Q application with tensor-core products (qrtc.cu) -------
 // Optional per-phase timing: begin() before a phase's launches returns a
@@ -304,6 +307,17 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
 // C <- Q C for the Q of geqrf_tc (p reflectors).
 cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* Gin, cplx* C, int ldc, int q,
                      void* scratch, size_t scratch_bytes, int* err, int S, cudaStream_t s, const PhaseTimer& pt);
+
+// The same at FP64 accuracy: panels of 32 columns by the cooperative kernel
+// (FP64, or double-float if mixed), their Gram and all trailing products from
+// the wide digits.  T: per panel the record of geqrf (may be NULL).
+bool qr_wide_applies(int m, int p);
+size_t qr_wide_scratch_bytes(int m, int k);
+cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void* scratch, size_t scratch_bytes,
+                       const CoopWs& cws, int mixed, cudaStream_t s, const PhaseTimer& pt);
+// C <- Q C for the Q of geqrf_wide (T as it left it).
+cudaError_t ormqr_wide(const cplx* A, int lda, int m, int p, const cplx* T, cplx* C, int ldc, int q, void* scratch,
+                       size_t scratch_bytes, int* err, cudaStream_t s, const PhaseTimer& pt);
 
 // ---- device memory of the library (hopf.cu) -----------------------------------
 // Every device allocation of the solver and the surrogate goes through these:

@@ -699,6 +699,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         }
       }
     __syncthreads();
+    // a single panel whose Gram the caller forms itself
+    if (Tg == nullptr && j0 + nbk >= k) break;
     // fix up P to hold pure reflectors: zero above, one on the diagonal
     for (int t = 0; t < nbk; ++t)
       for (int i = r0 + tid; i < r1; i += blockDim.x) {
@@ -767,7 +769,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       Ts[e] = (u < c) ? ld_cg(ws.wfin + e) : (u == c ? ld_cg(tau + j0 + c) : mk(0, 0));
     }
     __syncthreads();
-    if (g == 0)
+    if (g == 0 && Tg)
       for (int e = tid; e < nbk * nbk; e += blockDim.x) Tg[(size_t)panel * nb * nb + e] = Ts[e];
     {
       const cplx ctl = (lane < nbk) ? cconj(Ts[lane + nbk * lane]) : mk(0, 0);  // conj(tau_lane)

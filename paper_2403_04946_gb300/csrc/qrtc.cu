@@ -193,7 +193,7 @@ int tc_outer_panel() { return kOuter; }
 bool qr_tc_applies(int m, int p) { return m >= 4096 && p > 32; }
 
 size_t qr_tc_scratch_bytes(int m, int k, int S) {
-  const int Kc = tc_chunk();
+  const int Kc = tc_chunk(S);
   const int nt = std::max(k, 1);
   size_t b = 0;
   auto add = [&](size_t x) { b += (x + 255) & ~(size_t)255; };
@@ -202,7 +202,7 @@ size_t qr_tc_scratch_bytes(int m, int k, int S) {
   add(tc_operand_bytes(nt, m, S, Kc));      // trailing columns / C
   add(tc_operand_bytes(m, kOuter, S, Kc));  // V
   add(tc_operand_bytes(nt, kOuter, S, Kc)); // W2
-  add(std::max(tc_part_elems(kOuter, nt, m), tc_part_elems(kOuter, kOuter, m)) * sizeof(cplx));
+  add(std::max(tc_part_elems(kOuter, nt, m, S), tc_part_elems(kOuter, kOuter, m, S)) * sizeof(cplx));
   add((size_t)kOuter * nt * sizeof(cplx) * 2);  // W, W2
   add(wy_packed_elems(kOuter) * sizeof(df2));   // packed WY triangle
   return b + 1024;
@@ -216,7 +216,7 @@ static double zflops(double M, double N, double K) { return 8.0 * M * N * K; }
 cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* Gout, void* scratch,
                      size_t scratch_bytes, const CoopWs& cws, int S, cudaStream_t s, const PhaseTimer& pt) {
   const int p = std::min(m, k);
-  const int Kc = tc_chunk();
+  const int Kc = tc_chunk(S);
   cudaError_t e = cudaSuccess;
   for (int j0 = 0; j0 < p && e == cudaSuccess; j0 += kOuter) {
     const int nbk = std::min(kOuter, p - j0);
@@ -234,7 +234,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     void* bX = c.take(tc_operand_bytes(std::max(nt, 1), mv, S, Kc));
     void* bV = c.take(tc_operand_bytes(mv, nbk, S, Kc));
     void* bW2 = c.take(tc_operand_bytes(std::max(nt, 1), nbk, S, Kc));
-    const size_t npart = std::max(tc_part_elems(nbk, std::max(nt, 1), mv), tc_part_elems(nbk, nbk, mv));
+    const size_t npart = std::max(tc_part_elems(nbk, std::max(nt, 1), mv, S), tc_part_elems(nbk, nbk, mv, S));
     cplx* part = static_cast<cplx*>(c.take(npart * sizeof(cplx)));
     cplx* W = static_cast<cplx*>(c.take((size_t)nbk * std::max(nt, 1) * sizeof(cplx)));
     cplx* W2 = static_cast<cplx*>(c.take((size_t)nbk * std::max(nt, 1) * sizeof(cplx)));
@@ -246,7 +246,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
     if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 0, 2, 0}, S, &oVB, bVB, s);
     cplx* G = Gout + (size_t)(j0 / kOuter) * kOuter * kOuter;
-    if (e == cudaSuccess) e = tc_zgemm(oVH, oVB, G, kOuter, 1.0, 0, part, npart, &cws.bar->err, s);
+    if (e == cudaSuccess) e = tc_zgemm(oVH, oVB, G, 1, kOuter, 1.0, 0, part, npart, &cws.bar->err, s);
     if (e == cudaSuccess) {
       hermitize_kernel<<<(nbk * nbk + 255) / 256, 256, 0, s>>>(G, kOuter, nbk);
       e = cudaGetLastError();
@@ -258,7 +258,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     cplx* At = A + j0 + (size_t)lda * (j0 + nbk);
     slot = pt.b();
     e = tc_split(TcOperandView{At, lda, 1, nt, mv, 0, 0, 0}, S, &oX, bX, s);
-    if (e == cudaSuccess) e = tc_zgemm(oVH, oX, W, nbk, 1.0, 0, part, npart, &cws.bar->err, s);
+    if (e == cudaSuccess) e = tc_zgemm(oVH, oX, W, 1, nbk, 1.0, 0, part, npart, &cws.bar->err, s);
     pt.e(slot, pt.cls_tc, zflops(nbk, nt, mv), 2 + (mv > Kc));
     slot = pt.b();
     if (e == cudaSuccess) e = wy_solve(G, kOuter, tau + j0, nbk, W, nbk, nt, W2, nbk, 1, packed, s);
@@ -266,7 +266,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     slot = pt.b();
     if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, S, &oW2, bW2, s);
     if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
-    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, At, lda, -1.0, 1, nullptr, 0, &cws.bar->err, s);
+    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, At, 1, lda, -1.0, 1, nullptr, 0, &cws.bar->err, s);
     pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 3);  // two splits, one chunk
   }
   return e;
@@ -275,7 +275,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
 cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* Gin, cplx* C, int ldc, int q,
                      void* scratch, size_t scratch_bytes, int* err, int S, cudaStream_t s, const PhaseTimer& pt) {
   if (m <= 0 || p <= 0 || q <= 0) return cudaSuccess;
-  const int Kc = tc_chunk();
+  const int Kc = tc_chunk(S);
   const int npanel = (p + kOuter - 1) / kOuter;
   cudaError_t e = cudaSuccess;
   for (int j = npanel - 1; j >= 0 && e == cudaSuccess; --j) {
@@ -287,7 +287,7 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
     void* bX = c.take(tc_operand_bytes(q, mv, S, Kc));
     void* bV = c.take(tc_operand_bytes(mv, nbk, S, Kc));
     void* bW2 = c.take(tc_operand_bytes(q, nbk, S, Kc));
-    const size_t npart = tc_part_elems(nbk, q, mv);
+    const size_t npart = tc_part_elems(nbk, q, mv, S);
     cplx* part = static_cast<cplx*>(c.take(std::max<size_t>(npart, 1) * sizeof(cplx)));
     cplx* W = static_cast<cplx*>(c.take((size_t)nbk * q * sizeof(cplx)));
     cplx* W2 = static_cast<cplx*>(c.take((size_t)nbk * q * sizeof(cplx)));
@@ -297,7 +297,7 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
     int slot = pt.b();
     e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
     if (e == cudaSuccess) e = tc_split(TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, S, &oX, bX, s);
-    if (e == cudaSuccess) e = tc_zgemm(oVH, oX, W, nbk, 1.0, 0, part, npart, err, s);
+    if (e == cudaSuccess) e = tc_zgemm(oVH, oX, W, 1, nbk, 1.0, 0, part, npart, err, s);
     pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 3 + (mv > Kc));
     slot = pt.b();
     if (e == cudaSuccess)
@@ -306,7 +306,165 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
     slot = pt.b();
     if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, S, &oW2, bW2, s);
     if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
-    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, Cj, ldc, -1.0, 1, nullptr, 0, err, s);
+    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, Cj, 1, ldc, -1.0, 1, nullptr, 0, err, s);
+    pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 3);
+  }
+  return e;
+}
+
+// ---- the same at FP64 accuracy ------------------------------------------------
+namespace {
+
+constexpr int kWidePanel = 32;
+constexpr int kWy64Warps = 4;
+
+// W2 = T^H W (forward) or T W (backward) for a panel of at most 32 reflectors
+// with Gram g (v_s^H v_u at g[s + nbk u]) and tau (NULL: g holds the panel's
+// record instead, the strict upper triangle of the Gram with tau on the
+// diagonal); one warp per column, a chain of nbk steps in FP64.  rec (may be
+// NULL) receives the record.
+__global__ void __launch_bounds__(32 * kWy64Warps)
+wy_solve64_kernel(const cplx* __restrict__ g, const cplx* __restrict__ tau, int nbk, const cplx* __restrict__ W, int nt,
+                  cplx* __restrict__ W2, int forward, cplx* __restrict__ rec) {
+  __shared__ cplx ts[kWidePanel * kWidePanel];
+  for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
+    const int u = e % nbk, c = e / nbk;
+    const cplx v = u < c ? g[e] : (u == c ? (tau ? tau[c] : g[e]) : mk(0, 0));
+    ts[e] = v;
+    if (rec && blockIdx.x == 0) rec[e] = v;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, l = blockIdx.x * kWy64Warps + (threadIdx.x >> 5);
+  if (l >= nt) return;
+  const bool in = lane < nbk;
+  cplx acc = in ? W[lane + (size_t)nbk * l] : mk(0, 0), mine = mk(0, 0);
+  const cplx own = in ? ts[lane + nbk * lane] : mk(0, 0);
+  const cplx tl = forward ? cconj(own) : own;
+  for (int step = 0; step < nbk; ++step) {
+    const int u = forward ? step : nbk - 1 - step;
+    const cplx wu = cmul(tl, acc);  // valid on lane u
+    const cplx w2 = mk(__shfl_sync(0xffffffffu, wu.x, u), __shfl_sync(0xffffffffu, wu.y, u));
+    if (lane == u) mine = w2;
+    // forward: Gram[lane, u] = conj(Gram[u, lane]), lane > u
+    if (forward) {
+      if (lane > u && in) acc = csub(acc, cmulc(ts[u + nbk * lane], w2));
+    } else {
+      if (lane < u) acc = csub(acc, cmul(ts[lane + nbk * u], w2));
+    }
+  }
+  if (in) W2[lane + (size_t)nbk * l] = mine;
+}
+
+cudaError_t wy_solve64(const cplx* g, const cplx* tau, int nbk, const cplx* W, int nt, cplx* W2, int forward, cplx* rec,
+                       cudaStream_t s) {
+  if (nt <= 0 && !rec) return cudaSuccess;
+  wy_solve64_kernel<<<std::max(1, (nt + kWy64Warps - 1) / kWy64Warps), 32 * kWy64Warps, 0, s>>>(g, tau, nbk, W, nt, W2,
+                                                                                               forward, rec);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// The panel kernel's trailing update costs 16 m 32 FP64 operations per
+// trailing column on all SMs together (1.1 TFLOP/s), the products about 60 us
+// per panel in launches whatever the size: from 2048 rows and a few panels on
+// the products are ahead.
+bool qr_wide_applies(int m, int p) { return m >= 2048 && p > kWidePanel; }
+
+size_t qr_wide_scratch_bytes(int m, int k) {
+  const int S = tc_wide_digits(), Kc = tc_chunk(S), nb = kWidePanel;
+  size_t b = 0;
+  auto add = [&](size_t x) { b += (x + 255) & ~(size_t)255; };
+  add(tc_operand_bytes(nb, m, S, Kc));      // conj(V)
+  add(tc_operand_bytes(k + nb, m, S, Kc));  // [V | trailing columns] / C
+  add(tc_operand_bytes(m, nb, S, Kc));      // V
+  add(tc_operand_bytes(std::max(k, 1), nb, S, Kc));  // W2
+  add(tc_part_elems(k + nb, nb, m, S) * sizeof(cplx));
+  add((size_t)nb * (k + nb) * sizeof(cplx));  // Gram and W
+  add((size_t)nb * std::max(k, 1) * sizeof(cplx));
+  return b + 1024;
+}
+
+cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void* scratch, size_t scratch_bytes,
+                       const CoopWs& cws, int mixed, cudaStream_t s, const PhaseTimer& pt) {
+  const int S = tc_wide_digits(), Kc = tc_chunk(S);
+  const int p = std::min(m, k);
+  cudaError_t e = cudaSuccess;
+  for (int j0 = 0; j0 < p && e == cudaSuccess; j0 += kWidePanel) {
+    const int nbk = std::min(kWidePanel, p - j0), mv = m - j0, nt = k - j0 - nbk;
+    cplx* Ap = A + j0 + (size_t)lda * j0;
+    int nb = kWidePanel;
+    int slot = pt.b();
+    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, mixed);
+    pt.e(slot, pt.cls_panel, 8.0 * mv * (double)nbk * nbk - 8.0 * (double)nbk * nbk * nbk / 3.0, 1);
+    if (e != cudaSuccess || (nt <= 0 && !T)) continue;
+    Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
+    void* bVH = c.take(tc_operand_bytes(nbk, mv, S, Kc));
+    void* bX = c.take(tc_operand_bytes(nbk + nt, mv, S, Kc));
+    void* bV = c.take(tc_operand_bytes(mv, nbk, S, Kc));
+    void* bW2 = c.take(tc_operand_bytes(std::max(nt, 1), nbk, S, Kc));
+    const size_t npart = tc_part_elems(nbk + nt, nbk, mv, S);
+    cplx* part = static_cast<cplx*>(c.take(std::max<size_t>(npart, 1) * sizeof(cplx)));
+    cplx* GW = static_cast<cplx*>(c.take((size_t)nbk * (nbk + nt) * sizeof(cplx)));
+    cplx* W2 = static_cast<cplx*>(c.take((size_t)nbk * std::max(nt, 1) * sizeof(cplx)));
+    if (!c.ok) return cudaErrorInvalidValue;
+    // [G | W] = V^H [V | A_t], rows l of the product are the columns on the
+    // right (128 to a tile), the reflectors its 32 columns
+    TcOperand oVH, oX, oV, oW2;
+    slot = pt.b();
+    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
+    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, lda, 1, nbk + nt, mv, 0, 4, nbk}, S, &oX, bX, s);
+    if (e == cudaSuccess) e = tc_zgemm(oX, oVH, GW, nbk, 1, 1.0, 0, part, npart, &cws.bar->err, s);
+    pt.e(slot, pt.cls_tc, zflops(nbk, nbk + nt, mv), 3 + (mv > Kc));
+    slot = pt.b();
+    cplx* rec = T ? T + (size_t)(j0 / kWidePanel) * kWidePanel * kWidePanel : nullptr;
+    if (e == cudaSuccess) e = wy_solve64(GW, tau + j0, nbk, GW + (size_t)nbk * nbk, nt, W2, 1, rec, s);
+    pt.e(slot, pt.cls_small, 0.0, 1);
+    if (e != cudaSuccess || nt <= 0) continue;
+    cplx* At = A + j0 + (size_t)lda * (j0 + nbk);
+    slot = pt.b();
+    e = tc_split(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, S, &oW2, bW2, s);
+    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, At, 1, lda, -1.0, 1, nullptr, 0, &cws.bar->err, s);
+    pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 3);
+  }
+  return e;
+}
+
+cudaError_t ormqr_wide(const cplx* A, int lda, int m, int p, const cplx* T, cplx* C, int ldc, int q, void* scratch,
+                       size_t scratch_bytes, int* err, cudaStream_t s, const PhaseTimer& pt) {
+  if (m <= 0 || p <= 0 || q <= 0) return cudaSuccess;
+  const int S = tc_wide_digits(), Kc = tc_chunk(S);
+  const int npanel = (p + kWidePanel - 1) / kWidePanel;
+  cudaError_t e = cudaSuccess;
+  for (int j = npanel - 1; j >= 0 && e == cudaSuccess; --j) {
+    const int j0 = j * kWidePanel, nbk = std::min(kWidePanel, p - j0), mv = m - j0;
+    const cplx* Ap = A + j0 + (size_t)lda * j0;
+    cplx* Cj = C + j0;
+    Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
+    void* bVH = c.take(tc_operand_bytes(nbk, mv, S, Kc));
+    void* bX = c.take(tc_operand_bytes(q, mv, S, Kc));
+    void* bV = c.take(tc_operand_bytes(mv, nbk, S, Kc));
+    void* bW2 = c.take(tc_operand_bytes(q, nbk, S, Kc));
+    const size_t npart = tc_part_elems(q, nbk, mv, S);
+    cplx* part = static_cast<cplx*>(c.take(std::max<size_t>(npart, 1) * sizeof(cplx)));
+    cplx* W = static_cast<cplx*>(c.take((size_t)nbk * q * sizeof(cplx)));
+    cplx* W2 = static_cast<cplx*>(c.take((size_t)nbk * q * sizeof(cplx)));
+    if (!c.ok) return cudaErrorInvalidValue;
+    TcOperand oVH, oX, oV, oW2;
+    int slot = pt.b();
+    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
+    if (e == cudaSuccess) e = tc_split(TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, S, &oX, bX, s);
+    if (e == cudaSuccess) e = tc_zgemm(oX, oVH, W, nbk, 1, 1.0, 0, part, npart, err, s);
+    pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 3 + (mv > Kc));
+    slot = pt.b();
+    if (e == cudaSuccess)
+      e = wy_solve64(T + (size_t)j * kWidePanel * kWidePanel, nullptr, nbk, W, q, W2, 0, nullptr, s);
+    pt.e(slot, pt.cls_small, 0.0, 1);
+    slot = pt.b();
+    if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, S, &oW2, bW2, s);
+    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    if (e == cudaSuccess) e = tc_zgemm(oV, oW2, Cj, 1, ldc, -1.0, 1, nullptr, 0, err, s);
     pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 3);
   }
   return e;

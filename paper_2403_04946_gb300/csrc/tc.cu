@@ -52,6 +52,7 @@ constexpr int kTcM = 128;        // rows of an output tile (one TMEM lane each)
 constexpr int kTcN = 32;         // columns of an output tile
 constexpr int kSlab = 64;        // K-values per digit slab (128 bytes of BF16)
 constexpr int kMaxDigits = 5;    // 3 products x 5 levels x 32 columns = 480 TMEM columns
+constexpr int kWideDigits = 8;   // FP64 products (tc_zgemm_wide_kernel): 63 bits per operand row
 constexpr int kTmemCols = 512;
 constexpr int kStages = 2;
 constexpr int kTcThreads = 320;  // warps 0-7 epilogue, 8 producer, 9 MMA
@@ -71,6 +72,7 @@ struct TcArgs {
   const int* eB;  // [3][nchunks][N]
   cplx* out;      // out[z * zstride + m + ldo * n]
   long long ldo, zstride;
+  long long rso;  // wide kernel: out[z * zstride + rso * m + ldo * n]
   int alpha_exp, alpha_neg;  // alpha = (-1)^alpha_neg 2^alpha_exp: out = alpha * result (+ out if accumulate)
   int accumulate;
   int* err;       // expiry record (the context's grid-barrier err field)
@@ -278,6 +280,277 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
 }
 
+// ---- products at FP64 accuracy -----------------------------------------------
+// The same product from kWideDigits = 8 digits per operand (63 bits below the
+// row's power of two: every bit of entries down to 2^-10 of the row's largest;
+// the dropped pairs weigh 8 2^-64 of |A||B|), so that the FP64 path's
+// contractions leave the FP64 units, 1/800 of the tensor pipe.  (With seven
+// digits a C2 step was 28 times further from a 64-bit reference than FP64
+// products: the entries of a K-chunk decay, and the digits count from the
+// largest.)  36 digit pairs per real product; a level sums at most 8 pairs, so
+// a K-chunk of 128 stays within 8 2^7 2^14 = 2^24: exact.
+//
+// 8 levels x 32 columns are 256 tensor-memory columns, two of the three 3M
+// products at a time: product c accumulates in half c mod 2 while the
+// epilogue reads the previous one, the third waits until the first is read.
+// A stage of all 8 + 8 planes would be 160 KB, so the ring holds single A
+// planes (16 KB, nine of them) beside two sets of B planes (32 KB, one per
+// K-slab); A plane i meets B planes 0 .. 7-i in one MMA of N = 32 (8 - i).
+// The epilogue sums the integer levels exactly (64 + 16 bits), aligns the three
+// products on the largest, combines them as integers and rounds once to FP64:
+// no FP64 instruction but the addition to an accumulated output.  The component re + im of an operand is summed as
+// fixed-point integers as well (split_kernel), not rounded to FP64 first.
+constexpr int kWideA = 9;
+constexpr int kWideChunk = 2 * kSlab;
+__host__ __device__ constexpr int wide_b_bytes() { return kWideDigits * kTcN * kSlab * 2; }  // 32 KB
+size_t wide_smem_bytes() { return (size_t)kWideA * a_plane_bytes() + 2 * wide_b_bytes() + 1024; }
+
+DV void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// I 2^E as a double, rounded to nearest (ties away from zero), by integer
+// arithmetic; outside the normal range 0 or infinity.
+DV double int_scaled(long long I, int E) {
+  if (I == 0) return 0.0;
+  const unsigned long long m0 = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
+  const int msb = 63 - __clzll((long long)m0);
+  const long long ex = (long long)msb + E + 1023;
+  unsigned long long m = msb > 52 ? (m0 + (1ull << (msb - 53))) >> (msb - 52) : m0 << (52 - msb);
+  // m in [2^52, 2^53]: a carry moves into the exponent field by itself
+  const unsigned long long sgn = I < 0 ? 1ull << 63 : 0ull;
+  if (ex <= 0) return __longlong_as_double((long long)sgn);
+  if (ex >= 2046) return __longlong_as_double((long long)(sgn | (0x7FFull << 52)));
+  return __longlong_as_double((long long)(sgn | (((unsigned long long)ex << 52) + (m - (1ull << 52)))));
+}
+
+// I 2^-d rounded to nearest, d >= 0.
+DV long long shift_round(long long I, int d) {
+  if (d == 0) return I;
+  return d > 62 ? 0 : (I + (1ll << (d - 1))) >> d;
+}
+
+// Exponent of a K-chunk of a row that holds an infinity or a NaN (wide digits):
+// every output it enters becomes NaN, as in FP64 arithmetic.
+constexpr int kNotFinite = 20000;
+
+__global__ void __launch_bounds__(kTcThreads, 1)
+    tc_zgemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcArgs a) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t a_full[kWideA], a_empty[kWideA], b_full[2], b_empty[2], acc_full[3], acc_free, done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  __shared__ int eb_sh[3][kTcN];
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* smem_b = smem + (size_t)kWideA * a_plane_bytes();
+  constexpr int S = kWideDigits;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * kTcN, z = blockIdx.z;
+  const int k_begin = z * kWideChunk;
+  const int k_len = min(kWideChunk, a.K - k_begin);
+  const int nslab = (k_len + kSlab - 1) / kSlab;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kWideA; ++i) {
+      mbar_init(&a_full[i], 1);
+      mbar_init(&a_empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&b_full[i], 1);
+      mbar_init(&b_empty[i], 1);
+    }
+    for (int i = 0; i < 3; ++i) mbar_init(&acc_full[i], 1);
+    mbar_init(&acc_free, 256);
+    mbar_init(&done, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  volatile int* vabort = &abort_flag;
+  // units u = c * nslab + slab in order; A plane i of unit u is use u S + i
+  const int nunit = 3 * nslab;
+
+  if (warp == 8) {
+    if (lane == 0) {
+      int nb = 0, na = 0;  // B sets and A planes issued
+      bool ok = true;
+      for (int u = 0; u < nunit && ok; ++u) {
+        const int c = u / nslab, k0 = k_begin + (u - c * nslab) * kSlab;
+        const int sb = u & 1;
+        if (u >= 2 && !mbar_wait(&b_empty[sb], ((u >> 1) - 1) & 1, vabort, a.err)) break;
+        mbar_expect_tx(&b_full[sb], (uint32_t)wide_b_bytes());
+        for (int j = 0; j < S; ++j)
+          tma_load_3d(smem_b + (size_t)sb * wide_b_bytes() + (size_t)j * b_plane_bytes(), &mapB, &b_full[sb], k0, n0,
+                      c * S + j);
+        nb = u + 1;
+        for (int i = 0; i < S; ++i) {
+          const int w = u * S + i, sl = w % kWideA;
+          if (w >= kWideA && !mbar_wait(&a_empty[sl], ((w / kWideA) - 1) & 1, vabort, a.err)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&a_full[sl], (uint32_t)a_plane_bytes());
+          tma_load_3d(smem + (size_t)sl * a_plane_bytes(), &mapA, &a_full[sl], k0, m0, c * S + i);
+          na = w + 1;
+        }
+      }
+      // every issued copy has landed before the CTA may exit (bounded)
+      for (int u = max(0, nb - 2); u < nb; ++u) {
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(&b_full[u & 1], (u >> 1) & 1))
+          if (global_ns() - t0 > kWaitNs) break;
+      }
+      for (int w = max(0, na - kWideA); w < na; ++w) {
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(&a_full[w % kWideA], (w / kWideA) & 1))
+          if (global_ns() - t0 > kWaitNs) break;
+      }
+    }
+  } else if (warp == 9) {
+    if (lane == 0) {
+      bool ok = true;
+      for (int u = 0; u < nunit && ok; ++u) {
+        const int c = u / nslab, slab = u - c * nslab, sb = u & 1;
+        // the third product takes the first one's columns
+        if (c == 2 && slab == 0 && !mbar_wait(&acc_free, 0, vabort, a.err)) break;
+        if (!mbar_wait(&b_full[sb], (u >> 1) & 1, vabort, a.err)) break;
+        const uint64_t b0 = sw128_desc(smem_u32(smem_b + (size_t)sb * wide_b_bytes()));
+        const int nkk = min(kSlab, k_len - slab * kSlab + 15) / 16;  // 16-value steps that hold data
+        const uint32_t acc = tmem + (uint32_t)((c & 1) * S * kTcN);
+        for (int i = 0; i < S; ++i) {
+          const int w = u * S + i, sl = w % kWideA;
+          if (!mbar_wait(&a_full[sl], (w / kWideA) & 1, vabort, a.err)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t a0 = sw128_desc(smem_u32(smem + (size_t)sl * a_plane_bytes()));
+          const uint32_t idesc = umma_idesc_bf16(kTcM, kTcN * (S - i));
+          for (int kk = 0; kk < nkk; ++kk)
+            umma(acc + (uint32_t)(i * kTcN), a0 + (uint64_t)(kk * 2), b0 + (uint64_t)(kk * 2), idesc,
+                 (slab > 0 || i > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(&a_empty[sl]);
+        }
+        if (!ok) break;
+        umma_commit(&b_empty[sb]);
+        if (slab == nslab - 1) umma_commit(&acc_full[c]);
+      }
+      // the MMAs issued have finished before the tensor memory is freed (bounded)
+      umma_commit(&done);
+      const uint64_t t0 = global_ns();
+      while (!mbar_try_wait(&done, 0))
+        if (global_ns() - t0 > kWaitNs) break;
+    }
+  } else {
+    // ---- epilogue: warps 0-7; two per lane quadrant, 16 columns each -------
+    const int quad = warp & 3, half = warp >> 2;
+    const int m = m0 + 32 * quad + lane;
+    cplx* out = a.out + (size_t)z * a.zstride;
+    {
+      const int t = threadIdx.x;
+      if (t < 3 * kTcN) {
+        const int c = t / kTcN, n = n0 + t % kTcN;
+        eb_sh[c][t % kTcN] = (n < a.N) ? a.eB[(size_t)c * a.nchunks * a.N + (size_t)z * a.N + n] : 0;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+    }
+    const size_t eAs = (size_t)a.nchunks * a.M;
+    int ea[3] = {0, 0, 0};
+    if (m < a.M)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ea[c] = a.eA[c * eAs + (size_t)z * a.M + m];
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(16 * half);
+    // product c of column q: X 2^(ex - 54) + lo 2^(ex - 70), lo 16 bits
+    long long X[3][16];
+    unsigned int lo[3][8];
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ok = ok && mbar_wait(&acc_full[c], 0, vabort, a.err);
+      tc_fence_after();
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          float v[8][4];
+          tmem_ld_levels8x4(lane_base + (uint32_t)((c & 1) * S * kTcN + 4 * h), v);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            long long x = __float2int_rn(v[0][q]);
+#pragma unroll
+            for (int L = 1; L < 6; ++L) x = x * 256 + __float2int_rn(v[L][q]);
+            const long long low = (long long)__float2int_rn(v[6][q]) * 256 + __float2int_rn(v[7][q]);
+            X[c][4 * h + q] = x + (low >> 16);
+            const unsigned int l16 = (unsigned int)low & 0xFFFFu;
+            unsigned int& w = lo[c][(4 * h + q) / 2];
+            w = (q & 1) ? w | (l16 << 16) : l16;
+          }
+        }
+      }
+      if (c == 0) {  // read: its columns are free for the third product
+        tc_fence_before();
+        mbar_arrive(&acc_free);
+      }
+    }
+    if (ok && !*vabort) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int n = n0 + 16 * half + q;
+        if (m >= a.M || n >= a.N) continue;
+        // all three at one unit, the largest at bit 60 (a zero product has no
+        // scale): the sum is exact to 2^-60 of the largest product, whatever
+        // the scales
+        int ex[3], top = -100000;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          ex[c] = ea[c] + eb_sh[c][16 * half + q];
+          const long long x = X[c][q];
+          if (x != 0 || lo[c][q / 2] != 0)
+            top = max(top, ex[c] + 63 - __clzll((x < 0 ? ~x : x) | 1ll));
+        }
+        long long T[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const unsigned int l16 = (q & 1) ? lo[c][q / 2] >> 16 : lo[c][q / 2] & 0xFFFFu;
+          const int up = 60 - top + ex[c];
+          const long long x = X[c][q];
+          if (x == 0 && l16 == 0) T[c] = 0;
+          else if (up >= 0) T[c] = (x << up) + (long long)(up >= 16 ? (unsigned long long)l16 << (up - 16) : l16 >> (16 - up));
+          else T[c] = shift_round(x, -up);
+        }
+        // re = T1 - T2, im = T3 - T1 - T2: each |T| <= 2^61, sums below 2^63
+        long long re = T[0] - T[1], im = T[2] - T[0] - T[1];
+        if (a.alpha_neg) {
+          re = -re;
+          im = -im;
+        }
+        const int Es = top - 114 + a.alpha_exp;
+        cplx r = mk(int_scaled(re, Es), int_scaled(im, Es));
+        if (max(ex[0], max(ex[1], ex[2])) > kNotFinite / 2) r = mk(__longlong_as_double(-1ll), __longlong_as_double(-1ll));
+        cplx* p = out + (size_t)a.rso * m + (size_t)a.ldo * n;
+        if (a.accumulate) r = cadd(*p, r);
+        *p = r;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+}
+
 // ---- digit splitting ----------------------------------------------------------
 // The operand view of TcOperandView (kernels.h), passed by value.
 struct SplitView {
@@ -296,6 +569,8 @@ DV int view_kind(const SplitView& v, int r, int k) {
   if (v.tri_mode == 2) return k < r + v.tri ? 1 : (k == r + v.tri ? 2 : 0);
   // same reflector block, view with rows = entry index i, columns = s
   if (v.tri_mode == 3) return r < k + v.tri ? 1 : (r == k + v.tri ? 2 : 0);
+  // the first `tri` rows are such reflectors (r, entry k), the rest stored
+  if (v.tri_mode == 4 && r < v.tri) return k < r ? 1 : (k == r ? 2 : 0);
   return 0;
 }
 
@@ -343,7 +618,7 @@ DV long long fixed_point(double v, int e, int nbits) {
   const int sh = E - e + nbits;
   long long X;
   if (M == 0 || sh < -62) X = 0;
-  else if (sh >= 0) X = M << sh;  // not reached for |v| < 2^e, nbits <= 46
+  else if (sh >= 0) X = M << sh;  // only for nbits > 53: sh <= nbits - 53, X < 2^nbits
   else X = (M + (1ll << (-sh - 1))) >> (-sh);
   return b < 0 ? -X : X;
 }
@@ -384,10 +659,31 @@ DV void digit_pair(long long X0, long long X1, int S, unsigned int* dst, size_t 
   dst[0] = bf16_bits(y0) | (bf16_bits(y1) << 16);
 }
 
+// The same for S = kWideDigits: |X| < 2^63, the first five digits are cut in
+// 64 bits (below 2^24 is left), the rest in 32.
+DV void digit_pair_wide(long long X0, long long X1, unsigned int* dst, size_t pstride) {
+#pragma unroll
+  for (int j = kWideDigits - 1; j >= 3; --j) {
+    const int d0 = (int)((X0 + 128) & 255) - 128, d1 = (int)((X1 + 128) & 255) - 128;
+    X0 = (X0 - d0) >> 8;
+    X1 = (X1 - d1) >> 8;
+    dst[(size_t)j * pstride] = bf16_bits(d0) | (bf16_bits(d1) << 16);
+  }
+  int y0 = (int)X0, y1 = (int)X1;
+#pragma unroll
+  for (int j = 2; j >= 1; --j) {
+    const int d0 = ((y0 + 128) & 255) - 128, d1 = ((y1 + 128) & 255) - 128;
+    y0 = (y0 - d0) >> 8;
+    y1 = (y1 - d1) >> 8;
+    dst[(size_t)j * pstride] = bf16_bits(d0) | (bf16_bits(d1) << 16);
+  }
+  dst[0] = bf16_bits(y0) | (bf16_bits(y1) << 16);
+}
+
 __global__ void __launch_bounds__(kSplitThreads)
     split_kernel(SplitView v, int Kc, int nchunks, int S, int* e, __nv_bfloat16* planes, long long ldk) {
   extern __shared__ cplx tile[];  // [kSplitRows][kSplitLd]
-  __shared__ int esh[3][kSplitRows];
+  __shared__ int esh[4][kSplitRows];  // components' exponents; one above max(|re|, |im|)
   const int r0 = blockIdx.x * kSplitRows, z = blockIdx.y;
   const int kb = z * Kc, klen = min(v.K - kb, Kc);
   const int tid = threadIdx.x;
@@ -415,8 +711,13 @@ __global__ void __launch_bounds__(kSplitThreads)
   {
     const int r = tid >> 4, j = tid & 15;
     long long k0m = 0, k1m = 0, k2m = 0;
+    // infinities and NaNs by their exponent bits (a NaN's sign may stay in the
+    // masked key: the mask can become a floating-point absolute value)
+    int bad = 0;
     for (int k = j; k < klen; k += 16) {
       const cplx x = tile[r * kSplitLd + k];
+      if (S == kWideDigits)
+        bad |= ((unsigned)__double2hiint(x.x) << 1) >= 0xFFE00000u || ((unsigned)__double2hiint(x.y) << 1) >= 0xFFE00000u;
       const double im = sgn * x.y;
       k0m = max(k0m, mag_key(x.x));
       k1m = max(k1m, mag_key(im));
@@ -427,10 +728,12 @@ __global__ void __launch_bounds__(kSplitThreads)
       k0m = max(k0m, __shfl_xor_sync(0xffffffffu, k0m, o));
       k1m = max(k1m, __shfl_xor_sync(0xffffffffu, k1m, o));
       k2m = max(k2m, __shfl_xor_sync(0xffffffffu, k2m, o));
+      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
     }
     if (j < 3) {
-      const int ex = key_exponent(j == 0 ? k0m : (j == 1 ? k1m : k2m));
+      const int ex = bad ? kNotFinite : key_exponent(j == 0 ? k0m : (j == 1 ? k1m : k2m));
       esh[j][r] = ex;
+      if (j == 0) esh[3][r] = key_exponent(max(k0m, k1m)) + 1;
       if (r0 + r < v.R) e[((size_t)j * nchunks + z) * v.R + r0 + r] = ex;
     }
   }
@@ -447,9 +750,23 @@ __global__ void __launch_bounds__(kSplitThreads)
     if (r0 + r >= v.R) break;
     const cplx x0 = tile[r * kSplitLd + kk], x1 = tile[r * kSplitLd + kk + 1];
     const double i0 = sgn * x0.y, i1 = sgn * x1.y;
+    unsigned int* dst = reinterpret_cast<unsigned int*>(planes + (size_t)(r0 + r) * ldk + kb + kk);
+    if (S == kWideDigits) {
+      digit_pair_wide(fixed_point(x0.x, esh[0][r], nbits), fixed_point(x1.x, esh[0][r], nbits), dst, plane / 2);
+      digit_pair_wide(fixed_point(i0, esh[1][r], nbits), fixed_point(i1, esh[1][r], nbits), dst + (size_t)S * (plane / 2),
+                      plane / 2);
+      // re + im as integers at a scale above both (exact to 2^-62 of the larger
+      // one), then at the sum's own scale, which it does not exceed
+      const int ec = esh[3][r], up = ec - esh[2][r];
+      long long s0 = fixed_point(x0.x, ec, nbits) + fixed_point(i0, ec, nbits);
+      long long s1 = fixed_point(x1.x, ec, nbits) + fixed_point(i1, ec, nbits);
+      s0 = up < 63 ? s0 << max(up, 0) : 0;
+      s1 = up < 63 ? s1 << max(up, 0) : 0;
+      digit_pair_wide(s0, s1, dst + (size_t)(2 * S) * (plane / 2), plane / 2);
+      continue;
+    }
     const double c0[3] = {x0.x, i0, x0.x + i0};
     const double c1[3] = {x1.x, i1, x1.x + i1};
-    unsigned int* dst = reinterpret_cast<unsigned int*>(planes + (size_t)(r0 + r) * ldk + kb + kk);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const int ex = esh[q][r];
@@ -459,18 +776,61 @@ __global__ void __launch_bounds__(kSplitThreads)
   }
 }
 
-// out[m + ldo n] = alpha * sum_z part[z * zstride + m + M n] (+ out)
-__global__ void reduce_parts_kernel(const cplx* part, int M, int N, int nz, long long zstride, double alpha, int accumulate,
-                                    cplx* out, long long ldo) {
+// out[rso m + ldo n] = alpha * sum_z part[z * zstride + m + M n] (+ out), one
+// thread per output, the partials in order (the narrow digits' results are
+// kept to the last bit), eight loads in flight.
+__global__ void reduce_parts_kernel(const cplx* __restrict__ part, int M, int N, int nz, long long zstride, double alpha,
+                                    int accumulate, cplx* __restrict__ out, long long rso, long long ldo) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
   const int m = (int)(idx % M), n = (int)(idx / M);
   cplx s = mk(0, 0);
-  for (int z = 0; z < nz; ++z) s = cadd(s, part[(size_t)z * zstride + idx]);
-  cplx* p = out + m + (size_t)ldo * n;
+  for (int z0 = 0; z0 < nz; z0 += 8) {
+    cplx v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = z0 + u < nz ? part[(size_t)(z0 + u) * zstride + idx] : mk(0, 0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (z0 + u < nz) s = cadd(s, v[u]);
+  }
+  cplx* p = out + (size_t)rso * m + (size_t)ldo * n;
   cplx r = mk(alpha * s.x, alpha * s.y);
   if (accumulate) r = cadd(*p, r);
   *p = r;
+}
+
+// The same for the wide digits, whose chunks are shorter: eight threads per
+// output take every eighth partial, four loads in flight, and their sums are
+// added in a fixed order (384 partials of 49152 rows would be one chain of
+// 384 dependent FP64 additions).
+constexpr int kRedOut = 32;
+constexpr int kRedZ = 8;
+__global__ void __launch_bounds__(kRedOut * kRedZ)
+    reduce_wide_kernel(const cplx* __restrict__ part, int M, int N, int nz, long long zstride, double alpha, int accumulate,
+                       cplx* __restrict__ out, long long rso, long long ldo) {
+  __shared__ cplx sums[kRedZ][kRedOut];
+  const int o = threadIdx.x % kRedOut, zl = threadIdx.x / kRedOut;
+  const long long idx = (long long)blockIdx.x * kRedOut + o, total = (long long)M * N;
+  cplx s = mk(0, 0);
+  if (idx < total) {
+    const cplx* p = part + idx;
+    int z = zl;
+    for (; z + 3 * kRedZ < nz; z += 4 * kRedZ) {
+      const cplx v0 = p[(size_t)z * zstride], v1 = p[(size_t)(z + kRedZ) * zstride],
+                 v2 = p[(size_t)(z + 2 * kRedZ) * zstride], v3 = p[(size_t)(z + 3 * kRedZ) * zstride];
+      s = cadd(cadd(s, v0), cadd(v1, cadd(v2, v3)));
+    }
+    for (; z < nz; z += kRedZ) s = cadd(s, p[(size_t)z * zstride]);
+  }
+  sums[zl][o] = s;
+  __syncthreads();
+  if (zl != 0 || idx >= total) return;
+  for (int i = 1; i < kRedZ; ++i) s = cadd(s, sums[i][o]);
+  const int m = (int)(idx % M), n = (int)(idx / M);
+  cplx* q = out + (size_t)rso * m + (size_t)ldo * n;
+  cplx r = mk(alpha * s.x, alpha * s.y);
+  if (accumulate) r = cadd(*q, r);
+  *q = r;
 }
 
 }  // namespace
@@ -485,12 +845,13 @@ size_t tc_operand_bytes(int R, int K, int S, int Kc) {
   return ((planes + 255) & ~(size_t)255) + exps + 256;
 }
 
-int tc_chunk() { return 3 * kSlab; }
+int tc_chunk(int S) { return S == kWideDigits ? kWideChunk : 3 * kSlab; }
 int tc_max_digits() { return kMaxDigits; }
+int tc_wide_digits() { return kWideDigits; }
 
 cudaError_t tc_split(const TcOperandView& ov, int S, TcOperand* out, void* buf, cudaStream_t s) {
-  if (S < 1 || S > kMaxDigits || ov.R <= 0 || ov.K <= 0) return cudaErrorInvalidValue;
-  const int Kc = tc_chunk();
+  if (S < 1 || (S > kMaxDigits && S != kWideDigits) || ov.R <= 0 || ov.K <= 0) return cudaErrorInvalidValue;
+  const int Kc = tc_chunk(S);
   const long long ldk = ((long long)ov.K + kSlab - 1) / kSlab * kSlab;
   const int nchunks = (ov.K + Kc - 1) / Kc;
   const size_t planes = (size_t)3 * S * ov.R * ldk * sizeof(__nv_bfloat16);
@@ -509,28 +870,25 @@ cudaError_t tc_split(const TcOperandView& ov, int S, TcOperand* out, void* buf, 
   return cudaGetLastError();
 }
 
-cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long ldo, double alpha, int accumulate,
-                     cplx* part, size_t part_elems, int* err, cudaStream_t s) {
+cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long rso, long long ldo, double alpha,
+                     int accumulate, cplx* part, size_t part_elems, int* err, cudaStream_t s) {
   if (A.K != B.K || A.S != B.S || A.nchunks != B.nchunks) return cudaErrorInvalidValue;
   const int M = A.R, N = B.R, K = A.K, S = A.S, nz = A.nchunks;
+  const bool wide = S == kWideDigits;
+  if (!wide && nz == 1 && rso != 1) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
   cudaError_t e = plane_map(&ma, static_cast<const __nv_bfloat16*>(A.planes), K, A.ldk, M, 3 * S, kTcM);
   if (e == cudaSuccess) e = plane_map(&mb, static_cast<const __nv_bfloat16*>(B.planes), K, B.ldk, N, 3 * S, kTcN);
   if (e != cudaSuccess) return e;
-  const size_t smem = tc_smem_bytes(S);
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, []() {
-    attr = cudaFuncSetAttribute(tc_zgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tc_smem_bytes(kMaxDigits));
-  });
-  if (attr != cudaSuccess) return attr;
+  const size_t smem = wide ? wide_smem_bytes() : tc_smem_bytes(S);
+  e = allow_smem(wide ? (const void*)tc_zgemm_wide_kernel : (const void*)tc_zgemm_kernel, smem);
+  if (e != cudaSuccess) return e;
   TcArgs a{};
   a.M = M;
   a.N = N;
   a.K = K;
   a.S = S;
-  a.Kc = tc_chunk();
+  a.Kc = tc_chunk(S);
   a.nchunks = nz;
   a.eA = A.e;
   a.eB = B.e;
@@ -542,32 +900,38 @@ cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long lon
   if (am != 0.5) return cudaErrorInvalidValue;
   if (nz == 1) {
     a.out = out;
+    a.rso = rso;
     a.ldo = ldo;
     a.zstride = 0;
     a.alpha_exp = aexp - 1;
     a.alpha_neg = alpha < 0.0;
     a.accumulate = accumulate;
-    tc_zgemm_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
-    return cudaGetLastError();
+  } else {
+    if (!part || part_elems < (size_t)nz * M * N) return cudaErrorInvalidValue;
+    a.out = part;
+    a.rso = 1;
+    a.ldo = M;
+    a.zstride = (long long)M * N;
+    a.alpha_exp = 0;
+    a.alpha_neg = 0;
+    a.accumulate = 0;
   }
-  if (!part || part_elems < (size_t)nz * M * N) return cudaErrorInvalidValue;
-  a.out = part;
-  a.ldo = M;
-  a.zstride = (long long)M * N;
-  a.alpha_exp = 0;
-  a.alpha_neg = 0;
-  a.accumulate = 0;
-  tc_zgemm_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
+  if (wide) tc_zgemm_wide_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
+  else tc_zgemm_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || nz == 1) return e;
   const long long n = (long long)M * N;
-  reduce_parts_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, M, N, nz, (long long)M * N, alpha, accumulate,
-                                                                   out, ldo);
+  if (wide)
+    reduce_wide_kernel<<<(unsigned)((n + kRedOut - 1) / kRedOut), kRedOut * kRedZ, 0, s>>>(
+        part, M, N, nz, (long long)M * N, alpha, accumulate, out, rso, ldo);
+  else
+    reduce_parts_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(part, M, N, nz, (long long)M * N, alpha, accumulate,
+                                                                    out, rso, ldo);
   return cudaGetLastError();
 }
 
-size_t tc_part_elems(int M, int N, int K) {
-  const int nz = (K + tc_chunk() - 1) / tc_chunk();
+size_t tc_part_elems(int M, int N, int K, int S) {
+  const int nz = (K + tc_chunk(S) - 1) / tc_chunk(S);
   return nz > 1 ? (size_t)nz * M * N : 0;
 }
 
