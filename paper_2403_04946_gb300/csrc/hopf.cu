@@ -621,11 +621,10 @@ hopf_status tc_product(hopf_ctx* ctx, const hk::TcOperandView& a, const hk::TcOp
   unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
   hk::TcOperand oa, ob;
   const int slot = prof_begin(ctx);
-  CK(hk::tc_split(a, S, &oa, buf, ctx->stream));
-  CK(hk::tc_split(b, S, &ob, buf + ba, ctx->stream));
+  CK(hk::tc_split2(a, &oa, buf, b, &ob, buf + ba, S, ctx->stream));
   CK(hk::tc_zgemm(oa, ob, out, 1, ldo, 1.0, 0, np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr, np,
                   &ctx->coop.bar->err, ctx->stream));
-  prof_end(ctx, slot, HOPF_K_TC, flops, 0.0, np ? 4 : 3);
+  prof_end(ctx, slot, HOPF_K_TC, flops, 0.0, np ? 3 : 2);
   return HOPF_OK;
 }
 

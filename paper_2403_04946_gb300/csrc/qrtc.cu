@@ -243,16 +243,16 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     // G = V^H V (reflector s along rows, entries i along K)
     TcOperand oVH, oVB, oX, oV, oW2;
     slot = pt.b();
-    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 0, 2, 0}, S, &oVB, bVB, s);
+    e = tc_split2(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, &oVH, bVH,
+                  TcOperandView{Ap, lda, 1, nbk, mv, 0, 2, 0}, &oVB, bVB, S, s);
     cplx* G = Gout + (size_t)(j0 / kOuter) * kOuter * kOuter;
     if (e == cudaSuccess) e = tc_zgemm(oVH, oVB, G, 1, kOuter, 1.0, 0, part, npart, &cws.bar->err, s);
     if (e == cudaSuccess) {
       hermitize_kernel<<<(nbk * nbk + 255) / 256, 256, 0, s>>>(G, kOuter, nbk);
       e = cudaGetLastError();
     }
-    // launches: two splits, the product, its chunk reduction (K > one chunk), hermitize
-    pt.e(slot, pt.cls_tc, zflops(nbk, nbk, mv), 4 + (mv > Kc));
+    // launches: the splits, the product, its chunk reduction (K > one chunk), hermitize
+    pt.e(slot, pt.cls_tc, zflops(nbk, nbk, mv), 3 + (mv > Kc));
     if (e != cudaSuccess || nt <= 0) continue;
     // trailing columns: W = V^H A_t, W2 = T^H W, A_t -= V W2
     cplx* At = A + j0 + (size_t)lda * (j0 + nbk);
@@ -264,10 +264,11 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     if (e == cudaSuccess) e = wy_solve(G, kOuter, tau + j0, nbk, W, nbk, nt, W2, nbk, 1, packed, s);
     pt.e(slot, pt.cls_small, 0.0, 2);  // pack + solve
     slot = pt.b();
-    if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, S, &oW2, bW2, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    if (e == cudaSuccess)
+      e = tc_split2(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, &oW2, bW2,
+                  TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, &oV, bV, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oV, oW2, At, 1, lda, -1.0, 1, nullptr, 0, &cws.bar->err, s);
-    pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 3);  // two splits, one chunk
+    pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 2);  // the splits, one chunk
   }
   return e;
 }
@@ -295,19 +296,20 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
     if (!c.ok) return cudaErrorInvalidValue;
     TcOperand oVH, oX, oV, oW2;
     int slot = pt.b();
-    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, S, &oX, bX, s);
+    e = tc_split2(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, &oVH, bVH,
+                  TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, &oX, bX, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oVH, oX, W, 1, nbk, 1.0, 0, part, npart, err, s);
-    pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 3 + (mv > Kc));
+    pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 2 + (mv > Kc));
     slot = pt.b();
     if (e == cudaSuccess)
       e = wy_solve(Gin + (size_t)j * kOuter * kOuter, kOuter, tau + j0, nbk, W, nbk, q, W2, nbk, 0, packed, s);
     pt.e(slot, pt.cls_small, 0.0, 2);
     slot = pt.b();
-    if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, S, &oW2, bW2, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    if (e == cudaSuccess)
+      e = tc_split2(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, &oW2, bW2,
+                  TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, &oV, bV, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oV, oW2, Cj, 1, ldc, -1.0, 1, nullptr, 0, err, s);
-    pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 3);
+    pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 2);
   }
   return e;
 }
@@ -316,50 +318,56 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
 namespace {
 
 constexpr int kWidePanel = 32;
-constexpr int kWy64Warps = 4;
 
 // W2 = T^H W (forward) or T W (backward) for a panel of at most 32 reflectors
 // with Gram g (v_s^H v_u at g[s + nbk u]) and tau (NULL: g holds the panel's
 // record instead, the strict upper triangle of the Gram with tau on the
-// diagonal); one warp per column, a chain of nbk steps in FP64.  rec (may be
-// NULL) receives the record.
-__global__ void __launch_bounds__(32 * kWy64Warps)
+// diagonal).  With t_s = conj(tau_s) (forward) or tau_s,
+//   w2_s = t_s W_s - sum_u (t_s Gram[s, u]) w2_u
+// over the u before s (forward) or after it: one warp per column, the scaled
+// Gram in shared memory, so that a step of the chain is one exchange and one
+// complex multiply-add.  One warp per CTA: the chain is what bounds it, and
+// four warps on one SM's FP64 unit would wait for each other (18.5 us with
+// four and the scaling inside the chain).  rec (may be NULL) receives the
+// record.
+constexpr int kWy64Cols = 1;  // columns (warps) per CTA
+__global__ void __launch_bounds__(32 * kWy64Cols)
 wy_solve64_kernel(const cplx* __restrict__ g, const cplx* __restrict__ tau, int nbk, const cplx* __restrict__ W, int nt,
                   cplx* __restrict__ W2, int forward, cplx* __restrict__ rec) {
-  __shared__ cplx ts[kWidePanel * kWidePanel];
-  for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
-    const int u = e % nbk, c = e / nbk;
-    const cplx v = u < c ? g[e] : (u == c ? (tau ? tau[c] : g[e]) : mk(0, 0));
-    ts[e] = v;
-    if (rec && blockIdx.x == 0) rec[e] = v;
+  // m[u * 33 + s] = -t_s Gram[s, u] for the pairs of the chain, else zero
+  __shared__ cplx m[kWidePanel * (kWidePanel + 1)];
+  const int lane = threadIdx.x & 31, l = blockIdx.x * kWy64Cols + (threadIdx.x >> 5);
+  const bool in = lane < nbk;
+  const cplx tl = in ? (tau ? tau[lane] : g[lane + nbk * lane]) : mk(0, 0);
+  const cplx t = forward ? cconj(tl) : tl;
+  for (int u = threadIdx.x >> 5; u < nbk; u += kWy64Cols) {
+    // stored pair (min, max): Gram[s, u] itself for s < u, its conjugate else
+    const int lo = min(lane, u), hi = max(lane, u);
+    const bool pair = in && (forward ? lane > u : lane < u);
+    cplx v = mk(0, 0);
+    if (pair) {
+      const cplx q = cmul(t, forward ? cconj(g[lo + nbk * hi]) : g[lo + nbk * hi]);
+      v = mk(-q.x, -q.y);
+    }
+    m[u * (kWidePanel + 1) + lane] = v;
+    if (rec && blockIdx.x == 0 && in) rec[lane + nbk * u] = lane < u ? g[lane + nbk * u] : (lane == u ? tl : mk(0, 0));
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, l = blockIdx.x * kWy64Warps + (threadIdx.x >> 5);
   if (l >= nt) return;
-  const bool in = lane < nbk;
-  cplx acc = in ? W[lane + (size_t)nbk * l] : mk(0, 0), mine = mk(0, 0);
-  const cplx own = in ? ts[lane + nbk * lane] : mk(0, 0);
-  const cplx tl = forward ? cconj(own) : own;
+  cplx acc = in ? cmul(t, W[lane + (size_t)nbk * l]) : mk(0, 0);
   for (int step = 0; step < nbk; ++step) {
     const int u = forward ? step : nbk - 1 - step;
-    const cplx wu = cmul(tl, acc);  // valid on lane u
-    const cplx w2 = mk(__shfl_sync(0xffffffffu, wu.x, u), __shfl_sync(0xffffffffu, wu.y, u));
-    if (lane == u) mine = w2;
-    // forward: Gram[lane, u] = conj(Gram[u, lane]), lane > u
-    if (forward) {
-      if (lane > u && in) acc = csub(acc, cmulc(ts[u + nbk * lane], w2));
-    } else {
-      if (lane < u) acc = csub(acc, cmul(ts[lane + nbk * u], w2));
-    }
+    const cplx w = mk(__shfl_sync(0xffffffffu, acc.x, u), __shfl_sync(0xffffffffu, acc.y, u));
+    acc = cfma(m[u * (kWidePanel + 1) + lane], w, acc);
   }
-  if (in) W2[lane + (size_t)nbk * l] = mine;
+  if (in) W2[lane + (size_t)nbk * l] = acc;
 }
 
 cudaError_t wy_solve64(const cplx* g, const cplx* tau, int nbk, const cplx* W, int nt, cplx* W2, int forward, cplx* rec,
                        cudaStream_t s) {
   if (nt <= 0 && !rec) return cudaSuccess;
-  wy_solve64_kernel<<<std::max(1, (nt + kWy64Warps - 1) / kWy64Warps), 32 * kWy64Warps, 0, s>>>(g, tau, nbk, W, nt, W2,
-                                                                                               forward, rec);
+  wy_solve64_kernel<<<std::max(1, (nt + kWy64Cols - 1) / kWy64Cols), 32 * kWy64Cols, 0, s>>>(g, tau, nbk, W, nt, W2,
+                                                                                            forward, rec);
   return cudaGetLastError();
 }
 
@@ -412,10 +420,10 @@ cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void*
     // right (128 to a tile), the reflectors its 32 columns
     TcOperand oVH, oX, oV, oW2;
     slot = pt.b();
-    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, lda, 1, nbk + nt, mv, 0, 4, nbk}, S, &oX, bX, s);
+    e = tc_split2(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, &oVH, bVH,
+                  TcOperandView{Ap, lda, 1, nbk + nt, mv, 0, 4, nbk}, &oX, bX, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oX, oVH, GW, nbk, 1, 1.0, 0, part, npart, &cws.bar->err, s);
-    pt.e(slot, pt.cls_tc, zflops(nbk, nbk + nt, mv), 3 + (mv > Kc));
+    pt.e(slot, pt.cls_tc, zflops(nbk, nbk + nt, mv), 2 + (mv > Kc));
     slot = pt.b();
     cplx* rec = T ? T + (size_t)(j0 / kWidePanel) * kWidePanel * kWidePanel : nullptr;
     if (e == cudaSuccess) e = wy_solve64(GW, tau + j0, nbk, GW + (size_t)nbk * nbk, nt, W2, 1, rec, s);
@@ -423,10 +431,10 @@ cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void*
     if (e != cudaSuccess || nt <= 0) continue;
     cplx* At = A + j0 + (size_t)lda * (j0 + nbk);
     slot = pt.b();
-    e = tc_split(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, S, &oW2, bW2, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    e = tc_split2(TcOperandView{W2, nbk, 1, nt, nbk, 0, 0, 0}, &oW2, bW2,
+                  TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, &oV, bV, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oV, oW2, At, 1, lda, -1.0, 1, nullptr, 0, &cws.bar->err, s);
-    pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 3);
+    pt.e(slot, pt.cls_tc, zflops(mv, nt, nbk), 2);
   }
   return e;
 }
@@ -453,19 +461,20 @@ cudaError_t ormqr_wide(const cplx* A, int lda, int m, int p, const cplx* T, cplx
     if (!c.ok) return cudaErrorInvalidValue;
     TcOperand oVH, oX, oV, oW2;
     int slot = pt.b();
-    e = tc_split(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, S, &oVH, bVH, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, S, &oX, bX, s);
+    e = tc_split2(TcOperandView{Ap, lda, 1, nbk, mv, 1, 2, 0}, &oVH, bVH,
+                  TcOperandView{Cj, ldc, 1, q, mv, 0, 0, 0}, &oX, bX, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oX, oVH, W, nbk, 1, 1.0, 0, part, npart, err, s);
-    pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 3 + (mv > Kc));
+    pt.e(slot, pt.cls_tc, zflops(nbk, q, mv), 2 + (mv > Kc));
     slot = pt.b();
     if (e == cudaSuccess)
       e = wy_solve64(T + (size_t)j * kWidePanel * kWidePanel, nullptr, nbk, W, q, W2, 0, nullptr, s);
     pt.e(slot, pt.cls_small, 0.0, 1);
     slot = pt.b();
-    if (e == cudaSuccess) e = tc_split(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, S, &oW2, bW2, s);
-    if (e == cudaSuccess) e = tc_split(TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, S, &oV, bV, s);
+    if (e == cudaSuccess)
+      e = tc_split2(TcOperandView{W2, nbk, 1, q, nbk, 0, 0, 0}, &oW2, bW2,
+                  TcOperandView{Ap, 1, lda, mv, nbk, 0, 3, 0}, &oV, bV, S, s);
     if (e == cudaSuccess) e = tc_zgemm(oV, oW2, Cj, 1, ldc, -1.0, 1, nullptr, 0, err, s);
-    pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 3);
+    pt.e(slot, pt.cls_tc, zflops(mv, q, nbk), 2);
   }
   return e;
 }

@@ -559,6 +559,14 @@ struct SplitView {
   int R, K, conj;
   int tri_mode, tri;
 };
+// A view and where its digits go.
+struct SplitJob {
+  SplitView v;
+  int nchunks, row_ctas;  // K-chunks; CTAs along the rows
+  int* e;
+  __nv_bfloat16* planes;
+  long long ldk;
+};
 
 // What the view holds at an in-range (r, k): 0 the stored value, 1 zero
 // (outside the triangle), 2 one (the unit diagonal of a reflector block).
@@ -681,10 +689,19 @@ DV void digit_pair_wide(long long X0, long long X1, unsigned int* dst, size_t ps
 }
 
 __global__ void __launch_bounds__(kSplitThreads)
-    split_kernel(SplitView v, int Kc, int nchunks, int S, int* e, __nv_bfloat16* planes, long long ldk) {
+    split_kernel(SplitJob j0, SplitJob j1, int Kc, int S) {
   extern __shared__ cplx tile[];  // [kSplitRows][kSplitLd]
   __shared__ int esh[4][kSplitRows];  // components' exponents; one above max(|re|, |im|)
-  const int r0 = blockIdx.x * kSplitRows, z = blockIdx.y;
+  // the two jobs' CTAs one after the other
+  int blk = blockIdx.x;
+  const bool second = blk >= j0.row_ctas * j0.nchunks;
+  if (second) blk -= j0.row_ctas * j0.nchunks;
+  const SplitView v = second ? j1.v : j0.v;
+  const int nchunks = second ? j1.nchunks : j0.nchunks, row_ctas = second ? j1.row_ctas : j0.row_ctas;
+  int* e = second ? j1.e : j0.e;
+  __nv_bfloat16* planes = second ? j1.planes : j0.planes;
+  const long long ldk = second ? j1.ldk : j0.ldk;
+  const int r0 = (blk % row_ctas) * kSplitRows, z = blk / row_ctas;
   const int kb = z * Kc, klen = min(v.K - kb, Kc);
   const int tid = threadIdx.x;
   const int nval = kSplitRows * klen;
@@ -849,8 +866,7 @@ int tc_chunk(int S) { return S == kWideDigits ? kWideChunk : 3 * kSlab; }
 int tc_max_digits() { return kMaxDigits; }
 int tc_wide_digits() { return kWideDigits; }
 
-cudaError_t tc_split(const TcOperandView& ov, int S, TcOperand* out, void* buf, cudaStream_t s) {
-  if (S < 1 || (S > kMaxDigits && S != kWideDigits) || ov.R <= 0 || ov.K <= 0) return cudaErrorInvalidValue;
+static SplitJob split_job(const TcOperandView& ov, int S, TcOperand* out, void* buf) {
   const int Kc = tc_chunk(S);
   const long long ldk = ((long long)ov.K + kSlab - 1) / kSlab * kSlab;
   const int nchunks = (ov.K + Kc - 1) / Kc;
@@ -862,12 +878,29 @@ cudaError_t tc_split(const TcOperandView& ov, int S, TcOperand* out, void* buf, 
   out->S = S;
   out->ldk = ldk;
   out->nchunks = nchunks;
-  SplitView v{ov.X, ov.rs, ov.ks, ov.R, ov.K, ov.conj, ov.tri_mode, ov.tri};
-  const dim3 grid((ov.R + kSplitRows - 1) / kSplitRows, nchunks);
+  return SplitJob{SplitView{ov.X, ov.rs, ov.ks, ov.R, ov.K, ov.conj, ov.tri_mode, ov.tri}, nchunks,
+                  (ov.R + kSplitRows - 1) / kSplitRows, out->e, reinterpret_cast<__nv_bfloat16*>(buf), ldk};
+}
+
+// Two operands in one launch (a product's operands are split back to back, and
+// most of these launches are short).
+cudaError_t tc_split2(const TcOperandView& a, TcOperand* oa, void* bufa, const TcOperandView& b, TcOperand* ob, void* bufb,
+                      int S, cudaStream_t s) {
+  if (S < 1 || (S > kMaxDigits && S != kWideDigits) || a.R <= 0 || a.K <= 0 || b.R < 0 || (b.R > 0 && b.K <= 0))
+    return cudaErrorInvalidValue;
+  const SplitJob j0 = split_job(a, S, oa, bufa);
+  SplitJob j1{};
+  if (b.R > 0) j1 = split_job(b, S, ob, bufb);
+  const long long ctas = (long long)j0.row_ctas * j0.nchunks + (long long)j1.row_ctas * j1.nchunks;
+  if (ctas > 0x7fffffffll) return cudaErrorInvalidValue;
   cudaError_t e = allow_smem((const void*)split_kernel, split_smem_bytes());
   if (e != cudaSuccess) return e;
-  split_kernel<<<grid, kSplitThreads, split_smem_bytes(), s>>>(v, Kc, nchunks, S, out->e, reinterpret_cast<__nv_bfloat16*>(buf), ldk);
+  split_kernel<<<(unsigned)ctas, kSplitThreads, split_smem_bytes(), s>>>(j0, j1, tc_chunk(S), S);
   return cudaGetLastError();
+}
+
+cudaError_t tc_split(const TcOperandView& ov, int S, TcOperand* out, void* buf, cudaStream_t s) {
+  return tc_split2(ov, out, buf, TcOperandView{}, nullptr, nullptr, S, s);
 }
 
 cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long rso, long long ldo, double alpha,
