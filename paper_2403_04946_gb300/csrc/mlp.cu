@@ -9,7 +9,7 @@
 // leave: 24 significant bits, all of FP32's), so the sum of the part
 // products in one FP32 accumulator is the FP32-activation product up to
 // FP32 accumulation rounding.  Parts products below 2^-24 of the leading one
-// are skipped (pairs i + j > 2).  128 x 128 output tiles, the ensemble
+// are skipped (pairs i + j > 2).  128 x 128, 64 or 32 output tiles, the ensemble
 // members on gridDim.z, fused bias / GELU / GELU' epilogues.  A training
 // step is about thirty launches; it is captured once as a CUDA graph and
 // replayed, with the step number read from device memory so that the same
@@ -81,18 +81,23 @@ struct GemmArgs {
 };
 
 // ---- tensor-core products ----------------------------------------------------
-constexpr int kMmM = 128, kMmN = 128;   // output tile
+// Output tiles of 128 rows and NT = 128, 64 or 32 columns (mm_tile).  A tile is
+// bound by latency (the first slabs' loads, then the epilogue's stores), not by
+// its MMAs, so what counts is how many are in flight: the products of a
+// training step (128 x 256 x 256 per member) have 8 tiles of 128 columns and 32
+// of 32; a large batch has enough of the wide ones, which read A less often.
+// Shared memory is sized by the parts the product has, so that two or three
+// CTAs share an SM and one's loads run under another's epilogue.
+constexpr int kMmM = 128;
 constexpr int kMmParts = 3;             // BF16 parts of an FP32 operand
 constexpr int kMmThreads = 192;         // warps 0-3 epilogue, 4 TMA producer, 5 MMA issuer
 constexpr int kMmStages = 2;
-constexpr int kMmTmemCols = kMmN;       // one FP32 accumulator column per output column
-constexpr uint32_t kMmIdesc = hk::umma_idesc_bf16(kMmM, kMmN);
 static_assert(hk::kTmaSlab == 64, "one K slab is one 128-byte TMA box row");
 
 __host__ __device__ constexpr int mm_a_plane() { return kMmM * 64 * 2; }  // 16 KB
-__host__ __device__ constexpr int mm_b_plane() { return kMmN * 64 * 2; }  // 16 KB
-__host__ __device__ constexpr int mm_stage(int sa, int sb) { return sa * mm_a_plane() + sb * mm_b_plane(); }
-size_t mm_smem_bytes() { return (size_t)kMmStages * mm_stage(kMmParts, kMmParts) + 1024; }
+__host__ __device__ constexpr int mm_b_plane(int nt) { return nt * 64 * 2; }
+__host__ __device__ constexpr int mm_stage(int sa, int sb, int nt) { return sa * mm_a_plane() + sb * mm_b_plane(nt); }
+size_t mm_smem_bytes(int sa, int sb, int nt) { return (size_t)kMmStages * mm_stage(sa, sb, nt) + 1024; }
 
 // Parts of an operand view for the tensor cores: X(r, k) = X[e xme + r srow
 // + k sk] (FP32 or BF16) for r < R, k < K, written as S BF16 parts in
@@ -119,17 +124,19 @@ struct MmArgs {
   int M, N, nslab;  // output M x N, K in slabs of 64 (zero-padded)
   int SA, SB;       // parts of A and B
   int a_shared;     // every member reads member 0's A parts
+  int nt;           // columns of an output tile (also the tensor-memory columns)
+  int vec;          // C, H and Zp rows may be accessed 16 bytes at a time
   GemmArgs g;       // epilogue and output layout (A/B fields unused)
   int* err;         // expiry record of a bounded wait
 };
 
 // C(m, n) = sum_k A(m, k) B(n, k) for member e = blockIdx.z, over the part
 // pairs (i, j), i + j < max(SA, SB), all into one FP32 accumulator; one CTA
-// per 128 x 128 output tile.  Warp 4 streams the K slabs of the parts into
+// per 128 x nt output tile.  Warp 4 streams the K slabs of the parts into
 // a two-stage ring with TMA, warp 5 issues the MMAs, warps 0-3 read the
 // accumulator back (a thread per row) and apply the epilogue.  Waits are
 // bounded like those of the complex product kernel.
-__global__ void __launch_bounds__(kMmThreads, 1)
+__global__ void __launch_bounds__(kMmThreads)
     mlp_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, MmArgs a) {
   extern __shared__ unsigned char mm_smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kMmStages], empty_bar[kMmStages], acc_bar;
@@ -138,9 +145,10 @@ __global__ void __launch_bounds__(kMmThreads, 1)
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(mm_smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kMmM, n0 = blockIdx.x * kMmN, e = blockIdx.z;
+  const int NT = a.nt;
+  const int m0 = blockIdx.y * kMmM, n0 = blockIdx.x * NT, e = blockIdx.z;
   const int SA = a.SA, SB = a.SB, smax = SA > SB ? SA : SB;
-  const int sbytes = mm_stage(SA, SB);
+  const int sbytes = mm_stage(SA, SB, NT);
   if (threadIdx.x == 0) {
     for (int st = 0; st < kMmStages; ++st) {
       hk::mbar_init(&full_bar[st], 1);
@@ -152,7 +160,7 @@ __global__ void __launch_bounds__(kMmThreads, 1)
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(hk::smem_u32(&tmem_slot)),
-                 "r"(kMmTmemCols)
+                 "r"((uint32_t)NT)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -174,7 +182,7 @@ __global__ void __launch_bounds__(kMmThreads, 1)
         for (int j = 0; j < SA; ++j)
           hk::tma_load_3d(base + (size_t)j * mm_a_plane(), &mapA, &full_bar[slot], st * 64, m0, za + j);
         for (int j = 0; j < SB; ++j)
-          hk::tma_load_3d(base + (size_t)SA * mm_a_plane() + (size_t)j * mm_b_plane(), &mapB, &full_bar[slot], st * 64,
+          hk::tma_load_3d(base + (size_t)SA * mm_a_plane() + (size_t)j * mm_b_plane(NT), &mapB, &full_bar[slot], st * 64,
                           n0, zb + j);
         issued = st + 1;
       }
@@ -186,6 +194,7 @@ __global__ void __launch_bounds__(kMmThreads, 1)
     }
   } else if (warp == 5) {
     if (lane == 0) {
+      const uint32_t idesc = hk::umma_idesc_bf16(kMmM, NT);
       for (int st = 0; st < a.nslab; ++st) {
         const int slot = st % kMmStages;
         if (!hk::mbar_wait(&full_bar[slot], (st / kMmStages) & 1, vabort, a.err)) break;
@@ -199,8 +208,8 @@ __global__ void __launch_bounds__(kMmThreads, 1)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               const uint64_t ad = hk::sw128_desc(abase + (uint32_t)(i * mm_a_plane() + kk * 32));
-              const uint64_t bd = hk::sw128_desc(bbase + (uint32_t)(j * mm_b_plane() + kk * 32));
-              hk::umma(tmem, ad, bd, kMmIdesc, first ? 0u : 1u);
+              const uint64_t bd = hk::sw128_desc(bbase + (uint32_t)(j * mm_b_plane(NT) + kk * 32));
+              hk::umma(tmem, ad, bd, idesc, first ? 0u : 1u);
               first = false;
             }
           }
@@ -215,19 +224,42 @@ __global__ void __launch_bounds__(kMmThreads, 1)
     const GemmArgs& g = a.g;
     if (ok && !*vabort) {
 #pragma unroll 1
-      for (int h = 0; h < kMmN / 16; ++h) {
+      for (int h = 0; h < NT / 16; ++h) {
         float v[16];
         hk::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(16 * h), v);
-        if (m >= a.M) continue;
+        const int nb = n0 + 16 * h;
+        if (m >= a.M || nb >= a.N) continue;
+        float* crow = g.C + e * g.cme + (long long)m * g.ldc + nb;
+        float* hrow = g.epi == EPI_BIAS_GELU ? g.H + e * g.hme + (long long)m * g.ldh + nb : nullptr;
+        const float* zrow = g.epi == EPI_GELU_GRAD ? g.Zp + e * g.zpme + (long long)m * g.ldzp + nb : nullptr;
+        if (a.vec && nb + 16 <= a.N) {
+          // 16-byte accesses: a thread's row segment of 64 bytes in four
+#pragma unroll
+          for (int q = 0; q < 16; q += 4) {
+            float x[4] = {v[q], v[q + 1], v[q + 2], v[q + 3]};
+            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (zrow) z = *reinterpret_cast<const float4*>(zrow + q);
+            const float zz[4] = {z.x, z.y, z.z, z.w};
+            float y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              if (g.epi == EPI_BIAS || g.epi == EPI_BIAS_GELU) x[u] += g.bias[e * g.biasme + nb + q + u];
+              if (zrow) x[u] *= gelu_grad(zz[u]);
+              y[u] = hrow ? gelu(x[u]) : 0.f;
+            }
+            *reinterpret_cast<float4*>(crow + q) = make_float4(x[0], x[1], x[2], x[3]);
+            if (hrow) *reinterpret_cast<float4*>(hrow + q) = make_float4(y[0], y[1], y[2], y[3]);
+          }
+          continue;
+        }
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
-          const int n = n0 + 16 * h + q;
-          if (n >= a.N) continue;
+          if (nb + q >= a.N) continue;
           float x = v[q];
-          if (g.epi == EPI_BIAS || g.epi == EPI_BIAS_GELU) x += g.bias[e * g.biasme + n];
-          if (g.epi == EPI_GELU_GRAD) x *= gelu_grad(g.Zp[e * g.zpme + (long long)m * g.ldzp + n]);
-          g.C[e * g.cme + (long long)m * g.ldc + n] = x;
-          if (g.epi == EPI_BIAS_GELU) g.H[e * g.hme + (long long)m * g.ldh + n] = gelu(x);
+          if (g.epi == EPI_BIAS || g.epi == EPI_BIAS_GELU) x += g.bias[e * g.biasme + nb + q];
+          if (zrow) x *= gelu_grad(zrow[q]);
+          crow[q] = x;
+          if (hrow) hrow[q] = gelu(x);
         }
       }
     }
@@ -236,19 +268,29 @@ __global__ void __launch_bounds__(kMmThreads, 1)
   __syncthreads();
   if (warp == 0) {
     hk::tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMmTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)NT) : "memory");
   }
 }
 
-// db[e][n] = sum_m G[e][m][n] (bias gradient; one thread per column).
-__global__ void colsum_kernel(const float* G, long long ldg, long long gme, int M, int N, float* db,
-                              long long dbme) {
-  const int e = blockIdx.y;
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  const float* g = G + e * gme + n;
+// db[e][n] = sum_m G[e][m][n] (bias gradient): 32 columns x 8 row groups per
+// CTA, the groups' sums added in order (one thread per column walked all rows
+// with one load in flight).
+constexpr int kCsN = 32, kCsM = 8;
+__global__ void __launch_bounds__(kCsN* kCsM)
+    colsum_kernel(const float* G, long long ldg, long long gme, int M, int N, float* db, long long dbme) {
+  __shared__ float part[kCsM][kCsN];
+  const int e = blockIdx.y, c = threadIdx.x % kCsN, r = threadIdx.x / kCsN;
+  const int n = blockIdx.x * kCsN + c;
   float s = 0.f;
-  for (int m = 0; m < M; ++m) s += g[m * ldg];
+  if (n < N) {
+    const float* g = G + e * gme + n;
+#pragma unroll 4
+    for (int m = r; m < M; m += kCsM) s += g[m * ldg];
+  }
+  part[r][c] = s;
+  __syncthreads();
+  if (r != 0 || n >= N) return;
+  for (int i = 1; i < kCsM; ++i) s += part[i][c];
   db[e * dbme + n] = s;
 }
 
@@ -301,18 +343,19 @@ __global__ void loss_kernel(const float* Y, long long yme, const float* T, long 
   }
 }
 
-// Adam on the FP32 master parameters; refreshes the BF16 copies.  counter:
-// [0] step of this call (learning-rate table index), [1] steps taken so far.
-__global__ void adam_kernel(float* w, float* m, float* v, const float* g, bf16* wb, long long total,
-                            const float* lr_tab, const int* counter) {
-  __shared__ float sc[3];
-  if (threadIdx.x == 0) {
-    const int t = counter[1] + 1;
-    sc[0] = lr_tab[counter[0]];
-    sc[1] = (float)(1.0 - pow((double)kBeta1, (double)t));
-    sc[2] = (float)(1.0 - pow((double)kBeta2, (double)t));
-  }
-  __syncthreads();
+// Learning rate and bias corrections of the coming Adam step, once per step
+// (two FP64 powers, which every CTA of the update otherwise waited for: 31 us
+// of its 31).  counter: [0] step of this call (learning-rate table index),
+// [1] steps taken so far.
+__global__ void adam_scalars_kernel(const float* lr_tab, const int* counter, float* sc) {
+  const int t = counter[1] + 1;
+  sc[0] = lr_tab[counter[0]];
+  sc[1] = (float)(1.0 - pow((double)kBeta1, (double)t));
+  sc[2] = (float)(1.0 - pow((double)kBeta2, (double)t));
+}
+
+// Adam on the FP32 master parameters; refreshes the BF16 copies.
+__global__ void adam_kernel(float* w, float* m, float* v, const float* g, bf16* wb, long long total, const float* sc) {
   const float lr = sc[0], bc1 = sc[1], bc2 = sc[2];
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < total;
        j += (long long)gridDim.x * blockDim.x) {
@@ -440,6 +483,7 @@ struct hopf_mlp {
   std::vector<float*> X, Z;    // per layer [members][max_batch][width]
   float *G0 = nullptr, *G1 = nullptr, *T = nullptr;
   int* counter = nullptr;      // [2]
+  float* adam_sc = nullptr;    // [3]: learning rate, bias corrections
   double* stats = nullptr;     // [2 (n_in + n_out)]
   bool have_stats = false;
   double *xd = nullptr, *yd = nullptr;
@@ -507,7 +551,8 @@ cudaError_t mm_prepare() {
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, []() {
-    attr = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mm_smem_bytes());
+    attr = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)mm_smem_bytes(kMmParts, kMmParts, 128));
   });
   return attr;
 }
@@ -523,6 +568,19 @@ void parts_sizes(const hopf_mlp_params& p, const std::vector<int>& dims, size_t*
   const size_t a1 = (size_t)mb * rup64(dmax), a2 = (size_t)dmax * rup64(mb);
   *pa = (size_t)p.members * kMmParts * std::max(a1, a2);
   *pb = (size_t)p.members * kMmParts * (size_t)dmax * rup64(std::max<long long>(mb, dmax));
+}
+
+// Widest tile that still gives the device two tiles per SM.
+int mm_tile(int M, int N, int members) {
+  static const int sms = []() {
+    int dev = 0, n = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  }();
+  for (int nt = 128; nt > 32; nt >>= 1)
+    if ((long long)((M + kMmM - 1) / kMmM) * ((N + nt - 1) / nt) * members >= 2 * sms) return nt;
+  return 32;
 }
 
 // C = A B (GemmArgs layout) on the tensor cores: the operands are cut into
@@ -551,8 +609,9 @@ cudaError_t launch_gemm(hopf_mlp* mm, const GemmArgs& g, int members) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap mapA, mapB;
+  const int nt = mm_tile(M, N, members);
   e = hk::plane_map(&mapA, mm->pa, ldk, ldk, M, ma * SA, kMmM);
-  if (e == cudaSuccess) e = hk::plane_map(&mapB, mm->pb, ldk, ldk, N, members * SB, kMmN);
+  if (e == cudaSuccess) e = hk::plane_map(&mapB, mm->pb, ldk, ldk, N, members * SB, nt);
   if (e != cudaSuccess) return e;
   MmArgs args{};
   args.M = M;
@@ -561,10 +620,15 @@ cudaError_t launch_gemm(hopf_mlp* mm, const GemmArgs& g, int members) {
   args.SA = SA;
   args.SB = SB;
   args.a_shared = a_shared;
+  args.nt = nt;
+  auto aligned = [](const void* p, long long ld, long long me) {
+    return !p || (reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld % 4 == 0 && me % 4 == 0);
+  };
+  args.vec = aligned(g.C, g.ldc, g.cme) && aligned(g.H, g.ldh, g.hme) && aligned(g.Zp, g.ldzp, g.zpme);
   args.g = g;
   args.err = hopf_internal_wait_record(mm->ctx);
-  const dim3 grid((N + kMmN - 1) / kMmN, (M + kMmM - 1) / kMmM, members);
-  mlp_tc_kernel<<<grid, kMmThreads, mm_smem_bytes(), s>>>(mapA, mapB, args);
+  const dim3 grid((N + nt - 1) / nt, (M + kMmM - 1) / kMmM, members);
+  mlp_tc_kernel<<<grid, kMmThreads, mm_smem_bytes(SA, SB, nt), s>>>(mapA, mapB, args);
   return cudaGetLastError();
 }
 
@@ -631,7 +695,7 @@ cudaError_t backward(hopf_mlp* mm, int batch) {
     a.cme = P;
     cudaError_t e = launch_gemm(mm, a, mm->p.members);
     if (e != cudaSuccess) return e;
-    colsum_kernel<<<dim3((fo + 255) / 256, mm->p.members), 256, 0, mm->s>>>(Gc, fo, gme, batch, fo,
+    colsum_kernel<<<dim3((fo + kCsN - 1) / kCsN, mm->p.members), kCsN * kCsM, 0, mm->s>>>(Gc, fo, gme, batch, fo,
                                                                             mm->g + mm->boff[l], P);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (l == 0) break;
@@ -679,8 +743,9 @@ cudaError_t train_step(hopf_mlp* mm, int batch, const int* idx, float* loss, boo
   if ((e = backward(mm, batch)) != cudaSuccess) return e;
   if (!update) return cudaSuccess;
   const long long total = (long long)M * mm->P;
-  adam_kernel<<<blocks_for(total, 256, 2048), 256, 0, mm->s>>>(mm->w, mm->m, mm->v, mm->g, mm->wb, total, mm->lr,
-                                                                mm->counter);
+  adam_scalars_kernel<<<1, 1, 0, mm->s>>>(mm->lr, mm->counter, mm->adam_sc);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  adam_kernel<<<blocks_for(total, 256, 2048), 256, 0, mm->s>>>(mm->w, mm->m, mm->v, mm->g, mm->wb, total, mm->adam_sc);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   step_counter_kernel<<<1, 1, 0, mm->s>>>(mm->counter);
   return cudaGetLastError();
@@ -780,6 +845,7 @@ hopf_status hopf_mlp_create(hopf_ctx* ctx, const hopf_mlp_params* p, const float
     if (e == cudaSuccess) e = malloc_track(mm, &mm->G1, (size_t)M * mb * mm->gmax);
     if (e == cudaSuccess) e = malloc_track(mm, &mm->T, (size_t)M * mb * p->n_out);
     if (e == cudaSuccess) e = malloc_track(mm, &mm->counter, 2);
+    if (e == cudaSuccess) e = malloc_track(mm, &mm->adam_sc, 3);
     if (e == cudaSuccess) e = malloc_track(mm, &mm->stats, (size_t)2 * (p->n_in + p->n_out));
     if (e == cudaSuccess) e = malloc_track(mm, &mm->qx, (size_t)mb * p->n_in);
     if (e == cudaSuccess) e = malloc_track(mm, &mm->qy, (size_t)mb * p->n_out);
