@@ -1046,27 +1046,17 @@ hopf_status orth_sweep_apply(hopf_ctx* ctx, const hopf_tt* X, std::vector<int>& 
     const int rl = r[c - 1];
     const size_t blk = (size_t)rl * n * p[c];
     if (use_tc(ctx, rl * n, 64)) {
-      // the six products on the tensor cores: X_{c-1} (rl n x r) split once,
-      // each block of R^H (conjugated, upper trapezoid) split in turn
-      const int S = product_digits(ctx), Kc = hk::tc_chunk(S);
-      const size_t ba = (hk::tc_operand_bytes(rl * n, r[c], S, Kc) + 255) & ~(size_t)255;
-      const size_t bb = (hk::tc_operand_bytes(p[c], r[c], S, Kc) + 255) & ~(size_t)255;
-      const size_t np = hk::tc_part_elems(rl * n, p[c], r[c], S);
-      TRY(tc_reserve_bytes(ctx, ba + bb + np * sizeof(cplx) + 256));
-      unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
-      cplx* part = np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr;
-      hk::TcOperand oX, oR;
-      int slot = prof_begin(ctx);
-      CK(hk::tc_split(hk::TcOperandView{X->cores[c - 1], 1, (long long)rl * n, rl * n, r[c], 0, 0, 0}, S, &oX, buf,
-                      ctx->stream));
-      prof_end(ctx, slot, HOPF_K_TC, 0.0, 0.0, 1);
-      for (int be = 0; be < 6; ++be) {
-        slot = prof_begin(ctx);
-        CK(hk::tc_split(hk::TcOperandView{w.B[c] + (size_t)m * be * r[c], 1, m, p[c], r[c], 1, 1, be * r[c]}, S,
-                        &oR, buf + ba, ctx->stream));
-        CK(hk::tc_zgemm(oX, oR, w.W1 + be * blk, 1, rl * n, 1.0, 0, part, np, &ctx->coop.bar->err, ctx->stream));
-        prof_end(ctx, slot, HOPF_K_TC, rblk_flops((double)rl * n, r[c], p[c], be * r[c]), 0.0, np ? 3 : 2);
-      }
+      // the six products on the tensor cores as one: the blocks of R^H
+      // (conjugated, upper trapezoid) are row groups of the right operand, and
+      // the results T_beta lie one after another (six products of 30 to 80 us
+      // and as many splits were short launches each)
+      double flops = 0.0;
+      for (int be = 0; be < 6; ++be) flops += rblk_flops((double)rl * n, r[c], p[c], be * r[c]);
+      hk::TcOperandView vr{w.B[c], 1, m, 6 * p[c], r[c], 1, 5, r[c]};
+      vr.group = p[c];
+      vr.gs = (long long)m * r[c];
+      TRY(tc_product(ctx, hk::TcOperandView{X->cores[c - 1], 1, (long long)rl * n, rl * n, r[c], 0, 0, 0}, vr, w.W1,
+                     (long long)rl * n, flops));
     } else {
       for (int be = 0; be < 6; ++be) {
         LAUNCH(HOPF_K_GEMM, rblk_flops((double)rl * n, r[c], p[c], be * r[c]), 0, 1,

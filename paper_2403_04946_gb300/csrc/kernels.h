@@ -247,12 +247,16 @@ cudaError_t check_finite(const cplx* x, size_t count, int* flag, cudaStream_t s)
 // Householder reflectors s and columns their entries i, zero where
 // k < r + tri, one where k == r + tri; 3: the same reflectors with rows i and
 // columns s (zero where r < k + tri, one where r == k + tri); 4: the first
-// tri rows are reflectors as in mode 2 (with tri = 0), the others stored.
+// tri rows are reflectors as in mode 2 (with tri = 0), the others stored; 5:
+// rows in groups of `group`, row i of group g at X + i rs + g gs, zero where
+// i > k + g tri.
 struct TcOperandView {
   const cplx* X;
   long long rs, ks;
   int R, K, conj;
   int tri_mode, tri;
+  int group = 0;     // 0: no groups
+  long long gs = 0;
 };
 // Digit planes of an operand split for the tensor cores: 3 components
 // (re, im, re + im) x S digits, each R x ldk BF16 (K contiguous), and the

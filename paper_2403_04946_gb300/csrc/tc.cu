@@ -503,8 +503,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
     if (ok && !*vabort) {
+      // the values an accumulating product adds to, two to four columns ahead (each
+      // column's own load would otherwise wait out an L2 round trip: 16 us
+      // of a tile's 26)
+      cplx pre[2][2];
+      auto prefetch = [&](int h) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int n = n0 + 16 * half + 2 * h + q;
+          pre[h & 1][q] = (a.accumulate && m < a.M && n < a.N) ? out[(size_t)a.rso * m + (size_t)a.ldo * n] : mk(0, 0);
+        }
+      };
+      prefetch(0);
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
+        if (q % 2 == 0 && q < 14) prefetch(q / 2 + 1);
         const int n = n0 + 16 * half + q;
         if (m >= a.M || n >= a.N) continue;
         // all three at one unit, the largest at bit 60 (a zero product has no
@@ -537,9 +550,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int Es = top - 114 + a.alpha_exp;
         cplx r = mk(int_scaled(re, Es), int_scaled(im, Es));
         if (max(ex[0], max(ex[1], ex[2])) > kNotFinite / 2) r = mk(__longlong_as_double(-1ll), __longlong_as_double(-1ll));
-        cplx* p = out + (size_t)a.rso * m + (size_t)a.ldo * n;
-        if (a.accumulate) r = cadd(*p, r);
-        *p = r;
+        if (a.accumulate) r = cadd(pre[(q / 2) & 1][q % 2], r);
+        out[(size_t)a.rso * m + (size_t)a.ldo * n] = r;
       }
     }
   }
@@ -558,6 +570,8 @@ struct SplitView {
   long long rs, ks;
   int R, K, conj;
   int tri_mode, tri;
+  int group;        // rows per group (R: one group)
+  long long gs;     // elements between groups
 };
 // A view and where its digits go.
 struct SplitJob {
@@ -572,6 +586,9 @@ struct SplitJob {
 // (outside the triangle), 2 one (the unit diagonal of a reflector block).
 DV int view_kind(const SplitView& v, int r, int k) {
   if (v.tri_mode == 1) return r > k + v.tri ? 1 : 0;
+  // rows in groups: row i of group g is row i of an upper trapezoid's columns
+  // from g tri on
+  if (v.tri_mode == 5) return r % v.group > k + v.tri * (r / v.group) ? 1 : 0;
   // reflector s = r (rows of the view are reflector indices), entry i = k:
   // zero above the unit diagonal k < r + tri, one on it
   if (v.tri_mode == 2) return k < r + v.tri ? 1 : (k == r + v.tri ? 2 : 0);
@@ -717,7 +734,12 @@ __global__ void __launch_bounds__(kSplitThreads)
     }
     cplx* dst = tile + r * kSplitLd + k;
     const int kind = (r0 + r < v.R) ? view_kind(v, r0 + r, kb + k) : 1;
-    if (kind == 0) cp_async16(dst, v.X + (long long)(r0 + r) * v.rs + (long long)(kb + k) * v.ks);
+    if (kind == 0) {
+      const cplx* src = v.X + (long long)(kb + k) * v.ks;
+      src += v.group < v.R ? (long long)((r0 + r) % v.group) * v.rs + (long long)((r0 + r) / v.group) * v.gs
+                           : (long long)(r0 + r) * v.rs;
+      cp_async16(dst, src);
+    }
     else *dst = mk(kind == 2 ? 1.0 : 0.0, 0.0);
   }
   if ((klen & 1) && tid < kSplitRows) tile[tid * kSplitLd + klen] = mk(0, 0);  // second value of the last pair
@@ -878,7 +900,9 @@ static SplitJob split_job(const TcOperandView& ov, int S, TcOperand* out, void* 
   out->S = S;
   out->ldk = ldk;
   out->nchunks = nchunks;
-  return SplitJob{SplitView{ov.X, ov.rs, ov.ks, ov.R, ov.K, ov.conj, ov.tri_mode, ov.tri}, nchunks,
+  return SplitJob{SplitView{ov.X, ov.rs, ov.ks, ov.R, ov.K, ov.conj, ov.tri_mode, ov.tri,
+                            ov.group > 0 ? ov.group : ov.R, ov.gs},
+                  nchunks,
                   (ov.R + kSplitRows - 1) / kSplitRows, out->e, reinterpret_cast<__nv_bfloat16*>(buf), ldk};
 }
 
