@@ -884,11 +884,18 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
   if (MIXED) rows_to_fp64(C, ldc, r0, r1, 0, q, E);
 }
 
-static void pick_layout(int m, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {
+// CTAs of a factorisation: 8 rows each until every SM has one.  A column costs
+// the CTAs their rows' multiply-adds (8 per row and remaining column, on an
+// FP64 unit of 2 per clock) and the sum over the CTAs' partials; the first
+// outweighs the second down to a few rows.  With 64 rows per CTA, 16 CTAs at
+// least (what it was): a C1 step (336 x 96 factors) 68 ms against 52 ms with 8
+// rows, 53 with 16, 60 with 32; the 942 x 768 factors of the CDF workload ran on 16
+// CTAs, 437 against 310 ms a step.  Mixed precision keeps 64 rows from 2048
+// rows on: there the order of the sums shows in its digit-cut products.
+static void pick_layout(int m, int mixed, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {
   const DevInfo& di = dev_info();
-  // row blocks of >= 64 rows, but small matrices (the wide first and last
-  // cores) still spread over up to 16 CTAs of >= 8 rows
-  int g = std::max(1, std::min(coop_sms(ws), std::max((m + 63) / 64, std::min(16, (m + 7) / 8))));
+  const int rows = mixed && m >= 2048 ? 64 : 8;
+  const int g = std::max(1, std::min(coop_sms(ws), (m + rows - 1) / rows));
   int r = (m + g - 1) / g;
   int b = kNbMax;
   const size_t lim = (size_t)di.max_smem_optin - 16384;  // static shared memory too
@@ -904,7 +911,7 @@ cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_ou
   if (m <= 0 || k <= 0) return cudaSuccess;
   int G, R, nb;
   size_t smem;
-  pick_layout(m, ws, &G, &R, &nb, &smem);
+  pick_layout(m, mixed, ws, &G, &R, &nb, &smem);
   // per CTA: S1 partials nb (nb + k), then the panel's exchange tail 4 nb
   if ((size_t)G * ((size_t)nb * (nb + k) + 4 * (size_t)nb) > ws.pc_elems || (size_t)nb * (nb + k) > ws.wfin_elems)
     return cudaErrorInvalidValue;
@@ -934,7 +941,7 @@ cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const c
   if (m <= 0 || p <= 0 || q <= 0) return cudaSuccess;
   int G, R, nb2;
   size_t smem;
-  pick_layout(m, ws, &G, &R, &nb2, &smem);
+  pick_layout(m, mixed, ws, &G, &R, &nb2, &smem);
   if (nb2 != nb) {
     // the layout depends only on m, so geqrf and ormqr agree
     return cudaErrorInvalidValue;
