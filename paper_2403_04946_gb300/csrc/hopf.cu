@@ -920,7 +920,13 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
       } else {
         int nbl = 32;
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Rb, pp, pp, cols, w.Mb, cols, ctx->stream));
-        LAUNCH(HOPF_K_SVD, qr_flops(cols, pp), 0, 1, hk::geqrf(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, w.T + (size_t)c * w.tstride, &nbl, ctx->coop, ctx->stream, 0));
+        if (hk::qr_wide_applies(cols, pp)) {
+          TRY(tc_reserve_bytes(ctx, hk::qr_wide_scratch_bytes(cols, pp)));
+          CK(hk::geqrf_wide(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, nullptr, ctx->tcbuf, ctx->tcbytes, ctx->coop, 0,
+                            ctx->stream, phase_timer(ctx, HOPF_K_SVD)));
+        } else {
+          LAUNCH(HOPF_K_SVD, qr_flops(cols, pp), 0, 1, hk::geqrf(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, w.T + (size_t)c * w.tstride, &nbl, ctx->coop, ctx->stream, 0));
+        }
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::extract_r(w.Mb, cols, pp, pp, w.Jb, pp, ctx->stream));
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Jb, pp, pp, pp, w.Mb, pp, ctx->stream));
       }

@@ -889,8 +889,8 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
 // FP64 unit of 2 per clock) and the sum over the CTAs' partials; the first
 // outweighs the second down to a few rows.  With 64 rows per CTA, 16 CTAs at
 // least (what it was): a C1 step (336 x 96 factors) 68 ms against 52 ms with 8
-// rows, 53 with 16, 60 with 32; the 942 x 768 factors of the CDF workload ran on 16
-// CTAs, 437 against 310 ms a step.  Mixed precision keeps 64 rows from 2048
+// rows, 53 with 16, 60 with 32; the CDF workload's factors (64 to 942 rows, up to 942
+// columns) ran on 16 CTAs, 437 against 310 ms a step.  Mixed precision keeps 64 rows from 2048
 // rows on: there the order of the sums shows in its digit-cut products.
 static void pick_layout(int m, int mixed, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {
   const DevInfo& di = dev_info();

@@ -373,11 +373,14 @@ cudaError_t wy_solve64(const cplx* g, const cplx* tau, int nbk, const cplx* W, i
 
 }  // namespace
 
-// The panel kernel's trailing update costs 16 m 32 FP64 operations per
-// trailing column on all SMs together (1.1 TFLOP/s), the products about 60 us
-// per panel in launches whatever the size: from 2048 rows and a few panels on
-// the products are ahead.
-bool qr_wide_applies(int m, int p) { return m >= 2048 && p > kWidePanel; }
+// The panel kernel's own trailing update costs 16 m 32 FP64 operations per
+// trailing column on all SMs together (1.1 TFLOP/s), the products about 100 us
+// per panel in launches whatever the size.  Measured with both sides: from
+// 2048 rows the products are ahead as soon as there is a second panel, from
+// 1024 rows with two full panels (C2 steps 351 -> 345 ms, C3 278 -> 263 ms, the CDF
+// workload's LQ factors 311 -> 265 ms); below that the C1 factors (336 x 96)
+// are faster on the kernel alone.
+bool qr_wide_applies(int m, int p) { return (m >= 2048 && p > kWidePanel) || (m >= 1024 && p >= 2 * kWidePanel); }
 
 size_t qr_wide_scratch_bytes(int m, int k) {
   const int S = tc_wide_digits(), Kc = tc_chunk(S), nb = kWidePanel;

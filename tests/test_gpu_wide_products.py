@@ -1,7 +1,7 @@
 """FP64 roundings whose tall factors take the digit products (2048 rows and
-more than 32 columns): row counts at the threshold and between K-chunks,
-column counts with a remainder in the last panel, magnitudes graded over the
-columns.
+more than 32 columns, or 1024 rows and 64 columns): row counts at the threshold
+and between K-chunks, column counts with a remainder in the last panel,
+magnitudes graded over the columns, a wide factor through its LQ.
 
 At tol = 0 the rounding keeps every value, so the tensor must come back and
 every core but the last must be left-orthonormal.  The products are accurate
@@ -24,7 +24,8 @@ def B():
 
 
 @pytest.mark.parametrize("graded", [False, True])
-@pytest.mark.parametrize("n,r1,r2", [(64, 33, 32), (64, 64, 33), (66, 100, 37), (130, 97, 64), (64, 50, 31)])
+@pytest.mark.parametrize("n,r1,r2", [(64, 33, 32), (64, 64, 33), (66, 100, 37), (130, 97, 64), (64, 50, 31),
+                                     (32, 64, 32), (34, 70, 31)])
 def test_fp64_rounding_through_the_digit_products(B, n, r1, r2, graded):
     d = 4
     ranks = [1, min(n, r1), r1, r2, 1]
@@ -40,6 +41,20 @@ def test_fp64_rounding_through_the_digit_products(B, n, r1, r2, graded):
     for C in got[:-1]:
         V = tt.V(C)
         assert np.abs(V.conj().T @ V - np.eye(V.shape[1])).max() < 1e-12
+    ctx.tt_free(t)
+    ctx.close()
+
+
+def test_wide_factor_through_its_lq(B):
+    """Bond 1 of rank 1100 at n = 80: the first flattening is 80 x 1100, its LQ a
+    QR of 1100 x 80."""
+    n = 80
+    x = synthetic.random_tt_cores(3, n, [1, 1100, 30, 1], seed=2)
+    ctx = B.Context(d=3, n=n, nu=0.02, tol=0.0, rank_cap=1100, L=4.0)
+    t = ctx.tt_from_host(x, max_rank=1100)
+    ctx.tt_round(t, 0.0, 1100, forced_ranks=[1, n, 30, 1])
+    got = ctx.tt_to_host(t)
+    assert tt.diff_norm(got, x) < 1e-12 * tt.norm(x)
     ctx.tt_free(t)
     ctx.close()
 
