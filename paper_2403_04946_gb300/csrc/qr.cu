@@ -246,20 +246,24 @@ __device__ void update_x_f(const df2* P, int R, int r0, int lo, int hi, int nbk,
 __device__ void rows_to_df(cplx* A, int lda, int r0, int r1, int c0, int c1, int E) {
   const int nr = r1 - r0;
   if (nr <= 0) return;
-  for (long long e = threadIdx.x; e < (long long)nr * (c1 - c0); e += blockDim.x) {
-    const int c = c0 + (int)(e / nr), i = r0 + (int)(e % nr);
-    cplx* p = A + i + (size_t)lda * c;
-    const cplx v = *p;
-    *reinterpret_cast<df2*>(p) = df_from_scaled(v, E);
+  // a warp per column: no index divisions (64-bit ones cost as much as the
+  // conversion)
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int c = c0 + (threadIdx.x >> 5); c < c1; c += nw) {
+    cplx* col = A + (size_t)lda * c;
+    for (int i = r0 + lane; i < r1; i += 32) {
+      const cplx v = col[i];
+      *reinterpret_cast<df2*>(col + i) = df_from_scaled(v, E);
+    }
   }
 }
 __device__ void rows_to_fp64(cplx* A, int lda, int r0, int r1, int c0, int c1, int E) {
   const int nr = r1 - r0;
   if (nr <= 0) return;
-  for (long long e = threadIdx.x; e < (long long)nr * (c1 - c0); e += blockDim.x) {
-    const int c = c0 + (int)(e / nr), i = r0 + (int)(e % nr);
-    cplx* p = A + i + (size_t)lda * c;
-    *p = df_to_scaled(*reinterpret_cast<const df2*>(p), E);
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int c = c0 + (threadIdx.x >> 5); c < c1; c += nw) {
+    cplx* col = A + (size_t)lda * c;
+    for (int i = r0 + lane; i < r1; i += 32) col[i] = df_to_scaled(*reinterpret_cast<const df2*>(col + i), E);
   }
 }
 
@@ -273,9 +277,9 @@ __device__ int grid_scale_exponent(const cplx* A, int lda, int r0, int r1, int k
   const int nr = r1 - r0;
   double mx = 0.0;
   if (nr > 0)
-    for (long long e = threadIdx.x; e < (long long)nr * k; e += blockDim.x) {
-      const cplx v = A[r0 + (int)(e % nr) + (size_t)lda * (int)(e / nr)];
-      mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+    for (int c = threadIdx.x >> 5; c < k; c += blockDim.x >> 5) {
+      const cplx* col = A + (size_t)lda * c;
+      for (int i = r0 + (threadIdx.x & 31); i < r1; i += 32) mx = fmax(mx, fmax(fabs(col[i].x), fabs(col[i].y)));
     }
   for (int o = 16; o >= 1; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   __syncthreads();
@@ -652,13 +656,18 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           df2* Pd = reinterpret_cast<df2*>(P);
           const df2* xt = Pd + (size_t)t * R;
           const df2* nf = reinterpret_cast<const df2*>(wl);
-          for (int e = tid; e < nrow * nrem; e += blockDim.x) {
-            const int c = e / nrow, i = ifrom + e % nrow;
-            const df2 v = (i == jj) ? df2{1.f, 0.f, 0.f, 0.f} : xt[i - r0];
-            df2& a = Pd[(size_t)(t + 1 + c) * R + (i - r0)];
-            df2 dlt = df_zero();
-            df_cmac(dlt, v, nf[c]);
-            a = df_cadd(a, dlt);
+          int L = 32;
+          while (L > 4 && L / 2 >= nrow) L >>= 1;
+          const int cw = 32 / L;
+          for (int c = wid * cw + lane / L; c < nrem; c += nw * cw) {
+            df2* ac = Pd + (size_t)(t + 1 + c) * R;
+            const df2 f = nf[c];
+            for (int i = ifrom + lane % L; i < r1; i += L) {
+              const df2 v = (i == jj) ? df2{1.f, 0.f, 0.f, 0.f} : xt[i - r0];
+              df2 dlt = df_zero();
+              df_cmac(dlt, v, f);
+              ac[i - r0] = df_cadd(ac[i - r0], dlt);
+            }
           }
         } else {
           // L lanes along the rows (few rows: several columns per warp)
