@@ -326,35 +326,45 @@ constexpr int kWidePanel = 32;
 //   w2_s = t_s W_s - sum_u (t_s Gram[s, u]) w2_u
 // over the u before s (forward) or after it: one warp per column, the scaled
 // Gram in shared memory, so that a step of the chain is one exchange and one
-// complex multiply-add.  One warp per CTA: the chain is what bounds it, and
-// four warps on one SM's FP64 unit would wait for each other (18.5 us with
-// four and the scaling inside the chain).  rec (may be NULL) receives the
-// record.
-constexpr int kWy64Cols = 1;  // columns (warps) per CTA
+// complex multiply-add (about 180 cycles).  The scaled Gram costs 2048 cycles
+// of a CTA's FP64 unit and a load per entry: four warps load it with eight
+// loads in flight each, and a CTA takes as many columns (four at most: their
+// chains share the unit without waiting) as it needs for one CTA per SM.  With
+// one warp per CTA loading entry after entry the kernel took 18.6 us, the
+// 32 load latencies alone 10.  rec (may be NULL) receives the record.
+constexpr int kWy64Cols = 4;  // warps, and columns at most, per CTA
 __global__ void __launch_bounds__(32 * kWy64Cols)
 wy_solve64_kernel(const cplx* __restrict__ g, const cplx* __restrict__ tau, int nbk, const cplx* __restrict__ W, int nt,
-                  cplx* __restrict__ W2, int forward, cplx* __restrict__ rec) {
+                  int cols, cplx* __restrict__ W2, int forward, cplx* __restrict__ rec) {
   // m[u * 33 + s] = -t_s Gram[s, u] for the pairs of the chain, else zero
   __shared__ cplx m[kWidePanel * (kWidePanel + 1)];
-  const int lane = threadIdx.x & 31, l = blockIdx.x * kWy64Cols + (threadIdx.x >> 5);
-  const bool in = lane < nbk;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, l = blockIdx.x * cols + wid;
+  const bool in = lane < nbk, mine = wid < cols && l < nt;
   const cplx tl = in ? (tau ? tau[lane] : g[lane + nbk * lane]) : mk(0, 0);
+  const cplx wl = in && mine ? W[lane + (size_t)nbk * l] : mk(0, 0);
   const cplx t = forward ? cconj(tl) : tl;
-  for (int u = threadIdx.x >> 5; u < nbk; u += kWy64Cols) {
+  constexpr int Q = kWidePanel / kWy64Cols;
+  cplx gv[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
     // stored pair (min, max): Gram[s, u] itself for s < u, its conjugate else
-    const int lo = min(lane, u), hi = max(lane, u);
-    const bool pair = in && (forward ? lane > u : lane < u);
+    const int u = wid + kWy64Cols * q, lo = min(lane, u), hi = max(lane, u);
+    gv[q] = in && u < nbk && u != lane ? g[lo + nbk * hi] : mk(0, 0);
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int u = wid + kWy64Cols * q;
     cplx v = mk(0, 0);
-    if (pair) {
-      const cplx q = cmul(t, forward ? cconj(g[lo + nbk * hi]) : g[lo + nbk * hi]);
-      v = mk(-q.x, -q.y);
+    if (forward ? lane > u : lane < u) {
+      const cplx p = cmul(t, forward ? cconj(gv[q]) : gv[q]);
+      v = mk(-p.x, -p.y);
     }
     m[u * (kWidePanel + 1) + lane] = v;
-    if (rec && blockIdx.x == 0 && in) rec[lane + nbk * u] = lane < u ? g[lane + nbk * u] : (lane == u ? tl : mk(0, 0));
+    if (rec && blockIdx.x == 0 && in && u < nbk) rec[lane + nbk * u] = lane < u ? gv[q] : (lane == u ? tl : mk(0, 0));
   }
   __syncthreads();
-  if (l >= nt) return;
-  cplx acc = in ? cmul(t, W[lane + (size_t)nbk * l]) : mk(0, 0);
+  if (!mine) return;
+  cplx acc = cmul(t, wl);
   for (int step = 0; step < nbk; ++step) {
     const int u = forward ? step : nbk - 1 - step;
     const cplx w = mk(__shfl_sync(0xffffffffu, acc.x, u), __shfl_sync(0xffffffffu, acc.y, u));
@@ -366,8 +376,9 @@ wy_solve64_kernel(const cplx* __restrict__ g, const cplx* __restrict__ tau, int 
 cudaError_t wy_solve64(const cplx* g, const cplx* tau, int nbk, const cplx* W, int nt, cplx* W2, int forward, cplx* rec,
                        cudaStream_t s) {
   if (nt <= 0 && !rec) return cudaSuccess;
-  wy_solve64_kernel<<<std::max(1, (nt + kWy64Cols - 1) / kWy64Cols), 32 * kWy64Cols, 0, s>>>(g, tau, nbk, W, nt, W2,
-                                                                                            forward, rec);
+  const int sms = dev_info().sm_count, cols = std::min(kWy64Cols, std::max(1, (nt + sms - 1) / sms));
+  wy_solve64_kernel<<<std::max(1, (nt + cols - 1) / cols), 32 * kWy64Cols, 0, s>>>(g, tau, nbk, W, nt, cols, W2, forward,
+                                                                                  rec);
   return cudaGetLastError();
 }
 
