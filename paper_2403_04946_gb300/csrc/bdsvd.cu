@@ -75,22 +75,23 @@ DV cplx sum_published(const cplx* p, size_t stride, int G) {
   }
   return s;
 }
-// Sum over the block delivered to warp 0 only (the other warps' FP64 work
-// in a block-wide reduction costs more, on this GPU's narrow FP64 pipe,
+// Sum over the block delivered to lane 0 of warp 0 only (the other warps' FP64
+// work in a block-wide reduction costs more, on this GPU's narrow FP64 pipe,
 // than the column's arithmetic).  Warps whose `has` is false contribute
-// zero without reducing.  Ends with __syncthreads (so it also publishes
-// the block's shared-memory writes made before it).
+// zero without reducing.  Its __syncthreads also publishes the block's
+// shared-memory writes made before it; the next use of red has to lie behind
+// another one.
 DV double sum_to_warp0(double v, bool has, double* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr int nw = kBdThreads / 32;
   if (has) v = warp_sum(v);
   if (lane == 0) red[w] = has ? v : 0.0;
   __syncthreads();
   double s = 0.0;
   if (w == 0) {
     s = (lane < nw) ? red[lane] : 0.0;
-    s = warp_sum(s);
+    for (int o = nw / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   }
-  __syncthreads();
   return s;
 }
 
@@ -173,16 +174,32 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     // first own local row strictly below i (rows of this CTA: g + lr G)
     const int lr0 = (i + 1 > g) ? (i + 1 - g + G - 1) / G : 0;
     const bool owner = (i % G == g);
-    // (a) partial sums over own rows r > i
-    double sq = 0.0;
-    for (int lr = lr0 + tid; lr < nact; lr += blockDim.x) sq += cabs2(R(lr, i));
-    sq = sum_to_warp0(sq, lr0 + 32 * wid < nact, dred);
+    // (a) partial sums over own rows r > i.  Up to eight rows (three at full
+    // grid size) are summed by one thread, in the order of a warp's exchange
+    // (the same bits): a block-wide sum held every column up by two exchanges
+    // and two barriers, 0.2 of 6.4 us.
+    if (nact - lr0 <= 8) {
+      if (tid == kBdThreads - 1) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = lr0 + q < nact ? cabs2(R(lr0 + q, i)) : 0.0;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+          for (int q = 0; q < o; ++q) v[q] += v[q + o];
+        pr[g] = v[0];
+      }
+    } else {
+      double sq = 0.0;
+      for (int lr = lr0 + tid; lr < nact; lr += blockDim.x) sq += cabs2(R(lr, i));
+      sq = sum_to_warp0(sq, lr0 + 32 * wid < nact, dred);
+      if (tid == 0) pr[g] = sq;
+    }
     for (int c = i + 1 + tid; c < n; c += blockDim.x) {
       cplx acc = mk(0, 0);
       for (int lr = lr0; lr < nact; ++lr) acc = cfmac(R(lr, i), R(lr, c), acc);
       pc[(size_t)g * pstride + c] = acc;
     }
-    if (tid == 0) pr[g] = sq;
     if (owner)
       for (int c = i + tid; c < n; c += blockDim.x) rowb[c] = R(i / G, c);
     if (grid_sync(gs)) return;
@@ -235,7 +252,7 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
       nrow[c] = nr;
       if (c >= i + 2) sqp += cabs2(nr);
     }
-    sqp = sum_to_warp0(sqp, i + 1 + 32 * wid < n, dred);  // its barriers also publish fv / nrow / vloc
+    sqp = sum_to_warp0(sqp, i + 1 + 32 * wid < n, dred);  // its barrier also publishes fv / nrow / vloc
     if (owner && tid == 0) {
       R(i / G, i) = bc[2];
       dg[i] = bc[2].x;
