@@ -49,21 +49,22 @@ DV df2 ld_cg_df(const cplx* p) {
 // (rs_writer picks one of them).  31 exchanges for 32 values instead of 5
 // per value: on this GPU the FP64 additions of a per-value warp sum cost
 // more than the products they reduce.
-template <int CH>
+// With O0 = 4 the same over groups of eight lanes.
+template <int CH, int O0 = 16>
 DV int rs_index(int lane) {
-  int s = 0, o = 16;
+  int s = 0, o = O0;
 #pragma unroll
   for (int h = CH / 2; h >= 1; h >>= 1, o >>= 1)
     if (lane & o) s += h;
   return s;
 }
-template <int CH>
+template <int CH, int O0 = 16>
 DV bool rs_writer(int lane) {
-  return (lane & (32 / CH - 1)) == 0;
+  return (lane & (2 * O0 / CH - 1)) == 0;
 }
-template <int CH>
+template <int CH, int O0 = 16>
 DV void reduce_scatter(cplx (&a)[CH], int lane) {
-  int o = 16;
+  int o = O0;
 #pragma unroll
   for (int h = CH / 2; h >= 1; h >>= 1, o >>= 1) {
     const bool up = (lane & o) != 0;
@@ -150,6 +151,66 @@ __device__ void update_x(const cplx* P, int R, int r0, int lo, int hi, int nbk, 
 #pragma unroll
       for (int s = 0; s < NB; ++s)
         if (s < nbk) acc = cfma(pv[(size_t)s * R], wc[s], acc);  // wc holds -W2: 4 FMAs
+      x[i] = acc;
+    }
+  }
+}
+
+// The same two for CTAs of few rows: eight lanes run along the rows, and the
+// four groups of a warp take every fourth reflector (products) or a column
+// each (update).  An FP64 instruction of a warp takes the unit for the time of
+// 32 lanes however few hold rows, and the sum over eight lanes of eight values
+// takes 14 additions instead of 62.  Up to 24 rows the padding to a multiple of
+// 8 is less than the one to 32 (beyond, the fewer passes over the columns
+// count).  FP64 panels with trailing columns are short (the tall ones take the
+// digit products): one C1 step (336 x 96 factors, 8 rows per CTA) 51 -> 44 ms.
+// tri: column l needs the reflectors before it only (the Gram).
+constexpr int kFewRows = 24;
+template <int NB>
+__device__ void partial_vhx_few(const cplx* P, int R, int r0, int lo, int hi, int nbk, const cplx* X, int ldx, int ncol,
+                                cplx* out, bool tri) {
+  constexpr int Q = NB / 4;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int rl = lane & 7, sg = lane >> 3;
+  for (int l = w; l < ncol; l += nw) {
+    const int smax = tri ? l : nbk;
+    cplx acc[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = mk(0, 0);
+    const cplx* x = X + (size_t)ldx * l;
+    cplx xn = (lo + rl < hi) ? x[lo + rl] : mk(0, 0);
+    for (int i = lo + rl; i < hi; i += 8) {
+      const cplx xi = xn;
+      if (i + 8 < hi) xn = x[i + 8];
+      const cplx* pv = P + (i - r0);
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (4 * q + sg < smax) acc[q] = cfmac(pv[(size_t)(4 * q + sg) * R], xi, acc[q]);
+    }
+    reduce_scatter<Q, 4>(acc, lane);
+    const int s = 4 * rs_index<Q, 4>(lane) + sg;
+    if (rs_writer<Q, 4>(lane) && s < nbk) out[s + (size_t)nbk * l] = acc[0];
+  }
+}
+template <int NB>
+__device__ void update_x_few(const cplx* P, int R, int r0, int lo, int hi, int nbk, cplx* X, int ldx, int ncol,
+                             const cplx* w2) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int rl = lane & 7;
+  for (int l = 4 * w + (lane >> 3); l < ncol; l += 4 * nw) {
+    cplx wc[NB];
+#pragma unroll
+    for (int s = 0; s < NB; ++s) {
+      const cplx v = (s < nbk) ? ld_cg(w2 + s + (size_t)nbk * l) : mk(0, 0);
+      wc[s] = mk(-v.x, -v.y);
+    }
+    cplx* x = X + (size_t)ldx * l;
+    for (int i = lo + rl; i < hi; i += 8) {
+      cplx acc = x[i];
+      const cplx* pv = P + (i - r0);
+#pragma unroll
+      for (int s = 0; s < NB; ++s)
+        if (s < nbk) acc = cfma(pv[(size_t)s * R], wc[s], acc);
       x[i] = acc;
     }
   }
@@ -740,27 +801,20 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
     } else {
       cplx* out = ws.pc + (size_t)g * pstride;
       // Gram block: columns are the reflectors themselves (from shared memory)
-      for (int l = wid; l < nbk; l += nw) {
-        cplx acc[NB];
-#pragma unroll
-        for (int s = 0; s < NB; ++s) acc[s] = mk(0, 0);
-        for (int i = lo + lane; i < r1; i += 32) {
-          const cplx xi = P[(size_t)l * R + (i - r0)];
-#pragma unroll
-          for (int s = 0; s < NB; ++s)
-            if (s < nbk) acc[s] = cfmac(P[(size_t)s * R + (i - r0)], xi, acc[s]);
-        }
-        reduce_scatter<NB>(acc, lane);
-        const int s = rs_index<NB>(lane);
-        if (rs_writer<NB>(lane) && s < nbk) out[s + (size_t)nbk * l] = acc[0];
+      if (R <= kFewRows) {
+        partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, P - r0, R, nbk, out, true);
+        if (nt > 0)
+          partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, out + (size_t)nbk * nbk, false);
+      } else {
+        partial_vhx<NB>(P, R, r0, lo, r1, nbk, P - r0, R, nbk, out);
+        if (nt > 0) partial_vhx<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, out + (size_t)nbk * nbk);
       }
-      __syncthreads();
-      if (nt > 0) partial_vhx<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, out + (size_t)nbk * nbk);
     }
     if (grid_sync(gs)) return;
-    // S2: reduce columns l % G == g into wfin
+    // S2: reduce columns l % G == g into wfin (of the Gram, what lies above
+    // the diagonal)
     for (int l = g; l < ncol; l += G) {
-      for (int s = wid; s < nbk; s += nw) {
+      for (int s = wid; s < min(l, nbk); s += nw) {
         cplx v = reduce_partials(ws.pc, pstride, G, s + (size_t)nbk * l);
         if (lane == 0) ws.wfin[s + (size_t)nbk * l] = v;
       }
@@ -801,6 +855,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       if (MIXED)
         update_x_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<df2*>(A) + (size_t)lda * c0,
                        lda, nt, ws.wfin + (size_t)nbk * nbk);
+      else if (R <= kFewRows)
+        update_x_few<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, ws.wfin + (size_t)nbk * nbk);
       else
         update_x<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, ws.wfin + (size_t)nbk * nbk);
     }
@@ -853,6 +909,8 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     if (MIXED)
       partial_vhx_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<const df2*>(C), ldc, q,
                         ws.pc + (size_t)g * pstride);
+    else if (R <= kFewRows)
+      partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride, false);
     else
       partial_vhx<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride);
     if (grid_sync(gs)) return;
@@ -884,6 +942,8 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     if (grid_sync(gs)) return;
     if (MIXED)
       update_x_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<df2*>(C), ldc, q, ws.wfin);
+    else if (R <= kFewRows)
+      update_x_few<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.wfin);
     else
       update_x<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.wfin);
     __syncthreads();
