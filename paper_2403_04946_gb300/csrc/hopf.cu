@@ -692,7 +692,7 @@ hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int
   if (conf_tc(ctx, c, m, std::min(m, k))) {
     TRY(tc_reserve(ctx, m, k));
     *nb = 32;
-    CK(hk::geqrf_tc(A, lda, m, k, tau, T, G, ctx->tcbuf, ctx->tcbytes, ctx->coop, kTcDigits, ctx->stream,
+    CK(hk::geqrf_tc(A, lda, m, k, tau, G, ctx->tcbuf, ctx->tcbytes, ctx->coop, kTcDigits, ctx->stream,
                     phase_timer(ctx, HOPF_K_QR)));
     return HOPF_OK;
   }

@@ -309,7 +309,7 @@ size_t qr_tc_gram_elems(int k);                         // complex elements of G
 // As geqrf (mixed), plus Gout: per outer panel j the Gram v_s^H v_u of its
 // reflectors (128 x 128 block at Gout + j 128^2, leading dimension 128),
 // which ormqr_tc needs.  T receives the inner panels' records as geqrf.
-cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* Gout, void* scratch,
+cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* Gout, void* scratch,
                      size_t scratch_bytes, const CoopWs& cws, int S, cudaStream_t s, const PhaseTimer& pt);
 // C <- Q C for the Q of geqrf_tc (p reflectors).
 cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* Gin, cplx* C, int ldc, int q,

@@ -224,14 +224,14 @@ __device__ void update_x_few(const cplx* P, int R, int r0, int lo, int hi, int n
 // sees no per-element conversions.
 template <int NB>
 __device__ void partial_vhx_f(const df2* P, int R, int r0, int lo, int hi, int nbk,
-                              const df2* X, int ldx, int ncol, cplx* out) {
+                              const df2* X, int ldx, int ncol, cplx* out, bool tri) {
   // 16 reflectors per pass over the rows keep the double-float accumulators
-  // in registers
+  // in registers; tri: passes without a reflector before column l left out
   constexpr int CH = NB < 16 ? NB : 16;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int l = w; l < ncol; l += nw) {
     const df2* x = X + (size_t)ldx * l;
-    for (int s0 = 0; s0 < nbk; s0 += CH) {
+    for (int s0 = 0; s0 < (tri ? l : nbk); s0 += CH) {
       df2 acc[CH];
 #pragma unroll
       for (int s = 0; s < CH; ++s) acc[s] = df_zero();
@@ -794,10 +794,10 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       // the Gram block (its columns are the reflectors themselves) and the
       // trailing products from the double-float panel, on the FP32 pipe
       const df2* Pd = reinterpret_cast<const df2*>(P);
-      partial_vhx_f<NB>(Pd, R, r0, lo, r1, nbk, Pd - r0, R, nbk, out);
+      partial_vhx_f<NB>(Pd, R, r0, lo, r1, nbk, Pd - r0, R, nbk, out, true);
       if (nt > 0)
         partial_vhx_f<NB>(Pd, R, r0, lo, r1, nbk, reinterpret_cast<const df2*>(A) + (size_t)lda * c0, lda, nt,
-                          out + (size_t)nbk * nbk);
+                          out + (size_t)nbk * nbk, false);
     } else {
       cplx* out = ws.pc + (size_t)g * pstride;
       // Gram block: columns are the reflectors themselves (from shared memory)
@@ -908,7 +908,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     __syncthreads();
     if (MIXED)
       partial_vhx_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<const df2*>(C), ldc, q,
-                        ws.pc + (size_t)g * pstride);
+                        ws.pc + (size_t)g * pstride, false);
     else if (R <= kFewRows)
       partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride, false);
     else

@@ -213,7 +213,7 @@ size_t qr_tc_gram_elems(int k) { return (size_t)((k + kOuter - 1) / kOuter) * kO
 // Complex GEMM FLOPs (8 per complex multiply-add) of an M x N x K product.
 static double zflops(double M, double N, double K) { return 8.0 * M * N * K; }
 
-cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* Gout, void* scratch,
+cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* Gout, void* scratch,
                      size_t scratch_bytes, const CoopWs& cws, int S, cudaStream_t s, const PhaseTimer& pt) {
   const int p = std::min(m, k);
   const int Kc = tc_chunk(S);
@@ -224,7 +224,9 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, cplx* G
     cplx* Ap = A + j0 + (size_t)lda * j0;
     int nb = 32;
     int slot = pt.b();
-    e = geqrf(Ap, lda, mv, nbk, tau + j0, T + (size_t)(j0 / 32) * 32 * 32, &nb, cws, s, 1);
+    // without the record of the 32-column blocks: G below takes its place, and
+    // the kernel leaves the last block's products and their barriers out
+    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, 1);
     pt.e(slot, pt.cls_panel, 8.0 * mv * (double)nbk * nbk - 8.0 * (double)nbk * nbk * nbk / 3.0, 1);
     if (e != cudaSuccess) break;
     Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
