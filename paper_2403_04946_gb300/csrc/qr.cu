@@ -518,28 +518,31 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           for (int c = tid; c < nbk - t; c += blockDim.x)
             reinterpret_cast<df2*>(rowp)[c] = Pd[(size_t)(t + c) * R + (jj - r0)];
       } else {
-        // columns t (its norm) .. nbk-1 at once: S lanes per column, so that
-        // 32, 16 or 8 columns fill the CTA (a warp per column would spend
-        // more FP64 time on the additions across 32 lanes than on the sums)
-        const int S = nrem + 1 > 16 ? 8 : (nrem + 1 > 8 ? 16 : 32);
+        // columns t (its norm) .. nbk-1 at once: S lanes per column.  Eight for
+        // CTAs of up to 64 rows, where the FP64 additions across more lanes
+        // cost more than the sums, and warps without a column leave; beyond,
+        // as many as fill the CTA
+        const int S = R <= 64 || nrem + 1 > 16 ? 8 : (nrem + 1 > 8 ? 16 : 32);
         const int c = tid / S, seg = tid % S;
-        cplx a0 = mk(0, 0), a1 = mk(0, 0);
-        if (c <= nrem) {
-          const cplx* xt = P + (size_t)t * R;
-          const cplx* ac = xt + (size_t)c * R;
-          int i = ilo - r0 + seg;
-          for (; i + S < r1 - r0; i += 2 * S) {
-            a0 = cfmac(xt[i], ac[i], a0);
-            a1 = cfmac(xt[i + S], ac[i + S], a1);
+        if (wid * (32 / S) <= nrem) {
+          cplx a0 = mk(0, 0), a1 = mk(0, 0);
+          if (c <= nrem) {
+            const cplx* xt = P + (size_t)t * R;
+            const cplx* ac = xt + (size_t)c * R;
+            int i = ilo - r0 + seg;
+            for (; i + S < r1 - r0; i += 2 * S) {
+              a0 = cfmac(xt[i], ac[i], a0);
+              a1 = cfmac(xt[i + S], ac[i + S], a1);
+            }
+            if (i < r1 - r0) a0 = cfmac(xt[i], ac[i], a0);
           }
-          if (i < r1 - r0) a0 = cfmac(xt[i], ac[i], a0);
+          a0 = cadd(a0, a1);
+          for (int o = 1; o < S; o <<= 1) {
+            a0.x += __shfl_xor_sync(0xffffffffu, a0.x, o);
+            a0.y += __shfl_xor_sync(0xffffffffu, a0.y, o);
+          }
+          if (seg == 0 && c <= nrem) myp[c] = a0;
         }
-        a0 = cadd(a0, a1);
-        for (int o = 1; o < S; o <<= 1) {
-          a0.x += __shfl_xor_sync(0xffffffffu, a0.x, o);
-          a0.y += __shfl_xor_sync(0xffffffffu, a0.y, o);
-        }
-        if (seg == 0 && c <= nrem) myp[c] = a0;
         if (g == gown)
           for (int q = tid; q < nbk - t; q += blockDim.x) rowp[q] = P[(size_t)(t + q) * R + (jj - r0)];
       }
