@@ -75,7 +75,7 @@ DV cplx sum_published(const cplx* p, size_t stride, int G) {
   }
   return s;
 }
-// Sum over the block delivered to lane 0 of warp 0 only (the other warps' FP64
+// Sum over the block delivered to lanes 0 to 7 of warp 0 only (the other warps' FP64
 // work in a block-wide reduction costs more, on this GPU's narrow FP64 pipe,
 // than the column's arithmetic).  Warps whose `has` is false contribute
 // zero without reducing.  Its __syncthreads also publishes the block's
@@ -93,26 +93,6 @@ DV double sum_to_warp0(double v, bool has, double* red) {
     for (int o = nw / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   }
   return s;
-}
-
-DV void house_scalars(cplx alpha, double xnorm2, cplx* tau, cplx* scale, double* beta) {
-  // H^H [alpha; x] = [beta; 0] with H = I - tau v v^H, v = [1; x * scale]
-  if (xnorm2 == 0.0 && alpha.y == 0.0) {
-    *tau = mk(0, 0);
-    *scale = mk(0, 0);
-    *beta = alpha.x;
-    return;
-  }
-  // two FP64 divisions (each ~640 cycles of latency on this GPU), issued
-  // independently of each other
-  const double an = sqrt(alpha.x * alpha.x + alpha.y * alpha.y + xnorm2);
-  const double b = (alpha.x >= 0.0) ? -an : an;
-  const double ib = 1.0 / b;
-  const double dr = alpha.x - b, di = alpha.y;
-  const double id2 = 1.0 / (dr * dr + di * di);
-  *tau = mk((b - alpha.x) * ib, -alpha.y * ib);
-  *scale = mk(dr * id2, -di * id2);
-  *beta = b;
 }
 
 // ---- 1. bidiagonalisation -------------------------------------------------------
@@ -211,11 +191,11 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     if (wid == 0) {
       const cplx al = __ldcg(rowb + i);
       const double s2 = warp_sum(sum_published(pr, G));
+      cplx tq, sc;
+      double beta;
+      if (FAST) house_fast(al, s2, &tq, &sc, &beta);
+      else house_warp(al, s2, &tq, &sc, &beta);
       if (lane == 0) {
-        cplx tq, sc;
-        double beta;
-        if (FAST) house_fast(al, s2, &tq, &sc, &beta);
-        else house_scalars(al, s2, &tq, &sc, &beta);
         bc[0] = tq;
         bc[1] = sc;
         bc[2] = mk(beta, 0.0);
@@ -263,11 +243,13 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     // reflector to the own rows: A[r,c] -= v_r conj(tau) w_c, column i
     // keeps v_r
     if (wid == 0) {
-      if (lane == 0 && i + 1 < n) {
-        cplx tp, sp;
-        double beta;
+      cplx tp = mk(0, 0), sp = mk(0, 0);
+      double beta = 0.0;
+      if (i + 1 < n) {
         if (FAST) house_fast(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
-        else house_scalars(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
+        else house_warp(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
+      }
+      if (lane == 0 && i + 1 < n) {
         bcr[0] = tp;
         bcr[1] = sp;
         bcr[2] = mk(beta, 0.0);

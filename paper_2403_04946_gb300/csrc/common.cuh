@@ -74,6 +74,22 @@ DV void house_fast(cplx al, double s2, cplx* tau, cplx* scale, double* beta) {
   *beta = b;
 }
 
+// The same with IEEE root and divisions, by a whole warp whose lanes 0 and 1 (at
+// least) hold the inputs; the results are theirs.  The two divisions (about 640
+// cycles each, and one after the other in one lane's code) run side by side in
+// the two lanes.
+DV void house_warp(cplx al, double s2, cplx* tau, cplx* scale, double* beta) {
+  const double an = sqrt(al.x * al.x + al.y * al.y + s2);
+  const double b = (al.x >= 0.0) ? -an : an;
+  const double dr = al.x - b, den = dr * dr + al.y * al.y;
+  const double r = 1.0 / ((threadIdx.x & 1) ? den : b);
+  const double ib = __shfl_sync(0xffffffffu, r, 0), id2 = __shfl_sync(0xffffffffu, r, 1);
+  const bool none = s2 == 0.0 && al.y == 0.0;
+  *tau = none ? mk(0, 0) : mk((b - al.x) * ib, -al.y * ib);
+  *scale = none ? mk(0, 0) : mk(dr * id2, -al.y * id2);
+  *beta = none ? al.x : b;
+}
+
 // Single-precision complex (mixed-precision trailing updates and products).
 typedef float2 cplxf;
 HD cplxf mkf(float re, float im) { return make_float2(re, im); }

@@ -587,36 +587,25 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           bc[1] = sc;
           bc[2] = mk(beta, 0.0);
         }
-        if (MIXED && lane == 0) {
+        if constexpr (MIXED) {
           cplx tu, sc;
           double beta;
-          if (s2 == 0.0 && al.y == 0.0) {
-            tu = mk(0, 0);
-            beta = al.x;
-            sc = mk(0, 0);
-          } else {
-            // one division for tau, one for the scale
-            const double an = sqrt(al.x * al.x + al.y * al.y + s2);
-            beta = (al.x >= 0.0) ? -an : an;
-            const double ib = 1.0 / beta;
-            tu = mk((beta - al.x) * ib, -al.y * ib);
-            sc = cinv(mk(al.x - beta, al.y));
-          }
-          {
-            // the scale can leave the FP32 range (tiny columns): keep it as
-            // mantissa x 2^esc
-            const double smax = fmax(fabs(sc.x), fabs(sc.y));
-            const int es = (smax > 0.0) ? ilogb(smax) : 0;
-            sc = mk(scalbn(sc.x, -es), scalbn(sc.y, -es));
+          house_warp(al, s2, &tu, &sc, &beta);
+          // the scale can leave the FP32 range (tiny columns): keep it as
+          // mantissa x 2^esc
+          const double smax = fmax(fabs(sc.x), fabs(sc.y));
+          const int es = (smax > 0.0) ? ilogb(smax) : 0;
+          sc = mk(scalbn(sc.x, -es), scalbn(sc.y, -es));
+          // one conversion per lane
+          const cplx v = lane == 0 ? cconj(tu) : (lane == 1 ? cconj(sc) : (lane == 2 ? sc : mk(beta, 0.0)));
+          const df2 vd = df_from_scaled(v, 0);
+          if (lane < 4) bcd[lane] = vd;
+          if (lane == 0) {
             esc_sh = es;
-            bcd[0] = df_from_scaled(cconj(tu), 0);
-            bcd[1] = df_from_scaled(cconj(sc), 0);
-            bcd[2] = df_from_scaled(sc, 0);
-            bcd[3] = df_from_scaled(mk(beta, 0.0), 0);
+            bc[0] = tu;
+            bc[1] = sc;
+            bc[2] = mk(beta, 0.0);
           }
-          bc[0] = tu;
-          bc[1] = sc;
-          bc[2] = mk(beta, 0.0);
         }
       }
       // raw sums over the CTAs of the dot products (tpc threads per
