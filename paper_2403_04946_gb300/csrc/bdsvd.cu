@@ -191,14 +191,17 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     if (wid == 0) {
       const cplx al = __ldcg(rowb + i);
       const double s2 = warp_sum(sum_published(pr, G));
-      cplx tq, sc;
-      double beta;
-      if (FAST) house_fast(al, s2, &tq, &sc, &beta);
-      else house_warp(al, s2, &tq, &sc, &beta);
-      if (lane == 0) {
-        bc[0] = tq;
-        bc[1] = sc;
-        bc[2] = mk(beta, 0.0);
+      if constexpr (FAST) {
+        house_fast(al, s2, bc);
+      } else {
+        cplx tq, sc;
+        double beta;
+        house_warp(al, s2, &tq, &sc, &beta);
+        if (lane == 0) {
+          bc[0] = tq;
+          bc[1] = sc;
+          bc[2] = mk(beta, 0.0);
+        }
       }
     } else if (cc < C) {
       a_ic = __ldcg(rowb + i + 1 + cc);
@@ -243,16 +246,17 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     // reflector to the own rows: A[r,c] -= v_r conj(tau) w_c, column i
     // keeps v_r
     if (wid == 0) {
-      cplx tp = mk(0, 0), sp = mk(0, 0);
-      double beta = 0.0;
-      if (i + 1 < n) {
-        if (FAST) house_fast(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
-        else house_warp(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
-      }
-      if (lane == 0 && i + 1 < n) {
-        bcr[0] = tp;
-        bcr[1] = sp;
-        bcr[2] = mk(beta, 0.0);
+      if (FAST && i + 1 < n) {
+        house_fast(cconj(nrow[i + 1]), sqp, bcr);
+      } else if (i + 1 < n) {
+        cplx tp, sp;
+        double beta;
+        house_warp(cconj(nrow[i + 1]), sqp, &tp, &sp, &beta);
+        if (lane == 0) {
+          bcr[0] = tp;
+          bcr[1] = sp;
+          bcr[2] = mk(beta, 0.0);
+        }
       }
     } else {
       const int t1 = tid - 32, nt1 = blockDim.x - 32;
@@ -278,18 +282,25 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
     __syncthreads();
     // right update of own rows r > i: A[r,:] -= taup (A[r,:] . u) u^H
     for (int lr = lr0 + wid; lr < nact; lr += nw) {
-      // four interleaved partial dot products (a dependent FP64 FMA chain
-      // costs 64-128 cycles per step on this GPU)
-      cplx d0 = mk(0, 0), d1 = mk(0, 0), d2 = mk(0, 0), d3 = mk(0, 0);
-      int c = i + 1 + lane;
-      for (; c + 96 < n; c += 128) {
-        d0 = cfma(R(lr, c), uv[c], d0);
-        d1 = cfma(R(lr, c + 32), uv[c + 32], d1);
-        d2 = cfma(R(lr, c + 64), uv[c + 64], d2);
-        d3 = cfma(R(lr, c + 96), uv[c + 96], d3);
+      cplx dot = mk(0, 0);
+      if constexpr (FAST) {
+        // a warp's FP64 instructions follow one another at the pace of a
+        // dependent chain: one sum (four cost six more additions)
+#pragma unroll 4
+        for (int c = i + 1 + lane; c < n; c += 32) dot = cfma(R(lr, c), uv[c], dot);
+        dot = warp_sum(dot);
+      } else {
+        cplx d0 = mk(0, 0), d1 = mk(0, 0), d2 = mk(0, 0), d3 = mk(0, 0);
+        int c = i + 1 + lane;
+        for (; c + 96 < n; c += 128) {
+          d0 = cfma(R(lr, c), uv[c], d0);
+          d1 = cfma(R(lr, c + 32), uv[c + 32], d1);
+          d2 = cfma(R(lr, c + 64), uv[c + 64], d2);
+          d3 = cfma(R(lr, c + 96), uv[c + 96], d3);
+        }
+        for (; c < n; c += 32) d0 = cfma(R(lr, c), uv[c], d0);
+        dot = warp_sum(cadd(cadd(d0, d1), cadd(d2, d3)));
       }
-      for (; c < n; c += 32) d0 = cfma(R(lr, c), uv[c], d0);
-      cplx dot = warp_sum(cadd(cadd(d0, d1), cadd(d2, d3)));
       const cplx f = cmul(tp, dot);
       const cplx nf = mk(-f.x, -f.y);
       for (int c = i + 1 + lane; c < n; c += 32) R(lr, c) = cfma(nf, cconj(uv[c]), R(lr, c));

@@ -51,27 +51,24 @@ DV double rsqrt_fast(double x) {
   return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 // Householder reflector H = I - tau v v^H, v = [1; x scale], with H^H [alpha; x]
-// = [beta; 0], beta real (zlarfg conventions), from alpha and |x|^2.  One
-// reciprocal root and one reciprocal, issued after one another's inputs are
-// known, instead of a root and two divisions; the IEEE forms where a square
-// leaves the range of the fast ones.
-DV void house_fast(cplx al, double s2, cplx* tau, cplx* scale, double* beta) {
-  if (s2 == 0.0 && al.y == 0.0) {
-    *tau = mk(0, 0);
-    *scale = mk(0, 0);
-    *beta = al.x;
-    return;
-  }
+// = [beta; 0], beta real (zlarfg conventions), from alpha and |x|^2, by a whole
+// warp whose lanes 0 to 3 (at least) hold the inputs; out[0..2] <- tau, scale,
+// beta.  One reciprocal root and one reciprocal, issued after one another's
+// inputs are known, instead of a root and two divisions; the IEEE forms where a
+// square leaves the range of the fast ones.  Every FP64 instruction of a warp
+// takes 64 cycles, so the four last products are one, a lane each.
+DV void house_fast(cplx al, double s2, cplx* out) {
+  const int lane = threadIdx.x & 31;
   const double a2 = fma(al.x, al.x, fma(al.y, al.y, s2));
-  const bool in = a2 > 1e-280 && a2 < 1e280;
+  const bool none = s2 == 0.0 && al.y == 0.0, in = a2 > 1e-280 && a2 < 1e280;
   const double rs = in ? rsqrt_fast(a2) : 1.0 / sqrt(a2);
   const double an = in ? a2 * rs : sqrt(a2);
   const double b = al.x >= 0.0 ? -an : an, ib = al.x >= 0.0 ? -rs : rs;
   const double dr = al.x - b, den = fma(dr, dr, al.y * al.y);
   const double id2 = in ? rcp_fast(den) : 1.0 / den;
-  *tau = mk((b - al.x) * ib, -al.y * ib);
-  *scale = mk(dr * id2, -al.y * id2);
-  *beta = b;
+  const double r = ((lane & 1) ? -al.y : (lane & 2) ? dr : -dr) * ((lane & 2) ? id2 : ib);
+  if (lane < 4) reinterpret_cast<double*>(out)[lane] = none ? 0.0 : r;
+  if (lane == 0) out[2] = mk(none ? al.x : b, 0.0);
 }
 
 // The same with IEEE root and divisions, by a whole warp whose lanes 0 and 1 (at
@@ -232,10 +229,16 @@ DV double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// The halves of the warp take the real and the imaginary parts after the first
+// exchange: five additions instead of ten (an FP64 instruction of a warp takes
+// 64 cycles), in the same order.
 DV cplx warp_sum(cplx v) {
-  v.x = warp_sum(v.x);
-  v.y = warp_sum(v.y);
-  return v;
+  unsigned int lane;
+  asm("mov.u32 %0, %%laneid;" : "=r"(lane));
+  const bool im = lane & 16u;
+  double s = (im ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, im ? v.x : v.y, 16);
+  for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return mk(__shfl_sync(0xffffffffu, s, 0), __shfl_sync(0xffffffffu, s, 16));
 }
 DV float warp_sumf(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -100,6 +100,16 @@ DV void reduce_scatter(df2 (&a)[CH], int lane) {
   for (; o >= 1; o >>= 1) a[0] = df_cadd(a[0], df_shfl_xor(a[0], o));
 }
 
+// Sum of a complex value over S >= 2 adjacent lanes (a power of two): the even
+// ones return its real part, the odd ones its imaginary part, for half the
+// additions of summing both.
+DV double half_sum(cplx a, int S) {
+  const bool im = threadIdx.x & 1;
+  double h = (im ? a.y : a.x) + __shfl_xor_sync(0xffffffffu, im ? a.x : a.y, 1);
+  for (int o = 2; o < S; o <<= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+  return h;
+}
+
 // Partial products V^H X over this CTA's rows [lo, hi) (global row index),
 // V in shared memory (P, leading dimension R, rows offset r0), X column l
 // given by a pointer.  One warp per column; results to out[s + nbk * l].
@@ -536,12 +546,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
             }
             if (i < r1 - r0) a0 = cfmac(xt[i], ac[i], a0);
           }
-          a0 = cadd(a0, a1);
-          for (int o = 1; o < S; o <<= 1) {
-            a0.x += __shfl_xor_sync(0xffffffffu, a0.x, o);
-            a0.y += __shfl_xor_sync(0xffffffffu, a0.y, o);
-          }
-          if (seg == 0 && c <= nrem) myp[c] = a0;
+          const double h = half_sum(cadd(a0, a1), S);
+          if (seg < 2 && c <= nrem) reinterpret_cast<double*>(myp + c)[seg] = h;
         }
         if (g == gown)
           for (int q = tid; q < nbk - t; q += blockDim.x) rowp[q] = P[(size_t)(t + q) * R + (jj - r0)];
@@ -559,11 +565,13 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (grid_wait(gs)) return;
       }
       // (b) the reflector (zlarfg conventions: beta real, v_jj = 1), in FP64
-      cplx rv = mk(0, 0);  // entry t + 1 + tid of the pivot row (warp 0)
+      cplx rv = mk(0, 0);  // mixed: entry t + 1 + tid of the pivot row (warp 0)
+      double rvh = 0.0;    // FP64: part tid & 1 of its entry t + 1 + tid / 2 (warps 0 and 1)
+      if (!MIXED && tid < 2 * nrem) rvh = ld_cg(reinterpret_cast<const double*>(rowp + 1) + tid);
       if (wid == 0) {
         // the pivot row is loaded with the first batch of partial norms (all
         // one L2 round trip away)
-        if (lane < nrem) rv = ld_cg(rowp + 1 + lane);
+        if (MIXED && lane < nrem) rv = ld_cg(rowp + 1 + lane);
         cplx al;
         if constexpr (MIXED) al = df_to_scaled(ld_cg_df(rowp), 0);
         else al = ld_cg(rowp);
@@ -579,14 +587,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
             if (g0 + 32 * u < G) s2 += v[u];
         }
         s2 = warp_sum(s2);
-        if (!MIXED && lane == 0) {
-          cplx tu, sc;
-          double beta;
-          house_fast(al, s2, &tu, &sc, &beta);
-          bc[0] = tu;
-          bc[1] = sc;
-          bc[2] = mk(beta, 0.0);
-        }
+        if (!MIXED) house_fast(al, s2, bc);
         if constexpr (MIXED) {
           cplx tu, sc;
           double beta;
@@ -654,11 +655,9 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
                 for (int u = 0; u < kLoadBatch; u += 2)
                   if (g0 + tpc * u < G) acc = cadd(acc, v[u]);
               }
-            for (int o = 1; o < tpc; o <<= 1) {
-              acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-              acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-            }
-            if (valid && sub == 0) praw[c] = acc;
+            // four threads or more: 31 columns at most for 224 threads
+            const double h = half_sum(acc, tpc);
+            if (valid && sub < 2) reinterpret_cast<double*>(praw + c)[sub] = h;
           }
         }
       }
@@ -688,13 +687,23 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (tid == 0 && jj >= r0 && jj < r1) xt[jj - r0] = bcd[3];
       } else {
         // -f for the pivot row (v = 1), -scale f for the rows below, which
-        // hold x until the next column's barrier
-        if (tid < nrem) {
-          const int c = tid;
-          const cplx w = cadd(rv, cmul(cconj(sc), praw[c]));
-          const cplx f = cmul(cconj(tu), w), sf = cmul(sc, f);
-          wl[c] = mk(-f.x, -f.y);
-          wl[kNbMax + c] = mk(-sf.x, -sf.y);
+        // hold x until the next column's barrier; even threads the real parts,
+        // odd ones the imaginary parts (the chain is six FP64 instructions of
+        // a warp instead of fourteen)
+        if (wid < 2) {
+          const int c = tid >> 1, im = tid & 1;
+          const cplx raw = c < nrem ? praw[c] : mk(0, 0);
+          auto mul = [&](cplx a, double p, double q, double z) {  // that part of a (p, q) + z
+            return fma(a.x, p, fma(im ? a.y : -a.y, q, z));
+          };
+          auto other = [](double v) { return __shfl_xor_sync(0xffffffffu, v, 1); };
+          const double w = mul(cconj(sc), im ? raw.y : raw.x, im ? raw.x : raw.y, rvh);
+          const double f = mul(cconj(tu), w, other(w), 0.0);
+          const double sf = mul(sc, f, other(f), 0.0);
+          if (c < nrem) {
+            reinterpret_cast<double*>(wl + c)[im] = -f;
+            reinterpret_cast<double*>(wl + kNbMax + c)[im] = -sf;
+          }
         }
         if (tid == 0 && jj >= r0 && jj < r1) P[(size_t)t * R + (jj - r0)] = bc[2];
       }
