@@ -1191,43 +1191,84 @@ cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, co
 // ---- 4. back-transformation -------------------------------------------------------------------
 // u_k <- Q u_k with Q = H_0 H_1 ... H_{n-1} (reflector j: unit entry at j,
 // tail A[j+1:n, j], tau[j]).  One vector per CTA, so that the FP64 work
-// (about 10 n^2 / 2 operations per vector) spreads over many SMs; warp 0
-// applies reflector j while warp 1 stages reflector j-1 in shared memory.
+// (about 10 n^2 / 2 operations per vector) spreads over many SMs.  A warp's
+// FP64 instruction holds its quarter of the SM for 64 cycles, so one warp per
+// vector ran at a quarter of the SM's rate (7400 cycles for two reflectors at
+// n = 192; a factor of the C3 mixed step 520 us, 289 with four).  Four warps share a reflector: the real and the imaginary part of
+// the dot product on two of them each, by halves of the rows (SPLIT, FP64
+// contexts; the mixed path keeps the order of one warp's sums and every bit,
+// bd_invit_kernel says why), then a quarter of the rows' update each.
+// kBackStage further warps stage the next reflectors in shared memory.
 // The result goes to U (n x nvec, ldu) and to Xp (mrows x nvec, ldp, zero
 // below row n).
-__global__ void __launch_bounds__(64)
+constexpr int kBackStage = 2, kBackWarps = 4;
+template <bool SPLIT>
+__global__ void __launch_bounds__(32 * (kBackStage + kBackWarps))
 bd_back_kernel(const cplx* __restrict__ A, int lda, const cplx* __restrict__ tauq, int n,
                const double* __restrict__ Xr, int ldx, int nvec, cplx* __restrict__ U, int ldu,
                cplx* __restrict__ Xp, int ldp, int mrows) {
   extern __shared__ __align__(16) unsigned char bk_smem[];
-  cplx* vb = reinterpret_cast<cplx*>(bk_smem);  // [2][n] staged reflectors
-  cplx* x = vb + 2 * (size_t)n;                 // [n]
+  constexpr int S = kBackStage;
+  cplx* vb = reinterpret_cast<cplx*>(bk_smem);  // [2][S][n] staged reflectors
+  cplx* x = vb + 2 * (size_t)S * n;             // [n]
+  __shared__ cplx tb[2 * S];                    // their tau
+  __shared__ double red[2][kBackWarps];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k = blockIdx.x;
   if (k >= nvec) return;
-  auto stage = [&](int j) {  // reflector j into vb[j & 1][j..n)
-    cplx* v = vb + (size_t)(j & 1) * n;
-    for (int i = j + lane; i < n; i += 32) v[i] = (i == j) ? mk(1, 0) : __ldg(A + i + (size_t)lda * j);
+  // reflector j (none if negative) into slot q
+  auto stage = [&](int j, int q) {
+    if (j < 0) return;
+    cplx* v = vb + (size_t)q * n;
+    const cplx* a = A + (size_t)lda * j;
+    if (lane == 0) {
+      v[j] = mk(1, 0);
+      tb[q] = __ldg(tauq + j);
+    }
+    for (int i0 = j + 1 + lane; i0 < n; i0 += 128) {
+      cplx r[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) r[t] = (i0 + 32 * t < n) ? __ldg(a + i0 + 32 * t) : mk(0, 0);
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (i0 + 32 * t < n) v[i0 + 32 * t] = r[t];
+    }
   };
-  if (wid == 0) {
-    for (int i = lane; i < n; i += 32) x[i] = mk(Xr[i + (size_t)ldx * k], 0.0);
+  if (wid < kBackWarps) {
+    for (int i = threadIdx.x; i < n; i += 32 * kBackWarps) x[i] = mk(Xr[i + (size_t)ldx * k], 0.0);
   } else {
-    stage(n - 1);
+    stage(n - 1 - (wid - kBackWarps), wid - kBackWarps);
   }
   __syncthreads();
-  for (int j = n - 1; j >= 0; --j) {
-    if (wid == 1) {
-      if (j > 0) stage(j - 1);
+  for (int j0 = n - 1, h = 0; j0 >= 0; j0 -= S, h ^= 1) {
+    if (wid >= kBackWarps) {
+      stage(j0 - S - (wid - kBackWarps), (h ^ 1) * S + wid - kBackWarps);
     } else {
-      const cplx t = __ldg(tauq + j);
-      if (t.x != 0.0 || t.y != 0.0) {
-        const cplx* v = vb + (size_t)(j & 1) * n;
-        cplx acc = mk(0, 0);
-        for (int i = j + lane; i < n; i += 32) acc = cfmac(v[i], x[i], acc);
-        acc = warp_sum(acc);
-        const cplx f = cmul(t, acc);
+      for (int w = 0; w < S && j0 - w >= 0; ++w) {
+        const int j = j0 - w;
+        const cplx t = tb[h * S + w];
+        if (t.x == 0.0 && t.y == 0.0) continue;  // the same for every thread
+        const cplx* v = vb + (size_t)(h * S + w) * n;
+        double* rd = red[w & 1];
+        // part wid & 1 of v^H x
+        double acc = 0.0;
+        if (SPLIT || wid < 2) {
+          const int step = SPLIT ? 64 : 32;
+          int i = j + lane + (SPLIT ? 32 * (wid >> 1) : 0);
+          if (wid & 1) {
+            for (; i < n; i += step) acc = fma(v[i].x, x[i].y, fma(-v[i].y, x[i].x, acc));
+          } else {
+            for (; i < n; i += step) acc = fma(v[i].x, x[i].x, fma(v[i].y, x[i].y, acc));
+          }
+          acc = warp_sum(acc);
+          if (lane == 0) rd[wid] = acc;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kBackWarps) : "memory");
+        const cplx dot = SPLIT ? mk(rd[0] + rd[2], rd[1] + rd[3]) : mk(rd[0], rd[1]);
+        const cplx f = cmul(t, dot);
         const cplx nf = mk(-f.x, -f.y);
-        for (int i = j + lane; i < n; i += 32) x[i] = cfma(v[i], nf, x[i]);
+        for (int i = j + threadIdx.x; i < n; i += 32 * kBackWarps) x[i] = cfma(v[i], nf, x[i]);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kBackWarps) : "memory");
       }
     }
     __syncthreads();
@@ -1240,12 +1281,14 @@ bd_back_kernel(const cplx* __restrict__ A, int lda, const cplx* __restrict__ tau
 }
 
 cudaError_t bd_back(const cplx* A, int lda, const cplx* tauq, int n, const double* X, int ldx, int nvec,
-                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, cudaStream_t s) {
+                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int mixed, cudaStream_t s) {
   if (nvec <= 0) return cudaSuccess;
-  const size_t smem = sizeof(cplx) * (size_t)n * 3;
-  cudaError_t err = allow_smem((const void*)bd_back_kernel, smem);
+  // 80 bytes per row: less than the vectors' own solves keep (bd_vectors_smem)
+  const size_t smem = sizeof(cplx) * (size_t)n * (2 * kBackStage + 1);
+  const auto fn = mixed ? bd_back_kernel<false> : bd_back_kernel<true>;
+  cudaError_t err = allow_smem((const void*)fn, smem);
   if (err != cudaSuccess) return err;
-  bd_back_kernel<<<nvec, 64, smem, s>>>(A, lda, tauq, n, X, ldx, nvec, U, ldu, Xp, ldp, mrows);
+  fn<<<nvec, 32 * (kBackStage + kBackWarps), smem, s>>>(A, lda, tauq, n, X, ldx, nvec, U, ldu, Xp, ldp, mrows);
   return cudaGetLastError();
 }
 

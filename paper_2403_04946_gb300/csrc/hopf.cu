@@ -976,7 +976,7 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
       const int kt = std::min(ctx->h_int[2], rnew);
       if (MIXED_FLAG) TRY(bd_lu_reserve(ctx, hk::bd_lu_elems(pp, kt)));
       LAUNCH(HOPF_K_SVD, 0, 0, (kt > 0 ? 6 + MIXED_FLAG : 0) + (kt < rnew), hk::bd_vectors(w.bd_d, w.bd_e, pp, w.bd_info, w.sig, kt, rnew, w.bd_X, pp, w.bd_Zs, MIXED_FLAG ? w.bd_lu : nullptr, ctx->stream));
-      LAUNCH(HOPF_K_SVD, 0, 0, 1, hk::bd_back(w.Mb, pp, w.bd_tauq, pp, w.bd_X, pp, rnew, w.Ub, pp, t->cores[c], Mrows, Mrows, ctx->stream));
+      LAUNCH(HOPF_K_SVD, 0, 0, 1, hk::bd_back(w.Mb, pp, w.bd_tauq, pp, w.bd_X, pp, rnew, w.Ub, pp, t->cores[c], Mrows, Mrows, MIXED_FLAG, ctx->stream));
     } else if (case1) {
       LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::gather_u(w.Mb, pp, pp, w.perm, w.sig, 1, rnew, t->cores[c], Mrows, Mrows, w.Ub, pp, ctx->stream));
     } else {

@@ -109,7 +109,7 @@ cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, co
                        int kt, int nvec, double* X, int ldx, double* Zs, double* lu, cudaStream_t s);
 // U = Q X -> U (n x nvec, ldu) and Xp (mrows x nvec, ldp, zero below row n).
 cudaError_t bd_back(const cplx* A, int lda, const cplx* tauq, int n, const double* X, int ldx, int nvec,
-                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, cudaStream_t s);
+                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int mixed, cudaStream_t s);
 
 // ---- TT-cross construction of a Gaussian (cross.cu) --------------------------
 // A (rl n x rr, column-major, row alpha + rl i) = Phi0(Il[alpha], i, Jr[beta])
