@@ -399,6 +399,17 @@ __device__ __forceinline__ cplx reduce_partials(const cplx* pc, size_t pstride, 
   return warp_sum(acc);
 }
 
+// The chain of a WY solve by one warp, lane s holding tau_s-scaled W[s]: acc +=
+// M[s, u] w2_u for u from u0 in steps of du, the scaled Gram's column u at
+// u (nbk + 1), zero outside the chain's pairs.
+__device__ __forceinline__ void wy_chain(cplx& acc, const cplx* M, int nbk, int u0, int du) {
+  const int lane = threadIdx.x & 31;
+  for (int step = 0, u = u0; step < nbk; ++step, u += du) {
+    const cplx w = mk(__shfl_sync(0xffffffffu, acc.x, u), __shfl_sync(0xffffffffu, acc.y, u));
+    if (lane < nbk) acc = cfma(M[u * (nbk + 1) + lane], w, acc);
+  }
+}
+
 template <int NB, bool MIXED>
 __global__ void __launch_bounds__(qr_threads(MIXED), 1)
 geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
@@ -828,14 +839,31 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
     // a chain of nbk steps per column (lanes = s; one warp per column).  The
     // panel's Gram (strict upper triangle) and tau (diagonal) are kept in
     // Tg for ormqr, which runs the mirrored recurrence.
+    // In FP64 the Gram is scaled first (an entry of the packed triangle in Ts,
+    // column u at u (nbk + 1), is -conj(tau_s Gram[u,s])), so that a step is one
+    // exchange and one complex multiply-add, four FP64 instructions instead of
+    // ten on the chain; the double-float kernel keeps its order of operations.
     for (int e = tid; e < nbk * nbk; e += blockDim.x) {
       const int u = e % nbk, c = e / nbk;
-      Ts[e] = (u < c) ? ld_cg(ws.wfin + e) : (u == c ? ld_cg(tau + j0 + c) : mk(0, 0));
+      const cplx tc = (MIXED && u != c) ? mk(0, 0) : ld_cg(tau + j0 + c);
+      const cplx v = (u < c) ? ld_cg(ws.wfin + e) : (u == c ? tc : mk(0, 0));
+      if (g == 0 && Tg) Tg[(size_t)panel * nb * nb + e] = v;
+      if (MIXED) {
+        Ts[e] = v;
+      } else {
+        const cplx q = cmul(tc, v);
+        Ts[u * (nbk + 1) + c] = (u < c) ? mk(-q.x, q.y) : mk(0, 0);
+      }
     }
     __syncthreads();
-    if (g == 0 && Tg)
-      for (int e = tid; e < nbk * nbk; e += blockDim.x) Tg[(size_t)panel * nb * nb + e] = Ts[e];
-    {
+    if constexpr (!MIXED) {
+      const cplx ctl = (lane < nbk) ? cconj(ld_cg(tau + j0 + lane)) : mk(0, 0);
+      for (int l = nbk + g + wid * G; l < ncol; l += nw * G) {
+        cplx acc = (lane < nbk) ? cmul(ctl, ld_cg(ws.wfin + lane + (size_t)nbk * l)) : mk(0, 0);
+        wy_chain(acc, Ts, nbk, 0, 1);
+        if (lane < nbk) ws.wfin[lane + (size_t)nbk * l] = acc;
+      }
+    } else {
       const cplx ctl = (lane < nbk) ? cconj(Ts[lane + nbk * lane]) : mk(0, 0);  // conj(tau_lane)
       for (int l = nbk + g + wid * G; l < ncol; l += nw * G) {
         cplx acc = (lane < nbk) ? ld_cg(ws.wfin + lane + (size_t)nbk * l) : mk(0, 0);
@@ -904,8 +932,18 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
         else P[(size_t)t * R + (i - r0)] = v;
       }
     // the panel's Gram (strict upper triangle) and tau (diagonal), packed
-    // with leading dimension nbk
-    for (int e = tid; e < nbk * nbk; e += blockDim.x) Ts[e] = Tg[(size_t)panel * nb * nb + e];
+    // with leading dimension nbk; in FP64 scaled, as in the factorisation
+    // (column u at u (nbk + 1), entries -tau_s Gram[s,u])
+    for (int e = tid; e < nbk * nbk; e += blockDim.x) {
+      const cplx v = Tg[(size_t)panel * nb * nb + e];
+      if (MIXED) {
+        Ts[e] = v;
+      } else {
+        const int sr = e % nbk, u = e / nbk;
+        const cplx q = cmul(Tg[(size_t)panel * nb * nb + sr + (size_t)nbk * sr], v);
+        Ts[u * (nbk + 1) + sr] = (sr < u) ? mk(-q.x, -q.y) : mk(0, 0);
+      }
+    }
     __syncthreads();
     if (MIXED)
       partial_vhx_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<const df2*>(C), ldc, q,
@@ -925,7 +963,14 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
       }
     }
     __syncthreads();
-    {
+    if constexpr (!MIXED) {
+      const cplx tl = (lane < nbk) ? Tg[(size_t)panel * nb * nb + lane + (size_t)nbk * lane] : mk(0, 0);
+      for (int l = g + wid * G; l < q; l += nw * G) {
+        cplx acc = (lane < nbk) ? cmul(tl, ws.wfin[lane + (size_t)nbk * l]) : mk(0, 0);
+        wy_chain(acc, Ts, nbk, nbk - 1, -1);
+        if (lane < nbk) ws.wfin[lane + (size_t)nbk * l] = acc;
+      }
+    } else {
       const cplx tl = (lane < nbk) ? Ts[lane + nbk * lane] : mk(0, 0);  // tau_lane
       for (int l = g + wid * G; l < q; l += nw * G) {
         cplx acc = (lane < nbk) ? ws.wfin[lane + (size_t)nbk * l] : mk(0, 0);
