@@ -718,12 +718,12 @@ DV void gk_factor(int N, double lam, double* w) {
   double* PV = w + L_PV * N;
   const double* off = w + L_OFF * N;
   const double tiny = 4.0 * DBL_EPSILON;
-  auto guard = [&](double p) { return fabs(p) < tiny ? (p < 0.0 ? -tiny : tiny) : p; };
+  auto guard = [&](double p) { return d_mag_less(p, tiny) ? (d_neg(p) ? -tiny : tiny) : p; };
   double di = -lam, dui = (N > 1) ? off[0] : 0.0;
   double sub = dui;
   for (int i = 0; i < N - 1; ++i) {
     const double un = (i + 1 < N - 1) ? off[i + 1] : 0.0;
-    if (fabs(di) >= fabs(sub)) {
+    if (!d_mag_less(di, sub)) {
       const double rp = 1.0 / guard(di);
       const double f = sub * rp;
       Dinv[i] = rp;
@@ -750,7 +750,11 @@ DV void gk_factor(int N, double lam, double* w) {
   Dinv[N - 1] = 1.0 / guard(di);
 }
 
-// Solve with the factors, in place on B; one thread.
+// Solve with the factors, in place on B, by a whole warp (its results need a __syncwarp).  An
+// FP64 instruction of a warp takes 64 cycles, one lane or all: comparisons are
+// on the bits, the products with the reciprocal pivots run on all lanes, and
+// the chains of lane 0 have one multiply-add per row (two where rows were
+// swapped).
 DV void gk_solve(int N, double* w) {
   const double* Dinv = w + L_DINV * N;
   const double* C1 = w + L_C1 * N;
@@ -758,26 +762,43 @@ DV void gk_solve(int N, double* w) {
   const double* DL = w + L_DL * N;
   const double* PV = w + L_PV * N;
   double* B = w + L_B * N;
+  const int lane = threadIdx.x & 31;
   double cur = B[0];
-  for (int i = 0; i < N - 1; ++i) {
-    const double bn = B[i + 1], f = DL[i];
-    if (PV[i] != 0.0) {
-      B[i] = bn;
-      cur = fma(-f, bn, cur);
-    } else {
-      B[i] = cur;
-      cur = fma(-f, cur, bn);
+  if (lane == 0) {
+    double bn = B[min(1, N - 1)], f = DL[0];
+    bool swap = !d_zero(PV[0]);
+    for (int i = 0; i < N - 1; ++i) {
+      // the next row's inputs are loaded ahead of the chain
+      const int in = min(i + 1, N - 2);
+      const double bnn = B[in + 1], fn = DL[in], pn = PV[in];
+      const double row = swap ? bn : cur;
+      B[i] = row;
+      cur = fma(-f, row, swap ? cur : bn);
+      bn = bnn;
+      f = fn;
+      swap = !d_zero(pn);
     }
   }
-  double x2 = 0.0, x1 = cur * Dinv[N - 1];
-  B[N - 1] = x1;
-  for (int i = N - 2; i >= 0; --i) {
-    // x2 is known one row earlier than x1: only the last multiply-add waits on x1
-    const double t = fma(-C2[i], x2, B[i] * Dinv[i]);
-    const double x = fma(-C1[i], x1, t);
-    B[i] = x;
-    x2 = x1;
-    x1 = x;
+  __syncwarp();
+  for (int i = lane; i < N - 1; i += 32) B[i] *= Dinv[i];
+  __syncwarp();
+  if (lane == 0) {
+    double x2 = 0.0, x1 = cur * Dinv[N - 1];
+    B[N - 1] = x1;
+    int i = N - 2;
+    double t = B[max(i, 0)], c1 = C1[max(i, 0)], c2 = C2[max(i, 0)];
+    for (; i >= 0; --i) {
+      const int in = max(i - 1, 0);
+      const double tn = B[in], c1n = C1[in], c2n = C2[in];
+      if (!d_zero(c2)) t = fma(-c2, x2, t);  // swapped rows only
+      const double x = fma(-c1, x1, t);
+      B[i] = x;
+      x2 = x1;
+      x1 = x;
+      t = tn;
+      c1 = c1n;
+      c2 = c2n;
+    }
   }
 }
 
@@ -836,8 +857,8 @@ bd_vectors_kernel(const double* __restrict__ d, const double* __restrict__ e, in
         const double mul = up ? EP[in] : Q[in];
         const double addn = up ? Q[in] : EP[in];
         double piv = v + add;
-        if (fabs(piv) < tiny) {
-          piv = piv < 0.0 ? -tiny : tiny;
+        if (d_mag_less(piv, tiny)) {
+          piv = d_neg(piv) ? -tiny : tiny;
           v = piv - add;
         }
         V[i] = v;
@@ -987,7 +1008,7 @@ __global__ void bd_cluster_kernel(const double* __restrict__ d, const double* __
     for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
     __syncwarp();
     for (int it = 0; it < 3; ++it) {
-      if (lane == 0) gk_solve(N, vsm);
+      gk_solve(N, vsm);
       __syncwarp();
       for (int j = k0; j < k; ++j) {
         const double* zj = Zs + (size_t)j * N;
@@ -1060,7 +1081,7 @@ bd_invit_kernel(const double* __restrict__ d, const double* __restrict__ e, int 
     for (int i = lane; i < N; i += 32) B[i] = z[i];
     __syncwarp();
   }
-  if (lane == 0) gk_solve(N, vsm);
+  gk_solve(N, vsm);
   __syncwarp();
   double nrm = 0.0;
   for (int i = lane; i < N; i += 32) nrm += B[i] * B[i];

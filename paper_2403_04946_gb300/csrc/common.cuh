@@ -32,6 +32,14 @@ HD cplx cinv(cplx a) {
   return mk(a.x * s, -a.y * s);
 }
 
+// Comparisons on the bits: one on the values is an FP64 instruction, 64 cycles
+// of a warp.  x == 0; x < 0; |a| < |b| (the last two not for NaN).
+DV bool d_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+DV bool d_neg(double x) { return __double_as_longlong(x) < 0 && !d_zero(x); }
+DV bool d_mag_less(double a, double b) {
+  return (unsigned long long)__double_as_longlong(a) << 1 < (unsigned long long)__double_as_longlong(b) << 1;
+}
+
 // Reciprocal to FP64 rounding level: the hardware's 20-bit seed and one
 // third-order step of Householder's iteration, y (1 + e + e^2) with
 // e = 1 - x y (error e^3).  About 230 cycles of dependent operations against
@@ -60,10 +68,12 @@ DV double rsqrt_fast(double x) {
 DV void house_fast(cplx al, double s2, cplx* out) {
   const int lane = threadIdx.x & 31;
   const double a2 = fma(al.x, al.x, fma(al.y, al.y, s2));
-  const bool none = s2 == 0.0 && al.y == 0.0, in = a2 > 1e-280 && a2 < 1e280;
+  // in: a2 between 2^-928 and 2^929
+  const int hi = __double2hiint(a2);
+  const bool none = d_zero(s2) && d_zero(al.y), neg = d_neg(al.x), in = hi > 0x05f00000 && hi < 0x7a000000;
   const double rs = in ? rsqrt_fast(a2) : 1.0 / sqrt(a2);
   const double an = in ? a2 * rs : sqrt(a2);
-  const double b = al.x >= 0.0 ? -an : an, ib = al.x >= 0.0 ? -rs : rs;
+  const double b = neg ? an : -an, ib = neg ? rs : -rs;
   const double dr = al.x - b, den = fma(dr, dr, al.y * al.y);
   const double id2 = in ? rcp_fast(den) : 1.0 / den;
   const double r = ((lane & 1) ? -al.y : (lane & 2) ? dr : -dr) * ((lane & 2) ? id2 : ib);
@@ -77,11 +87,11 @@ DV void house_fast(cplx al, double s2, cplx* out) {
 // the two lanes.
 DV void house_warp(cplx al, double s2, cplx* tau, cplx* scale, double* beta) {
   const double an = sqrt(al.x * al.x + al.y * al.y + s2);
-  const double b = (al.x >= 0.0) ? -an : an;
+  const double b = d_neg(al.x) ? an : -an;
   const double dr = al.x - b, den = dr * dr + al.y * al.y;
   const double r = 1.0 / ((threadIdx.x & 1) ? den : b);
   const double ib = __shfl_sync(0xffffffffu, r, 0), id2 = __shfl_sync(0xffffffffu, r, 1);
-  const bool none = s2 == 0.0 && al.y == 0.0;
+  const bool none = d_zero(s2) && d_zero(al.y);
   *tau = none ? mk(0, 0) : mk((b - al.x) * ib, -al.y * ib);
   *scale = none ? mk(0, 0) : mk(dr * id2, -al.y * id2);
   *beta = none ? al.x : b;
