@@ -685,7 +685,7 @@ hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int
   if (ctx->p.precision == HOPF_FP64 && hk::qr_wide_applies(m, std::min(m, k))) {
     TRY(tc_reserve(ctx, m, k));
     *nb = 32;
-    CK(hk::geqrf_wide(A, lda, m, k, tau, T, ctx->tcbuf, ctx->tcbytes, ctx->coop, 0, ctx->stream,
+    CK(hk::geqrf_wide(A, lda, m, k, tau, T, ctx->tcbuf, ctx->tcbytes, ctx->coop, ctx->stream,
                       phase_timer(ctx, HOPF_K_QR)));
     return HOPF_OK;
   }
@@ -922,7 +922,7 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Rb, pp, pp, cols, w.Mb, cols, ctx->stream));
         if (hk::qr_wide_applies(cols, pp)) {
           TRY(tc_reserve_bytes(ctx, hk::qr_wide_scratch_bytes(cols, pp)));
-          CK(hk::geqrf_wide(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, nullptr, ctx->tcbuf, ctx->tcbytes, ctx->coop, 0,
+          CK(hk::geqrf_wide(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, nullptr, ctx->tcbuf, ctx->tcbytes, ctx->coop,
                             ctx->stream, phase_timer(ctx, HOPF_K_SVD)));
         } else {
           LAUNCH(HOPF_K_SVD, qr_flops(cols, pp), 0, 1, hk::geqrf(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, w.T + (size_t)c * w.tstride, &nbl, ctx->coop, ctx->stream, 0));

@@ -308,7 +308,7 @@ size_t qr_tc_scratch_bytes(int m, int k, int S);        // scratch of one call
 size_t qr_tc_gram_elems(int k);                         // complex elements of Gout
 // As geqrf (mixed), plus Gout: per outer panel j the Gram v_s^H v_u of its
 // reflectors (128 x 128 block at Gout + j 128^2, leading dimension 128),
-// which ormqr_tc needs.  T receives the inner panels' records as geqrf.
+// which ormqr_tc needs.
 cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* Gout, void* scratch,
                      size_t scratch_bytes, const CoopWs& cws, int S, cudaStream_t s, const PhaseTimer& pt);
 // C <- Q C for the Q of geqrf_tc (p reflectors).
@@ -316,12 +316,12 @@ cudaError_t ormqr_tc(const cplx* A, int lda, int m, int p, const cplx* tau, cons
                      void* scratch, size_t scratch_bytes, int* err, int S, cudaStream_t s, const PhaseTimer& pt);
 
 // The same at FP64 accuracy: panels of 32 columns by the cooperative kernel
-// (FP64, or double-float if mixed), their Gram and all trailing products from
+// (FP64), their Gram and all trailing products from
 // the wide digits.  T: per panel the record of geqrf (may be NULL).
 bool qr_wide_applies(int m, int p);
 size_t qr_wide_scratch_bytes(int m, int k);
 cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void* scratch, size_t scratch_bytes,
-                       const CoopWs& cws, int mixed, cudaStream_t s, const PhaseTimer& pt);
+                       const CoopWs& cws, cudaStream_t s, const PhaseTimer& pt);
 // C <- Q C for the Q of geqrf_wide (T as it left it).
 cudaError_t ormqr_wide(const cplx* A, int lda, int m, int p, const cplx* T, cplx* C, int ldc, int q, void* scratch,
                        size_t scratch_bytes, int* err, cudaStream_t s, const PhaseTimer& pt);

@@ -410,7 +410,7 @@ size_t qr_wide_scratch_bytes(int m, int k) {
 }
 
 cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void* scratch, size_t scratch_bytes,
-                       const CoopWs& cws, int mixed, cudaStream_t s, const PhaseTimer& pt) {
+                       const CoopWs& cws, cudaStream_t s, const PhaseTimer& pt) {
   const int S = tc_wide_digits(), Kc = tc_chunk(S);
   const int p = std::min(m, k);
   cudaError_t e = cudaSuccess;
@@ -419,7 +419,7 @@ cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void*
     cplx* Ap = A + j0 + (size_t)lda * j0;
     int nb = kWidePanel;
     int slot = pt.b();
-    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, mixed);
+    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, 0);
     pt.e(slot, pt.cls_panel, 8.0 * mv * (double)nbk * nbk - 8.0 * (double)nbk * nbk * nbk / 3.0, 1);
     if (e != cudaSuccess || (nt <= 0 && !T)) continue;
     Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
