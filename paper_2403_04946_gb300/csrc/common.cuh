@@ -250,6 +250,15 @@ DV cplx warp_sum(cplx v) {
   for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return mk(__shfl_sync(0xffffffffu, s, 0), __shfl_sync(0xffffffffu, s, 16));
 }
+// Sum of a complex value over S >= 2 adjacent lanes (a power of two): the even
+// ones return its real part, the odd ones its imaginary part, for half the
+// additions of summing both.
+DV double half_sum(cplx a, int S) {
+  const bool im = threadIdx.x & 1;
+  double h = (im ? a.y : a.x) + __shfl_xor_sync(0xffffffffu, im ? a.x : a.y, 1);
+  for (int o = 2; o < S; o <<= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+  return h;
+}
 DV float warp_sumf(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

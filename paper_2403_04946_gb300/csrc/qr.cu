@@ -100,16 +100,6 @@ DV void reduce_scatter(df2 (&a)[CH], int lane) {
   for (; o >= 1; o >>= 1) a[0] = df_cadd(a[0], df_shfl_xor(a[0], o));
 }
 
-// Sum of a complex value over S >= 2 adjacent lanes (a power of two): the even
-// ones return its real part, the odd ones its imaginary part, for half the
-// additions of summing both.
-DV double half_sum(cplx a, int S) {
-  const bool im = threadIdx.x & 1;
-  double h = (im ? a.y : a.x) + __shfl_xor_sync(0xffffffffu, im ? a.x : a.y, 1);
-  for (int o = 2; o < S; o <<= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
-  return h;
-}
-
 // Partial products V^H X over this CTA's rows [lo, hi) (global row index),
 // V in shared memory (P, leading dimension R, rows offset r0), X column l
 // given by a pointer.  One warp per column; results to out[s + nbk * l].
@@ -699,18 +689,20 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       } else {
         // -f for the pivot row (v = 1), -scale f for the rows below, which
         // hold x until the next column's barrier; even threads the real parts,
-        // odd ones the imaginary parts (the chain is six FP64 instructions of
+        // odd ones the imaginary parts (the chain is seven FP64 instructions of
         // a warp instead of fourteen)
         if (wid < 2) {
           const int c = tid >> 1, im = tid & 1;
           const cplx raw = c < nrem ? praw[c] : mk(0, 0);
-          auto mul = [&](cplx a, double p, double q, double z) {  // that part of a (p, q) + z
-            return fma(a.x, p, fma(im ? a.y : -a.y, q, z));
+          auto mul = [&](cplx a, double p, double q) {  // that part of a (p, q)
+            return fma(a.x, p, (im ? a.y : -a.y) * q);
           };
           auto other = [](double v) { return __shfl_xor_sync(0xffffffffu, v, 1); };
-          const double w = mul(cconj(sc), im ? raw.y : raw.x, im ? raw.x : raw.y, rvh);
-          const double f = mul(cconj(tu), w, other(w), 0.0);
-          const double sf = mul(sc, f, other(f), 0.0);
+          // (the product rounded before the sum, as in a complex product: the
+          // mixed path's LQ passes here, and what follows it shows a rounding)
+          const double w = rvh + mul(cconj(sc), im ? raw.y : raw.x, im ? raw.x : raw.y);
+          const double f = mul(cconj(tu), w, other(w));
+          const double sf = mul(sc, f, other(f));
           if (c < nrem) {
             reinterpret_cast<double*>(wl + c)[im] = -f;
             reinterpret_cast<double*>(wl + kNbMax + c)[im] = -sf;
@@ -1004,7 +996,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
 // FP64 unit of 2 per clock) and the sum over the CTAs' partials; the first
 // outweighs the second down to a few rows.  With 64 rows per CTA, 16 CTAs at
 // least (what it was): a C1 step (336 x 96 factors) 68 ms against 52 ms with 8
-// rows, 53 with 16, 60 with 32; the CDF workload's factors (64 to 942 rows, up to 942
+// rows, 53 with 16, 60 with 32 (39.7 and 42.9 ms with 8 and 16 now); the CDF workload's factors (64 to 942 rows, up to 942
 // columns) ran on 16 CTAs, 437 against 310 ms a step.  Mixed precision keeps 64 rows from 2048
 // rows on: there the order of the sums shows in its digit-cut products.
 static void pick_layout(int m, int mixed, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {

@@ -187,20 +187,25 @@ cudaError_t sum_core(const SumTerm* terms_dev, int nterms, int kind, int n, cplx
 // Phi[i_1..i_d] = C_1[0,i_1,:] C_2[:,i_2,:] ... C_d[:,i_d,0]; one CTA per
 // point, the running row vector in shared memory.  S adjacent lanes share a
 // column of the slice (interleaved rows: contiguous in memory) and add their
-// parts by shuffles; S = 4 for many columns (the additions across lanes cost
-// FP64 time), more when the columns do not fill the CTA.  Many points are
+// parts by shuffles.  An FP64 instruction of a warp takes 64 cycles of a quarter
+// of the SM: 4 ceil(a / S) for the products, log2 S for the additions, so S is
+// the least that gives each quarter a warp: 4 from 17 columns, 8 below, more for
+// the few columns of a long row vector (one lane per column from 17 columns when
+// there are many points: fewest instructions and CTA barriers; 2000 points at
+// r = 64, d = 10: 543 us, 256 threads with four lanes per column 548, now 521).  Many points are
 // bound by the FP64 units (r^2 complex multiply-adds per mode, 2 per clock
 // and SM).  Few points are bound by latency, d dependent products: the
 // indices are known ahead, so every slice is prefetched into L2 first, and
 // each thread keeps four loads and two sums in flight (one thread per column
 // walking all rows took 6.7 us per mode at r = 32).
-constexpr int kEvThreads = 256;
-template <int S>
+constexpr int ev_threads(bool few) { return few ? 256 : 128; }
+template <int S, int T>
 DV void eval_mode(const cplx* __restrict__ C, size_t cs, int a, int c, const cplx* v, cplx* w) {
   const int seg = threadIdx.x % S;
-  constexpr int per = kEvThreads / S;
+  constexpr int per = T / S;
   for (int jb = 0; jb < c; jb += per) {
     const int j = jb + threadIdx.x / S;
+    if (jb + (threadIdx.x & ~31u) / S >= (unsigned)c) continue;  // no column in this warp
     cplx s0 = mk(0, 0), s1 = mk(0, 0);
     if (j < c) {
       const cplx* col = C + cs * j;
@@ -214,29 +219,31 @@ DV void eval_mode(const cplx* __restrict__ C, size_t cs, int a, int c, const cpl
       }
       for (; i < a; i += S) s0 = cfma(v[i], __ldg(col + i), s0);
     }
-    s0 = cadd(s0, s1);
-#pragma unroll
-    for (int o = 1; o < S; o <<= 1) {
-      s0.x += __shfl_xor_sync(0xffffffffu, s0.x, o);
-      s0.y += __shfl_xor_sync(0xffffffffu, s0.y, o);
+    if (a > 3 * S) s0 = cadd(s0, s1);
+    if constexpr (S == 1) {
+      if (j < c) w[j] = s0;
+    } else {
+      const double h = half_sum(s0, S);
+      if (seg < 2 && j < c) reinterpret_cast<double*>(w + j)[seg] = h;
     }
-    if (seg == 0 && j < c) w[j] = s0;
   }
 }
 
-__global__ void __launch_bounds__(kEvThreads)
+template <bool FEW>
+__global__ void __launch_bounds__(ev_threads(FEW))
 eval_points_kernel(const cplx* const* __restrict__ cores, const int* __restrict__ ranks, int d, int n, int rmax,
-                   int prefetch, const int* __restrict__ idx, cplx* __restrict__ vals) {
+                   const int* __restrict__ idx, cplx* __restrict__ vals) {
+  constexpr int T = ev_threads(FEW);
   extern __shared__ __align__(16) unsigned char sm[];
   cplx* vb = reinterpret_cast<cplx*>(sm);  // [2][rmax]
   const int pt = blockIdx.x;
   const int* ip = idx + (size_t)pt * d;
-  if (prefetch) {
+  if constexpr (FEW) {
     // one 128-byte line (8 values of a column) per thread and step
     for (int k = 0; k < d; ++k) {
       const int a = ranks[k], c = ranks[k + 1], lines = (a + 7) / 8;
       const cplx* C = cores[k] + (size_t)a * ip[k];
-      for (int t = threadIdx.x; t < lines * c; t += kEvThreads)
+      for (int t = threadIdx.x; t < lines * c; t += T)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(C + (size_t)a * n * (t / lines) + 8 * (t % lines)));
     }
   }
@@ -249,10 +256,11 @@ eval_points_kernel(const cplx* const* __restrict__ cores, const int* __restrict_
     const cplx* v = vb + (size_t)cur * rmax;
     cplx* w = vb + (size_t)(cur ^ 1) * rmax;
     const size_t cs = (size_t)a * n;
-    if (c > 32) eval_mode<4>(C, cs, a, c, v, w);
-    else if (c > 16) eval_mode<8>(C, cs, a, c, v, w);
-    else if (c > 8) eval_mode<16>(C, cs, a, c, v, w);
-    else eval_mode<32>(C, cs, a, c, v, w);
+    if (!FEW && c > 16) eval_mode<1, T>(C, cs, a, c, v, w);
+    else if (c > 16) eval_mode<4, T>(C, cs, a, c, v, w);
+    else if (a <= 16 || c > 8) eval_mode<8, T>(C, cs, a, c, v, w);
+    else if (c > 4) eval_mode<16, T>(C, cs, a, c, v, w);
+    else eval_mode<32, T>(C, cs, a, c, v, w);
     __syncthreads();
   }
   if (threadIdx.x == 0) vals[pt] = vb[(size_t)cur * rmax];
@@ -263,11 +271,13 @@ cudaError_t eval_points(const cplx* const* cores_dev, const int* ranks_dev, int 
   if (npts <= 0) return cudaSuccess;
   const int rmax = std::max(maxr, 1);
   const size_t smem = sizeof(cplx) * 2 * (size_t)rmax;
-  cudaError_t e = allow_smem((const void*)eval_points_kernel, smem);
+  // with several points per SM the next point's loads hide the latency, and
+  // what counts is the number of FP64 instructions and of resident CTAs
+  const bool few = npts <= 2 * dev_info().sm_count;
+  const auto fn = few ? eval_points_kernel<true> : eval_points_kernel<false>;
+  cudaError_t e = allow_smem((const void*)fn, smem);
   if (e != cudaSuccess) return e;
-  // with several points per SM the next point's loads hide the latency
-  const int prefetch = npts <= 2 * dev_info().sm_count;
-  eval_points_kernel<<<npts, kEvThreads, smem, s>>>(cores_dev, ranks_dev, d, n, rmax, prefetch, idx_dev, vals);
+  fn<<<npts, ev_threads(few), smem, s>>>(cores_dev, ranks_dev, d, n, rmax, idx_dev, vals);
   return cudaGetLastError();
 }
 
