@@ -37,7 +37,6 @@
 //  4. U = Q [u_1 .. u_rho] by applying the left reflectors.
 #include <algorithm>
 #include <cfloat>
-#include <utility>
 
 #include "kernels.h"
 
@@ -110,10 +109,10 @@ DV double sum_to_warp0(double v, bool has, double* red) {
 // alternate between two halves by column parity: a CTA writing column
 // i+2's data has passed both barriers of column i+1, so every reader of
 // column i's half is done.
-// FAST (FP64 contexts): reflector scalars from the reciprocal root and
-// reciprocal of common.cuh, about 800 cycles less on each of a column's two
-// scalar chains.  The mixed path keeps the IEEE forms (bd_invit_kernel says
-// why its factors are kept to the last bit).
+// FAST: reflector scalars from the reciprocal root and reciprocal of
+// common.cuh, about 800 cycles less on each of a column's two scalar chains.
+// Without it the IEEE forms (bd_serial_kernel says where the factors are kept
+// to the last bit).
 template <bool FAST>
 __global__ void __launch_bounds__(kBdThreads, 1)
 gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* tauq, cplx* taup,
@@ -214,7 +213,9 @@ gebrd_kernel(cplx* A, int lda, int n, int nloc, double* dg, double* eg, cplx* ta
       while (cc < C) {
         const int c = i + 1 + cc;
         if (lane == 0) {
-          const cplx f = cmul(ctq, cadd(a_ic, cmul(cscq, acc)));
+          // (the compiler may fuse a product's rounding into the sum around it)
+          const cplx f = FAST ? cmul(ctq, cadd(a_ic, cmul(cscq, acc)))
+                              : cmul_rounded(ctq, cadd(a_ic, cmul_rounded(cscq, acc)));
           fvg[c] = f;
           nrg[c] = csub(a_ic, f);
         }
@@ -357,7 +358,7 @@ bool gebrd_fits(int n, const CoopWs& ws, bool have_rows_ws) {
 }
 
 cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cplx* taup,
-                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int mixed) {
+                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int kept) {
   if (n <= 0) return cudaSuccess;
   int nloc;
   size_t smem;
@@ -367,7 +368,7 @@ cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cpl
   cplx* rows_global = glob ? rows_ws : nullptr;
   if ((size_t)2 * G * (n + 1) > ws.pc_elems || (size_t)6 * n > ws.wfin_elems || 2 * G > 1024)
     return cudaErrorInvalidValue;
-  void* fn = mixed ? (void*)gebrd_kernel<false> : (void*)gebrd_kernel<true>;
+  void* fn = kept ? (void*)gebrd_kernel<false> : (void*)gebrd_kernel<true>;
   cudaError_t err = allow_smem(fn, smem);
   if (err != cudaSuccess) return err;
   err = cudaMemsetAsync(&ws.bar->count, 0, sizeof(unsigned int), s);
@@ -577,7 +578,7 @@ bd_sigma_kernel(const float2* __restrict__ a2, const double* __restrict__ info, 
   if (t == 0) sig[k] = 0.5 * (lo + hi) * amax;
 }
 
-// The mixed path's values (see bd_invit_kernel): one warp per value on T_GK,
+// The kept form of the values (see bd_serial_kernel): one warp per value on T_GK,
 // sig[k] = k-th largest singular value of B.  The
 // bracket [lo, hi) keeps #{sigma < lo} < target <= #{sigma < hi} with
 // target = n - k; each round the lanes count at 32 interior points.
@@ -608,12 +609,12 @@ __global__ void bd_sigma_gk_kernel(const float2* __restrict__ a2, const double* 
 }
 
 cudaError_t bd_sigma(const double* d, const double* e, int n, float2* a2, double* info, double* sig,
-                     int mixed, cudaStream_t s) {
+                     int kept, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   bd_prep_kernel<<<1, 256, 0, s>>>(d, e, n, a2, info);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  if (mixed) bd_sigma_gk_kernel<<<(n + 3) / 4, 128, 0, s>>>(a2, info, n, sig);
+  if (kept) bd_sigma_gk_kernel<<<(n + 3) / 4, 128, 0, s>>>(a2, info, n, sig);
   else if (n <= 512) bd_sigma_kernel<4><<<n, 128, 0, s>>>(a2, info, n, sig);
   else bd_sigma_kernel<1><<<n, 32, 0, s>>>(a2, info, n, sig);
   return cudaGetLastError();
@@ -750,18 +751,17 @@ DV void gk_factor(int N, double lam, double* w) {
   Dinv[N - 1] = 1.0 / guard(di);
 }
 
-// Solve with the factors, in place on B, by a whole warp (its results need a __syncwarp).  An
-// FP64 instruction of a warp takes 64 cycles, one lane or all: comparisons are
+// Solve with the factors at w, in place on B, by a whole warp (its results need
+// a __syncwarp).  An FP64 instruction of a warp takes 64 cycles, one lane or all: comparisons are
 // on the bits, the products with the reciprocal pivots run on all lanes, and
 // the chains of lane 0 have one multiply-add per row (two where rows were
 // swapped).
-DV void gk_solve(int N, double* w) {
+DV void gk_solve(int N, const double* w, double* B) {
   const double* Dinv = w + L_DINV * N;
   const double* C1 = w + L_C1 * N;
   const double* C2 = w + L_C2 * N;
   const double* DL = w + L_DL * N;
   const double* PV = w + L_PV * N;
-  double* B = w + L_B * N;
   const int lane = threadIdx.x & 31;
   double cur = B[0];
   if (lane == 0) {
@@ -1008,7 +1008,7 @@ __global__ void bd_cluster_kernel(const double* __restrict__ d, const double* __
     for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
     __syncwarp();
     for (int it = 0; it < 3; ++it) {
-      gk_solve(N, vsm);
+      gk_solve(N, vsm, B);
       __syncwarp();
       for (int j = k0; j < k; ++j) {
         const double* zj = Zs + (size_t)j * N;
@@ -1039,95 +1039,131 @@ __global__ void bd_cluster_kernel(const double* __restrict__ d, const double* __
   }
 }
 
-// ---- vectors of the mixed path ------------------------------------------------
-// The digit products cut U at 2^-40 of its largest entry, about the 1e-12 by
-// which a vector in a cluster of values (gaps below 1e-3 sigma_max) moves with
-// the rounding of its computation, so another method shows in the mixed
-// path's results at 1e-2 of their error (1e-9 of a covariance).  Here the
-// vectors stay those of three steps of inverse iteration on T_GK - lambda I
-// with Gram-Schmidt inside clusters, at the T_GK values, but all of them at
-// once: the LU factors and the solves of every value are independent, and
-// since each step leaves the vectors orthogonal to about 1e-9 already,
-// Gram-Schmidt in order is its first-order form
-//   z_k <- z_k (1 - (g_kk - 1) / 2) - sum_{j < k, same cluster} g_jk z_j
-// with g the Gram before the step.  One serial warp per cluster took 14.3 ms
-// per factor on average at n = 384 (up to 43 ms).  Values so close that a
-// step leaves 1e-4 or more set info[2]: the serial kernel then runs.
-// lu: per value the five factor arrays (5 N); Z: N per value.
+// ---- vectors kept to the last bit ----------------------------------------------
+// In a mixed context with digit products U is cut at 2^-40 of its largest
+// entry, about the 1e-12 by which a vector in a cluster of values moves with the
+// rounding of its computation; the flipped digits move a covariance (a second
+// difference of Phi) by 1e-10 to 2e-9.  There the vectors are those of
+// bd_cluster_kernel, in its order of operations, from two kernels instead of
+// one: bd_factor_kernel does for all values at once what does not wait for other
+// vectors (the LU factors, a division per row on the chain, and the first
+// solve), bd_serial_kernel the rest, one CTA per cluster.
+//   lu: 5 N doubles per value (the factor arrays), Z: N per value.
 __global__ void __launch_bounds__(32)
-bd_invit_kernel(const double* __restrict__ d, const double* __restrict__ e, int n, const double* __restrict__ info,
-                const double* __restrict__ sig, int first, double* __restrict__ lu, double* __restrict__ Z) {
+bd_factor_kernel(const double* __restrict__ d, const double* __restrict__ e, int n, const double* __restrict__ info,
+                 const double* __restrict__ sig, double* __restrict__ lu, double* __restrict__ Z) {
   extern __shared__ __align__(16) double vsm[];  // kSolveArrays * N
   const int k = blockIdx.x, lane = threadIdx.x, N = 2 * n;
   const double amax = info[0];
   if (amax == 0.0) return;
-  double* B = vsm + L_B * N;
-  double* f = lu + (size_t)k * 5 * N;
-  double* z = Z + (size_t)k * N;
-  if (first) {
-    const double inv = 1.0 / amax;
-    double* off = vsm + L_OFF * N;
-    for (int i = lane; i < N - 1; i += 32) off[i] = ((i & 1) ? e[i >> 1] : d[i >> 1]) * inv;
-    __syncwarp();
-    if (lane == 0) gk_factor(N, sig[k] * inv, vsm);
-    for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
-    __syncwarp();
-    // (the last rows of C1, C2, DL, PV are never written or read)
-    for (int i = lane; i < 5 * N; i += 32)
-      if (i < N || i % N < N - 1) f[i] = vsm[i];
-  } else {
-    for (int i = lane; i < 5 * N; i += 32)
-      if (i < N || i % N < N - 1) vsm[i] = f[i];
-    for (int i = lane; i < N; i += 32) B[i] = z[i];
-    __syncwarp();
-  }
-  gk_solve(N, vsm);
+  const double inv = 1.0 / amax;
+  double *off = vsm + L_OFF * N, *B = vsm + L_B * N;
+  for (int i = lane; i < N - 1; i += 32) off[i] = ((i & 1) ? e[i >> 1] : d[i >> 1]) * inv;
   __syncwarp();
-  double nrm = 0.0;
-  for (int i = lane; i < N; i += 32) nrm += B[i] * B[i];
-  nrm = warp_sum(nrm);
-  const double s = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
-  for (int i = lane; i < N; i += 32) z[i] = B[i] * s;
+  if (lane == 0) gk_factor(N, sig[k] * inv, vsm);
+  for (int i = lane; i < N; i += 32) B[i] = start_value(i, k);
+  __syncwarp();
+  // (the last rows of C1, C2, DL, PV are never written or read)
+  double* f = lu + (size_t)k * 5 * N;
+  for (int i = lane; i < 5 * N; i += 32)
+    if (i < N || i % N < N - 1) f[i] = vsm[i];
+  gk_solve(N, vsm, B);
+  __syncwarp();
+  for (int i = lane; i < N; i += 32) Z[(size_t)k * N + i] = B[i];
 }
 
-// The ordered Gram-Schmidt step, one CTA per vector; with X, the result is
-// the normalised left part (entries 1, 3, ..) instead.
-__global__ void __launch_bounds__(kOrthThreads)
-bd_gs_kernel(int n, const double* __restrict__ sig, const double* __restrict__ Z, double* __restrict__ Zo,
-             double* __restrict__ X, int ldx, double* __restrict__ info) {
-  extern __shared__ __align__(16) double osm[];  // z_k [N], g [k + 1]
-  __shared__ double red[32];
-  const int N = 2 * n, k = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kOrthThreads >> 5;
-  double *zk = osm, *g = osm + N;
-  for (int i = threadIdx.x; i < N; i += kOrthThreads) zk[i] = Z[(size_t)k * N + i];
+// Per vector of a cluster: Gram-Schmidt against the members before it,
+// normalisation, and twice solve, Gram-Schmidt, normalisation.  A dot product's
+// 32 chains (one per lane) fix warp 0 to it; the other warps stage the next
+// vector meanwhile and share the update, and while warp 0 solves they load the
+// next value's factors (two buffers of each, where they fit).  Bound by warp 0's
+// FP64 instructions: per pair N / 32 of the chain, 5 of the sum, N / 128 of the
+// update.
+constexpr int kSerialThreads = 128;
+size_t bd_serial_smem(int n, int buffers) { return sizeof(double) * (6 * (size_t)buffers + 1) * 2 * n; }
+
+__global__ void __launch_bounds__(kSerialThreads)
+bd_serial_kernel(int n, const double* __restrict__ info, const double* __restrict__ sig, int nvec,
+                 const double* __restrict__ lu, double* Z, double* __restrict__ X, int ldx, int buffers) {
+  extern __shared__ __align__(16) double ssm[];
+  __shared__ double bcast;
+  const int N = 2 * n, k0 = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  if (info[0] == 0.0) return;
   const double gap_tol = 1e-3 * sig[0];
-  int k0 = k;  // first member of the cluster
-  while (k0 > 0 && sig[k0 - 1] - sig[k0] < gap_tol) --k0;
-  __syncthreads();
-  for (int j = k0 + wid; j <= k; j += nw) {
-    const double* zj = Z + (size_t)j * N;
-    double s = 0.0;
-    for (int i = lane; i < N; i += 32) s = fma(zj[i], zk[i], s);
-    s = warp_sum(s);
-    if (lane == 0) {
-      g[j - k0] = (j == k) ? 0.5 * (s - 1.0) : s;
-      if (!(fabs(j == k ? s - 1.0 : s) <= 1e-4)) info[2] = 1.0;
+  if (k0 > 0 && sig[k0 - 1] - sig[k0] < gap_tol) return;  // not the first of its cluster
+  int k1 = k0 + 1;
+  while (k1 < nvec && sig[k1 - 1] - sig[k1] < gap_tol) ++k1;
+  double* F = ssm;                                // [buffers][5 N]
+  double* B = F + (size_t)buffers * 5 * N;        // [N]
+  double* zb = B + N;                             // [buffers][N]
+  const int odd = buffers - 1;  // with two buffers odd values and vectors use the second
+  // factors of value k by the threads from t0 on
+  auto load_factors = [&](int k, int t0) {
+    double* dst = F + (size_t)((k & 1) & odd) * 5 * N;
+    const double* src = lu + (size_t)k * 5 * N;
+    for (int i = tid - t0; i < 5 * N; i += kSerialThreads - t0)
+      if (i < N || i % N < N - 1) dst[i] = src[i];
+  };
+  auto load_vector = [&](double* dst, int j, int t0) {
+    for (int i = tid - t0; i < N; i += kSerialThreads - t0) dst[i] = Z[(size_t)j * N + i];
+  };
+  load_factors(k0, 0);
+  for (int k = k0; k < k1; ++k) {
+    load_vector(B, k, 0);
+    __syncthreads();
+    const double* f = F + (size_t)((k & 1) & odd) * 5 * N;
+    for (int it = 0; it < 3; ++it) {
+      if (it > 0) {
+        if (tid < 32) gk_solve(N, f, B);
+        else if (it == 1 && buffers == 2 && k + 1 < k1) load_factors(k + 1, 32);
+        __syncthreads();
+      }
+      if (k > k0) load_vector(zb, k0, 0);
+      __syncthreads();
+      for (int j = k0; j < k; ++j) {
+        const double* zj = zb + (size_t)((j - k0) & odd) * N;
+        if (tid < 32) {
+          double dot = 0.0;
+          for (int i = lane; i < N; i += 32) dot = fma(zj[i], B[i], dot);
+          dot = warp_sum(dot);
+          if (lane == 0) bcast = dot;
+        } else if (buffers == 2 && j + 1 < k) {
+          load_vector(zb + (size_t)((j + 1 - k0) & 1) * N, j + 1, 32);
+        }
+        __syncthreads();
+        const double dot = bcast;
+        for (int i = tid; i < N; i += kSerialThreads) B[i] = fma(-dot, zj[i], B[i]);
+        if (buffers == 1 && j + 1 < k) {
+          __syncthreads();
+          load_vector(zb, j + 1, 0);
+        }
+        __syncthreads();
+      }
+      if (tid < 32) {
+        double nrm = 0.0;
+        for (int i = lane; i < N; i += 32) nrm = fma(B[i], B[i], nrm);
+        nrm = warp_sum(nrm);
+        if (lane == 0) bcast = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
+      }
+      __syncthreads();
+      const double s = bcast;
+      for (int i = tid; i < N; i += kSerialThreads) B[i] *= s;
+      __syncthreads();
     }
+    for (int i = tid; i < N; i += kSerialThreads) Z[(size_t)k * N + i] = B[i];
+    if (tid < 32) {
+      double un = 0.0;
+      for (int i = lane; i < N; i += 32)
+        if (i & 1) un = fma(B[i], B[i], un);
+      un = warp_sum(un);
+      if (lane == 0) bcast = un > 0.0 ? 1.0 / sqrt(un) : 0.0;
+    }
+    if (buffers == 1 && k + 1 < k1) load_factors(k + 1, 0);
+    __syncthreads();
+    const double s = bcast;
+    for (int i = tid; i < n; i += kSerialThreads) X[i + (size_t)ldx * k] = B[2 * i + 1] * s;
+    __syncthreads();
   }
-  __syncthreads();
-  double un = 0.0;
-  for (int i = threadIdx.x; i < N; i += kOrthThreads) {
-    double v = 0.0;
-    for (int j = k0; j <= k; ++j) v = fma(Z[(size_t)j * N + i], g[j - k0], v);
-    v = zk[i] - v;
-    if (!X) Zo[(size_t)k * N + i] = v;
-    else if (i & 1) un = fma(v, v, un);
-    if (X) zk[i] = v;
-  }
-  if (!X) return;
-  un = block_sum(un, red);
-  const double s = un > 0.0 ? 1.0 / sqrt(un) : 0.0;
-  for (int i = threadIdx.x; i < n; i += kOrthThreads) X[i + (size_t)ldx * k] = zk[2 * i + 1] * s;
 }
 
 // Orthonormal completion for kept values at the noise level (indices
@@ -1167,38 +1203,35 @@ __global__ void bd_complete_kernel(int n, int kt, int nvec, double* __restrict__
 }
 
 
-size_t bd_lu_elems(int n, int kt) { return (size_t)14 * n * kt; }
+size_t bd_lu_elems(int n, int kt) { return (size_t)10 * n * kt; }
 
 cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, const double* sig,
                        int kt, int nvec, double* X, int ldx, double* Zs, double* lu, cudaStream_t s) {
-  const bool mixed = lu != nullptr;
   if (nvec <= 0) return cudaSuccess;
-  if (kt > 0) {
-    const size_t vsmem = sizeof(double) * kVecArrays * (size_t)n, csmem = bd_vectors_smem(n);
-    const size_t osmem = sizeof(double) * ((mixed ? 2 : 1) * (size_t)n + kt);
-    cudaError_t err = allow_smem(mixed ? (const void*)bd_gs_kernel : (const void*)bd_orth_kernel, osmem);
-    if (err == cudaSuccess) err = allow_smem((const void*)bd_cluster_kernel, csmem);
-    if (err == cudaSuccess)
-      err = mixed ? allow_smem((const void*)bd_invit_kernel, csmem) : allow_smem((const void*)bd_vectors_kernel, vsmem);
+  if (kt > 0 && lu) {
+    const size_t fsmem = bd_vectors_smem(n);
+    const int buffers = bd_serial_smem(n, 2) <= (size_t)dev_info().max_smem_optin - 1024 ? 2 : 1;
+    const size_t smem = bd_serial_smem(n, buffers);
+    cudaError_t err = allow_smem((const void*)bd_factor_kernel, fsmem);
+    if (err == cudaSuccess) err = allow_smem((const void*)bd_serial_kernel, smem);
     if (err != cudaSuccess) return err;
-    if (mixed) {
-      const size_t nz = (size_t)2 * n * kt;
-      double *Z = lu + 5 * nz, *Zo = Z + nz;
-      for (int it = 0; it < 3; ++it) {
-        bd_invit_kernel<<<kt, 32, csmem, s>>>(d, e, n, info, sig, it == 0, lu, Z);
-        bd_gs_kernel<<<kt, kOrthThreads, osmem, s>>>(n, sig, Z, Zo, it == 2 ? X : nullptr, ldx, info);
-        std::swap(Z, Zo);
-      }
-    } else {
-      bd_vectors_kernel<<<kt, 32, vsmem, s>>>(d, e, n, info, sig, X, ldx);
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthFirst);
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthNext);
-    }
+    bd_factor_kernel<<<kt, 32, fsmem, s>>>(d, e, n, info, sig, lu, Zs);
+    bd_serial_kernel<<<kt, kSerialThreads, smem, s>>>(n, info, sig, kt, lu, Zs, X, ldx, buffers);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  } else if (kt > 0) {
+    const size_t vsmem = sizeof(double) * kVecArrays * (size_t)n, csmem = bd_vectors_smem(n);
+    const size_t osmem = sizeof(double) * ((size_t)n + kt);
+    cudaError_t err = allow_smem((const void*)bd_orth_kernel, osmem);
+    if (err == cudaSuccess) err = allow_smem((const void*)bd_cluster_kernel, csmem);
+    if (err == cudaSuccess) err = allow_smem((const void*)bd_vectors_kernel, vsmem);
+    if (err != cudaSuccess) return err;
+    bd_vectors_kernel<<<kt, 32, vsmem, s>>>(d, e, n, info, sig, X, ldx);
+    bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthFirst);
+    bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthNext);
     bd_cluster_kernel<<<kt, 32, csmem, s>>>(d, e, n, info, sig, kt, X, ldx, Zs);
-    if (!mixed) {
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthClustered);
-      bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthClustered);
-    }
+    bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, X, ldx, Zs, n, info, kOrthClustered);
+    bd_orth_kernel<<<kt, kOrthThreads, osmem, s>>>(n, kt, Zs, n, X, ldx, info, kOrthClustered);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
@@ -1215,10 +1248,11 @@ cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, co
 // (about 10 n^2 / 2 operations per vector) spreads over many SMs.  A warp's
 // FP64 instruction holds its quarter of the SM for 64 cycles, so one warp per
 // vector ran at a quarter of the SM's rate (7400 cycles for two reflectors at
-// n = 192; a factor of the C3 mixed step 520 us, 289 with four).  Four warps share a reflector: the real and the imaginary part of
-// the dot product on two of them each, by halves of the rows (SPLIT, FP64
-// contexts; the mixed path keeps the order of one warp's sums and every bit,
-// bd_invit_kernel says why), then a quarter of the rows' update each.
+// n = 192; a factor of the C3 mixed step 520 us, 289 with four).  Four warps
+// share a reflector: the real and the imaginary part of the dot product on two
+// of them each, by halves of the rows (SPLIT; without it one warp's order of
+// the sums and its bits, bd_serial_kernel says where), then a quarter of the
+// rows' update each.
 // kBackStage further warps stage the next reflectors in shared memory.
 // The result goes to U (n x nvec, ldu) and to Xp (mrows x nvec, ldp, zero
 // below row n).
@@ -1302,11 +1336,11 @@ bd_back_kernel(const cplx* __restrict__ A, int lda, const cplx* __restrict__ tau
 }
 
 cudaError_t bd_back(const cplx* A, int lda, const cplx* tauq, int n, const double* X, int ldx, int nvec,
-                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int mixed, cudaStream_t s) {
+                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int kept, cudaStream_t s) {
   if (nvec <= 0) return cudaSuccess;
   // 80 bytes per row: less than the vectors' own solves keep (bd_vectors_smem)
   const size_t smem = sizeof(cplx) * (size_t)n * (2 * kBackStage + 1);
-  const auto fn = mixed ? bd_back_kernel<false> : bd_back_kernel<true>;
+  const auto fn = kept ? bd_back_kernel<false> : bd_back_kernel<true>;
   cudaError_t err = allow_smem((const void*)fn, smem);
   if (err != cudaSuccess) return err;
   fn<<<nvec, 32 * (kBackStage + kBackWarps), smem, s>>>(A, lda, tauq, n, X, ldx, nvec, U, ldu, Xp, ldp, mrows);

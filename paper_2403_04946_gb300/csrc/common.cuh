@@ -19,6 +19,11 @@ HD cplx cmul(cplx a, cplx b) { return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y 
 // conj(a) * b
 HD cplx cmulc(cplx a, cplx b) { return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
 HD double cabs2(cplx a) { return a.x * a.x + a.y * a.y; }
+// a * b rounded by itself whatever stands around it: cmul's second products may
+// be fused with a sum that takes its result.
+DV cplx cmul_rounded(cplx a, cplx b) {
+  return mk(fma(a.x, b.x, -__dmul_rn(a.y, b.y)), fma(a.x, b.y, __dmul_rn(a.y, b.x)));
+}
 // acc + a * b
 DV cplx cfma(cplx a, cplx b, cplx acc) {
   return mk(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));

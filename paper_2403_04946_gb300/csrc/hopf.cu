@@ -57,8 +57,7 @@ struct RoundWs {
   double* bd_info = nullptr;  // 4
   double* bd_X = nullptr;     // kcap * kcap
   double* bd_Zs = nullptr;    // kcap * 2 kcap
-  double* bd_lu = nullptr;    // mixed: factors of the inverse iteration, grown on demand
-  size_t bd_lu_elems = 0;
+  double* bd_lu = nullptr;    // kept forms: factors of the inverse iteration
   // mixed precision, tensor-core QR: per core the Gram blocks of the
   // phase-1 reflectors (gstride elements each), and those of phase 2's QR
   cplx* G = nullptr;
@@ -66,6 +65,7 @@ struct RoundWs {
   cplx* G2 = nullptr;
   // rows of a bidiagonalisation too large for shared memory
   cplx* bd_rows = nullptr;
+  bool kept = false;          // this rounding's forms (kept_order)
 };
 
 struct hopf_ctx {
@@ -183,6 +183,21 @@ hopf_status fail(hopf_ctx* c, hopf_status st, const char* fmt, ...) {
 // Mixed precision: FP32 trailing updates and products in QR / apply-Q /
 // merges; FP64 Householder panels and Jacobi SVD.
 #define MIXED_FLAG (ctx->p.precision == HOPF_MIXED ? 1 : 0)
+
+// Contexts whose roundings keep one order of operations for good, to the last
+// bit (kQrKept, bd_serial_kernel).  The five-digit products cut what they take
+// at 2^-40, so that a changed last bit anywhere before one flips digits: Phi
+// then moves by 3e-11 to 9e-11 and a covariance, a second difference of Phi, by
+// 1e-10 to 2e-9, whatever the change was.  That matters where moments are taken
+// (the CDF equation has none: its values move by up to 8e-11) and where a factor can
+// reach the products' 4096 rows: ranks go up to 6 rank_cap in a step's
+// roundings, or to those of the tensor at hand.
+bool kept_order(const hopf_ctx* ctx, const hopf_tt* t) {
+  if (ctx->p.precision != HOPF_MIXED || ctx->equation != HOPF_EQ_PHI) return false;
+  if (ctx->qr_method != HOPF_QR_TENSOR && !ctx->autotune) return false;
+  const long long r = std::max(6 * (long long)ctx->p.rank_cap, (long long)t->cap_rank);
+  return r * ctx->p.n >= 4096;
+}
 
 #define TRY(expr)                        \
   do {                                   \
@@ -422,7 +437,7 @@ hopf_status coop_reserve(hopf_ctx* ctx, int kcap) {
   return HOPF_OK;
 }
 
-hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
+hopf_status round_buffers(hopf_ctx* ctx, const hopf_tt* t) {
   size_t need = 0;
   for (size_t c : t->core_cap) need = std::max(need, c);
   const int kcap = t->cap_rank;
@@ -472,14 +487,12 @@ hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
   return coop_reserve(ctx, K);
 }
 
-hopf_status bd_lu_reserve(hopf_ctx* ctx, size_t elems) {
+// Workspace of a rounding of t, and the forms it takes.
+hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
+  TRY(round_buffers(ctx, t));
   RoundWs& w = ctx->rw;
-  if (elems <= w.bd_lu_elems) return HOPF_OK;
-  dfree(w.bd_lu);
-  w.bd_lu = nullptr;
-  w.bd_lu_elems = 0;
-  CK(dalloc(&w.bd_lu, elems));
-  w.bd_lu_elems = elems;
+  w.kept = kept_order(ctx, t);
+  if (w.kept && !w.bd_lu) CK(dalloc(&w.bd_lu, hk::bd_lu_elems(w.kcap, w.kcap)));
   return HOPF_OK;
 }
 
@@ -679,6 +692,10 @@ bool conf_tc(const hopf_ctx* ctx, const QrConf& c, int m, int p) {
   return ctx->p.precision == HOPF_MIXED && c.method == HOPF_QR_TENSOR && hk::qr_tc_applies(m, p);
 }
 
+int qr_mode(const hopf_ctx* ctx) {
+  return (MIXED_FLAG ? hk::kQrMixed : hk::kQrFp64) | (ctx->rw.kept ? hk::kQrKept : 0);
+}
+
 hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int m, int k, cplx* tau, cplx* T,
                            int* nb, cplx* G) {
   CtaCap cap(ctx, c.ctas);
@@ -696,7 +713,7 @@ hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int
                     phase_timer(ctx, HOPF_K_QR)));
     return HOPF_OK;
   }
-  LAUNCH(HOPF_K_QR, qr_flops(m, k), 0, 1, hk::geqrf(A, lda, m, k, tau, T, nb, ctx->coop, ctx->stream, MIXED_FLAG));
+  LAUNCH(HOPF_K_QR, qr_flops(m, k), 0, 1, hk::geqrf(A, lda, m, k, tau, T, nb, ctx->coop, ctx->stream, qr_mode(ctx)));
   return HOPF_OK;
 }
 
@@ -799,7 +816,7 @@ hopf_status qr_apply(hopf_ctx* ctx, const cplx* A, int lda, int m, int p, const 
     return HOPF_OK;
   }
   LAUNCH(HOPF_K_APPLYQ, applyq_flops(m, q, p), 0, 1,
-         hk::ormqr(A, lda, m, p, tau, T, nb, C, ldc, q, ctx->coop, ctx->stream, MIXED_FLAG));
+         hk::ormqr(A, lda, m, p, tau, T, nb, C, ldc, q, ctx->coop, ctx->stream, qr_mode(ctx)));
   return HOPF_OK;
 }
 
@@ -920,18 +937,18 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
       } else {
         int nbl = 32;
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Rb, pp, pp, cols, w.Mb, cols, ctx->stream));
-        if (hk::qr_wide_applies(cols, pp)) {
+        if (!w.kept && hk::qr_wide_applies(cols, pp)) {
           TRY(tc_reserve_bytes(ctx, hk::qr_wide_scratch_bytes(cols, pp)));
           CK(hk::geqrf_wide(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, nullptr, ctx->tcbuf, ctx->tcbytes, ctx->coop,
                             ctx->stream, phase_timer(ctx, HOPF_K_SVD)));
         } else {
-          LAUNCH(HOPF_K_SVD, qr_flops(cols, pp), 0, 1, hk::geqrf(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, w.T + (size_t)c * w.tstride, &nbl, ctx->coop, ctx->stream, 0));
+          LAUNCH(HOPF_K_SVD, qr_flops(cols, pp), 0, 1, hk::geqrf(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, w.T + (size_t)c * w.tstride, &nbl, ctx->coop, ctx->stream, w.kept ? hk::kQrKept : hk::kQrFp64));
         }
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::extract_r(w.Mb, cols, pp, pp, w.Jb, pp, ctx->stream));
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Jb, pp, pp, pp, w.Mb, pp, ctx->stream));
       }
-      LAUNCH(HOPF_K_SVD, gebrd_flops(pp), 0, 1, hk::gebrd(w.Mb, pp, pp, w.bd_d, w.bd_e, w.bd_tauq, w.bd_taup, ctx->coop, ctx->stream, w.bd_rows, MIXED_FLAG));
-      LAUNCH(HOPF_K_SVD, 0, 0, 2, hk::bd_sigma(w.bd_d, w.bd_e, pp, w.bd_a2, w.bd_info, w.sig, MIXED_FLAG, ctx->stream));
+      LAUNCH(HOPF_K_SVD, gebrd_flops(pp), 0, 1, hk::gebrd(w.Mb, pp, pp, w.bd_d, w.bd_e, w.bd_tauq, w.bd_taup, ctx->coop, ctx->stream, w.bd_rows, w.kept));
+      LAUNCH(HOPF_K_SVD, 0, 0, 2, hk::bd_sigma(w.bd_d, w.bd_e, pp, w.bd_a2, w.bd_info, w.sig, w.kept, ctx->stream));
       LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::bd_rank(w.sig, pp, ctx->d_dbl + 1, cap, forced_c, ctx->d_int, ctx->d_dbl + 2, w.sig + pp, ctx->stream));
       TRY(read_small_checked(ctx, 3, 5));
       ctx->prof.svd_count += 1;
@@ -974,9 +991,8 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
     // new core c = Q [U_rho; 0]
     if (use_bd) {
       const int kt = std::min(ctx->h_int[2], rnew);
-      if (MIXED_FLAG) TRY(bd_lu_reserve(ctx, hk::bd_lu_elems(pp, kt)));
-      LAUNCH(HOPF_K_SVD, 0, 0, (kt > 0 ? 6 + MIXED_FLAG : 0) + (kt < rnew), hk::bd_vectors(w.bd_d, w.bd_e, pp, w.bd_info, w.sig, kt, rnew, w.bd_X, pp, w.bd_Zs, MIXED_FLAG ? w.bd_lu : nullptr, ctx->stream));
-      LAUNCH(HOPF_K_SVD, 0, 0, 1, hk::bd_back(w.Mb, pp, w.bd_tauq, pp, w.bd_X, pp, rnew, w.Ub, pp, t->cores[c], Mrows, Mrows, MIXED_FLAG, ctx->stream));
+      LAUNCH(HOPF_K_SVD, 0, 0, (kt > 0 ? (w.kept ? 2 : 6) : 0) + (kt < rnew), hk::bd_vectors(w.bd_d, w.bd_e, pp, w.bd_info, w.sig, kt, rnew, w.bd_X, pp, w.bd_Zs, w.kept ? w.bd_lu : nullptr, ctx->stream));
+      LAUNCH(HOPF_K_SVD, 0, 0, 1, hk::bd_back(w.Mb, pp, w.bd_tauq, pp, w.bd_X, pp, rnew, w.Ub, pp, t->cores[c], Mrows, Mrows, w.kept, ctx->stream));
     } else if (case1) {
       LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::gather_u(w.Mb, pp, pp, w.perm, w.sig, 1, rnew, t->cores[c], Mrows, Mrows, w.Ub, pp, ctx->stream));
     } else {
@@ -1271,8 +1287,8 @@ hopf_status cross_sweep(hopf_ctx* ctx, CrossBufs& B, int cap, const std::vector<
       if ((size_t)M * cnt > cores->core_cap[k]) return fail(ctx, HOPF_EINVAL, "cross: core %d exceeds capacity", k);
       CK(hk::cross_gather(B.A, M, B.piv + cap, cnt, B.Q, B.W, B.seq, ctx->stream));
       int nb = 32;
-      CK(hk::geqrf(B.Q, M, M, cnt, B.tau, B.T, &nb, ctx->coop, ctx->stream, 0));
-      CK(hk::ormqr(B.Q, M, M, cnt, B.tau, B.T, nb, B.W, M, cnt, ctx->coop, ctx->stream, 0));
+      CK(hk::geqrf(B.Q, M, M, cnt, B.tau, B.T, &nb, ctx->coop, ctx->stream, hk::kQrFp64));
+      CK(hk::ormqr(B.Q, M, M, cnt, B.tau, B.T, nb, B.W, M, cnt, ctx->coop, ctx->stream, hk::kQrFp64));
       TRY(check_barrier(ctx));
       CK(hk::cross_core(B.W, M, B.piv, B.seq, cnt, B.Gw, B.Gi, cores->cores[k], ctx->stream));
     }

@@ -50,14 +50,18 @@ cudaError_t allow_smem(const void* fn, size_t need);
 // every panel of width `nb` its reflectors' Gram matrix v_u^H v_s (strict
 // upper triangle) with tau on the diagonal, in T (npanel x nb x nb); ormqr
 // applies the panel from these.  Returns the panel width used through
-// *nb_out.  mixed != 0: the matrix is held in double-float form (scaled by a
-// power of two) during the factorisation, the Householder scalars in FP64.
+// *nb_out.  mode, of:
+//   kQrMixed  the matrix is held in double-float form (scaled by a power of
+//             two) during the factorisation, the Householder scalars in FP64;
+//   kQrKept   one order of the sums for good (rows per CTA, lanes, CTAs), for
+//             contexts whose digit products show the last bit of what they cut.
+enum { kQrFp64 = 0, kQrMixed = 1, kQrKept = 2 };
 cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_out,
-                  const CoopWs& ws, cudaStream_t s, int mixed = 0);
+                  const CoopWs& ws, cudaStream_t s, int mode);
 // C <- Q C with Q = H_0 H_1 ... H_{p-1} from geqrf (A, lda, m, p, tau, T, nb);
-// C is m x q column-major (ldc).
+// C is m x q column-major (ldc); mode as geqrf had it.
 cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* T,
-                  int nb, cplx* C, int ldc, int q, const CoopWs& ws, cudaStream_t s, int mixed = 0);
+                  int nb, cplx* C, int ldc, int q, const CoopWs& ws, cudaStream_t s, int mode);
 
 // One-sided Jacobi SVD of the nr x nc column-major matrix M (ldm), in place:
 // on exit the columns of M are U_i * sigma_i (any order); if accumJ, J
@@ -87,14 +91,14 @@ cudaError_t rank_select(const cplx* M, int ldm, int nr, int nc, const double* ep
 // rows_ws (may be NULL): gebrd_rows_elems(n) elements where the rows go when
 // they do not fit in shared memory (L2-resident for the sizes met here).
 cudaError_t gebrd(cplx* A, int lda, int n, double* d, double* e, cplx* tauq, cplx* taup,
-                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int mixed);
+                  const CoopWs& ws, cudaStream_t s, cplx* rows_ws, int kept);
 bool gebrd_fits(int n, const CoopWs& ws, bool have_rows_ws = false);
 size_t gebrd_rows_elems(int n, int sms);
 // All singular values of B, sorted descending, into sig[n]; a2 (float2
-// [2n]) and info (double [4]) are scratch kept for bd_vectors.  mixed: the
-// values of the mixed path, see bd_invit_kernel.
+// [2n]) and info (double [4]) are scratch kept for bd_vectors.  kept (here and
+// below): the forms of the mixed path with digit products, see bd_serial_kernel.
 cudaError_t bd_sigma(const double* d, const double* e, int n, float2* a2, double* info, double* sig,
-                     int mixed, cudaStream_t s);
+                     int kept, cudaStream_t s);
 // Rank rule on sorted values: out_int[0] = rho, [1] = rho by tolerance,
 // [2] = number of kept values above the noise level 2 n eps ||B||_F;
 // out_dbl as rank_select; tail2[n+1] scratch.
@@ -102,14 +106,14 @@ cudaError_t bd_rank(const double* sig, int n, const double* eps_hat, int cap, in
                     double* out_dbl, double* tail2, cudaStream_t s);
 // Left singular vectors of B: columns k < kt by twisted factorisation, columns
 // kt..nvec-1 by orthonormal completion; X (n x nvec, ldx), real.
-// Zs: nvec x 2n doubles of scratch; lu (NULL in FP64): bd_lu_elems(n, kt)
-// doubles for the mixed path's inverse iteration.
+// Zs: nvec x 2n doubles of scratch; lu (NULL unless kept): bd_lu_elems(n, kt)
+// doubles for the factors of the inverse iteration.
 size_t bd_lu_elems(int n, int kt);
 cudaError_t bd_vectors(const double* d, const double* e, int n, double* info, const double* sig,
                        int kt, int nvec, double* X, int ldx, double* Zs, double* lu, cudaStream_t s);
 // U = Q X -> U (n x nvec, ldu) and Xp (mrows x nvec, ldp, zero below row n).
 cudaError_t bd_back(const cplx* A, int lda, const cplx* tauq, int n, const double* X, int ldx, int nvec,
-                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int mixed, cudaStream_t s);
+                    cplx* U, int ldu, cplx* Xp, int ldp, int mrows, int kept, cudaStream_t s);
 
 // ---- TT-cross construction of a Gaussian (cross.cu) --------------------------
 // A (rl n x rr, column-major, row alpha + rl i) = Phi0(Il[alpha], i, Jr[beta])

@@ -400,7 +400,11 @@ __device__ __forceinline__ void wy_chain(cplx& acc, const cplx* M, int nbk, int 
   }
 }
 
-template <int NB, bool MIXED>
+// KEPT (FP64): sums over rows and CTAs in the order of one warp per column and
+// one addition after another, IEEE reflector scalars, the reflector scaled
+// before the update.  Slower by a third per column; for factors whose last bit
+// is part of the result (kQrKept in kernels.h).
+template <int NB, bool MIXED, bool KEPT = false>
 __global__ void __launch_bounds__(qr_threads(MIXED), 1)
 geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
              CoopWs ws) {
@@ -528,6 +532,29 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (g == gown)
           for (int c = tid; c < nbk - t; c += blockDim.x)
             reinterpret_cast<df2*>(rowp)[c] = Pd[(size_t)(t + c) * R + (jj - r0)];
+      } else if constexpr (KEPT) {
+        const cplx* xt = P + (size_t)t * R;
+        double sq = 0.0;
+        for (int i = ilo + tid; i < r1; i += blockDim.x) sq += cabs2(xt[i - r0]);
+        sq = block_sum(sq, dred);
+        if (tid == 0) prp[g] = sq;
+        for (int cb = wid; cb < nrem; cb += 4 * nw) {
+          cplx acc[4] = {mk(0, 0), mk(0, 0), mk(0, 0), mk(0, 0)};
+          for (int i = ilo + lane; i < r1; i += 32) {
+            const cplx x = xt[i - r0];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (cb + q * nw < nrem) acc[q] = cfmac(x, P[(size_t)(t + 1 + cb + q * nw) * R + (i - r0)], acc[q]);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (cb + q * nw < nrem) {
+              acc[q] = warp_sum(acc[q]);
+              if (lane == 0) myp[cb + q * nw] = acc[q];
+            }
+        }
+        if (g == gown)
+          for (int c = tid; c < nbk - t; c += blockDim.x) rowp[c] = P[(size_t)(t + c) * R + (jj - r0)];
       } else {
         // columns t (its norm) .. nbk-1 at once: S lanes per column.  Eight for
         // CTAs of up to 64 rows, where the FP64 additions across more lanes
@@ -553,7 +580,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if (g == gown)
           for (int q = tid; q < nbk - t; q += blockDim.x) rowp[q] = P[(size_t)(t + q) * R + (jj - r0)];
       }
-      if constexpr (MIXED) {
+      if constexpr (MIXED || KEPT) {
         if (grid_sync(gs)) return;
       } else {
         // while the other CTAs arrive: column t-1 becomes its reflector
@@ -568,7 +595,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       // (b) the reflector (zlarfg conventions: beta real, v_jj = 1), in FP64
       cplx rv = mk(0, 0);  // mixed: entry t + 1 + tid of the pivot row (warp 0)
       double rvh = 0.0;    // FP64: part tid & 1 of its entry t + 1 + tid / 2 (warps 0 and 1)
-      if (!MIXED && tid < 2 * nrem) rvh = ld_cg(reinterpret_cast<const double*>(rowp + 1) + tid);
+      if (!MIXED && !KEPT && tid < 2 * nrem) rvh = ld_cg(reinterpret_cast<const double*>(rowp + 1) + tid);
       if (wid == 0) {
         // the pivot row is loaded with the first batch of partial norms (all
         // one L2 round trip away)
@@ -577,8 +604,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         if constexpr (MIXED) al = df_to_scaled(ld_cg_df(rowp), 0);
         else al = ld_cg(rowp);
         double s2 = 0.0;
-        const double* nsrc = MIXED ? prp : reinterpret_cast<const double*>(ws.pc + tail0 + (size_t)par * nb);
-        const size_t nstride = MIXED ? 1 : 2 * pstride;
+        const double* nsrc = MIXED || KEPT ? prp : reinterpret_cast<const double*>(ws.pc + tail0 + (size_t)par * nb);
+        const size_t nstride = MIXED || KEPT ? 1 : 2 * pstride;
         for (int g0 = lane; g0 < G; g0 += 32 * kLoadBatch) {
           double v[kLoadBatch];
 #pragma unroll
@@ -588,7 +615,17 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
             if (g0 + 32 * u < G) s2 += v[u];
         }
         s2 = warp_sum(s2);
-        if (!MIXED) house_fast(al, s2, bc);
+        if constexpr (!MIXED && !KEPT) house_fast(al, s2, bc);
+        if constexpr (KEPT) {
+          cplx tu, sc;
+          double beta;
+          house_warp(al, s2, &tu, &sc, &beta);
+          if (lane == 0) {
+            bc[0] = tu;
+            bc[1] = sc;
+            bc[2] = mk(beta, 0.0);
+          }
+        }
         if constexpr (MIXED) {
           cplx tu, sc;
           double beta;
@@ -612,8 +649,8 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       }
       // raw sums over the CTAs of the dot products (tpc threads per
       // column); warp 0 is left out, so that these sums run while it forms
-      // the reflector
-      constexpr int skip = 32;
+      // the reflector (KEPT: all threads, whose count sets the order)
+      constexpr int skip = KEPT ? 0 : 32;
       if (nrem > 0 && tid >= skip) {
         const int nthr = blockDim.x - skip, t2 = tid - skip;
         int tpc = 32;
@@ -622,7 +659,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
         for (int base = 0; base < nrem; base += per) {
           const int c = base + t2 / tpc;
           const bool valid = c < nrem && t2 / tpc < per;
-          const cplx* src = ws.pc + tail0 + (size_t)par * nb + c + (MIXED ? 0 : 1);
+          const cplx* src = ws.pc + tail0 + (size_t)par * nb + c + (MIXED || KEPT ? 0 : 1);
           if constexpr (MIXED) {
             df2 acc = df_zero();
             if (valid)
@@ -649,14 +686,17 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
                   const int gg = g0 + tpc * u;
                   v[u] = (gg < G) ? ld_cg(src + (size_t)gg * pstride) : mk(0, 0);
                 }
-                // pairs first: half the dependent FP64 additions
+                constexpr int step = KEPT ? 1 : 2;
+                if constexpr (!KEPT) {
+                  // pairs first: half the dependent FP64 additions
 #pragma unroll
-                for (int u = 0; u < kLoadBatch; u += 2) v[u] = cadd(v[u], v[u + 1]);
+                  for (int u = 0; u < kLoadBatch; u += 2) v[u] = cadd(v[u], v[u + 1]);
+                }
 #pragma unroll
-                for (int u = 0; u < kLoadBatch; u += 2)
+                for (int u = 0; u < kLoadBatch; u += step)
                   if (g0 + tpc * u < G) acc = cadd(acc, v[u]);
               }
-            // four threads or more: 31 columns at most for 224 threads
+            // four threads or more: 31 columns at most for 224 threads or 256
             const double h = half_sum(acc, tpc);
             if (valid && sub < 2) reinterpret_cast<double*>(praw + c)[sub] = h;
           }
@@ -686,6 +726,15 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           xt[i - r0] = df_scalb(df_cadd(v, df_zero()), es);
         }
         if (tid == 0 && jj >= r0 && jj < r1) xt[jj - r0] = bcd[3];
+      } else if constexpr (KEPT) {
+        for (int c = tid; c < nrem; c += blockDim.x) {
+          const cplx w = cadd(ld_cg(rowp + 1 + c), cmul(cconj(sc), praw[c]));
+          const cplx f = cmul(cconj(tu), w);
+          wl[c] = mk(-f.x, -f.y);  // -f
+        }
+        cplx* xt = P + (size_t)t * R;
+        for (int i = ilo + tid; i < r1; i += blockDim.x) xt[i - r0] = cmul(xt[i - r0], sc);
+        if (tid == 0 && jj >= r0 && jj < r1) xt[jj - r0] = bc[2];
       } else {
         // -f for the pivot row (v = 1), -scale f for the rows below, which
         // hold x until the next column's barrier; even threads the real parts,
@@ -743,7 +792,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
           const int cw = 32 / L;
           for (int c = wid * cw + lane / L; c < nrem; c += nw * cw) {
             cplx* ac = P + (size_t)(t + 1 + c) * R;
-            const cplx sf = wl[kNbMax + c];
+            const cplx sf = wl[KEPT ? c : kNbMax + c];  // (KEPT: x is the reflector already)
             for (int i = ilo - r0 + lane % L; i < r1 - r0; i += L) ac[i] = cfma(xt[i], sf, ac[i]);
           }
           if (g == gown)
@@ -755,7 +804,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       }
       __syncthreads();
     }
-    if constexpr (!MIXED) {
+    if constexpr (!MIXED && !KEPT) {
       const cplx psc = bc[1];
       cplx* xp = P + (size_t)(nbk - 1) * R;
       for (int i = max(lo, j0 + nbk) + tid; i < r1; i += blockDim.x) xp[i - r0] = cmul(xp[i - r0], psc);
@@ -805,7 +854,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
     } else {
       cplx* out = ws.pc + (size_t)g * pstride;
       // Gram block: columns are the reflectors themselves (from shared memory)
-      if (R <= kFewRows) {
+      if (!KEPT && R <= kFewRows) {
         partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, P - r0, R, nbk, out, true);
         if (nt > 0)
           partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, out + (size_t)nbk * nbk, false);
@@ -837,10 +886,10 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
     // ten on the chain; the double-float kernel keeps its order of operations.
     for (int e = tid; e < nbk * nbk; e += blockDim.x) {
       const int u = e % nbk, c = e / nbk;
-      const cplx tc = (MIXED && u != c) ? mk(0, 0) : ld_cg(tau + j0 + c);
+      const cplx tc = ((MIXED || KEPT) && u != c) ? mk(0, 0) : ld_cg(tau + j0 + c);
       const cplx v = (u < c) ? ld_cg(ws.wfin + e) : (u == c ? tc : mk(0, 0));
       if (g == 0 && Tg) Tg[(size_t)panel * nb * nb + e] = v;
-      if (MIXED) {
+      if (MIXED || KEPT) {
         Ts[e] = v;
       } else {
         const cplx q = cmul(tc, v);
@@ -848,7 +897,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       }
     }
     __syncthreads();
-    if constexpr (!MIXED) {
+    if constexpr (!MIXED && !KEPT) {
       const cplx ctl = (lane < nbk) ? cconj(ld_cg(tau + j0 + lane)) : mk(0, 0);
       for (int l = nbk + g + wid * G; l < ncol; l += nw * G) {
         cplx acc = (lane < nbk) ? cmul(ctl, ld_cg(ws.wfin + lane + (size_t)nbk * l)) : mk(0, 0);
@@ -876,7 +925,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
       if (MIXED)
         update_x_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<df2*>(A) + (size_t)lda * c0,
                        lda, nt, ws.wfin + (size_t)nbk * nbk);
-      else if (R <= kFewRows)
+      else if (!KEPT && R <= kFewRows)
         update_x_few<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, ws.wfin + (size_t)nbk * nbk);
       else
         update_x<NB>(P, R, r0, lo, r1, nbk, A + (size_t)lda * c0, lda, nt, ws.wfin + (size_t)nbk * nbk);
@@ -994,15 +1043,17 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
 // CTAs of a factorisation: 8 rows each until every SM has one.  A column costs
 // the CTAs their rows' multiply-adds (8 per row and remaining column, on an
 // FP64 unit of 2 per clock) and the sum over the CTAs' partials; the first
-// outweighs the second down to a few rows.  With 64 rows per CTA, 16 CTAs at
-// least (what it was): a C1 step (336 x 96 factors) 68 ms against 52 ms with 8
-// rows, 53 with 16, 60 with 32 (39.7 and 42.9 ms with 8 and 16 now); the CDF workload's factors (64 to 942 rows, up to 942
-// columns) ran on 16 CTAs, 437 against 310 ms a step.  Mixed precision keeps 64 rows from 2048
-// rows on: there the order of the sums shows in its digit-cut products.
-static void pick_layout(int m, int mixed, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {
+// outweighs the second down to a few rows.  With 64 rows per CTA and 16 CTAs at
+// least: a C1 step (336 x 96 factors) 68 ms against 52 ms with 8 rows, 53 with
+// 16, 60 with 32 (39.7 and 42.9 ms with 8 and 16 now); the CDF workload's
+// factors (64 to 942 rows, up to 942 columns) on 16 CTAs, 437 against 310 ms a
+// step.  kQrKept: those 64 rows, since the count of CTAs is the order of the
+// sums; mixed factors from 2048 rows on have them too (as fast there).
+static void pick_layout(int m, int mode, const CoopWs& ws, int* G, int* R, int* nb, size_t* smem) {
   const DevInfo& di = dev_info();
-  const int rows = mixed && m >= 2048 ? 64 : 8;
-  const int g = std::max(1, std::min(coop_sms(ws), (m + rows - 1) / rows));
+  const int few = (m + 7) / 8, many = (m + 63) / 64;
+  const int want = (mode & kQrKept) ? std::max(many, std::min(16, few)) : ((mode & kQrMixed) && m >= 2048 ? many : few);
+  const int g = std::max(1, std::min(coop_sms(ws), want));
   int r = (m + g - 1) / g;
   int b = kNbMax;
   const size_t lim = (size_t)di.max_smem_optin - 16384;  // static shared memory too
@@ -1014,11 +1065,12 @@ static void pick_layout(int m, int mixed, const CoopWs& ws, int* G, int* R, int*
 }
 
 cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_out,
-                  const CoopWs& ws, cudaStream_t s, int mixed) {
+                  const CoopWs& ws, cudaStream_t s, int mode) {
+  const bool mixed = mode & kQrMixed, kept = mode & kQrKept;
   if (m <= 0 || k <= 0) return cudaSuccess;
   int G, R, nb;
   size_t smem;
-  pick_layout(m, mixed, ws, &G, &R, &nb, &smem);
+  pick_layout(m, mode, ws, &G, &R, &nb, &smem);
   // per CTA: S1 partials nb (nb + k), then the panel's exchange tail 4 nb
   if ((size_t)G * ((size_t)nb * (nb + k) + 4 * (size_t)nb) > ws.pc_elems || (size_t)nb * (nb + k) > ws.wfin_elems)
     return cudaErrorInvalidValue;
@@ -1028,6 +1080,10 @@ cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_ou
     if (nb == 32) fn = (void*)geqrf_kernel<32, true>;
     else if (nb == 16) fn = (void*)geqrf_kernel<16, true>;
     else fn = (void*)geqrf_kernel<8, true>;
+  } else if (kept) {
+    if (nb == 32) fn = (void*)geqrf_kernel<32, false, true>;
+    else if (nb == 16) fn = (void*)geqrf_kernel<16, false, true>;
+    else fn = (void*)geqrf_kernel<8, false, true>;
   } else {
     if (nb == 32) fn = (void*)geqrf_kernel<32, false>;
     else if (nb == 16) fn = (void*)geqrf_kernel<16, false>;
@@ -1039,18 +1095,20 @@ cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_ou
   e = cudaMemsetAsync(&ws.bar->count, 0, sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   void* args[] = {&A, &lda, &m, &k, &tau, &T, &nb, &R, &w};
-  return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(qr_threads(mixed != 0)), args, smem, s);
+  return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(qr_threads(mixed)), args, smem, s);
 }
 
 cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* T,
-                  int nb, cplx* C, int ldc, int q, const CoopWs& ws, cudaStream_t s, int mixed) {
+                  int nb, cplx* C, int ldc, int q, const CoopWs& ws, cudaStream_t s, int mode) {
+  const bool mixed = mode & kQrMixed;
   (void)tau;
   if (m <= 0 || p <= 0 || q <= 0) return cudaSuccess;
   int G, R, nb2;
   size_t smem;
-  pick_layout(m, mixed, ws, &G, &R, &nb2, &smem);
+  pick_layout(m, mode, ws, &G, &R, &nb2, &smem);
   if (nb2 != nb) {
-    // the layout depends only on m, so geqrf and ormqr agree
+    // the layout depends on m, mode and the context's CTAs only, so geqrf and
+    // ormqr agree
     return cudaErrorInvalidValue;
   }
   if ((size_t)G * nb * (size_t)q > ws.pc_elems || (size_t)nb * q > ws.wfin_elems)
@@ -1071,7 +1129,7 @@ cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const c
   e = cudaMemsetAsync(&ws.bar->count, 0, sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&A, &lda, &m, &p, (void*)&T, &nb, &C, &ldc, &q, &R, &w};
-  return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(qr_threads(mixed != 0)), args, smem, s);
+  return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(qr_threads(mixed)), args, smem, s);
 }
 
 }  // namespace hk

@@ -226,7 +226,7 @@ cudaError_t geqrf_tc(cplx* A, int lda, int m, int k, cplx* tau, cplx* Gout, void
     int slot = pt.b();
     // without the record of the 32-column blocks: G below takes its place, and
     // the kernel leaves the last block's products and their barriers out
-    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, 1);
+    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, kQrMixed);
     pt.e(slot, pt.cls_panel, 8.0 * mv * (double)nbk * nbk - 8.0 * (double)nbk * nbk * nbk / 3.0, 1);
     if (e != cudaSuccess) break;
     Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
@@ -419,7 +419,7 @@ cudaError_t geqrf_wide(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, void*
     cplx* Ap = A + j0 + (size_t)lda * j0;
     int nb = kWidePanel;
     int slot = pt.b();
-    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, 0);
+    e = geqrf(Ap, lda, mv, nbk, tau + j0, nullptr, &nb, cws, s, kQrFp64);
     pt.e(slot, pt.cls_panel, 8.0 * mv * (double)nbk * nbk - 8.0 * (double)nbk * nbk * nbk / 3.0, 1);
     if (e != cudaSuccess || (nt <= 0 && !T)) continue;
     Carve c{static_cast<unsigned char*>(scratch), scratch_bytes};
