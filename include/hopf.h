@@ -71,7 +71,9 @@ typedef struct {
   int rank_cap;   /* rank cap used by hopf_step                           */
   int precision;  /* HOPF_FP64: every step at FP64 accuracy (products of   */
                   /* tall factors as eight-digit BF16 splits on the tensor */
-                  /* cores, exact to 2^-60).  HOPF_MIXED: the              */
+                  /* cores: exact to 2^-60 of the largest entries they     */
+                  /* meet, in a row and 128 columns of either side, the    */
+                  /* bonds' gauges balanced first).  HOPF_MIXED: the       */
                   /* dense products of the rounding (QR trailing updates,  */
                   /* Q applications, merges, U^H R) run on the tensor     */
                   /* cores as digit-split BF16 products with exact FP32   */

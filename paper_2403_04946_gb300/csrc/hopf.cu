@@ -630,14 +630,16 @@ hopf_status tc_product(hopf_ctx* ctx, const hk::TcOperandView& a, const hk::TcOp
   const size_t ba = (hk::tc_operand_bytes(a.R, a.K, S, Kc) + 255) & ~(size_t)255;
   const size_t bb = (hk::tc_operand_bytes(b.R, b.K, S, Kc) + 255) & ~(size_t)255;
   const size_t np = hk::tc_part_elems(a.R, b.R, a.K, S);
-  TRY(tc_reserve_bytes(ctx, ba + bb + np * sizeof(cplx) + 256));
+  const bool wide = S == hk::tc_wide_digits();
+  const size_t bt = wide ? (2 * (size_t)a.K * sizeof(int) + 255) & ~(size_t)255 : 0;
+  TRY(tc_reserve_bytes(ctx, ba + bb + bt + np * sizeof(cplx) + 256));
   unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
   hk::TcOperand oa, ob;
   const int slot = prof_begin(ctx);
-  CK(hk::tc_split2(a, &oa, buf, b, &ob, buf + ba, S, ctx->stream));
-  CK(hk::tc_zgemm(oa, ob, out, 1, ldo, 1.0, 0, np ? reinterpret_cast<cplx*>(buf + ba + bb) : nullptr, np,
+  CK(hk::tc_split2(a, &oa, buf, b, &ob, buf + ba, S, ctx->stream, wide ? reinterpret_cast<int*>(buf + ba + bb) : nullptr));
+  CK(hk::tc_zgemm(oa, ob, out, 1, ldo, 1.0, 0, np ? reinterpret_cast<cplx*>(buf + ba + bb + bt) : nullptr, np,
                   &ctx->coop.bar->err, ctx->stream));
-  prof_end(ctx, slot, HOPF_K_TC, flops, 0.0, np ? 3 : 2);
+  prof_end(ctx, slot, HOPF_K_TC, flops, 0.0, 2 + (np > 0) + wide);
   return HOPF_OK;
 }
 

@@ -279,9 +279,11 @@ int tc_max_digits();   // 5
 int tc_wide_digits();  // 8: products at FP64 accuracy
 // Splits the operand into S digit planes in `buf` (tc_operand_bytes).
 cudaError_t tc_split(const TcOperandView& v, int S, TcOperand* out, void* buf, cudaStream_t s);
-// Two operands in one launch.
+// Two operands in one launch.  top (wide digits; 2 K ints of scratch): the
+// contraction index is balanced first, column k of a times 2^s and of b times
+// 2^-s, so that the product does not depend on the gauge between them.
 cudaError_t tc_split2(const TcOperandView& a, TcOperand* oa, void* bufa, const TcOperandView& b, TcOperand* ob, void* bufb,
-                      int S, cudaStream_t s);
+                      int S, cudaStream_t s, int* top = nullptr);
 // out[rso m + ldo n] = alpha * A B^T (+ out if accumulate), with alpha a
 // signed power of two, A (M x K) and B (N x K) split operands (5 digits at
 // most, or the wide digits; rso != 1 only for those or beyond one chunk), i.e.

@@ -573,13 +573,16 @@ struct SplitView {
   int group;        // rows per group (R: one group)
   long long gs;     // elements between groups
 };
-// A view and where its digits go.
+// A view and where its digits go.  top (may be NULL; wide digits): the column
+// maxima of both operands (col_top_kernel), this one's side of the balance.
 struct SplitJob {
   SplitView v;
   int nchunks, row_ctas;  // K-chunks; CTAs along the rows
   int* e;
   __nv_bfloat16* planes;
   long long ldk;
+  const int* top;
+  int side;
 };
 
 // What the view holds at an in-range (r, k): 0 the stored value, 1 zero
@@ -648,6 +651,63 @@ DV long long fixed_point(double v, int e, int nbits) {
   return b < 0 ? -X : X;
 }
 
+// ---- balance of a contraction (wide digits) -----------------------------------
+// The digits count from the largest entry of a row, so a product is accurate
+// against (largest of A's row) x (largest of B's row), not term by term.  If the
+// columns of A grow with k and those of B shrink with it, the same tensor in
+// another gauge of its bond, the terms are alike but every row is graded, and
+// what lies 2^63 below its largest entry is cut: 1e-12 of the result where D and
+// 1/D span 8 decades, 1e-8 for 12 (FP64 products: 1e-15).  So column k of A is
+// multiplied by 2^s and that of B by 2^-s, exact, with s from the columns' largest
+// exponents, half of their difference: then both are at the root of their
+// product, and the error is of the largest term of |A||B| (1e-15 whatever the
+// gauge).  A column that is zero on one side is left out on the other.
+constexpr int kNoTop = -1000000;  // exponent of zero; a shift that leaves a value out
+
+// e with |x| 2^-e < 1 (a power of two above it at most); kNoTop for 0.
+DV int value_top(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  return (hi | __double2loint(x)) == 0 ? kNoTop : max(hi >> 20, 1) - 1022;
+}
+// Biased exponent of the larger part of what the view holds at (r, k), 0 for zero
+// and for what is not finite.
+DV int entry_top(const SplitView& v, int r, int k) {
+  const int kind = view_kind(v, r, k);
+  if (kind) return kind == 2 ? 1023 : 0;
+  const cplx x = __ldg(v.X + (long long)k * v.ks + (long long)(r % v.group) * v.rs + (long long)(r / v.group) * v.gs);
+  const int m = max(__double2hiint(x.x) & 0x7fffffff, __double2hiint(x.y) & 0x7fffffff);
+  if (d_zero(x.x) && d_zero(x.y)) return 0;
+  return m >= 0x7ff00000 ? 0 : max(m >> 20, 1);
+}
+// top[z * K + k] <- max over the rows of view z (0 or 1) of column k; zeroed
+// before.  Lanes along whichever index is contiguous; bound by one read of the
+// operands (8 to 10 us at 2048 to 8192 rows of 32 and 64 columns).
+constexpr int kTopRows = 256;
+__global__ void __launch_bounds__(256) col_top_kernel(SplitView a, SplitView b, int* __restrict__ top) {
+  const SplitView& v = blockIdx.z ? b : a;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ra = blockIdx.y * kTopRows, rb = min(v.R, ra + kTopRows);
+  int* t = top + (size_t)blockIdx.z * v.K;
+  int m = 0;
+  if (v.rs == 1) {  // a column per warp
+    const int k = blockIdx.x * 8 + w;
+    if (k >= v.K) return;
+#pragma unroll 4
+    for (int r = ra + lane; r < rb; r += 32) m = max(m, entry_top(v, r, k));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0 && m) atomicMax(t + k, m);
+  } else {
+    // eight columns per CTA here too; the rows over its 32 groups of eight lanes
+    const int k = blockIdx.x * 8 + (threadIdx.x & 7);
+    if (k < v.K)
+#pragma unroll 4
+      for (int r = ra + (threadIdx.x >> 3); r < rb; r += 32) m = max(m, entry_top(v, r, k));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    if (lane < 8 && k < v.K && m) atomicMax(t + k, m);
+  }
+}
+
 // BF16 bits of a small integer (|d| <= 128: exact in BF16, so the upper
 // half of its FP32 bits).
 DV unsigned int bf16_bits(int d) { return __float_as_uint((float)d) >> 16; }
@@ -709,6 +769,7 @@ __global__ void __launch_bounds__(kSplitThreads)
     split_kernel(SplitJob j0, SplitJob j1, int Kc, int S) {
   extern __shared__ cplx tile[];  // [kSplitRows][kSplitLd]
   __shared__ int esh[4][kSplitRows];  // components' exponents; one above max(|re|, |im|)
+  __shared__ int shift[kWideChunk];   // wide digits: column k is taken times 2^shift
   // the two jobs' CTAs one after the other
   int blk = blockIdx.x;
   const bool second = blk >= j0.row_ctas * j0.nchunks;
@@ -743,6 +804,18 @@ __global__ void __launch_bounds__(kSplitThreads)
     else *dst = mk(kind == 2 ? 1.0 : 0.0, 0.0);
   }
   if ((klen & 1) && tid < kSplitRows) tile[tid * kSplitLd + klen] = mk(0, 0);  // second value of the last pair
+  if (S == kWideDigits && tid < kWideChunk) {
+    const int* top = second ? j1.top : j0.top;
+    int sh = 0;
+    if (top && tid < klen) {
+      const int side = second ? j1.side : j0.side, own = top[(size_t)side * v.K + kb + tid],
+                other = top[(size_t)(side ^ 1) * v.K + kb + tid];
+      // (the same halving on both sides, so that the two shifts cancel)
+      const int half = (side ? own - other : other - own) >> 1;
+      sh = own == 0 || other == 0 ? kNoTop : (side ? -half : half);
+    }
+    shift[tid] = sh;
+  }
   cp_async_wait_all();
   __syncthreads();
   const double sgn = v.conj ? -1.0 : 1.0;
@@ -750,14 +823,19 @@ __global__ void __launch_bounds__(kSplitThreads)
   {
     const int r = tid >> 4, j = tid & 15;
     long long k0m = 0, k1m = 0, k2m = 0;
-    // infinities and NaNs by their exponent bits (a NaN's sign may stay in the
-    // masked key: the mask can become a floating-point absolute value)
-    int bad = 0;
+    int t0m = kNoTop, t1m = kNoTop, t2m = kNoTop;  // the same as exponents (wide digits)
+    int bad = 0;  // an infinity or a NaN, by its exponent
     for (int k = j; k < klen; k += 16) {
       const cplx x = tile[r * kSplitLd + k];
-      if (S == kWideDigits)
-        bad |= ((unsigned)__double2hiint(x.x) << 1) >= 0xFFE00000u || ((unsigned)__double2hiint(x.y) << 1) >= 0xFFE00000u;
       const double im = sgn * x.y;
+      if (S == kWideDigits) {
+        const int sh = shift[k], t0 = value_top(x.x), t1 = value_top(x.y);
+        bad |= max(t0, t1) > 1024;
+        t0m = max(t0m, t0 + sh);  // (a column left out stays far below any exponent)
+        t1m = max(t1m, t1 + sh);
+        t2m = max(t2m, value_top(x.x + im) + sh);
+        continue;
+      }
       k0m = max(k0m, mag_key(x.x));
       k1m = max(k1m, mag_key(im));
       k2m = max(k2m, mag_key(x.x + im));
@@ -767,12 +845,19 @@ __global__ void __launch_bounds__(kSplitThreads)
       k0m = max(k0m, __shfl_xor_sync(0xffffffffu, k0m, o));
       k1m = max(k1m, __shfl_xor_sync(0xffffffffu, k1m, o));
       k2m = max(k2m, __shfl_xor_sync(0xffffffffu, k2m, o));
-      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+      if (S == kWideDigits) {
+        t0m = max(t0m, __shfl_xor_sync(0xffffffffu, t0m, o));
+        t1m = max(t1m, __shfl_xor_sync(0xffffffffu, t1m, o));
+        t2m = max(t2m, __shfl_xor_sync(0xffffffffu, t2m, o));
+        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+      }
     }
     if (j < 3) {
-      const int ex = bad ? kNotFinite : key_exponent(j == 0 ? k0m : (j == 1 ? k1m : k2m));
+      const int t = j == 0 ? t0m : (j == 1 ? t1m : t2m);
+      const int own = S == kWideDigits ? (t < kNoTop / 2 ? 0 : t) : key_exponent(j == 0 ? k0m : (j == 1 ? k1m : k2m));
+      const int ex = bad ? kNotFinite : own;
       esh[j][r] = ex;
-      if (j == 0) esh[3][r] = key_exponent(max(k0m, k1m)) + 1;
+      if (j == 0) esh[3][r] = max(t0m, t1m) + 1;
       if (r0 + r < v.R) e[((size_t)j * nchunks + z) * v.R + r0 + r] = ex;
     }
   }
@@ -791,14 +876,16 @@ __global__ void __launch_bounds__(kSplitThreads)
     const double i0 = sgn * x0.y, i1 = sgn * x1.y;
     unsigned int* dst = reinterpret_cast<unsigned int*>(planes + (size_t)(r0 + r) * ldk + kb + kk);
     if (S == kWideDigits) {
-      digit_pair_wide(fixed_point(x0.x, esh[0][r], nbits), fixed_point(x1.x, esh[0][r], nbits), dst, plane / 2);
-      digit_pair_wide(fixed_point(i0, esh[1][r], nbits), fixed_point(i1, esh[1][r], nbits), dst + (size_t)S * (plane / 2),
-                      plane / 2);
+      // round(v 2^(shift + nbits - e)); a column left out is zero
+      const int sa = shift[kk], sb = kk + 1 < klen ? shift[kk + 1] : kNoTop;
+      auto cut = [&](double v, int e, int sh) { return sh == kNoTop ? 0ll : fixed_point(v, e - sh, nbits); };
+      digit_pair_wide(cut(x0.x, esh[0][r], sa), cut(x1.x, esh[0][r], sb), dst, plane / 2);
+      digit_pair_wide(cut(i0, esh[1][r], sa), cut(i1, esh[1][r], sb), dst + (size_t)S * (plane / 2), plane / 2);
       // re + im as integers at a scale above both (exact to 2^-62 of the larger
       // one), then at the sum's own scale, which it does not exceed
       const int ec = esh[3][r], up = ec - esh[2][r];
-      long long s0 = fixed_point(x0.x, ec, nbits) + fixed_point(i0, ec, nbits);
-      long long s1 = fixed_point(x1.x, ec, nbits) + fixed_point(i1, ec, nbits);
+      long long s0 = cut(x0.x, ec, sa) + cut(i0, ec, sa);
+      long long s1 = cut(x1.x, ec, sb) + cut(i1, ec, sb);
       s0 = up < 63 ? s0 << max(up, 0) : 0;
       s1 = up < 63 ? s1 << max(up, 0) : 0;
       digit_pair_wide(s0, s1, dst + (size_t)(2 * S) * (plane / 2), plane / 2);
@@ -903,18 +990,29 @@ static SplitJob split_job(const TcOperandView& ov, int S, TcOperand* out, void* 
   return SplitJob{SplitView{ov.X, ov.rs, ov.ks, ov.R, ov.K, ov.conj, ov.tri_mode, ov.tri,
                             ov.group > 0 ? ov.group : ov.R, ov.gs},
                   nchunks,
-                  (ov.R + kSplitRows - 1) / kSplitRows, out->e, reinterpret_cast<__nv_bfloat16*>(buf), ldk};
+                  (ov.R + kSplitRows - 1) / kSplitRows, out->e, reinterpret_cast<__nv_bfloat16*>(buf), ldk, nullptr, 0};
 }
 
 // Two operands in one launch (a product's operands are split back to back, and
 // most of these launches are short).
 cudaError_t tc_split2(const TcOperandView& a, TcOperand* oa, void* bufa, const TcOperandView& b, TcOperand* ob, void* bufb,
-                      int S, cudaStream_t s) {
+                      int S, cudaStream_t s, int* top) {
   if (S < 1 || (S > kMaxDigits && S != kWideDigits) || a.R <= 0 || a.K <= 0 || b.R < 0 || (b.R > 0 && b.K <= 0))
     return cudaErrorInvalidValue;
-  const SplitJob j0 = split_job(a, S, oa, bufa);
+  SplitJob j0 = split_job(a, S, oa, bufa);
   SplitJob j1{};
   if (b.R > 0) j1 = split_job(b, S, ob, bufb);
+  if (top) {
+    if (S != kWideDigits || b.R <= 0 || a.K != b.K) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(top, 0, 2 * (size_t)a.K * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((a.K + 7) / 8, (std::max(a.R, b.R) + kTopRows - 1) / kTopRows, 2);
+    if (grid.y > 65535) return cudaErrorInvalidValue;
+    col_top_kernel<<<grid, 256, 0, s>>>(j0.v, j1.v, top);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    j0.top = j1.top = top;
+    j1.side = 1;
+  }
   const long long ctas = (long long)j0.row_ctas * j0.nchunks + (long long)j1.row_ctas * j1.nchunks;
   if (ctas > 0x7fffffffll) return cudaErrorInvalidValue;
   cudaError_t e = allow_smem((const void*)split_kernel, split_smem_bytes());
