@@ -24,12 +24,17 @@ constexpr int kQrThreadsMixed = 512;
 constexpr int qr_threads(bool mixed) { return mixed ? kQrThreadsMixed : kQrThreads; }
 constexpr int kNbMax = 32;
 
+// Shared memory, in order: the panel P (nb x R), the Gram Ts (columns nb apart, or
+// nb + 1 apart where it is scaled, FP64), wl (2 kNbMax; the factorisation only).
 struct QrSmem {
-  // sizes in cplx
+  static constexpr size_t gram(int nb) { return (size_t)nb * (nb + 1); }
   static size_t bytes(int R, int nb) {
-    return sizeof(cplx) * ((size_t)nb * R + (size_t)nb * nb + 2 * kNbMax + 32) + 256;
+    return sizeof(cplx) * ((size_t)nb * R + (size_t)nb * nb + kNbMax + 2 * kNbMax) + 256;
   }
 };
+// the last entry of the scaled Gram, and its place before wl
+static_assert((kNbMax - 1) * (kNbMax + 1) + kNbMax - 1 < (int)QrSmem::gram(kNbMax), "scaled Gram");
+static_assert(QrSmem::gram(kNbMax) <= kNbMax * kNbMax + kNbMax, "scaled Gram");
 
 // v_s(i) for the panel held in P (after fix-up P holds pure V: zeros above
 // the unit diagonal).
@@ -411,7 +416,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx* P = reinterpret_cast<cplx*>(smem_raw);
   cplx* Ts = P + (size_t)nb * R;
-  cplx* wl = Ts + (size_t)nb * nb;  // [2*kNbMax]
+  cplx* wl = Ts + QrSmem::gram(nb);  // [2*kNbMax]
   __shared__ double dred[32];
   __shared__ cplx bc[4];
   __shared__ df2 bcd[4];  // mixed: conj(tau), conj(scale), scale, beta as double-float values
