@@ -288,7 +288,8 @@ cudaError_t tc_split2(const TcOperandView& a, TcOperand* oa, void* bufa, const T
 // signed power of two, A (M x K) and B (N x K) split operands (5 digits at
 // most, or the wide digits; rso != 1 only for those or beyond one chunk), i.e.
 // alpha sum_k A(m, k) B(n, k).  K beyond one chunk: per-chunk partials in
-// part (tc_part_elems), summed in a fixed order.  err: expiry record.
+// part (tc_part_elems; fewer: more launches), summed in a fixed order.  err:
+// expiry record.
 cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long long rso, long long ldo, double alpha,
                      int accumulate, cplx* part, size_t part_elems, int* err, cudaStream_t s);
 size_t tc_part_elems(int M, int N, int K, int S);

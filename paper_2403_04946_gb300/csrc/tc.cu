@@ -76,6 +76,7 @@ struct TcArgs {
   int alpha_exp, alpha_neg;  // alpha = (-1)^alpha_neg 2^alpha_exp: out = alpha * result (+ out if accumulate)
   int accumulate;
   int* err;       // expiry record (the context's grid-barrier err field)
+  int n_first;    // this launch's columns begin here, those of out with them
 };
 
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // N-tiles fastest: the CTAs that share an A-tile (the large digit planes)
   // run together and find it in L2
-  const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * kTcN, z = blockIdx.z;
+  const int m0 = blockIdx.y * kTcM, n0 = a.n_first + blockIdx.x * kTcN, z = blockIdx.z;
   const int k_begin = z * a.Kc;
   const int k_len = min(a.Kc, a.K - k_begin);
   const int nslab = (k_len + kSlab - 1) / kSlab;
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // columns 16 (w / 4) .. +15: two warps per quadrant share the rows
     const int quad = warp & 3, half = warp >> 2;
     const int m = m0 + 32 * quad + lane;
-    cplx* out = a.out + (size_t)z * a.zstride;
+    cplx* out = a.out + z * a.zstride - a.ldo * a.n_first;
     // the tile's column exponents of B, staged while the MMAs run (named
     // barrier 1: the eight epilogue warps only)
     {
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   unsigned char* smem_b = smem + (size_t)kWideA * a_plane_bytes();
   constexpr int S = kWideDigits;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * kTcN, z = blockIdx.z;
+  const int m0 = blockIdx.y * kTcM, n0 = a.n_first + blockIdx.x * kTcN, z = blockIdx.z;
   const int k_begin = z * kWideChunk;
   const int k_len = min(kWideChunk, a.K - k_begin);
   const int nslab = (k_len + kSlab - 1) / kSlab;
@@ -462,7 +463,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // ---- epilogue: warps 0-7; two per lane quadrant, 16 columns each -------
     const int quad = warp & 3, half = warp >> 2;
     const int m = m0 + 32 * quad + lane;
-    cplx* out = a.out + (size_t)z * a.zstride;
+    cplx* out = a.out + z * a.zstride - a.ldo * a.n_first;
     {
       const int t = threadIdx.x;
       if (t < 3 * kTcN) {
@@ -1055,46 +1056,57 @@ cudaError_t tc_zgemm(const TcOperand& A, const TcOperand& B, cplx* out, long lon
   a.eA = A.e;
   a.eB = B.e;
   a.err = err;
-  const dim3 grid((N + kTcN - 1) / kTcN, (M + kTcM - 1) / kTcM, nz);
   // alpha must be a signed power of two (the callers use +-1)
   int aexp = 0;
   const double am = std::frexp(std::fabs(alpha), &aexp);
   if (am != 0.5) return cudaErrorInvalidValue;
+  // the columns of one launch: as many as part holds the partial sums of
+  long long cols = N;
   if (nz == 1) {
-    a.out = out;
     a.rso = rso;
     a.ldo = ldo;
-    a.zstride = 0;
     a.alpha_exp = aexp - 1;
     a.alpha_neg = alpha < 0.0;
     a.accumulate = accumulate;
   } else {
-    if (!part || part_elems < (size_t)nz * M * N) return cudaErrorInvalidValue;
+    if (!part) return cudaErrorInvalidValue;
+    if (part_elems < (size_t)nz * M * N) cols = (long long)(part_elems / ((size_t)nz * M)) / kTcN * kTcN;
+    if (cols <= 0) return cudaErrorInvalidValue;
     a.out = part;
     a.rso = 1;
     a.ldo = M;
-    a.zstride = (long long)M * N;
-    a.alpha_exp = 0;
-    a.alpha_neg = 0;
-    a.accumulate = 0;
   }
-  if (wide) tc_zgemm_wide_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
-  else tc_zgemm_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
-  e = cudaGetLastError();
-  if (e != cudaSuccess || nz == 1) return e;
-  const long long n = (long long)M * N;
-  if (wide)
-    reduce_wide_kernel<<<(unsigned)((n + kRedOut - 1) / kRedOut), kRedOut * kRedZ, 0, s>>>(
-        part, M, N, nz, (long long)M * N, alpha, accumulate, out, rso, ldo);
-  else
-    reduce_parts_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(part, M, N, nz, (long long)M * N, alpha, accumulate,
-                                                                    out, rso, ldo);
-  return cudaGetLastError();
+  for (long long n0 = 0; n0 < N; n0 += cols) {
+    const int nc = (int)std::min<long long>(cols, N - n0);
+    const dim3 grid((nc + kTcN - 1) / kTcN, (M + kTcM - 1) / kTcM, nz);
+    a.n_first = (int)n0;
+    a.zstride = nz == 1 ? 0 : (long long)M * nc;
+    if (nz == 1) a.out = out;
+    if (wide) tc_zgemm_wide_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
+    else tc_zgemm_kernel<<<grid, kTcThreads, smem, s>>>(ma, mb, a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess || nz == 1) return e;
+    const long long n = (long long)M * nc;
+    cplx* o = out + (size_t)ldo * n0;
+    if (wide)
+      reduce_wide_kernel<<<(unsigned)((n + kRedOut - 1) / kRedOut), kRedOut * kRedZ, 0, s>>>(
+          part, M, nc, nz, a.zstride, alpha, accumulate, o, rso, ldo);
+    else
+      reduce_parts_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(part, M, nc, nz, a.zstride, alpha, accumulate, o, rso,
+                                                                      ldo);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
+// Partial sums take nz times the output: 20 times a core of 2560 columns.  Beyond
+// 1 GiB a product runs in groups of columns instead, at least one tile's: a group
+// is then a large launch by itself, and every sum has its order.
+constexpr size_t kMaxPart = (size_t)1 << 26;
 size_t tc_part_elems(int M, int N, int K, int S) {
-  const int nz = (K + tc_chunk(S) - 1) / tc_chunk(S);
-  return nz > 1 ? (size_t)nz * M * N : 0;
+  const size_t nz = (K + tc_chunk(S) - 1) / tc_chunk(S);
+  return nz > 1 ? std::min(nz * M * N, std::max(kMaxPart, nz * M * kTcN)) : 0;
 }
 
 }  // namespace hk

@@ -34,12 +34,14 @@ __global__ void house_kernel(int n, const cplx* alpha, const double* s2, cplx* o
 extern "C" {
 
 // C[rso m + ldo n] (nc values, read first) = alpha A B^T (+ C), A M x K and B N x K
-// row-major, by the eight-digit product; balance: with the contraction index
-// balanced.
-int probe_wide_product(int M, int N, int K, const double* A, const double* B, double* C, long long nc, long long rso,
-                       long long ldo, double alpha, int accumulate, int balance) {
-  const int S = hk::tc_wide_digits(), Kc = hk::tc_chunk(S);
-  const size_t np = hk::tc_part_elems(M, N, K, S);
+// row-major, from S digits (0: the wide ones); balance: with the contraction index
+// balanced; max_part: elements of the buffer of partial sums (0: all it may take).
+int probe_product(int M, int N, int K, const double* A, const double* B, double* C, long long nc, long long rso,
+                  long long ldo, double alpha, int accumulate, int balance, int S, long long max_part) {
+  if (S == 0) S = hk::tc_wide_digits();
+  const int Kc = hk::tc_chunk(S);
+  size_t np = hk::tc_part_elems(M, N, K, S);
+  if (max_part > 0 && np > (size_t)max_part) np = max_part;
   Buf a(sizeof(cplx) * M * K), b(sizeof(cplx) * N * K), c(sizeof(cplx) * nc), pa(hk::tc_operand_bytes(M, K, S, Kc)),
       pb(hk::tc_operand_bytes(N, K, S, Kc)), part(sizeof(cplx) * np), top(2 * sizeof(int) * K), err(sizeof(int));
   for (const Buf* q : {&a, &b, &c, &pa, &pb, &part, &top, &err})
@@ -61,6 +63,11 @@ int probe_wide_product(int M, int N, int K, const double* A, const double* B, do
   cudaMemcpy(&expired, err.p, sizeof(int), cudaMemcpyDeviceToHost);
   if (expired) return cudaErrorUnknown;
   return cudaMemcpy(C, c.p, sizeof(cplx) * nc, cudaMemcpyDeviceToHost);
+}
+
+// Bytes of partial sums a product asks for.
+long long probe_part_bytes(int M, int N, int K, int S) {
+  return (long long)(hk::tc_part_elems(M, N, K, S ? S : hk::tc_wide_digits()) * sizeof(cplx));
 }
 
 int probe_reciprocals(int n, const double* x, double* rcp, double* rsq) {

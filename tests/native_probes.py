@@ -29,12 +29,14 @@ class Probes:
     def __init__(self, lib):
         self.lib = lib
         d, i, ll = C.POINTER(C.c_double), C.c_int, C.c_longlong
-        lib.probe_wide_product.argtypes = [i, i, i, d, d, d, ll, ll, ll, C.c_double, i, i]
+        lib.probe_product.argtypes = [i, i, i, d, d, d, ll, ll, ll, C.c_double, i, i, i, ll]
+        lib.probe_part_bytes.argtypes = [i, i, i, i]
+        lib.probe_part_bytes.restype = ll
         lib.probe_reciprocals.argtypes = [i, d, d, d]
         lib.probe_house.argtypes = [i, d, d, d]
 
-    def wide_product(self, A, B, C0=None, alpha=1.0, transposed=False, balance=False):
-        """alpha A B^T (+ C0) for complex A (M x K), B (N x K)."""
+    def wide_product(self, A, B, C0=None, alpha=1.0, transposed=False, balance=False, digits=0, max_part=0):
+        """alpha A B^T (+ C0) for complex A (M x K), B (N x K), by the wide digits or by `digits`."""
         A, B = np.ascontiguousarray(A, np.complex128), np.ascontiguousarray(B, np.complex128)
         (M, K), N = A.shape, B.shape[0]
         pad = 3  # unused rows of the leading dimension, which must stay
@@ -43,8 +45,9 @@ class Probes:
         view = out[:, :N] if transposed else out[:, :M].T
         if C0 is not None:
             view[...] = C0
-        st = self.lib.probe_wide_product(M, N, K, _p(A.view(np.float64)), _p(B.view(np.float64)),
-                                         _p(out.view(np.float64)), out.size, rso, ldo, alpha, C0 is not None, balance)
+        st = self.lib.probe_product(M, N, K, _p(A.view(np.float64)), _p(B.view(np.float64)),
+                                    _p(out.view(np.float64)), out.size, rso, ldo, alpha, C0 is not None, balance, digits,
+                                    max_part)
         assert st == 0, st
         rest = out[:, N:] if transposed else out[:, M:]
         assert (rest == 7.0 - 3.0j).all()
