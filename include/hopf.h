@@ -99,7 +99,15 @@ typedef struct {
  * context, tensor or network exists (so that every pointer is released by
  * the functions that allocated it): HOPF_EINVAL otherwise, or when exactly
  * one of the two functions is NULL.  Pinned host staging buffers are not
- * affected. */
+ * affected.
+ *
+ * Besides its tensors a context keeps a workspace per rounding shape (d + 1
+ * buffers of the largest core) and, grown by the first rounding that meets a
+ * factor of 1024 rows or more, scratch for the digits of its products: 48
+ * bytes per entry of the largest factor in FP64 (three times the factor), 30
+ * in mixed precision, and at most 1 GiB of partial sums (or those of one
+ * tile's columns).  An FP64 context that is refused this scratch runs the
+ * factor on the FP64 units; a mixed one returns HOPF_ENOMEM. */
 typedef void* (*hopf_alloc_fn)(size_t bytes, void* user);
 typedef void (*hopf_free_fn)(void* ptr, void* user);
 hopf_status hopf_set_allocator(hopf_alloc_fn alloc, hopf_free_fn free, void* user);

@@ -606,33 +606,57 @@ bool use_tc(const hopf_ctx* ctx, int m, int p) {
 }
 int product_digits(const hopf_ctx* ctx) { return ctx->p.precision == HOPF_FP64 ? hk::tc_wide_digits() : kTcDigits; }
 
-hopf_status tc_reserve_bytes(hopf_ctx* ctx, size_t need) {
-  if (need <= ctx->tcbytes) return HOPF_OK;
+// Scratch of `need` bytes for the digits; false (and what there was before) if
+// the memory is not to be had.  Eight digits take 48 bytes per entry, three times
+// the operand: a state that nearly fills the device still runs in FP64, on the
+// FP64 units (qr_factor_conf, qr_apply and the merges ask first).
+bool tc_has(hopf_ctx* ctx, size_t need) {
+  const size_t had = ctx->tcbytes;
+  if (need <= had) return true;
   dfree(ctx->tcbuf);
   ctx->tcbuf = nullptr;
   ctx->tcbytes = 0;
-  CK(hk::dev_alloc(&ctx->tcbuf, need));
-  ctx->tcbytes = need;
-  return HOPF_OK;
+  for (const size_t want : {need, had}) {
+    if (want == 0) break;
+    if (hk::dev_alloc(&ctx->tcbuf, want) == cudaSuccess) {
+      ctx->tcbytes = want;
+      return want == need;
+    }
+    cudaGetLastError();
+    ctx->tcbuf = nullptr;
+  }
+  return false;
+}
+
+hopf_status tc_reserve_bytes(hopf_ctx* ctx, size_t need) {
+  return tc_has(ctx, need) ? HOPF_OK : fail(ctx, HOPF_ENOMEM, "digit scratch: %zu bytes", need);
 }
 
 hopf_status tc_reserve(hopf_ctx* ctx, int m, int k) {
-  return tc_reserve_bytes(ctx, ctx->p.precision == HOPF_FP64 ? hk::qr_wide_scratch_bytes(m, k)
-                                                             : hk::qr_tc_scratch_bytes(m, k, kTcDigits));
+  return tc_reserve_bytes(ctx, hk::qr_tc_scratch_bytes(m, k, kTcDigits));
+}
+
+// The FP64 route of an m-row factor with p reflectors and k columns besides.
+bool takes_wide(hopf_ctx* ctx, int m, int p, int k) {
+  return hk::qr_wide_applies(m, p) && tc_has(ctx, hk::qr_wide_scratch_bytes(m, k));
 }
 
 // out (a.R x b.R, column-major, ldo) = A B^T of two operand views on the
 // tensor cores (digit splits in the context's scratch), profiled as one
-// HOPF_K_TC phase with the given FLOP count.
+// HOPF_K_TC phase with the given FLOP count.  *done = false, and nothing
+// launched, if an FP64 product's scratch is not to be had.
 hopf_status tc_product(hopf_ctx* ctx, const hk::TcOperandView& a, const hk::TcOperandView& b, cplx* out, long long ldo,
-                       double flops) {
+                       double flops, bool* done) {
   const int S = product_digits(ctx), Kc = hk::tc_chunk(S);
   const size_t ba = (hk::tc_operand_bytes(a.R, a.K, S, Kc) + 255) & ~(size_t)255;
   const size_t bb = (hk::tc_operand_bytes(b.R, b.K, S, Kc) + 255) & ~(size_t)255;
   const size_t np = hk::tc_part_elems(a.R, b.R, a.K, S);
   const bool wide = S == hk::tc_wide_digits();
   const size_t bt = wide ? (2 * (size_t)a.K * sizeof(int) + 255) & ~(size_t)255 : 0;
-  TRY(tc_reserve_bytes(ctx, ba + bb + bt + np * sizeof(cplx) + 256));
+  const size_t need = ba + bb + bt + np * sizeof(cplx) + 256;
+  *done = !wide || tc_has(ctx, need);
+  if (!*done) return HOPF_OK;
+  TRY(tc_reserve_bytes(ctx, need));
   unsigned char* buf = static_cast<unsigned char*>(ctx->tcbuf);
   hk::TcOperand oa, ob;
   const int slot = prof_begin(ctx);
@@ -701,8 +725,7 @@ int qr_mode(const hopf_ctx* ctx) {
 hopf_status qr_factor_conf(hopf_ctx* ctx, const QrConf& c, cplx* A, int lda, int m, int k, cplx* tau, cplx* T,
                            int* nb, cplx* G) {
   CtaCap cap(ctx, c.ctas);
-  if (ctx->p.precision == HOPF_FP64 && hk::qr_wide_applies(m, std::min(m, k))) {
-    TRY(tc_reserve(ctx, m, k));
+  if (ctx->p.precision == HOPF_FP64 && takes_wide(ctx, m, std::min(m, k), k)) {
     *nb = 32;
     CK(hk::geqrf_wide(A, lda, m, k, tau, T, ctx->tcbuf, ctx->tcbytes, ctx->coop, ctx->stream,
                       phase_timer(ctx, HOPF_K_QR)));
@@ -805,8 +828,8 @@ hopf_status qr_apply(hopf_ctx* ctx, const cplx* A, int lda, int m, int p, const 
                      const cplx* G, cplx* C, int ldc, int q) {
   const QrConf c = qr_conf(ctx, m, p);
   CtaCap cap(ctx, c.ctas);
-  if (ctx->p.precision == HOPF_FP64 && hk::qr_wide_applies(m, p)) {
-    TRY(tc_reserve(ctx, m, q));
+  // (a panel's record is the same from either route, at 32 columns)
+  if (ctx->p.precision == HOPF_FP64 && nb == 32 && takes_wide(ctx, m, p, q)) {
     CK(hk::ormqr_wide(A, lda, m, p, T, C, ldc, q, ctx->tcbuf, ctx->tcbytes, &ctx->coop.bar->err, ctx->stream,
                       phase_timer(ctx, HOPF_K_APPLYQ)));
     return HOPF_OK;
@@ -869,12 +892,14 @@ hopf_status orth_sweep(hopf_ctx* ctx, const hopf_tt* t, std::vector<int>& p, std
     p[c] = std::min(m, k);
     // merge L_c = R_c^H into core c-1
     const int rl = r[c - 1];
-    if (c - 1 >= 1 && use_tc(ctx, rl * n, 64)) {
+    bool done = false;
+    if (c - 1 >= 1 && use_tc(ctx, rl * n, 64))
       // on the tensor cores: C = X_{c-1} R^H into the scratch W1
       // (column-major), then H(Y)^H into the next factor's buffer
       TRY(tc_product(ctx, hk::TcOperandView{t->cores[c - 1], 1, (long long)rl * n, rl * n, k, 0, 0, 0},
                      hk::TcOperandView{w.B[c], 1, m, p[c], k, 1, 1, 0}, w.W1, (long long)rl * n,
-                     arh_flops((double)rl * n, k, p[c])));
+                     arh_flops((double)rl * n, k, p[c]), &done));
+    if (done) {
       LAUNCH(HOPF_K_SUM, 0, 32.0 * rl * n * p[c], 1,
              hk::conj_transpose(w.W1, rl, rl, n * p[c], w.B[c - 1], n * p[c], ctx->stream));
     } else if (c - 1 >= 1) {
@@ -939,8 +964,7 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
       } else {
         int nbl = 32;
         LAUNCH(HOPF_K_SMALL, 0, 0, 1, hk::conj_transpose(w.Rb, pp, pp, cols, w.Mb, cols, ctx->stream));
-        if (!w.kept && hk::qr_wide_applies(cols, pp)) {
-          TRY(tc_reserve_bytes(ctx, hk::qr_wide_scratch_bytes(cols, pp)));
+        if (!w.kept && takes_wide(ctx, cols, pp, pp)) {
           CK(hk::geqrf_wide(w.Mb, cols, cols, pp, w.tau + (size_t)c * w.kcap, nullptr, ctx->tcbuf, ctx->tcbytes, ctx->coop,
                             ctx->stream, phase_timer(ctx, HOPF_K_SVD)));
         } else {
@@ -1004,10 +1028,11 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
     // S = U_rho^H R (rho x cols)
     // (FP64: below about 4e6 multiply-adds the product's and the splits'
     // launches cost more than the FP64 units' time on all SMs, 14 us)
-    if (use_tc(ctx, 4096, pp) && (MIXED_FLAG || (double)rnew * pp * cols > 4e6)) {
+    bool done = false;
+    if (use_tc(ctx, 4096, pp) && (MIXED_FLAG || (double)rnew * pp * cols > 4e6))
       TRY(tc_product(ctx, hk::TcOperandView{w.Ub, pp, 1, rnew, pp, 1, 0, 0}, hk::TcOperandView{w.Rb, pp, 1, cols, pp, 0, 0, 0},
-                     w.Sb, rnew, 8.0 * rnew * pp * cols));
-    } else {
+                     w.Sb, rnew, 8.0 * rnew * pp * cols, &done));
+    if (!done) {
       LAUNCH(HOPF_K_GEMM, 8.0 * rnew * pp * cols, 0, 1, hk::gemm_uh_r(w.Ub, pp, rnew, pp, w.Rb, pp, cols, w.Sb, rnew, ctx->stream));
     }
   }
@@ -1069,6 +1094,7 @@ hopf_status orth_sweep_apply(hopf_ctx* ctx, const hopf_tt* X, std::vector<int>& 
     p[c] = std::min(m, k);
     const int rl = r[c - 1];
     const size_t blk = (size_t)rl * n * p[c];
+    bool done = false;
     if (use_tc(ctx, rl * n, 64)) {
       // the six products on the tensor cores as one: the blocks of R^H
       // (conjugated, upper trapezoid) are row groups of the right operand, and
@@ -1080,8 +1106,9 @@ hopf_status orth_sweep_apply(hopf_ctx* ctx, const hopf_tt* X, std::vector<int>& 
       vr.group = p[c];
       vr.gs = (long long)m * r[c];
       TRY(tc_product(ctx, hk::TcOperandView{X->cores[c - 1], 1, (long long)rl * n, rl * n, r[c], 0, 0, 0}, vr, w.W1,
-                     (long long)rl * n, flops));
-    } else {
+                     (long long)rl * n, flops, &done));
+    }
+    if (!done) {
       for (int be = 0; be < 6; ++be) {
         LAUNCH(HOPF_K_GEMM, rblk_flops((double)rl * n, r[c], p[c], be * r[c]), 0, 1,
                hk::gemm_a_rblk_h(X->cores[c - 1], rl * n, rl * n, r[c], w.B[c], m, be * r[c], p[c], w.W1 + be * blk,
