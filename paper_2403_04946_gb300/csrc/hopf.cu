@@ -2046,6 +2046,27 @@ hopf_status hopf_eval_points(hopf_ctx* ctx, const hopf_tt* t, int npts, const in
   return HOPF_OK;
 }
 
+// Grid points of the moment stencil in the order moments_combine reads: the
+// centre, one step up and down every axis, then every pair of axes.
+static std::vector<int> moment_points(int d, int n) {
+  std::vector<int> idx((size_t)(1 + 2 * d + 2 * d * (d - 1)) * d, n / 2);
+  int* p = idx.data() + d;
+  for (int k = 0; k < d; ++k)
+    for (int s : {1, -1}) {
+      p[k] += s;
+      p += d;
+    }
+  for (int j = 0; j < d; ++j)
+    for (int k = j + 1; k < d; ++k)
+      for (int s : {1, -1})
+        for (int u : {1, -1}) {
+          p[j] += s;
+          p[k] += u;
+          p += d;
+        }
+  return idx;
+}
+
 hopf_status hopf_eval_moments(hopf_ctx* ctx, const hopf_tt* t, double* mean, double* cov, double* imag_resid) {
   if (!ctx || !t || !mean || !cov) return ctx ? fail(ctx, HOPF_EINVAL, "hopf_eval_moments: null argument") : HOPF_EINVAL;
   if (!(ctx->L > 0.0)) return fail(ctx, HOPF_EINVAL, "L is not set");
@@ -2054,10 +2075,23 @@ hopf_status hopf_eval_moments(hopf_ctx* ctx, const hopf_tt* t, double* mean, dou
   const int npts = 1 + 2 * d + 2 * d * (d - 1);
   int maxr = 1;
   for (int r : t->ranks) maxr = std::max(maxr, r);
-  TRY(ev_reserve(ctx, 0, (size_t)npts + hk::moment_env_elems(d, maxr), (size_t)d + (size_t)d * d + 1));
+  // Few or small products: every point by itself in one launch.  The row chains
+  // are d dependent exchanges of a cluster, 2.5 us each, and a second launch: at
+  // d = 8 they take 27 us for r = 17 and 31 for r = 48, the 129 points 16 and 30; at
+  // d = 16 46 us for r = 16 (513 points 28) and 58 for r = 33 (90).
+  const bool points = maxr <= 48 && (double)npts * d * maxr * maxr <= 2.4e6;
+  TRY(ev_reserve(ctx, points ? (size_t)npts * d : 0, (size_t)npts + (points ? 0 : hk::moment_env_elems(d, maxr)),
+                 (size_t)d + (size_t)d * d + 1));
   cplx* dv = ctx->ev_vals;
   double* dout = ctx->ev_out;
-  cudaError_t e = hk::moment_values(t->d_ptrs, t->d_ranks, d, n, maxr, dv + npts, dv, ctx->stream);
+  cudaError_t e;
+  if (points) {
+    const std::vector<int> idx = moment_points(d, n);
+    e = cudaMemcpyAsync(ctx->ev_idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = hk::eval_points(t->d_ptrs, t->d_ranks, d, n, maxr, npts, ctx->ev_idx, dv, ctx->stream);
+  } else {
+    e = hk::moment_values(t->d_ptrs, t->d_ranks, d, n, maxr, dv + npts, dv, ctx->stream);
+  }
   const double da = 2.0 * ctx->L / n;
   if (e == cudaSuccess) e = hk::moments_combine(dv, d, da, dout, dout + d, dout + d + (size_t)d * d, ctx->stream);
   double ir = 0.0;

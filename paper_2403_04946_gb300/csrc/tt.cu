@@ -188,26 +188,34 @@ cudaError_t sum_core(const SumTerm* terms_dev, int nterms, int kind, int n, cplx
 // point, the running row vector in shared memory.  S adjacent lanes share a
 // column of the slice (interleaved rows: contiguous in memory) and add their
 // parts by shuffles.  An FP64 instruction of a warp takes 64 cycles of a quarter
-// of the SM: 4 ceil(a / S) for the products, log2 S for the additions, so S is
-// the least that gives each quarter a warp: 4 from 17 columns, 8 below, more for
-// the few columns of a long row vector (one lane per column from 17 columns when
-// there are many points: fewest instructions and CTA barriers; 2000 points at
-// r = 64, d = 10: 543 us, 256 threads with four lanes per column 548, now 521).  Many points are
-// bound by the FP64 units (r^2 complex multiply-adds per mode, 2 per clock
-// and SM).  Few points are bound by latency, d dependent products: the
-// indices are known ahead, so every slice is prefetched into L2 first, and
-// each thread keeps four loads and two sums in flight (one thread per column
-// walking all rows took 6.7 us per mode at r = 32).
-constexpr int ev_threads(bool few) { return few ? 256 : 128; }
+// of the SM: 4 ceil(a / S) for the products, log2 S for the additions.
+//
+// Few points (two per SM at most) are bound by latency, d dependent products: S is
+// the least that gives each quarter a warp (4 from 17 columns, 8 below, more for
+// the few columns of a long row vector), every slice is prefetched into L2 first
+// (the indices are known ahead), and each thread keeps four loads and two sums
+// in flight: 44 us for one point at r = 33, d = 16, against 86 for one thread per
+// column and one load after another.  Up to 8 columns the prefetch costs more
+// than it gives (5.1 against 6.0 us at r = 8, d = 4).
+//
+// Many points are bound by those instructions, so the warps are filled: a thread
+// per column for every 32 columns, and for the rest of them as many lanes as make
+// one warp (17 to 24: 16 columns and the others).  2048 points, d = 16: 35 us at
+// r = 8, 65 at r = 16, 274 at r = 33 (one thread per column 64, 122, 441; eight lanes
+// per column, or one from 17, 71, 132, 467).  CTAs of one warp up to 24 columns, two up to
+// 48, four beyond (r = 16, 2048 points: 65 us, 68 with two, 71 with four; r = 48: 207
+// with two, 230 with four).  Up to 4 columns there is nothing to share and the plain
+// loop is shortest (r = 1, d = 16, 2048 points 11 us, with lanes 32).
 template <int S, int T>
-DV void eval_mode(const cplx* __restrict__ C, size_t cs, int a, int c, const cplx* v, cplx* w) {
-  const int seg = threadIdx.x % S;
+DV void eval_columns(const cplx* __restrict__ C, size_t cs, int a, int j0, int j1, int first, const cplx* v, cplx* w) {
+  // column j0 falls to thread `first`, a warp that has none of the columns before
+  const int t = (int)(threadIdx.x + T - first) % T, seg = t % S;
   constexpr int per = T / S;
-  for (int jb = 0; jb < c; jb += per) {
-    const int j = jb + threadIdx.x / S;
-    if (jb + (threadIdx.x & ~31u) / S >= (unsigned)c) continue;  // no column in this warp
+  for (int jb = j0; jb < j1; jb += per) {
+    const int j = jb + t / S;
+    if (jb + (t & ~31) / S >= j1) continue;  // no column in this warp
     cplx s0 = mk(0, 0), s1 = mk(0, 0);
-    if (j < c) {
+    if (j < j1) {
       const cplx* col = C + cs * j;
       int i = seg;
       for (; i + 3 * S < a; i += 4 * S) {
@@ -221,24 +229,24 @@ DV void eval_mode(const cplx* __restrict__ C, size_t cs, int a, int c, const cpl
     }
     if (a > 3 * S) s0 = cadd(s0, s1);
     if constexpr (S == 1) {
-      if (j < c) w[j] = s0;
+      if (j < j1) w[j] = s0;
     } else {
       const double h = half_sum(s0, S);
-      if (seg < 2 && j < c) reinterpret_cast<double*>(w + j)[seg] = h;
+      if (seg < 2 && j < j1) reinterpret_cast<double*>(w + j)[seg] = h;
     }
   }
 }
 
-template <bool FEW>
-__global__ void __launch_bounds__(ev_threads(FEW))
+enum { kEvalFew, kEvalMany, kEvalPlain };
+template <int MODE, int T>
+__global__ void __launch_bounds__(T)
 eval_points_kernel(const cplx* const* __restrict__ cores, const int* __restrict__ ranks, int d, int n, int rmax,
                    const int* __restrict__ idx, cplx* __restrict__ vals) {
-  constexpr int T = ev_threads(FEW);
   extern __shared__ __align__(16) unsigned char sm[];
   cplx* vb = reinterpret_cast<cplx*>(sm);  // [2][rmax]
   const int pt = blockIdx.x;
   const int* ip = idx + (size_t)pt * d;
-  if constexpr (FEW) {
+  if constexpr (MODE == kEvalFew) {
     // one 128-byte line (8 values of a column) per thread and step
     for (int k = 0; k < d; ++k) {
       const int a = ranks[k], c = ranks[k + 1], lines = (a + 7) / 8;
@@ -256,11 +264,35 @@ eval_points_kernel(const cplx* const* __restrict__ cores, const int* __restrict_
     const cplx* v = vb + (size_t)cur * rmax;
     cplx* w = vb + (size_t)(cur ^ 1) * rmax;
     const size_t cs = (size_t)a * n;
-    if (!FEW && c > 16) eval_mode<1, T>(C, cs, a, c, v, w);
-    else if (c > 16) eval_mode<4, T>(C, cs, a, c, v, w);
-    else if (a <= 16 || c > 8) eval_mode<8, T>(C, cs, a, c, v, w);
-    else if (c > 4) eval_mode<16, T>(C, cs, a, c, v, w);
-    else eval_mode<32, T>(C, cs, a, c, v, w);
+    if constexpr (MODE == kEvalPlain) {
+      for (int j = threadIdx.x; j < c; j += T) {
+        cplx acc = mk(0, 0);
+        for (int i = 0; i < a; ++i) acc = cfma(v[i], C[cs * j + i], acc);
+        w[j] = acc;
+      }
+    } else if constexpr (MODE == kEvalFew) {
+      if (c > 16) eval_columns<4, T>(C, cs, a, 0, c, 0, v, w);
+      else if (a <= 16 || c > 8) eval_columns<8, T>(C, cs, a, 0, c, 0, v, w);
+      else if (c > 4) eval_columns<16, T>(C, cs, a, 0, c, 0, v, w);
+      else eval_columns<32, T>(C, cs, a, 0, c, 0, v, w);
+    } else {
+      int j = c & ~31, first = j % T;
+      if (j) eval_columns<1, T>(C, cs, a, 0, j, 0, v, w);
+      if (c - j > 24 || (c > j && a <= 4)) {
+        eval_columns<1, T>(C, cs, a, j, c, first, v, w);
+        j = c;
+      } else if (c - j > 16) {  // 17 to 24 columns: 16 and the others
+        eval_columns<2, T>(C, cs, a, j, j + 16, first, v, w);
+        j += 16;
+        first = (first + 32) % T;
+      }
+      const int rest = c - j;
+      if (rest > 8) eval_columns<2, T>(C, cs, a, j, c, first, v, w);
+      else if (rest > 4) eval_columns<4, T>(C, cs, a, j, c, first, v, w);
+      else if (rest > 2) eval_columns<8, T>(C, cs, a, j, c, first, v, w);
+      else if (rest > 1) eval_columns<16, T>(C, cs, a, j, c, first, v, w);
+      else if (rest) eval_columns<32, T>(C, cs, a, j, c, first, v, w);
+    }
     __syncthreads();
   }
   if (threadIdx.x == 0) vals[pt] = vb[(size_t)cur * rmax];
@@ -271,13 +303,18 @@ cudaError_t eval_points(const cplx* const* cores_dev, const int* ranks_dev, int 
   if (npts <= 0) return cudaSuccess;
   const int rmax = std::max(maxr, 1);
   const size_t smem = sizeof(cplx) * 2 * (size_t)rmax;
-  // with several points per SM the next point's loads hide the latency, and
-  // what counts is the number of FP64 instructions and of resident CTAs
   const bool few = npts <= 2 * dev_info().sm_count;
-  const auto fn = few ? eval_points_kernel<true> : eval_points_kernel<false>;
+  auto fn = eval_points_kernel<kEvalPlain, 32>;
+  int T = 32;
+  if (rmax > 4) {
+    if (few && rmax > 8) fn = eval_points_kernel<kEvalFew, 256>, T = 256;
+    else if (rmax <= 24) fn = eval_points_kernel<kEvalMany, 32>, T = 32;
+    else if (rmax <= 48) fn = eval_points_kernel<kEvalMany, 64>, T = 64;
+    else fn = eval_points_kernel<kEvalMany, 128>, T = 128;
+  }
   cudaError_t e = allow_smem((const void*)fn, smem);
   if (e != cudaSuccess) return e;
-  fn<<<npts, ev_threads(few), smem, s>>>(cores_dev, ranks_dev, d, n, rmax, idx_dev, vals);
+  fn<<<npts, T, smem, s>>>(cores_dev, ranks_dev, d, n, rmax, idx_dev, vals);
   return cudaGetLastError();
 }
 
