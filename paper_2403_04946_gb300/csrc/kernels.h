@@ -141,7 +141,7 @@ cudaError_t fill_zero(cplx* A, size_t count, cudaStream_t s);
 // Upper triangle of the top p x k block of A (lda) -> R (p x k, ldr), zeros below.
 cudaError_t extract_r(const cplx* A, int lda, int p, int k, cplx* R, int ldr, cudaStream_t s);
 
-// GEMM variants (FP64 complex, tiles of 64 x 64).
+// GEMM variants (FP64 complex or double-float, tiles of 64, 32, 16 or 8).
 // C[M x N] = A[M x K] * R^H, R upper-trapezoidal N x K (ldr), A column-major (lda).
 // mode 0: C column-major (ldc); mode 1: C written conj-transposed into the
 // "H^H layout": row index i_all = i + rl * mm (i < rl), column j ->

@@ -65,6 +65,23 @@ int probe_product(int M, int N, int K, const double* A, const double* B, double*
   return cudaMemcpy(C, c.p, sizeof(cplx) * nc, cudaMemcpyDeviceToHost);
 }
 
+// C (M x N, column-major) = A R^H for A M x K and R N x (coff + K), column-major,
+// upper trapezoidal, by the tiled kernels; uh: C = A^H R instead (A K x M, R K x N, full).
+int probe_gemm(int M, int N, int K, const double* A, const double* R, double* C, int coff, int uh, int mixed) {
+  const int rows = uh ? K : N, cols = uh ? N : coff + K;
+  Buf a(sizeof(cplx) * M * K), r(sizeof(cplx) * rows * cols), c(sizeof(cplx) * M * N);
+  for (const Buf* q : {&a, &r, &c})
+    if (q->e != cudaSuccess) return q->e;
+  cudaMemcpy(a.p, A, sizeof(cplx) * M * K, cudaMemcpyHostToDevice);
+  cudaMemcpy(r.p, R, sizeof(cplx) * rows * cols, cudaMemcpyHostToDevice);
+  cudaError_t e;
+  if (uh) e = hk::gemm_uh_r(a.as<cplx>(), K, M, K, r.as<cplx>(), K, N, c.as<cplx>(), M, nullptr);
+  else if (coff) e = hk::gemm_a_rblk_h(a.as<cplx>(), M, M, K, r.as<cplx>(), N, coff, N, c.as<cplx>(), M, nullptr, mixed);
+  else e = hk::gemm_a_rh(a.as<cplx>(), M, M, K, r.as<cplx>(), N, N, c.as<cplx>(), M, 0, 1, 1, nullptr, mixed);
+  if (e != cudaSuccess) return e;
+  return cudaMemcpy(C, c.p, sizeof(cplx) * M * N, cudaMemcpyDeviceToHost);
+}
+
 // Bytes of partial sums a product asks for.
 long long probe_part_bytes(int M, int N, int K, int S) {
   return (long long)(hk::tc_part_elems(M, N, K, S ? S : hk::tc_wide_digits()) * sizeof(cplx));

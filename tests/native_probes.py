@@ -30,6 +30,7 @@ class Probes:
         self.lib = lib
         d, i, ll = C.POINTER(C.c_double), C.c_int, C.c_longlong
         lib.probe_product.argtypes = [i, i, i, d, d, d, ll, ll, ll, C.c_double, i, i, i, ll]
+        lib.probe_gemm.argtypes = [i, i, i, d, d, d, i, i, i]
         lib.probe_part_bytes.argtypes = [i, i, i, i]
         lib.probe_part_bytes.restype = ll
         lib.probe_reciprocals.argtypes = [i, d, d, d]
@@ -52,6 +53,17 @@ class Probes:
         rest = out[:, N:] if transposed else out[:, M:]
         assert (rest == 7.0 - 3.0j).all()
         return view.copy()
+
+    def gemm(self, A, R, coff=0, uh=False, mixed=False):
+        """A R^H for the upper trapezoid of R's columns from coff on, or A^H R."""
+        A, R = np.asfortranarray(A, np.complex128), np.asfortranarray(R, np.complex128)
+        K, M = A.shape if uh else A.shape[::-1]
+        N = R.shape[1] if uh else R.shape[0]
+        out = np.empty((M, N), np.complex128, order="F")
+        p = lambda x: x.ctypes.data_as(C.POINTER(C.c_double))
+        st = self.lib.probe_gemm(M, N, K, p(A), p(R), p(out), coff, uh, mixed)
+        assert st == 0, st
+        return out
 
     def reciprocals(self, x):
         x = np.ascontiguousarray(x, np.float64)
