@@ -191,11 +191,11 @@ hopf_status fail(hopf_ctx* c, hopf_status st, const char* fmt, ...) {
 // 1e-10 to 2e-9, whatever the change was.  That matters where moments are taken
 // (the CDF equation has none: its values move by up to 8e-11) and where a factor can
 // reach the products' 4096 rows: ranks go up to 6 rank_cap in a step's
-// roundings, or to those of the tensor at hand.
-bool kept_order(const hopf_ctx* ctx, const hopf_tt* t) {
+// roundings, or to the capacity of the tensor at hand.
+bool kept_order(const hopf_ctx* ctx, int cap_rank) {
   if (ctx->p.precision != HOPF_MIXED || ctx->equation != HOPF_EQ_PHI) return false;
   if (ctx->qr_method != HOPF_QR_TENSOR && !ctx->autotune) return false;
-  const long long r = std::max(6 * (long long)ctx->p.rank_cap, (long long)t->cap_rank);
+  const long long r = std::max(6 * (long long)ctx->p.rank_cap, (long long)cap_rank);
   return r * ctx->p.n >= 4096;
 }
 
@@ -491,7 +491,7 @@ hopf_status round_buffers(hopf_ctx* ctx, const hopf_tt* t) {
 hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
   TRY(round_buffers(ctx, t));
   RoundWs& w = ctx->rw;
-  w.kept = kept_order(ctx, t);
+  w.kept = kept_order(ctx, t->cap_rank);
   if (w.kept && !w.bd_lu) CK(dalloc(&w.bd_lu, hk::bd_lu_elems(w.kcap, w.kcap)));
   return HOPF_OK;
 }
@@ -1316,8 +1316,9 @@ hopf_status cross_sweep(hopf_ctx* ctx, CrossBufs& B, int cap, const std::vector<
       if ((size_t)M * cnt > cores->core_cap[k]) return fail(ctx, HOPF_EINVAL, "cross: core %d exceeds capacity", k);
       CK(hk::cross_gather(B.A, M, B.piv + cap, cnt, B.Q, B.W, B.seq, ctx->stream));
       int nb = 32;
-      CK(hk::geqrf(B.Q, M, M, cnt, B.tau, B.T, &nb, ctx->coop, ctx->stream, hk::kQrFp64));
-      CK(hk::ormqr(B.Q, M, M, cnt, B.tau, B.T, nb, B.W, M, cnt, ctx->coop, ctx->stream, hk::kQrFp64));
+      const int mode = kept_order(ctx, cap) ? hk::kQrKept : hk::kQrFp64;
+      CK(hk::geqrf(B.Q, M, M, cnt, B.tau, B.T, &nb, ctx->coop, ctx->stream, mode));
+      CK(hk::ormqr(B.Q, M, M, cnt, B.tau, B.T, nb, B.W, M, cnt, ctx->coop, ctx->stream, mode));
       TRY(check_barrier(ctx));
       CK(hk::cross_core(B.W, M, B.piv, B.seq, cnt, B.Gw, B.Gi, cores->cores[k], ctx->stream));
     }

@@ -941,7 +941,7 @@ geqrf_kernel(cplx* A, int lda, int m, int k, cplx* tau, cplx* Tg, int nb, int R,
   if (MIXED && k > p) rows_to_fp64(A, lda, r0, r1, p, k, E);
 }
 
-template <int NB, bool MIXED>
+template <int NB, bool MIXED, bool KEPT = false>
 __global__ void __launch_bounds__(qr_threads(MIXED), 1)
 ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx* C, int ldc,
              int q, int R, CoopWs ws) {
@@ -982,7 +982,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     // (column u at u (nbk + 1), entries -tau_s Gram[s,u])
     for (int e = tid; e < nbk * nbk; e += blockDim.x) {
       const cplx v = Tg[(size_t)panel * nb * nb + e];
-      if (MIXED) {
+      if (MIXED || KEPT) {
         Ts[e] = v;
       } else {
         const int sr = e % nbk, u = e / nbk;
@@ -994,7 +994,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     if (MIXED)
       partial_vhx_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<const df2*>(C), ldc, q,
                         ws.pc + (size_t)g * pstride, false);
-    else if (R <= kFewRows)
+    else if (!KEPT && R <= kFewRows)
       partial_vhx_few<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride, false);
     else
       partial_vhx<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.pc + (size_t)g * pstride);
@@ -1009,7 +1009,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
       }
     }
     __syncthreads();
-    if constexpr (!MIXED) {
+    if constexpr (!MIXED && !KEPT) {
       const cplx tl = (lane < nbk) ? Tg[(size_t)panel * nb * nb + lane + (size_t)nbk * lane] : mk(0, 0);
       for (int l = g + wid * G; l < q; l += nw * G) {
         cplx acc = (lane < nbk) ? cmul(tl, ws.wfin[lane + (size_t)nbk * l]) : mk(0, 0);
@@ -1034,7 +1034,7 @@ ormqr_kernel(const cplx* A, int lda, int m, int p, const cplx* Tg, int nb, cplx*
     if (grid_sync(gs)) return;
     if (MIXED)
       update_x_f<NB>(reinterpret_cast<const df2*>(P), R, r0, lo, r1, nbk, reinterpret_cast<df2*>(C), ldc, q, ws.wfin);
-    else if (R <= kFewRows)
+    else if (!KEPT && R <= kFewRows)
       update_x_few<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.wfin);
     else
       update_x<NB>(P, R, r0, lo, r1, nbk, C, ldc, q, ws.wfin);
@@ -1105,7 +1105,7 @@ cudaError_t geqrf(cplx* A, int lda, int m, int k, cplx* tau, cplx* T, int* nb_ou
 
 cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const cplx* T,
                   int nb, cplx* C, int ldc, int q, const CoopWs& ws, cudaStream_t s, int mode) {
-  const bool mixed = mode & kQrMixed;
+  const bool mixed = mode & kQrMixed, kept = mode & kQrKept;
   (void)tau;
   if (m <= 0 || p <= 0 || q <= 0) return cudaSuccess;
   int G, R, nb2;
@@ -1123,6 +1123,10 @@ cudaError_t ormqr(const cplx* A, int lda, int m, int p, const cplx* tau, const c
     if (nb == 32) fn = (void*)ormqr_kernel<32, true>;
     else if (nb == 16) fn = (void*)ormqr_kernel<16, true>;
     else fn = (void*)ormqr_kernel<8, true>;
+  } else if (kept) {
+    if (nb == 32) fn = (void*)ormqr_kernel<32, false, true>;
+    else if (nb == 16) fn = (void*)ormqr_kernel<16, false, true>;
+    else fn = (void*)ormqr_kernel<8, false, true>;
   } else {
     if (nb == 32) fn = (void*)ormqr_kernel<32, false>;
     else if (nb == 16) fn = (void*)ormqr_kernel<16, false>;

@@ -72,6 +72,28 @@ DV void op_acc(const cplx* __restrict__ cf, int n, int m, unsigned f, const cplx
   }
 }
 
+// (op x)[m] of the same taps and parts in the order of op_apply: the diagonal,
+// then the lower and the upper neighbour, imaginary parts first.
+DV cplx op_taps(const cplx* __restrict__ cf, int n, int m, unsigned f, const cplx& xl, const cplx& x0, const cplx& xu) {
+  if (f & 0x40) return x0;
+  cplx v = mk(0, 0);
+  if (f & 0x08) {
+    const cplx c = cf[n + m];
+    v = mk(-__dmul_rn(c.y, x0.y), __dmul_rn(c.y, x0.x));
+  }
+  if (f & 0x04) {
+    const cplx c = cf[n + m];
+    v = mk(fma(c.x, x0.x, v.x), fma(c.x, x0.y, v.y));
+  }
+  auto add = [&](const cplx& c, unsigned parts, const cplx& x) {
+    if (parts & 2) v = mk(fma(-c.y, x.y, v.x), fma(c.y, x.x, v.y));
+    if (parts & 1) v = mk(fma(c.x, x.x, v.x), fma(c.x, x.y, v.y));
+  };
+  if (f & 0x03) add(cf[m], f & 3, xl);
+  if (f & 0x30) add(cf[2 * n + m], (f >> 4) & 3, xu);
+  return v;
+}
+
 // ---- operator apply ------------------------------------------------------------
 // Y[(alpha, i), m, (beta, j)] = sum_m' W[alpha, beta][m, m'] X[i, m', j] with
 // every W block one of the per-mode operators: tridiagonal in (m, m'), or the
@@ -116,9 +138,7 @@ apply_cores_kernel(const cplx* const* __restrict__ in, const int* __restrict__ r
 #pragma unroll 4
     for (int m = m0; m < m1; ++m) {
       const cplx xu = m + 1 < n ? __ldg(x + (size_t)a * (m + 1)) : mk(0, 0);
-      cplx v = mk(0, 0);
-      op_acc(cf, n, m, f, xl, x0, xu, v);
-      y[(size_t)rows * m] = v;
+      y[(size_t)rows * m] = op_taps(cf, n, m, f, xl, x0, xu);
       xl = x0;
       x0 = xu;
     }

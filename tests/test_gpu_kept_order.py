@@ -1,6 +1,7 @@
-"""Mixed contexts with digit products keep their order of operations: one RK4
-step and two roundings against recorded values (tests/golden/kept_order.txt,
-hex floats; nvcc 13.0, GB300).
+"""Mixed contexts with digit products keep their order of operations: a step,
+roundings, a step from the library's own initial state and a sum with an
+applied operator against recorded values (tests/golden/kept_order.txt, hex
+floats; nvcc 13.0, GB300).
 
 The five-digit products cut at 2^-40, so a changed last bit in a factor, a
 bidiagonal or a singular vector shows in Phi at 1e-11 to 1e-10 and more in a
@@ -17,16 +18,18 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 GOLDEN = os.path.join(os.path.dirname(__file__), "golden", "kept_order.txt")
-# d, n, ranks, power-of-two decades of the bonds' weights, rounded by hand or stepped
-CASES = {"step": (4, 128, [1, 64, 64, 64, 1], 20, True),
-         "wide_factor": (3, 128, [1, 300, 64, 1], 30, False),
-         "tall_factors": (4, 128, [1, 128, 300, 128, 1], 12, False)}
+# d, n, ranks, powers of two over which the bonds' weights fall, what is done
+CASES = {"step": (4, 128, [1, 64, 64, 64, 1], 20, "step"),
+         "wide_factor": (3, 128, [1, 300, 64, 1], 30, "round"),
+         "tall_factors": (4, 128, [1, 128, 300, 128, 1], 12, "round"),
+         "init_step": (6, 32, [1, 32, 32, 32, 32, 32, 1], 0, "init"),
+         "apply_sum": (4, 128, [1, 64, 64, 64, 1], 20, "apply")}
 
 
 def read_out(name):
     """Mean, covariance and values near the centre, as one vector."""
     from paper_2403_04946_gb300 import binding as B
-    d, n, ranks, decay, step = CASES[name]
+    d, n, ranks, decay, what = CASES[name]
     rng = np.random.default_rng(5)
     cores = []
     for a, b in zip(ranks[:-1], ranks[1:]):
@@ -34,12 +37,23 @@ def read_out(name):
         # exact weights: the same input bits on every machine
         cores.append(np.asfortranarray(c * 2.0 ** -np.floor(decay * np.arange(b) / max(b - 1, 1))))
     idx = rng.integers(n // 4, 3 * n // 4, size=(12, d)).astype(np.int32)
-    ctx = B.Context(d=d, n=n, nu=0.01, tol=1e-7, rank_cap=64, L=12.4, precision=B.HOPF_MIXED)
-    t = ctx.tt_from_host(cores, max_rank=max(ranks))
-    if step:
+    cap = min(64, max(ranks))
+    ctx = B.Context(d=d, n=n, nu=0.01, tol=1e-7, rank_cap=cap, L=12.4, precision=B.HOPF_MIXED)
+    if what == "init":
+        t = ctx.hopf_init_gaussian(np.linspace(-0.125, 0.25, d), np.eye(d) * 0.5 + 0.25)
+    else:
+        t = ctx.tt_from_host(cores, max_rank=max(ranks))
+    if what == "apply":  # x + dt G x by hand
+        g, s = ctx.tt_create(6 * cap), ctx.tt_create(7 * cap)
+        ctx.hopf_apply_op(t, g)
+        ctx.tt_sum([t, g], np.array([1.0, 2.0 ** -16]), s)
+        ctx.tt_free(g)
+        ctx.tt_free(t)
+        t = s
+    if what in ("step", "init"):
         ctx.hopf_step(t, 1.2e-5, 1)
     else:
-        ctx.tt_round(t, 1e-7, 64)
+        ctx.tt_round(t, 1e-7, cap)
     mean, cov, _ = ctx.hopf_eval_moments(t)
     phi = ctx.hopf_eval_points(t, idx)
     ctx.tt_free(t)
