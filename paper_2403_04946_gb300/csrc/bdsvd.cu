@@ -74,9 +74,9 @@ DV cplx sum_published(const cplx* p, size_t stride, int G) {
   }
   return s;
 }
-// Sum over the block delivered to lanes 0 to 7 of warp 0 only (the other warps' FP64
-// work in a block-wide reduction costs more, on this GPU's narrow FP64 pipe,
-// than the column's arithmetic).  Warps whose `has` is false contribute
+// Sum over the block delivered to lanes 0 to 7 of warp 0 only (the other warps'
+// FP64 work in a block-wide reduction costs more, on this GPU's narrow FP64
+// pipe, than the column's arithmetic).  Warps whose `has` is false contribute
 // zero without reducing.  Its __syncthreads also publishes the block's
 // shared-memory writes made before it; the next use of red has to lie behind
 // another one.
