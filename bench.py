@@ -224,15 +224,14 @@ def timed_steps(ctx, t, w, steps, warmup, stream, barrier):
     return e0.elapsed_time(e1) / 1e3, prof
 
 
-# Tensor-core products of the mixed path: every complex multiply-add (8
-# FP64-equivalent FLOPs) costs 3 real products (3M) x 15 digit pairs (5
-# digits per operand) of BF16 multiply-adds, i.e. 45 real multiply-adds
-# where the FP64-equivalent count assigns 4.
-TC_DIGIT_PAIRS = 15
-TC_BF16_PER_FP64EQ = 3 * TC_DIGIT_PAIRS / 4.0
+# Tensor-core products: every complex multiply-add (8 FP64-equivalent FLOPs)
+# costs 3 real products (3M) x the digit pairs of BF16 multiply-adds, where the
+# FP64-equivalent count assigns 4: 15 pairs from 5 digits per operand on the
+# mixed path, 36 from 8 in FP64.
+TC_DIGIT_PAIRS = {True: 15, False: 36}  # mixed, FP64
 
 
-def tc_roofline(prof, peaks):
+def tc_roofline(prof, peaks, mixed):
     """The tensor-core class (digit splitting included) against the measured
     sustained BF16 peak (the products run inside a seconds-long step),
     expressed in FP64-equivalent complex FLOP/s."""
@@ -244,12 +243,13 @@ def tc_roofline(prof, peaks):
     if not bf16:
         bf16, src = 1700.0, "of fallback (1.7 PFLOP/s sustained bf16)"
     achieved = pd["flops"] / (pd["ms"] / 1e3) / 1e12
-    peak = bf16 / TC_BF16_PER_FP64EQ
+    per_flop = 3 * TC_DIGIT_PAIRS[mixed] / 4.0
+    peak = bf16 / per_flop
     return {"bound": "tensor", "kernel": "tc (tc_zgemm_kernel + digit splitting)", "achieved": achieved,
             "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "peak_source": f"{bf16:.1f} TFLOP/s bf16 {src} / {TC_BF16_PER_FP64EQ:.2f} bf16 multiply-adds "
-                           "per FP64-equivalent one (3M x 15 digit pairs / 4)",
-            "bf16_tflops_achieved": achieved * TC_BF16_PER_FP64EQ, "traffic": None}
+            "peak_source": f"{bf16:.1f} TFLOP/s bf16 {src} / {per_flop:.2f} bf16 multiply-adds "
+                           f"per FP64-equivalent one (3M x {TC_DIGIT_PAIRS[mixed]} digit pairs / 4)",
+            "bf16_tflops_achieved": achieved * per_flop, "traffic": None}
 
 
 # DRAM traffic of one 128-column mixed panel launch of geqrf_kernel, from the
@@ -278,7 +278,7 @@ def roofline(prof, mixed, peaks, tensor_qr=False):
     cls = [k for k in prof if isinstance(prof[k], dict) and prof[k].get("flops", 0) > 0 and prof[k]["ms"] > 0]
     dom = max(cls, key=lambda k: prof[k]["ms"])
     if dom == "tc":
-        return tc_roofline(prof, peaks)
+        return tc_roofline(prof, peaks, mixed)
     pd = prof[dom]
     launch_s = pd["ms"] / 1e3 / max(pd["timed_launches"], 1)
     achieved = pd["flops"] / max(pd["timed_launches"], 1) / launch_s / 1e12
@@ -653,7 +653,7 @@ def run_ours(args, rank, world, local_rank):
                       "in double-float (2 x f32); f64 Householder scalars and SVD"),
             "data": "synthetic", "config": cfg,
             "roofline": roofline(prof, True, peaks, tensor_qr=(qr_method == binding.HOPF_QR_TENSOR)),
-            "tensor_core_roofline": tc_roofline(prof, peaks),
+            "tensor_core_roofline": tc_roofline(prof, peaks, True),
             "kernel_shares": shares,
             "autotune": tune_table,
             "fp64": {"value": replica_rate(args.steps, el64, world), "unit": "steps/s", "ms_per_step": el64 / args.steps * 1e3,
