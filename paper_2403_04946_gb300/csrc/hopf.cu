@@ -65,7 +65,7 @@ struct RoundWs {
   cplx* G2 = nullptr;
   // rows of a bidiagonalisation too large for shared memory
   cplx* bd_rows = nullptr;
-  bool kept = false;          // this rounding's forms (kept_order)
+  bool kept = false;          // forms of the rounding at hand (kept_order)
 };
 
 struct hopf_ctx {
