@@ -189,13 +189,16 @@ hopf_status fail(hopf_ctx* c, hopf_status st, const char* fmt, ...) {
 // at 2^-40, so that a changed last bit anywhere before one flips digits: Phi
 // then moves by 3e-11 to 9e-11 and a covariance, a second difference of Phi, by
 // 1e-10 to 2e-9, whatever the change was.  That matters where moments are taken
-// (the CDF equation has none: its values move by up to 8e-11) and where a factor can
-// reach the products' 4096 rows: ranks go up to 6 rank_cap in a step's
-// roundings, or to the capacity of the tensor at hand.
-bool kept_order(const hopf_ctx* ctx, int cap_rank) {
+// (the CDF equation has none: its values move by up to 8e-11) and where a factor or
+// a merge can reach the products' 4096 rows: ranks go up to 6 times those of a
+// state in a step's roundings (rank_cap and what the bond's modes allow), or to
+// `rank`, the largest of the tensor at hand.
+bool kept_order(const hopf_ctx* ctx, int rank) {
   if (ctx->p.precision != HOPF_MIXED || ctx->equation != HOPF_EQ_PHI) return false;
   if (ctx->qr_method != HOPF_QR_TENSOR && !ctx->autotune) return false;
-  const long long r = std::max(6 * (long long)ctx->p.rank_cap, (long long)cap_rank);
+  long long state = 1;
+  for (int k = 0; k < ctx->p.d / 2 && state < ctx->p.rank_cap; ++k) state *= ctx->p.n;
+  const long long r = std::max(6 * std::min<long long>(ctx->p.rank_cap, state), (long long)rank);
   return r * ctx->p.n >= 4096;
 }
 
@@ -487,11 +490,12 @@ hopf_status round_buffers(hopf_ctx* ctx, const hopf_tt* t) {
   return coop_reserve(ctx, K);
 }
 
-// Workspace of a rounding of t, and the forms it takes.
-hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t) {
+// Workspace of a rounding in t of a tensor with these ranks, and the forms it
+// takes.
+hopf_status round_reserve(hopf_ctx* ctx, const hopf_tt* t, const std::vector<int>& ranks) {
   TRY(round_buffers(ctx, t));
   RoundWs& w = ctx->rw;
-  w.kept = kept_order(ctx, t->cap_rank);
+  w.kept = kept_order(ctx, *std::max_element(ranks.begin(), ranks.end()));
   if (w.kept && !w.bd_lu) CK(dalloc(&w.bd_lu, hk::bd_lu_elems(w.kcap, w.kcap)));
   return HOPF_OK;
 }
@@ -1054,7 +1058,7 @@ hopf_status phase2(hopf_ctx* ctx, hopf_tt* t, const std::vector<int>& p, const s
 
 hopf_status round_impl(hopf_ctx* ctx, hopf_tt* t, double tol, int cap, const int* forced,
                        double* disc_out, bool* capped) {
-  TRY(round_reserve(ctx, t));
+  TRY(round_reserve(ctx, t, t->ranks));
   std::vector<int> p, nbv;
   TRY(orth_sweep(ctx, t, p, nbv));
   return phase2(ctx, t, p, nbv, tol, cap, forced, disc_out, capped);
@@ -1131,7 +1135,7 @@ hopf_status round_apply_impl(hopf_ctx* ctx, const hopf_tt* X, hopf_tt* out, doub
   std::vector<int> r(X->d + 1, 1);
   for (int k = 1; k < X->d; ++k) r[k] = 6 * X->ranks[k];
   TRY(check_fit(ctx, out, r));
-  TRY(round_reserve(ctx, out));
+  TRY(round_reserve(ctx, out, r));
   std::vector<int> p, nbv;
   TRY(orth_sweep_apply(ctx, X, p, nbv));
   return phase2(ctx, out, p, nbv, tol, cap, forced, disc_out, capped);
@@ -1316,7 +1320,7 @@ hopf_status cross_sweep(hopf_ctx* ctx, CrossBufs& B, int cap, const std::vector<
       if ((size_t)M * cnt > cores->core_cap[k]) return fail(ctx, HOPF_EINVAL, "cross: core %d exceeds capacity", k);
       CK(hk::cross_gather(B.A, M, B.piv + cap, cnt, B.Q, B.W, B.seq, ctx->stream));
       int nb = 32;
-      const int mode = kept_order(ctx, cap) ? hk::kQrKept : hk::kQrFp64;
+      const int mode = kept_order(ctx, 0) ? hk::kQrKept : hk::kQrFp64;
       CK(hk::geqrf(B.Q, M, M, cnt, B.tau, B.T, &nb, ctx->coop, ctx->stream, mode));
       CK(hk::ormqr(B.Q, M, M, cnt, B.tau, B.T, nb, B.W, M, cnt, ctx->coop, ctx->stream, mode));
       TRY(check_barrier(ctx));
@@ -1866,7 +1870,7 @@ hopf_status tt_set_from_host(hopf_tt* t, const int* ranks, const double* cores) 
 
 hopf_status tt_norm(hopf_ctx* ctx, const hopf_tt* t, double* norm) {
   if (!ctx || !t || !norm) return ctx ? fail(ctx, HOPF_EINVAL, "tt_norm: null argument") : HOPF_EINVAL;
-  TRY(round_reserve(ctx, t));
+  TRY(round_reserve(ctx, t, t->ranks));
   std::vector<int> p, nbv;
   TRY(orth_sweep(ctx, t, p, nbv));
   TRY(read_small_checked(ctx, 0, 1));
