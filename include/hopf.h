@@ -80,7 +80,9 @@ typedef struct {
                   /* accumulation, and the QR panels in double-float      */
                   /* arithmetic (hopf_set_qr_method); Householder         */
                   /* scalars, the SVD that sets the ranks and all storage */
-                  /* stay FP64.                                           */
+                  /* stay FP64.  Its digits cut at 2^-40 of the largest   */
+                  /* entry of a row, and bonds are taken in the gauge     */
+                  /* they come in (after any rounding: orthonormal).      */
   int nonlinear;  /* 1: full Burgers generator; 0: drop the (i/2) D1 term */
 } hopf_params;
 
